@@ -179,10 +179,10 @@ def _arrays(tree):
 
 
 def _result(tree, precision):
-    """A result's blocks; a program that chose the tensor cores takes them on in float32, the
-    type of the accumulators they come from."""
+    """A result's blocks; a program that chose 32-bit arithmetic (in registers or in the tensor
+    cores' accumulators) takes them on in float32."""
     b = _arrays(tree)[0]
-    return b.float() if precision in TC else b
+    return b if precision == "fp64" else b.float()
 
 
 # ---------------------------------------------------------------- one pass
@@ -213,7 +213,7 @@ def run(s):
         phi, info = mra.kalos_step(s["phi"], s["potential"], s["length"], s["mu"], case["eps"], case["levels"],
                                    precision=case["precision"], screen=case["screen"], op_cache=s["cache"])
         r = np.array([info["energy"], info["mu_next"], info["norm_new"]])
-        return [_result(phi, case["precision"]), r.astype(np.float32) if case["precision"] in TC else r]
+        return [_result(phi, case["precision"]), r if case["precision"] == "fp64" else r.astype(np.float32)]
     if kind == "build":
         tree, _ = mra.build_tree(s["density"], case["k"], case["eps"], case["levels"], init_level=2)
         return list(_arrays(tree))
