@@ -293,68 +293,6 @@ static int schedule_smem_attr(int M, int lm) {
 }
 
 // ------------------------------------------------------------------ screen
-#define GH_EMPTY 0xffffffffffffffffull
-#define GH_TREE_BITS 22
-
-// level (6 bits) | tree (22 bits) | Morton key of the box (36 bits, level <= 12)
-__device__ inline uint64_t ghost_key(int j, int tree, int b1, int b2, int b3) {
-    return ((uint64_t)j << 58) | ((uint64_t)tree << 36) | morton3(b1, b2, b3);
-}
-
-__device__ inline uint32_t hash64(uint64_t k) {
-    k ^= k >> 33;
-    k *= 0xff51afd7ed558ccdull;
-    k ^= k >> 33;
-    k *= 0xc4ceb9fe1a85ec53ull;
-    k ^= k >> 33;
-    return (uint32_t)k;
-}
-
-// returns the slot (>= 0) or -1 when the probe limit is exceeded
-__device__ int ghost_insert(uint64_t* tab, uint32_t cap, uint64_t key) {
-    uint32_t h = hash64(key) & (cap - 1);
-    for (uint32_t it = 0; it < cap && it < 4096; ++it) {
-        uint64_t prev = atomicCAS((unsigned long long*)&tab[h], (unsigned long long)GH_EMPTY,
-                                  (unsigned long long)key);
-        if (prev == GH_EMPTY || prev == key) return (int)h;
-        h = (h + 1) & (cap - 1);
-    }
-    return -1;
-}
-
-__device__ int ghost_find(const uint64_t* tab, uint32_t cap, uint64_t key) {
-    uint32_t h = hash64(key) & (cap - 1);
-    for (uint32_t it = 0; it < cap && it < 4096; ++it) {
-        uint64_t v = tab[h];
-        if (v == key) return (int)h;
-        if (v == GH_EMPTY) return -1;
-        h = (h + 1) & (cap - 1);
-    }
-    return -1;
-}
-
-// The Step-2 set is keyed by the missing box's parent: slot -> parent key, an
-// 8-bit mask of the octants needed, and (after k_ghost_ids) the id of the
-// parent's first needed child.  A group's children get consecutive ids in
-// octant order, so no sort is needed to find siblings.
-struct ScreenArgs {
-    Forest F;
-    int M, sl;
-    const int32_t* sched;  // per tree: Jm | m1 | m2 | cnt
-    uint64_t* gtab;
-    uint32_t gcap;
-    uint32_t* gmask;       // slot -> octants needed (count pass)
-    const int32_t* gid;    // slot -> id of its first needed child (fill pass)
-    int32_t* count;        // per node pair count (count pass)
-    const int32_t* pair_off;
-    Pair* pairs;
-    int32_t* err;          // [0] hash overflow
-    // [n][216] (optional): the count pass's lookup per band position -- the input node,
-    // or -1 - slot of the missing box's parent in the Step-2 set -- so that the fill
-    // pass searches nothing
-    int32_t* qin;
-};
-
 // warp per output node; lane q covers band positions q, q+32, ... < 216
 template <bool FILL>
 __global__ void k_screen(ScreenArgs A) {
@@ -543,24 +481,7 @@ __global__ void k_ghost_refine(Forest F, const uint64_t* gkeys, double* gblk, in
 }
 
 
-// out = Mat along dimension `dim` of the k^3 array x (Mat k x k, out[c] = sum_i Mat[c][i] x[i]),
-// generic k (row-major k^3 arrays, one output element per thread)
-template <typename T>
-__device__ void mode_mul(int k, const T* Mat, const T* x, T* out, int dim) {
-    const int k3 = k * k * k, kk = k * k;
-    for (int idx = threadIdx.x; idx < k3; idx += blockDim.x) {
-        const int i1 = idx / kk, i2 = (idx / k) % k, i3 = idx % k;
-        const int c = dim == 0 ? i1 : (dim == 1 ? i2 : i3);
-        const int st = dim == 0 ? kk : (dim == 1 ? k : 1);
-        const T* src = x + idx - c * st;
-        T a = 0;
-        for (int i = 0; i < k; ++i) a += Mat[c * k + i] * src[i * st];
-        out[idx] = a;
-    }
-    __syncthreads();
-}
-
-// The same for k = K fixed at compile time on (K, K, K) arrays whose innermost
+// out = Mat along dimension `dim` of x (out[c] = sum_i Mat[c][i] x[i]), (K, K, K) arrays whose innermost
 // extent is padded to K + 1 (so that fibers along it, one per thread, hit
 // distinct banks), for upper-triangular Mat: the refinement matrices H^(p)T and
 // their products vanish below the diagonal (H^(p)_{ia} = 0 for a > i, since
@@ -588,6 +509,27 @@ __device__ __forceinline__ void mode_mul_tri(const T* Mat, const T* x, T* out, i
     __syncthreads();
 }
 
+// Both children of a fiber along its direction (d = 0 half of eqs. recon_even / recon_odd):
+// H^(1)_{ia} = (-1)^{i+a} H^(0)_{ia}, so with the sums s0 over the i >= a of a's parity and s1
+// over the others the children's entries a are s0 + s1 and s0 - s1: half the multiplications
+// of two products.  HT: H^(0) transposed.
+template <int K, typename T, typename TO>
+__device__ __forceinline__ void child_pair(const T* HT, const T* src, int st, TO* d0, TO* d1, int dst, bool n0, bool n1) {
+    T v[K];
+#pragma unroll
+    for (int i = 0; i < K; ++i) v[i] = src[i * st];
+#pragma unroll
+    for (int a = 0; a < K; ++a) {
+        T s0 = 0, s1 = 0;
+#pragma unroll
+        for (int i = a; i < K; i += 2) s0 += HT[a * K + i] * v[i];
+#pragma unroll
+        for (int i = a + 1; i < K; i += 2) s1 += HT[a * K + i] * v[i];
+        if (n0) d0[a * dst] = (TO)(s0 + s1);
+        if (n1) d1[a * dst] = (TO)(s0 - s1);
+    }
+}
+
 // Step 2 by sibling groups.  The children of one parent box have consecutive ids
 // (k_ghost_ids / k_ghost_keys); the block of a group's first ghost refines the
 // ancestor leaf to the parent (the path's per-direction two-scale matrices
@@ -595,13 +537,13 @@ __device__ __forceinline__ void mode_mul_tri(const T* Mat, const T* x, T* out, i
 // group, sharing the direction-3 and direction-2 partial products among the
 // children (d = 0 half of eqs. recon_even / recon_odd).
 // T = double, or float where the blocks only feed FP16 hi/lo tensor-core operands.
-// KT > 0: k fixed at compile time, padded arrays and triangular contractions.
+// k is fixed at compile time: padded arrays and triangular contractions.
 template <int KT, typename T>
 __global__ void k_ghost_refine_groups(Forest F, int ng, const uint64_t* gkeys, double* gblk, int32_t* err) {
     extern __shared__ double sm_raw[];
     T* sm = (T*)sm_raw;
-    const int k = KT ? KT : F.k, k3 = k * k * k, kk = k * k;
-    const int bs = KT ? KT * KT * (KT + 1) : k3;  // one block's footprint in shared memory
+    constexpr int k = KT, k3 = k * k * k, kk = k * k;
+    constexpr int bs = kk * (k + 1);  // one block's footprint in shared memory
     const int g0 = blockIdx.x;
     const uint64_t key0 = gkeys[g0];
     if (g0 > 0 && (gkeys[g0 - 1] >> 3) == (key0 >> 3)) return;  // not the first child of its group
@@ -611,12 +553,8 @@ __global__ void k_ghost_refine_groups(Forest F, int ng, const uint64_t* gkeys, d
     T* x = Q + 3 * kk;         // 1 block: the parent
     T* y = x + bs;             // 2 blocks: direction 3 by p3
     T* z = y + 2 * bs;         // 4 blocks: direction 2 by (p2, p3)
-    T* w = z + 4 * bs;         // 1 block
-    auto at = [&](int e) { return KT ? (e / KT) * (KT + 1) + e % KT : e; };  // element e of a block
-    auto mm = [&](const T* Mat, const T* in, T* out, int dim) {
-        if (KT) mode_mul_tri<KT ? KT : 1, T>(Mat, in, out, dim);
-        else mode_mul<T>(k, Mat, in, out, dim);
-    };
+    auto at = [&](int e) { return (e / k) * (k + 1) + e % k; };  // element e of a block
+    auto mm = [&](const T* Mat, const T* in, T* out, int dim) { mode_mul_tri<KT, T>(Mat, in, out, dim); };
     const int j = (int)(key0 >> 58);
     const int tree = (int)((key0 >> 36) & ((1ull << GH_TREE_BITS) - 1));
     const uint64_t mk = key0 & ((1ull << 36) - 1);
@@ -627,11 +565,12 @@ __global__ void k_ghost_refine_groups(Forest F, int ng, const uint64_t* gkeys, d
         int p = e / kk, r = e % kk, a = r / k, i = r % k;
         HT[e] = (T)F.filt[p * kk + i * k + a];
     }
-    __shared__ int anc, jj, gn;
+    __shared__ int anc, jj;
+    __shared__ unsigned need;  // the octants of the group's ghosts
     if (threadIdx.x == 0) {
-        int n = 1;
-        while (g0 + n < ng && n < 8 && (gkeys[g0 + n] >> 3) == (key0 >> 3)) ++n;
-        gn = n;
+        unsigned mk8 = 1u << (key0 & 7ull);
+        for (int n = 1; g0 + n < ng && n < 8 && (gkeys[g0 + n] >> 3) == (key0 >> 3); ++n) mk8 |= 1u << (gkeys[g0 + n] & 7ull);
+        need = mk8;
         anc = -1;
         for (int lv = jp; lv >= 0 && anc < 0; --lv) {
             const int sh = jp - lv;
@@ -672,16 +611,26 @@ __global__ void k_ghost_refine_groups(Forest F, int ng, const uint64_t* gkeys, d
     } else {
         __syncthreads();
     }
-    // the children: direction 3 for p3 = 0, 1; direction 2 for (p2, p3); direction 1 per child
-    mm(HT, x, y, 2);
-    mm(HT + kk, x, y + bs, 2);
-    for (int q = 0; q < 4; ++q) mm(HT + (q >> 1) * kk, y + (q & 1) * bs, z + q * bs, 1);
-    for (int g = 0; g < gn; ++g) {
-        const uint64_t cm = gkeys[g0 + g] & 7ull;  // octant (p1 p2 p3) of the child
-        const int p1 = (int)(cm >> 2) & 1, p23 = (int)(cm & 3);
-        mm(HT + p1 * kk, z + p23 * bs, w, 0);
-        for (int e = threadIdx.x; e < k3; e += blockDim.x) gblk[(size_t)(g0 + g) * k3 + e] = (double)w[at(e)];
-        __syncthreads();
+    // the children, both of a direction from one set of products (child_pair): direction 3, then
+    // 2, then 1 straight into the blocks that are needed
+    constexpr int P1 = k + 1, S0 = k * P1;
+    for (int f = threadIdx.x; f < kk; f += blockDim.x) {
+        const int at0 = (f / k) * S0 + (f % k) * P1;
+        child_pair<k, T>(HT, x + at0, 1, y + at0, y + bs + at0, 1, true, true);
+    }
+    __syncthreads();
+    for (int f = threadIdx.x; f < 2 * kk; f += blockDim.x) {
+        const int p3 = f / kk, at0 = (f % kk / k) * S0 + f % k;
+        child_pair<k, T>(HT, y + p3 * bs + at0, P1, z + p3 * bs + at0, z + (2 + p3) * bs + at0, P1, true, true);
+    }
+    __syncthreads();
+    for (int f = threadIdx.x; f < 4 * kk; f += blockDim.x) {
+        const int q = f / kk, r = f % kk;  // q = 2 p2 + p3: octants q and 4 + q
+        const bool n0 = (need >> q) & 1u, n1 = (need >> (4 + q)) & 1u;
+        if (!n0 && !n1) continue;
+        double* d0 = gblk + (size_t)(g0 + __popc(need & ((1u << q) - 1u))) * k3 + r;
+        double* d1 = gblk + (size_t)(g0 + __popc(need & ((16u << q) - 1u))) * k3 + r;
+        child_pair<k, T>(HT, z + q * bs + (r / k) * P1 + r % k, S0, d0, d1, kk, n0, n1);
     }
 }
 
@@ -783,6 +732,7 @@ __global__ void __launch_bounds__(128) k_apply_simt(ApplyArgs A) {
 void screen_release(const Alloc& A, ScreenOut* S) {
     A.put(S->dv); A.put(S->sched); A.put(S->count); A.put(S->pair_off); A.put(S->total); A.put(S->err);
     A.put(S->gtab); A.put(S->gid); A.put(S->gmask); A.put(S->gkeys); A.put(S->pairs);
+    oct_release(A, &S->oct);
     *S = ScreenOut();
 }
 
@@ -790,15 +740,20 @@ void screen_release(const Alloc& A, ScreenOut* S) {
 // host synchronisation that sizes the worklist.  The ghost hash set starts at
 // 64 slots per node; when a probe sequence reaches its limit the count pass
 // is redone with a set four times larger.
-int screen_forest(const mra_op* op, const Forest& F, int unscreened, const Alloc& A, cudaStream_t st, ScreenOut* S) {
+int screen_forest(const mra_op* op, const Forest& F, int unscreened, int what, const Alloc& A, cudaStream_t st,
+                  ScreenOut* S) {
     const int k3 = F.k * F.k * F.k, M = op->M, n = F.n;
     *S = ScreenOut();
     S->sl = M + 16 * F.lm;
     MRA_TRY(dalloc(A, &S->dv, 4 * (size_t)F.ntrees));
     MRA_TRY(dalloc(A, &S->sched, (size_t)F.ntrees * S->sl));
-    MRA_TRY(dalloc(A, &S->count, (size_t)n + 1));
-    MRA_TRY(dalloc(A, &S->pair_off, (size_t)n + 1));
-    MRA_TRY(dalloc(A, &S->total, 2));
+    const bool pairs = what & SCREEN_PAIRS, groups = what & SCREEN_GROUPS;
+    if (pairs) {
+        MRA_TRY(dalloc(A, &S->count, (size_t)n + 1));
+        MRA_TRY(dalloc(A, &S->pair_off, (size_t)n + 1));
+    }
+    if (groups) MRA_TRY(oct_alloc(F, A, &S->oct));
+    MRA_TRY(dalloc(A, &S->total, 3));
     MRA_TRY(dalloc(A, &S->err, 2));
     MRA_CK(cudaMemsetAsync(S->dv, 0, 4 * (size_t)F.ntrees * sizeof(double), st));
     MRA_CK(cudaMemsetAsync(S->err, 0, 2 * sizeof(int32_t), st));
@@ -826,32 +781,35 @@ int screen_forest(const mra_op* op, const Forest& F, int unscreened, const Alloc
     sa.count = S->count; sa.pair_off = S->pair_off; sa.pairs = nullptr; sa.err = S->err;
     // the count pass's lookups, kept for the fill pass (when they take at most 1 GiB)
     sa.qin = nullptr;
-    if ((size_t)n * 216 * sizeof(int32_t) <= ((size_t)1 << 30)) MRA_TRY(tmp.get(&sa.qin, (size_t)n * 216));
+    if (pairs && (size_t)n * 216 * sizeof(int32_t) <= ((size_t)1 << 30)) MRA_TRY(tmp.get(&sa.qin, (size_t)n * 216));
     const int sblocks = (int)std::max<long>(1, std::min<long>(num_sms() * 32, ((long)n * 32 + 255) / 256));
     // parents of missing boxes: 16 slots per node to start (a box's band has at most
     // 27 parent boxes, shared with its neighbours), regrown x4 on a probe overflow
     uint64_t cap = 1024;
     while (cap < (uint64_t)n * 16ull) cap <<= 1;
-    int32_t h[2] = {0, 0}, herr[2] = {0, 0};
+    int32_t h[3] = {0, 0, 0}, herr[2] = {0, 0};
     for (;;) {
         if (cap > (1ull << 30)) { set_error("ghost hash set overflow"); return MRA_ECUDA; }
         S->gcap = (uint32_t)cap;
         MRA_TRY(dalloc(A, &S->gtab, cap));
         MRA_TRY(dalloc(A, &S->gid, cap));
         MRA_TRY(dalloc(A, &S->gmask, cap));
-        MRA_CK(cudaMemsetAsync(S->total, 0, 2 * sizeof(int32_t), st));
+        MRA_CK(cudaMemsetAsync(S->total, 0, 3 * sizeof(int32_t), st));
         MRA_CK(cudaMemsetAsync(S->gmask, 0, cap * sizeof(uint32_t), st));
         k_fill_u64<<<1024, 256, 0, st>>>(S->gtab, cap, GH_EMPTY);
         MRA_CK_LAUNCH();
         sa.gtab = S->gtab; sa.gcap = S->gcap; sa.gid = S->gid; sa.gmask = S->gmask;
-        k_screen<false><<<sblocks, 256, 0, st>>>(sa);
-        MRA_CK_LAUNCH();
-        MRA_TRY(scan_exclusive(S->count, S->pair_off, n, S->total, st));
-        MRA_CK(cudaMemcpyAsync(S->pair_off + n, S->total, sizeof(int32_t), cudaMemcpyDeviceToDevice, st));
+        if (groups) MRA_TRY(oct_screen(sa, S->oct, S->total + 2, st));
+        if (pairs) {
+            k_screen<false><<<sblocks, 256, 0, st>>>(sa);
+            MRA_CK_LAUNCH();
+            MRA_TRY(scan_exclusive(S->count, S->pair_off, n, S->total, st));
+            MRA_CK(cudaMemcpyAsync(S->pair_off + n, S->total, sizeof(int32_t), cudaMemcpyDeviceToDevice, st));
+        }
         k_ghost_ids<<<1024, 256, 0, st>>>(S->gtab, S->gcap, S->gmask, S->gid, S->total + 1);
         MRA_CK_LAUNCH();
         // the one host synchronisation: pair and ghost counts size the worklist
-        MRA_CK(cudaMemcpyAsync(h, S->total, 2 * sizeof(int32_t), cudaMemcpyDeviceToHost, st));
+        MRA_CK(cudaMemcpyAsync(h, S->total, 3 * sizeof(int32_t), cudaMemcpyDeviceToHost, st));
         MRA_CK(cudaMemcpyAsync(herr, S->err, 2 * sizeof(int32_t), cudaMemcpyDeviceToHost, st));
         MRA_CK(cudaStreamSynchronize(st));
         if (!herr[0]) break;
@@ -862,25 +820,34 @@ int screen_forest(const mra_op* op, const Forest& F, int unscreened, const Alloc
     }
     S->npairs = h[0];
     S->nghost = h[1];
+    S->max_pieces = h[2];
     // the children's keys at their ids: siblings (children of one parent box) are consecutive
     MRA_TRY(dalloc(A, &S->gkeys, (size_t)S->nghost + 1));
     if (S->nghost > 0) {
         k_ghost_keys<<<1024, 256, 0, st>>>(S->gtab, S->gcap, S->gmask, S->gid, S->gkeys);
         MRA_CK_LAUNCH();
     }
-    MRA_TRY(dalloc(A, &S->pairs, (size_t)S->npairs + 1));
-    sa.pairs = S->pairs;
-    k_screen<true><<<sblocks, 256, 0, st>>>(sa);
-    MRA_CK_LAUNCH();
+    if (groups) MRA_TRY(oct_place_ghosts(*S, n, st));
+    if (pairs) {
+        MRA_TRY(dalloc(A, &S->pairs, (size_t)S->npairs + 1));
+        sa.pairs = S->pairs;
+        k_screen<true><<<sblocks, 256, 0, st>>>(sa);
+        MRA_CK_LAUNCH();
+    }
     return MRA_OK;
 }
 
 template <typename T>
 static int ghost_refine_launch(const Forest& F, const ScreenOut& S, double* gblk, cudaStream_t st) {
-    const int k = F.k, k3 = k * k * k;
-    const size_t gsm = (8 * (size_t)k * k + 8 * (size_t)k * k * (k + 1)) * sizeof(T);  // padded blocks
-    auto fn = k == 8 ? k_ghost_refine_groups<8, T> : (k == 6 ? k_ghost_refine_groups<6, T> :
-                                                    (k == 4 ? k_ghost_refine_groups<4, T> : k_ghost_refine_groups<0, T>));
+    const int k = F.k;
+    const size_t gsm = (8 * (size_t)k * k + 7 * (size_t)k * k * (k + 1)) * sizeof(T);  // padded blocks
+    using Fn = void (*)(Forest, int, const uint64_t*, double*, int32_t*);
+    static const Fn fns[] = {nullptr,
+                             k_ghost_refine_groups<1, T>, k_ghost_refine_groups<2, T>, k_ghost_refine_groups<3, T>,
+                             k_ghost_refine_groups<4, T>, k_ghost_refine_groups<5, T>, k_ghost_refine_groups<6, T>,
+                             k_ghost_refine_groups<7, T>, k_ghost_refine_groups<8, T>, k_ghost_refine_groups<9, T>,
+                             k_ghost_refine_groups<10, T>, k_ghost_refine_groups<11, T>, k_ghost_refine_groups<12, T>};
+    const Fn fn = fns[k];
     MRA_CK(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gsm));
     fn<<<S.nghost, 128, gsm, st>>>(F, S.nghost, S.gkeys, gblk, S.err + 1);
     MRA_CK_LAUNCH();
@@ -944,7 +911,7 @@ int apply_impl(const mra_op* op, const mra_tree* f, const mra_apply_opts* o, cud
     struct Guard {
         const Alloc& A;
         ScreenOut S;
-        void* p[4] = {nullptr, nullptr, nullptr, nullptr};
+        void* p[5] = {nullptr, nullptr, nullptr, nullptr, nullptr};
         cudaEvent_t ev[4] = {nullptr, nullptr, nullptr, nullptr};
         mra_tree* g = nullptr;
         explicit Guard(const Alloc& a) : A(a) {}
@@ -964,28 +931,34 @@ int apply_impl(const mra_op* op, const mra_tree* f, const mra_apply_opts* o, cud
     ScreenOut& S = G.S;
     const int unscreened = o ? o->unscreened : 0;
     int rc = MRA_OK;
-    MRA_TRY(screen_forest(op, F, unscreened, A, st, &S));
+    const int smode = o ? o->screen_mode : MRA_SCREEN_STATIC;
+    // the static schedule's items run by sibling groups (apply_oct.cu); a learned screen that
+    // narrows no pair is the static schedule, which the device decides
+    const bool groups = prec != MRA_PREC_TC_LADDER && !(o && (o->block_screen || o->itemwise)) && smode != MRA_SCREEN_PAIR;
+    const bool pairs = !groups || smode != MRA_SCREEN_STATIC;
+    MRA_TRY(screen_forest(op, F, unscreened, (pairs ? SCREEN_PAIRS : 0) | (groups ? SCREEN_GROUPS : 0), A, st, &S));
     MRA_CK(cudaEventRecord(ev[1], st));
     double* gblk;
     MRA_TRY(dalloc(A, &gblk, (size_t)(S.nghost + 1) * k3));
     G.p[0] = gblk;
     // per-pair term ranges: the exact screen, or the learned one judged by it
-    const int smode = o ? o->screen_mode : MRA_SCREEN_STATIC;
     // Step 2 in FP64 (a two-scale transform); MRA_PREC_TC_FAST refines in FP32 when the
     // blocks only become FP16 hi/lo operands (rounding 2^-24, below the operands' 2^-22)
     // and no screen decision reads them
     MRA_TRY(ghost_refine_forest(F, S, gblk, st, prec == MRA_PREC_TC_FAST && smode == MRA_SCREEN_STATIC));
     unsigned long long* scounts = nullptr;
+    int32_t* narrowed = nullptr;  // learned: 1 when some pair's range was narrowed
     if (smode != MRA_SCREEN_STATIC) {
         if (smode != MRA_SCREEN_PAIR && smode != MRA_SCREEN_LEARNED) {
             set_error("screen mode %d is not available", smode);
             return MRA_EINVAL;
         }
-        MRA_TRY(dalloc(A, &scounts, 2));
+        MRA_TRY(dalloc(A, &scounts, 3));
         G.p[1] = scounts;
-        MRA_CK(cudaMemsetAsync(scounts, 0, 2 * sizeof(unsigned long long), st));
+        MRA_CK(cudaMemsetAsync(scounts, 0, 3 * sizeof(unsigned long long), st));
+        if (groups) narrowed = (int32_t*)(scounts + 2);
         MRA_TRY(schedule_narrow(op, F, S, gblk, smode, o->schedule, std::max(0, o->margin), nullptr, nullptr,
-                                scounts, A, st));
+                                scounts, narrowed, A, st));
     }
     MRA_CK(cudaEventRecord(ev[2], st));
 
@@ -1010,20 +983,32 @@ int apply_impl(const mra_op* op, const mra_tree* f, const mra_apply_opts* o, cud
         aa.eta_blk = op->eps * sig / sqrt((double)n * 216.0 * M);
     }
     const bool itemwise = (o && o->itemwise) || aa.eta_blk >= 0.0;
+    if (!tc) aa.F = prec == MRA_PREC_FP64 ? (const void*)op->F : (const void*)op->F32;
+    OctArgs OP;
+    void* part = nullptr;
+    if (groups) {
+        OP = oct_args(aa, S, F);
+        OP.skip = narrowed;
+        MRA_TRY(oct_part_alloc(S, tc ? oct_slice_tc() : oct_slice_simt(), tc ? sizeof(float) : sizeof(double), k, A, &part));
+        G.p[4] = part;
+        MRA_TRY(oct_items(S, 1, narrowed, nitems, st));
+    }
+    aa.skip = narrowed;
+    aa.run_if = 1;
     if (tc) {
-        // tcgen05 FP16 hi/lo split products (apply_tc.cu); with the ladder,
+        // tcgen05 FP16 hi/lo split products (apply_oct_tc.cu, apply_tc.cu); with the ladder,
         // single FP16 products for the terms the error budget allows
         if (prec == MRA_PREC_TC_LADDER) {
             MRA_TRY(dalloc(A, &lpb, 1));
             G.p[3] = lpb;
             MRA_TRY(lp_budget(F, S, op->eps, lpb, st));
         }
-        MRA_TRY(launch_apply_tc(aa, S.nghost, op, S.err + 1, lpb, nitems + 1, o ? (unsigned)o->wait_limit : 0u,
-                                o ? (o->test_flags & MRA_TEST_WITHHOLD_MMA) : 0, st));
+        MRA_TRY(launch_apply_tc(aa, S, groups ? &OP : nullptr, part, pairs, op, S.err + 1, lpb, nitems + 1,
+                                o ? (unsigned)o->wait_limit : 0u, o ? (o->test_flags & MRA_TEST_WITHHOLD_MMA) : 0, st));
     } else if (!itemwise) {
+        if (groups) MRA_TRY(oct_launch(OP, S, prec, (double*)part, g->s, st));
         // Algorithm 3's nested sums, factorised (apply_fact.cu)
-        aa.F = prec == MRA_PREC_FP64 ? (const void*)op->F : (const void*)op->F32;
-        MRA_TRY(launch_apply_fact(aa, prec, st));
+        if (pairs) MRA_TRY(launch_apply_fact(aa, prec, st));
     } else if (prec == MRA_PREC_FP64) {
         aa.F = op->F;
         size_t smem = (size_t)k3 * sizeof(double) + (4 * (size_t)k3 + 3 * k * k) * sizeof(double);
@@ -1047,7 +1032,12 @@ int apply_impl(const mra_op* op, const mra_tree* f, const mra_apply_opts* o, cud
         MRA_CK(cudaMemcpyAsync(hv, S.dv, 3 * sizeof(double), cudaMemcpyDeviceToHost, st));
         MRA_CK(cudaMemcpyAsync(herr, S.err, 2 * sizeof(int32_t), cudaMemcpyDeviceToHost, st));
         MRA_CK(cudaStreamSynchronize(st));
-        stats->n_pairs = S.npairs;
+        unsigned long long np64 = (unsigned long long)S.npairs;
+        if (!pairs) {
+            MRA_CK(cudaMemcpyAsync(&np64, S.oct.pairs, sizeof(np64), cudaMemcpyDeviceToHost, st));
+            MRA_CK(cudaStreamSynchronize(st));
+        }
+        stats->n_pairs = (int64_t)np64;
         stats->n_items = (int64_t)ni[0];
         stats->n_items_lowp = (int64_t)ni[1];
         unsigned long long sc[2] = {0, 0};

@@ -31,6 +31,8 @@ struct ApplyArgs {
     double eta_blk;        // < 0: no per-block screen
     double* out;
     unsigned long long* n_items;  // items applied, per tree
+    const int32_t* skip = nullptr;  // run only when *skip == run_if (NULL: always)
+    int run_if = 0;
 };
 
 // tensor-core apply (apply_tc.cu)
@@ -79,6 +81,84 @@ struct Forest {
     const double* filt;          // H0, H1 (k x k each)
 };
 
+// ---- the Step-2 set and the screen's arguments
+#define GH_EMPTY 0xffffffffffffffffull
+#define GH_TREE_BITS 22
+
+// level (6 bits) | tree (22 bits) | Morton key of the box (36 bits, level <= 12)
+__device__ inline uint64_t ghost_key(int j, int tree, int b1, int b2, int b3) {
+    return ((uint64_t)j << 58) | ((uint64_t)tree << 36) | morton3(b1, b2, b3);
+}
+
+__device__ inline uint32_t hash64(uint64_t k) {
+    k ^= k >> 33;
+    k *= 0xff51afd7ed558ccdull;
+    k ^= k >> 33;
+    k *= 0xc4ceb9fe1a85ec53ull;
+    k ^= k >> 33;
+    return (uint32_t)k;
+}
+
+// returns the slot (>= 0) or -1 when the probe limit is exceeded
+__device__ inline int ghost_insert(uint64_t* tab, uint32_t cap, uint64_t key) {
+    uint32_t h = hash64(key) & (cap - 1);
+    for (uint32_t it = 0; it < cap && it < 4096; ++it) {
+        uint64_t prev = atomicCAS((unsigned long long*)&tab[h], (unsigned long long)GH_EMPTY,
+                                  (unsigned long long)key);
+        if (prev == GH_EMPTY || prev == key) return (int)h;
+        h = (h + 1) & (cap - 1);
+    }
+    return -1;
+}
+
+__device__ inline int ghost_find(const uint64_t* tab, uint32_t cap, uint64_t key) {
+    uint32_t h = hash64(key) & (cap - 1);
+    for (uint32_t it = 0; it < cap && it < 4096; ++it) {
+        uint64_t v = tab[h];
+        if (v == key) return (int)h;
+        if (v == GH_EMPTY) return -1;
+        h = (h + 1) & (cap - 1);
+    }
+    return -1;
+}
+
+// The Step-2 set is keyed by the missing box's parent: slot -> parent key, an
+// 8-bit mask of the octants needed, and (after k_ghost_ids) the id of the
+// parent's first needed child.  A group's children get consecutive ids in
+// octant order, so no sort is needed to find siblings.
+struct ScreenArgs {
+    Forest F;
+    int M, sl;
+    const int32_t* sched;  // per tree: Jm | m1 | m2 | cnt
+    uint64_t* gtab;
+    uint32_t gcap;
+    uint32_t* gmask;       // slot -> octants needed (count pass)
+    const int32_t* gid;    // slot -> id of its first needed child (fill pass)
+    int32_t* count;        // per node pair count (count pass)
+    const int32_t* pair_off;
+    Pair* pairs;
+    int32_t* err;          // [0] hash overflow
+    // [n][216] (optional): the count pass's lookup per band position -- the input node,
+    // or -1 - slot of the missing box's parent in the Step-2 set -- so that the fill
+    // pass searches nothing
+    int32_t* qin;
+};
+
+// Sibling groups of a forest (apply_oct.cu): the root of a tree alone, then its other nodes
+// by eights in node order.
+struct OctGroups {
+    int n = 0;
+    int32_t* first = nullptr;            // [n] first output node
+    int32_t* in = nullptr;               // [n][216] input blocks (node, or node count + Step-2 id; -1 none)
+    int32_t* np = nullptr;               // [n] pieces
+    unsigned long long* pairs = nullptr; // [ntrees] static pairs and items
+    unsigned long long* items = nullptr;
+};
+
+// what a screen leaves: pair lists per output node, sibling groups, or both
+#define SCREEN_PAIRS 1
+#define SCREEN_GROUPS 2
+
 // device results of the screen over a forest (screen_forest in apply.cu)
 struct ScreenOut {
     double* dv = nullptr;         // [ntrees][4]: ||f_b||^2, sigma_b, eta_b, unused
@@ -86,7 +166,7 @@ struct ScreenOut {
     int sl = 0;
     int32_t* count = nullptr;     // [n + 1] pairs per output node
     int32_t* pair_off = nullptr;  // [n + 1]
-    int32_t* total = nullptr;     // [2]: pairs, Step-2 blocks
+    int32_t* total = nullptr;     // [3]: pairs, Step-2 blocks, most pieces of a group
     int32_t* err = nullptr;       // [0] screen, [1] Step 2 / apply
     uint64_t* gtab = nullptr;     // Step-2 set: parent keys of the missing boxes
     int32_t* gid = nullptr;       // slot -> id of its first needed child
@@ -94,10 +174,54 @@ struct ScreenOut {
     uint64_t* gkeys = nullptr;    // [nghost] level | tree | Morton key of each child, by id
     uint32_t gcap = 0;
     Pair* pairs = nullptr;        // [npairs], out and in are forest node indices
-    int npairs = 0, nghost = 0;
+    int npairs = 0, nghost = 0, max_pieces = 0;
+    OctGroups oct;
 };
 
-int screen_forest(const mra_op* op, const Forest& F, int unscreened, const Alloc& A, cudaStream_t st, ScreenOut* S);
+// the sibling-group apply (apply_oct.cu)
+struct OctArgs {
+    int k, M, lm, sl, n;   // n: node blocks (Step-2 blocks follow them)
+    int g0 = 0, ns = 1;    // first group of the launch, slices per group
+    const int32_t *first, *in, *np;
+    const int32_t *coord, *leaf, *node_tree, *sched;
+    const double *s, *gblk;
+    const void* F;
+    const double* w;
+    double* part = nullptr;
+    const int32_t* skip = nullptr;  // run only when *skip == run_if (NULL: always)
+    int run_if = 0;
+};
+
+// tensor-core apply by sibling groups (apply_oct_tc.cu)
+struct OctTcArgs {
+    OctArgs P;
+    const __half *xh, *xl, *Fh, *Fl;   // as in TcArgs
+    const float *sx, *xmax, *sF, *maxF;
+    int* err;
+    unsigned wait_limit;
+    int withhold;
+    int* counter;
+    void* part;
+    int nunits;
+};
+
+int oct_alloc(const Forest& F, const Alloc& A, OctGroups* O);
+void oct_release(const Alloc& A, OctGroups* O);
+int oct_screen(const ScreenArgs& sa, const OctGroups& O, int32_t* max_pieces, cudaStream_t st);
+int oct_place_ghosts(const ScreenOut& S, int n, cudaStream_t st);
+int oct_items(const ScreenOut& S, int ntrees, const int32_t* skip, unsigned long long* n_items, cudaStream_t st);
+OctArgs oct_args(const ApplyArgs& A, const ScreenOut& S, const Forest& F);
+int oct_slice_simt();
+int oct_part_alloc(const ScreenOut& S, int slice, size_t elem, int k, const Alloc& A, void** part);
+int oct_part_groups(const ScreenOut& S, int slice, size_t elem, int k);
+int oct_reduce(const OctArgs& P, int slice, int ng, const float* part, double* out, cudaStream_t st);
+int oct_tc_configure();
+int oct_slice_tc();
+int oct_tc_launch(OctTcArgs Q, const ScreenOut& S, void* part, double* out, cudaStream_t st);
+int oct_launch(const OctArgs& P, const ScreenOut& S, int precision, double* part, double* out, cudaStream_t st);
+
+int screen_forest(const mra_op* op, const Forest& F, int unscreened, int what, const Alloc& A, cudaStream_t st,
+                  ScreenOut* S);
 void screen_release(const Alloc& A, ScreenOut* S);
 // Step 2 for every missing input block of a forest; fp32: refine in FP32 (for blocks that
 // only feed FP16 hi/lo tensor-core operands), else FP64
@@ -115,12 +239,15 @@ int tc3_configure();                               // apply_tc3.cu
 int tc3_launch(const TcArgs& T, cudaStream_t st);  // counter zeroed by the caller
 
 int launch_apply_fact(const ApplyArgs& A, int precision, cudaStream_t st);
-int launch_apply_tc(const ApplyArgs& A, int nghost, const mra_op* op, int* err, const double* lpb,
-                    unsigned long long* n_lowp, unsigned wait_limit, int withhold, cudaStream_t st);
+OctTcArgs oct_tc_args(const OctArgs& P, const TcBuffers& B, int* err);
+// OP: the sibling groups (with their partial sums `part`) and / or the pair lists
+int launch_apply_tc(const ApplyArgs& A, const ScreenOut& S, const OctArgs* OP, void* part, bool pairs,
+                    const mra_op* op, int* err, const double* lpb, unsigned long long* n_lowp, unsigned wait_limit,
+                    int withhold, cudaStream_t st);
 int lp_budget(const Forest& F, const ScreenOut& S, double eps, double* lpb, cudaStream_t st);
 int schedule_narrow(const mra_op* op, const Forest& F, const ScreenOut& S, const double* gblk, int mode,
                     const void* model, int margin, float* X_out, float* T_out, unsigned long long* counts,
-                    const Alloc& A, cudaStream_t st);
+                    int32_t* narrowed, const Alloc& A, cudaStream_t st);
 int screen_data_impl(const mra_op* op, const mra_tree* f, float* X, float* T, cudaStream_t st);
 
 }  // namespace mra

@@ -36,6 +36,7 @@ __global__ void __launch_bounds__(NT) k_apply_fact(ApplyArgs A) {
     unsigned char* msk = (unsigned char*)(tfl + 216);  // 36 * MC
     __shared__ int s_mlo, s_mhi, s_anyv[MC];
     __shared__ unsigned long long s_items;
+    if (A.skip && *A.skip != A.run_if) return;
 
     const int tid = threadIdx.x;
     const T* Ftab = (const T*)A.F;

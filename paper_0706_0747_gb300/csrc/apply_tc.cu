@@ -199,6 +199,7 @@ __global__ void __launch_bounds__(TC_THREADS, MC == 4 ? 4 : 3) k_apply_tc(TcArgs
     __shared__ unsigned long long s_lowi;
 
     const ApplyArgs& A = T.A;
+    if (A.skip && *A.skip != A.run_if) return;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int kr = T.kr;
     __half* B1H = (__half*)(sm + L::B1H);
@@ -855,8 +856,23 @@ TcArgs tc_args(const ApplyArgs& A, const TcBuffers& B, int* err) {
     return T;
 }
 
-int launch_apply_tc(const ApplyArgs& A, int nghost, const mra_op* op, int* err, const double* lpb,
-                    unsigned long long* n_lowp, unsigned wait_limit, int withhold, cudaStream_t st) {
+OctTcArgs oct_tc_args(const OctArgs& P, const TcBuffers& B, int* err) {
+    OctTcArgs Q;
+    Q.P = P;
+    Q.xh = B.xh; Q.xl = B.xl; Q.sx = B.sx; Q.xmax = B.xmax;
+    Q.Fh = B.Fh; Q.Fl = B.Fl; Q.sF = B.sF; Q.maxF = B.maxF;
+    Q.err = err;
+    Q.wait_limit = 0;
+    Q.withhold = 0;
+    Q.counter = B.counter;
+    Q.part = nullptr;
+    Q.nunits = 0;
+    return Q;
+}
+
+int launch_apply_tc(const ApplyArgs& A, const ScreenOut& S, const OctArgs* OP, void* part, bool pairs,
+                    const mra_op* op, int* err, const double* lpb, unsigned long long* n_lowp, unsigned wait_limit,
+                    int withhold, cudaStream_t st) {
     if (A.k > 8) {
         set_error("the tensor-core apply supports k <= 8 (got k = %d)", A.k);
         return MRA_EINVAL;
@@ -867,9 +883,18 @@ int launch_apply_tc(const ApplyArgs& A, int nghost, const mra_op* op, int* err, 
         TcBuffers B;
         ~Guard() { tc_release(op, &B); }
     } G{op, TcBuffers()};
-    MRA_TRY(tc_alloc(op, A.n + nghost, &G.B));
+    const int nb = A.n + S.nghost;
+    MRA_TRY(tc_alloc(op, nb, &G.B));
     MRA_TRY(tc_prep_F(op, G.B, st));
-    MRA_TRY(tc_prep_blocks(A.n + nghost, A.k, A.n, A.s, A.gblk, G.B, st));
+    MRA_TRY(tc_prep_blocks(nb, A.k, A.n, A.s, A.gblk, G.B, st));
+    if (OP) {
+        MRA_TRY(oct_tc_configure());
+        OctTcArgs Q = oct_tc_args(*OP, G.B, err);
+        Q.wait_limit = wait_limit;
+        Q.withhold = withhold;
+        MRA_TRY(oct_tc_launch(Q, S, part, A.out, st));
+    }
+    if (!pairs) return MRA_OK;
     MRA_TRY(tc_configure());
     TcArgs T = tc_args(A, G.B, err);
     T.lpb = lpb;

@@ -79,6 +79,7 @@ __global__ void __launch_bounds__(TC3_THREADS, 2) k_apply_tc3(TcArgs T) {
     __shared__ unsigned long long s_lowi;
 
     const ApplyArgs& A = T.A;
+    if (A.skip && *A.skip != A.run_if) return;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int kr = T.kr;
     __half* B1H = (__half*)(sm + L::B1H);

@@ -1,0 +1,104 @@
+// The pieces of a sibling group's schedule (see apply_oct.cu).
+#pragma once
+#include "apply_common.cuh"
+
+namespace mra {
+
+// ------------------------------------------------------------------ pieces
+// The classes {S : bit S of A set} of `dims` directions as products of per-direction sets
+// (1 core, 2 off, 3 both), two bits per direction from direction 1 at the top.
+struct PieceSet {
+    int n;
+    uint8_t box[4];
+};
+
+constexpr void piece_split(int dims, int A, int prefix, PieceSet& P) {
+    if (A == 0) return;
+    if (A == (1 << (dims + 1)) - 1) {  // every class: all translations of the rest
+        int b = prefix;
+        for (int d = 0; d < dims; ++d) b = (b << 2) | 3;
+        P.box[P.n++] = (uint8_t)b;
+        return;
+    }
+    const int in = A >> 1, off = A & ((1 << dims) - 1);  // classes left with this direction core / off core
+    if (in == off) {
+        piece_split(dims - 1, in, (prefix << 2) | 3, P);
+        return;
+    }
+    piece_split(dims - 1, in, (prefix << 2) | 1, P);
+    piece_split(dims - 1, off, (prefix << 2) | 2, P);
+}
+
+struct PieceTable {
+    PieceSet p[16];
+};
+
+constexpr PieceTable make_pieces() {
+    PieceTable T{};
+    for (int A = 0; A < 16; ++A) piece_split(3, A, 0, T.p[A]);
+    return T;
+}
+
+static __constant__ PieceTable c_pieces = make_pieces();
+
+#define PIECE_CCC 0x15  // core in every direction
+
+// The pieces of a group at level j, by one warp: non-core pieces first, then the core
+// ones, each in increasing m.  out[i] = m | box << 16 | leaf_only << 24 (NULL: count only).
+static __device__ int oct_pieces(const int32_t* sched, int M, int lm, int j, bool any_leaf, bool any_int, uint32_t* out) {
+    const int lane = threadIdx.x & 31;
+    const int32_t* m1 = sched + M + 4 * j;
+    const int32_t* m2 = sched + M + 4 * lm + 4 * j;
+    int lo[4], hi[4], first = M, last = -1;
+    for (int S = 0; S < 4; ++S) {
+        lo[S] = m1[S];
+        hi[S] = m2[S];
+        if (hi[S] >= lo[S]) {
+            first = min(first, lo[S]);
+            last = max(last, hi[S]);
+        }
+    }
+    int total = 0;
+    for (int pass = 0; pass < 2; ++pass)
+        for (int m0 = first; m0 <= last; m0 += 32) {
+            const int m = m0 + lane;
+            int A = 0;
+            bool extra = false;  // the core for the leaf outputs only
+            if (m <= last) {
+                const int jm = sched[m];
+                if (jm >= j) {
+                    for (int S = 0; S < 4; ++S) A |= (m >= lo[S] && m <= hi[S]) << S;
+                    if (jm > j && any_int && (A & 8)) {
+                        A &= 7;
+                        extra = any_leaf;
+                    }
+                }
+            }
+            const PieceSet& P = c_pieces.p[A];
+            int n = 0;
+            for (int i = 0; i < P.n; ++i) n += (P.box[i] == PIECE_CCC) == (pass == 1);
+            n += pass == 1 && extra;
+            int at = n;
+            for (int o = 1; o < 32; o <<= 1) {
+                const int v = __shfl_up_sync(0xffffffffu, at, o);
+                if (lane >= o) at += v;
+            }
+            const int sum = __shfl_sync(0xffffffffu, at, 31);
+            if (out) {
+                at += total - n;
+                for (int i = 0; i < P.n; ++i)
+                    if ((P.box[i] == PIECE_CCC) == (pass == 1)) out[at++] = (uint32_t)m | ((uint32_t)P.box[i] << 16);
+                if (pass == 1 && extra) out[at++] = (uint32_t)m | ((uint32_t)PIECE_CCC << 16) | (1u << 24);
+            }
+            total += sum;
+        }
+    return total;
+}
+
+// whether input b lies in the core of output a in a direction
+__device__ inline bool band_core(int a, int b) { return b >= 1 + a && b <= 3 + a; }
+
+// boxes b of a direction that some a in {0, 1} reaches by a translation of the set
+__device__ __forceinline__ unsigned set_boxes(int set) { return set == 1 ? 0x1eu : (set == 2 ? 0x33u : 0x3fu); }
+
+}  // namespace mra

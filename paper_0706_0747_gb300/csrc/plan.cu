@@ -87,6 +87,11 @@ struct mra_plan {
     unsigned long long* nitems = nullptr;  // per tree, then the single-FP16 items of all trees
     double* lpb = nullptr;                 // precision-ladder budgets per tree
     bool tc = false;
+    // Step 3 by sibling groups (apply_oct.cu), by the pair lists, or (learned screen) by the one
+    // that `narrowed` on the device asks for
+    bool groups = false, pairs = true;
+    void* part = nullptr;
+    int32_t* narrowed = nullptr;
     mra::TcBuffers tcb;
     int32_t* order_heavy = nullptr;
     // apply variant
@@ -117,12 +122,22 @@ static int plan_apply_args(const mra_plan* p, ApplyArgs* aa) {
     aa->Jm = p->S.sched; aa->node_tree = p->node_tree; aa->jm_stride = p->S.sl;
     aa->eta_blk = -1.0; aa->out = p->out; aa->n_items = p->nitems;
     aa->F = p->precision == MRA_PREC_FP64 ? (const void*)op->F : (const void*)op->F32;
+    aa->skip = p->narrowed;
+    aa->run_if = 1;
     return MRA_OK;
 }
 
+// the sibling-group apply where the plan has one (the variant does not concern it), and the
+// pair-list kernel of the variant
 static int plan_tc_launch(const mra_plan* p, int mc, int ctas, int ordered, cudaStream_t st) {
     ApplyArgs aa;
     plan_apply_args(p, &aa);
+    if (p->groups) {
+        OctArgs P = oct_args(aa, p->S, p->F);
+        P.skip = p->narrowed;
+        MRA_TRY(oct_tc_launch(oct_tc_args(P, p->tcb, p->S.err + 1), p->S, p->part, p->out, st));
+    }
+    if (!p->pairs) return MRA_OK;
     TcArgs T = tc_args(aa, p->tcb, p->S.err + 1);
     T.order = ordered ? p->order_heavy : nullptr;
     T.lpb = p->lpb;
@@ -140,13 +155,19 @@ static int plan_enqueue(const mra_plan* p, cudaStream_t st) {
     MRA_TRY(ghost_refine_forest(p->F, p->S, p->gblk, st,
                                 p->precision == MRA_PREC_TC_FAST && p->screen_mode == MRA_SCREEN_STATIC));
     MRA_CK(cudaMemsetAsync(p->nitems, 0, ((size_t)p->ntrees + 1) * sizeof(unsigned long long), st));
+    if (p->groups) MRA_TRY(oct_items(p->S, p->ntrees, p->narrowed, p->nitems, st));
     if (p->tc) {
         MRA_TRY(tc_prep_blocks(p->n + p->S.nghost, p->k, p->n, p->s, p->gblk, p->tcb, st));
         MRA_TRY(plan_tc_launch(p, p->mc, p->ctas, p->use_order, st));
     } else {
         ApplyArgs aa;
         plan_apply_args(p, &aa);
-        MRA_TRY(launch_apply_fact(aa, p->precision, st));
+        if (p->groups) {
+            OctArgs P = oct_args(aa, p->S, p->F);
+            P.skip = p->narrowed;
+            MRA_TRY(oct_launch(P, p->S, p->precision, (double*)p->part, p->out, st));
+        }
+        if (p->pairs) MRA_TRY(launch_apply_fact(aa, p->precision, st));
     }
     return MRA_OK;
 }
@@ -167,7 +188,7 @@ static void plan_release(mra_plan* p) {
     if (p->op) tc_release(p->op, &p->tcb);
     A.put(p->tref); A.put(p->dbase); A.put(p->coord); A.put(p->leaf); A.put(p->off); A.put(p->node_tree);
     A.put(p->nlev); A.put(p->key); A.put(p->s); A.put(p->gblk); A.put(p->out); A.put(p->nitems);
-    A.put(p->order_heavy); A.put(p->lpb);
+    A.put(p->order_heavy); A.put(p->lpb); A.put(p->part); A.put(p->narrowed);
     p->magic = 0;
     delete p;
 }
@@ -220,7 +241,9 @@ static int plan_build(mra_plan* p, cudaStream_t st) {
     MRA_CK(cudaEventCreate(&ev.e[0]));
     MRA_CK(cudaEventCreate(&ev.e[1]));
     MRA_CK(cudaEventRecord(ev.e[0], st));
-    MRA_TRY(screen_forest(op, F, 0, A, st, &p->S));
+    p->groups = p->precision != MRA_PREC_TC_LADDER && p->screen_mode != MRA_SCREEN_PAIR;
+    p->pairs = !p->groups || p->screen_mode != MRA_SCREEN_STATIC;
+    MRA_TRY(screen_forest(op, F, 0, (p->pairs ? SCREEN_PAIRS : 0) | (p->groups ? SCREEN_GROUPS : 0), A, st, &p->S));
     MRA_CK(cudaEventRecord(ev.e[1], st));
     MRA_CK(cudaEventSynchronize(ev.e[1]));
     cudaEventElapsedTime(&p->ms_screen, ev.e[0], ev.e[1]);
@@ -234,8 +257,12 @@ static int plan_build(mra_plan* p, cudaStream_t st) {
         MRA_TRY(tmp.get(&counts, 2));
         MRA_CK(cudaMemsetAsync(counts, 0, 2 * sizeof(unsigned long long), st));
         MRA_TRY(ghost_refine_forest(F, p->S, p->gblk, st));
+        if (p->groups) {
+            MRA_TRY(dalloc(A, &p->narrowed, 1));
+            MRA_CK(cudaMemsetAsync(p->narrowed, 0, sizeof(int32_t), st));
+        }
         MRA_TRY(schedule_narrow(op, F, p->S, p->gblk, p->screen_mode == MRA_SCREEN_PAIR ? 1 : 2, p->schedule,
-                                p->margin, nullptr, nullptr, counts, A, st));
+                                p->margin, nullptr, nullptr, counts, p->narrowed, A, st));
         unsigned long long hc[2] = {0, 0};
         MRA_CK(cudaMemcpyAsync(hc, counts, sizeof(hc), cudaMemcpyDeviceToHost, st));
         MRA_CK(cudaStreamSynchronize(st));
@@ -251,20 +278,27 @@ static int plan_build(mra_plan* p, cudaStream_t st) {
     }
 
     // heaviest-first node order: counting sort of the per-node pair counts
-    std::vector<int32_t> cnt(n), order(n);
-    MRA_CK(cudaMemcpyAsync(cnt.data(), p->S.count, n * sizeof(int32_t), cudaMemcpyDeviceToHost, st));
-    MRA_CK(cudaStreamSynchronize(st));
-    std::vector<int32_t> start(218, 0);
-    for (int i = 0; i < n; ++i) start[216 - std::min(216, std::max(0, cnt[i])) + 1]++;
-    for (int c = 1; c < 218; ++c) start[c] += start[c - 1];
-    for (int i = 0; i < n; ++i) order[start[216 - std::min(216, std::max(0, cnt[i]))]++] = i;
-    MRA_TRY(dalloc(A, &p->order_heavy, n));
-    MRA_CK(cudaMemcpyAsync(p->order_heavy, order.data(), n * sizeof(int32_t), cudaMemcpyHostToDevice, st));
+    if (p->pairs) {
+        std::vector<int32_t> cnt(n), order(n);
+        MRA_CK(cudaMemcpyAsync(cnt.data(), p->S.count, n * sizeof(int32_t), cudaMemcpyDeviceToHost, st));
+        MRA_CK(cudaStreamSynchronize(st));
+        std::vector<int32_t> start(218, 0);
+        for (int i = 0; i < n; ++i) start[216 - std::min(216, std::max(0, cnt[i])) + 1]++;
+        for (int c = 1; c < 218; ++c) start[c] += start[c - 1];
+        for (int i = 0; i < n; ++i) order[start[216 - std::min(216, std::max(0, cnt[i]))]++] = i;
+        MRA_TRY(dalloc(A, &p->order_heavy, n));
+        MRA_CK(cudaMemcpyAsync(p->order_heavy, order.data(), n * sizeof(int32_t), cudaMemcpyHostToDevice, st));
+        MRA_CK(cudaStreamSynchronize(st));  // `order` goes out of scope
+    }
+    if (p->groups)
+        MRA_TRY(oct_part_alloc(p->S, p->tc ? oct_slice_tc() : oct_slice_simt(), p->tc ? sizeof(float) : sizeof(double),
+                               p->k, A, &p->part));
 
     if (p->tc) {
         MRA_TRY(tc_alloc(op, n + p->S.nghost, &p->tcb));
         MRA_TRY(tc_prep_F(op, p->tcb, st));
         MRA_TRY(tc_configure());
+        MRA_TRY(oct_tc_configure());
     }
     MRA_CK(cudaStreamCreateWithFlags(&p->cap, cudaStreamNonBlocking));
     MRA_CK(cudaStreamSynchronize(st));  // host vectors above are read by the copies
@@ -467,6 +501,12 @@ int mra_plan_get_info(const mra_plan* p, mra_plan_info* info, void* stream) {
     info->n_trees = p->ntrees;
     info->n_nodes = p->n;
     info->n_pairs = p->S.npairs;
+    if (!p->pairs) {
+        std::vector<unsigned long long> np(p->ntrees);
+        MRA_CK(cudaMemcpyAsync(np.data(), p->S.oct.pairs, p->ntrees * sizeof(unsigned long long), cudaMemcpyDeviceToHost, st));
+        MRA_CK(cudaStreamSynchronize(st));
+        for (unsigned long long v : np) info->n_pairs += (int64_t)v;
+    }
     info->n_ghosts = p->S.nghost;
     for (int b = 0; b < p->ntrees; ++b) info->n_items += (int64_t)ni[b];
     info->n_items_lowp = (int64_t)ni[p->ntrees];
@@ -494,14 +534,19 @@ int mra_plan_tree_stats(const mra_plan* p, int b, void* stream, mra_apply_stats*
     cudaStream_t s = (cudaStream_t)stream;
     double dv[3];
     unsigned long long ni = 0;
-    int32_t po[2];
+    int32_t po[2] = {0, 0};
+    unsigned long long np64 = 0;
     MRA_CK(cudaMemcpyAsync(dv, p->S.dv + 4 * (size_t)b, 3 * sizeof(double), cudaMemcpyDeviceToHost, s));
     MRA_CK(cudaMemcpyAsync(&ni, p->nitems + b, sizeof(ni), cudaMemcpyDeviceToHost, s));
-    MRA_CK(cudaMemcpyAsync(&po[0], p->S.pair_off + p->base[b], sizeof(int32_t), cudaMemcpyDeviceToHost, s));
-    MRA_CK(cudaMemcpyAsync(&po[1], p->S.pair_off + p->base[b + 1], sizeof(int32_t), cudaMemcpyDeviceToHost, s));
+    if (p->pairs) {
+        MRA_CK(cudaMemcpyAsync(&po[0], p->S.pair_off + p->base[b], sizeof(int32_t), cudaMemcpyDeviceToHost, s));
+        MRA_CK(cudaMemcpyAsync(&po[1], p->S.pair_off + p->base[b + 1], sizeof(int32_t), cudaMemcpyDeviceToHost, s));
+    } else {
+        MRA_CK(cudaMemcpyAsync(&np64, p->S.oct.pairs + b, sizeof(np64), cudaMemcpyDeviceToHost, s));
+    }
     MRA_CK(cudaStreamSynchronize(s));
     memset(st, 0, sizeof(*st));
-    st->n_pairs = po[1] - po[0];
+    st->n_pairs = p->pairs ? po[1] - po[0] : (int64_t)np64;
     st->n_items = (int64_t)ni;
     st->n_ghosts = -1;  // Step-2 blocks are counted for the whole batch (mra_plan_get_info)
     st->n_out_nodes = p->base[b + 1] - p->base[b];

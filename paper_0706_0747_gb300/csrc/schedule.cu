@@ -200,6 +200,7 @@ struct RangeArgs {
     const double* rmq;            // range-maximum tables (rmq_L levels)
     int rmq_L;
     const int32_t* runs;          // [ntrees][lm][2] candidate-term runs (k_term_runs)
+    int32_t* narrowed;            // set to 1 when a range differs from the static one (NULL: not kept)
 };
 
 // thread per pair: narrow its term range in place
@@ -315,6 +316,7 @@ __global__ void k_pair_ranges(RangeArgs R) {
         hi = -1;
         if (R.counts) atomicAdd(&R.counts[1], 1ull);
     }
+    if (R.narrowed && (lo != p.m_lo || hi != p.m_hi)) *R.narrowed = 1;
     p.m_lo = (int16_t)lo;
     p.m_hi = (int16_t)hi;
     R.pairs[i] = p;
@@ -348,7 +350,7 @@ __global__ void k_fill_i32v(int32_t* p, int n, int32_t v) {
 // exact screen's targets.  counts (device, 2): misses, empty pairs.
 int schedule_narrow(const mra_op* op, const Forest& F, const ScreenOut& S, const double* gblk, int mode,
                     const void* model, int margin, float* X_out, float* T_out, unsigned long long* counts,
-                    const Alloc& A, cudaStream_t st) {
+                    int32_t* narrowed, const Alloc& A, cudaStream_t st) {
     const int k3 = F.k * F.k * F.k, n = F.n, nb = n + S.nghost;
     const mra_mlp* M = nullptr;
     if (mode == 2) {
@@ -394,7 +396,7 @@ int schedule_narrow(const mra_op* op, const Forest& F, const ScreenOut& S, const
     R.F = F; R.M = op->M; R.sl = S.sl; R.npairs = S.npairs; R.margin = margin;
     R.pairs = S.pairs; R.sched = S.sched; R.w = op->w; R.nF = op->nF; R.bn = bn; R.etab = etab;
     R.pred = Y; R.tlo = tlo; R.thi = thi; R.counts = counts;
-    R.rmq = rmq; R.rmq_L = op->rmq_L; R.runs = runs;
+    R.rmq = rmq; R.rmq_L = op->rmq_L; R.runs = runs; R.narrowed = narrowed;
     if (S.npairs > 0) {
         k_pair_ranges<<<(S.npairs + 255) / 256, 256, 0, st>>>(R);
         MRA_CK_LAUNCH();
@@ -415,11 +417,11 @@ int screen_data_impl(const mra_op* op, const mra_tree* f, float* X, float* T, cu
     const Forest F = forest_of_tree(f);
     ScreenOut S;
     Scratch tmp(A);
-    int rc = screen_forest(op, F, 0, A, st, &S);
+    int rc = screen_forest(op, F, 0, SCREEN_PAIRS, A, st, &S);
     double* gblk = nullptr;
     if (rc == MRA_OK) rc = tmp.get(&gblk, (size_t)(S.nghost + 1) * k3);
     if (rc == MRA_OK) rc = ghost_refine_forest(F, S, gblk, st);
-    if (rc == MRA_OK) rc = schedule_narrow(op, F, S, gblk, 1, nullptr, 0, X, T, nullptr, A, st);
+    if (rc == MRA_OK) rc = schedule_narrow(op, F, S, gblk, 1, nullptr, 0, X, T, nullptr, nullptr, A, st);
     if (rc == MRA_OK) {
         int32_t herr[2] = {0, 0};
         cudaError_t e = cudaMemcpyAsync(herr, S.err, 2 * sizeof(int32_t), cudaMemcpyDeviceToHost, st);

@@ -133,6 +133,48 @@ __device__ __forceinline__ void tmem_ld16x256_rep<4>(uint32_t taddr, float (*v)[
     for (int q = 0; q < 16; ++q) v[q >> 2][q & 3] = __uint_as_float(r[q]);
 }
 
+// 32 lanes x 16 consecutive 32-bit columns: lane l of the warp gets its TMEM lane's values
+__device__ __forceinline__ void tmem_ld32x16(uint32_t taddr, float* v) {
+    uint32_t r[16];
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+        : "r"(taddr));
+    asm volatile("tcgen05.wait::ld.sync.aligned;"
+                 : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]),
+                   "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15])
+                 :
+                 : "memory");
+#pragma unroll
+    for (int q = 0; q < 16; ++q) v[q] = __uint_as_float(r[q]);
+}
+
+// one arrival of the calling thread
+__device__ __forceinline__ void mbar_arrive(uint64_t* mbar) {
+    asm volatile("{\n.reg .b64 t;\nmbarrier.arrive.shared::cta.b64 t, [%0];\n}\n" ::"r"(smem_u32(mbar)) : "memory");
+}
+
+// As mbar_wait, but also gives up once *abort (shared memory) is set by another waiter;
+// a wait that reaches its limit sets it.
+__device__ __forceinline__ bool mbar_wait_or(uint64_t* mbar, uint32_t phase, uint32_t limit, volatile int* abort) {
+    for (uint32_t it = 0; it < limit; ++it) {
+        uint32_t done;
+        asm volatile(
+            "{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}\n"
+            : "=r"(done)
+            : "r"(smem_u32(mbar)), "r"(phase)
+            : "memory");
+        if (done) return true;
+        if ((it & 15) == 15) {
+            if (*abort) return false;
+            __nanosleep(TC_POLL_NS);
+        }
+    }
+    *abort = 1;
+    return false;
+}
+
 // 16-byte asynchronous global -> shared copies (completion by wait_all)
 __device__ __forceinline__ void cp_async16(void* smem_dst, const void* gsrc) {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(smem_dst)), "l"(gsrc) : "memory");
