@@ -69,25 +69,6 @@ __device__ void mode_product(const double* in, double* out, const double* Mat, i
     __syncthreads();
 }
 
-// In-place 2k-point transform along one direction of a (2k)^3 cube:
-// line <- M line (transpose = 0) or M^T line (transpose = 1), M = 2k x 2k.
-__device__ void cube_transform(double* cube, int n2, const double* Mt, int transpose, int dim) {
-    const int lines = n2 * n2;
-    const int stride = dim == 0 ? n2 * n2 : (dim == 1 ? n2 : 1);
-    for (int ln = threadIdx.x; ln < lines; ln += blockDim.x) {
-        int u = ln / n2, v = ln % n2;
-        int base = dim == 0 ? (u * n2 + v) : (dim == 1 ? (u * n2 * n2 + v) : (u * n2 * n2 + v * n2));
-        double x[2 * MRA_MAX_K];
-        for (int c = 0; c < n2; ++c) x[c] = cube[base + c * stride];
-        for (int r = 0; r < n2; ++r) {
-            double acc = 0.0;
-            for (int c = 0; c < n2; ++c) acc += (transpose ? Mt[c * n2 + r] : Mt[r * n2 + c]) * x[c];
-            cube[base + r * stride] = acc;
-        }
-    }
-    __syncthreads();
-}
-
 __device__ double block_sum(double v, double* red) {
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     const int w = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
@@ -574,68 +555,6 @@ int build_tree_impl(const mra_density* f, int k, double eps, int max_level, int 
 }
 
 // ------------------------------------------------------------ two-scale transforms
-// Block per node of level j (internal nodes only do work).
-// compress: the 8 children's blocks form a (2k)^3 cube, W is applied along each
-// direction, the k^3 corner is the parent's s and the rest its wavelet cube.
-__global__ void k_compress_level(int k, int lo, int hi, const int32_t* child, double* s, double* dnorm,
-                                 double* dcube, const double* filt) {
-    extern __shared__ double cube[];
-    __shared__ double red[32];
-    const int i = lo + blockIdx.x;
-    if (i >= hi || child[i] < 0) return;
-    const int n2 = 2 * k, k3 = k * k * k, c0 = child[i];
-    const double* W = filt + 2 * k * k;
-    for (int e = threadIdx.x; e < 8 * k3; e += blockDim.x) {
-        int o = e / k3, r = e % k3;
-        int i3 = r % k, i2 = (r / k) % k, i1 = r / (k * k);
-        int x1 = ((o >> 2) & 1) * k + i1, x2 = ((o >> 1) & 1) * k + i2, x3 = (o & 1) * k + i3;
-        cube[(x1 * n2 + x2) * n2 + x3] = s[(size_t)(c0 + o) * k3 + r];
-    }
-    __syncthreads();
-    for (int d = 0; d < 3; ++d) cube_transform(cube, n2, W, 0, d);
-    double acc = 0.0;
-    const int n3 = n2 * n2 * n2;
-    for (int e = threadIdx.x; e < n3; e += blockDim.x) {
-        int x3 = e % n2, x2 = (e / n2) % n2, x1 = e / (n2 * n2);
-        bool corner = x1 < k && x2 < k && x3 < k;
-        double v = cube[e];
-        if (corner) s[(size_t)i * k3 + (x1 * k + x2) * k + x3] = v;
-        else acc += v * v;
-        if (dcube) dcube[(size_t)i * n3 + e] = corner ? 0.0 : v;
-    }
-    acc = block_sum(acc, red);
-    if (threadIdx.x == 0) dnorm[i] = sqrt(acc);
-}
-
-// inverse (dcube != NULL: full s+d) or assemble (dcube == NULL: d = 0, the
-// children accumulate the upsampled parent block, eq. g_assemble).
-__global__ void k_expand_level(int k, int lo, int hi, const int32_t* child, double* s, const double* dcube,
-                               const double* filt) {
-    extern __shared__ double cube[];
-    const int i = lo + blockIdx.x;
-    if (i >= hi || child[i] < 0) return;
-    const int n2 = 2 * k, k3 = k * k * k, c0 = child[i], n3 = n2 * n2 * n2;
-    const double* W = filt + 2 * k * k;
-    for (int e = threadIdx.x; e < n3; e += blockDim.x) {
-        int x3 = e % n2, x2 = (e / n2) % n2, x1 = e / (n2 * n2);
-        bool corner = x1 < k && x2 < k && x3 < k;
-        double v = corner ? s[(size_t)i * k3 + (x1 * k + x2) * k + x3] : 0.0;
-        if (dcube && !corner) v = dcube[(size_t)i * n3 + e];
-        cube[e] = v;
-    }
-    __syncthreads();
-    for (int d = 0; d < 3; ++d) cube_transform(cube, n2, W, 1, d);
-    for (int e = threadIdx.x; e < 8 * k3; e += blockDim.x) {
-        int o = e / k3, r = e % k3;
-        int i3 = r % k, i2 = (r / k) % k, i1 = r / (k * k);
-        int x1 = ((o >> 2) & 1) * k + i1, x2 = ((o >> 1) & 1) * k + i2, x3 = (o & 1) * k + i3;
-        double v = cube[(x1 * n2 + x2) * n2 + x3];
-        size_t dst = (size_t)(c0 + o) * k3 + r;
-        if (dcube) s[dst] = v;
-        else s[dst] += v;
-    }
-}
-
 // One stage of a separable transform in shared memory: `in` has extents
 // (n[0], n[1], n[2]) with n[dim] = nin; `out` has the same extents except
 // nout along dim; out = Mat (nout x nin, row-major) applied along dim.
@@ -669,36 +588,6 @@ __device__ void load_UD(int k, const double* filt, double* U, double* D) {
         D[i * 2 * k + p * k + a] = h;
     }
     __syncthreads();
-}
-
-// Assembly (eq. g_assemble) with d = 0: children += (U x U x U) s_parent, in
-// three stages (2k^4 + 4k^4 + 8k^4 multiply-adds).  Block per node of level j.
-__global__ void k_up_level(int k, int lo, int hi, const int32_t* child, double* s, const double* filt) {
-    extern __shared__ double sm[];
-    const int i = lo + blockIdx.x;
-    if (i >= hi || child[i] < 0) return;
-    const int k2 = 2 * k, k3 = k * k * k, c0 = child[i];
-    double* U = sm;
-    double* D = U + 2 * k * k;
-    double* x = D + 2 * k * k;     // k^3
-    double* t1 = x + k3;           // 2k^3
-    double* t2 = t1 + 2 * k3;      // 4k^3
-    load_UD(k, filt, U, D);
-    for (int e = threadIdx.x; e < k3; e += blockDim.x) x[e] = s[(size_t)i * k3 + e];
-    __syncthreads();
-    int n0[3] = {k, k, k};
-    stage_mul(x, t1, n0, 0, U, k2);
-    int n1[3] = {k2, k, k};
-    stage_mul(t1, t2, n1, 1, U, k2);
-    // last stage on the fly, added into the children (octant (p1 p2 p3))
-    for (int idx = threadIdx.x; idx < 8 * k3; idx += blockDim.x) {
-        const int x1 = idx / (k2 * k2), x2 = (idx / k2) % k2, x3 = idx % k2;
-        const double* src = t2 + (x1 * k2 + x2) * k;
-        double acc = 0.0;
-        for (int c = 0; c < k; ++c) acc += U[x3 * k + c] * src[c];
-        const int o = ((x1 / k) << 2) | ((x2 / k) << 1) | (x3 / k);
-        s[(size_t)(c0 + o) * k3 + ((x1 % k) * k + (x2 % k)) * k + (x3 % k)] += acc;
-    }
 }
 
 // Redundant tree without stored wavelet cubes: s_parent = (D x D x D) cube of
@@ -763,7 +652,48 @@ __global__ void k_compress_fast_level(int k, int lo, int hi, const int32_t* chil
 // triangular loop bounds are compile-time constants and no warp diverges.
 // Shared-memory arrays keep their innermost extent padded to an odd number of
 // doubles, so that fibers along it (one per thread) hit distinct banks.
-enum { TRI_DENSE = 0, TRI_D = 1, TRI_U = 2 };
+//
+// Also H^(1)_{ia} = (-1)^{i+a} H^(0)_{ia} (phi_i(1 - u) = (-1)^i phi_i(u)), so both halves
+// come from the entries of H^(0) alone: with p_a = x0_a + (-1)^a x1_a and m_a = x0_a - (-1)^a x1_a
+// the parent's even rows read p and its odd rows m, and back the children are P + M and
+// (-1)^a (P - M), P / M the sums over even / odd i: k(k+1)/2 multiply-adds and 2k additions
+// per fiber (k = 8: 52 FP64 operations instead of 72, and the FP64 pipe is the bound).
+enum { TRI_D = 1, TRI_U = 2 };
+
+// y = D (x0 | x1): the parent's fiber from its two children's; H: H^(0) row-major in rows of LD
+template <int K, int LD>
+__device__ __forceinline__ void down_fiber(const double* H, const double* x, double* y) {
+    double p[K], m[K];
+#pragma unroll
+    for (int a = 0; a < K; ++a) {
+        const double x1 = (a & 1) ? -x[K + a] : x[K + a];
+        p[a] = x[a] + x1;
+        m[a] = x[a] - x1;
+    }
+#pragma unroll
+    for (int i = 0; i < K; ++i) {
+        double acc = 0.0;
+#pragma unroll
+        for (int a = 0; a <= i; ++a) acc += H[i * LD + a] * ((i & 1) ? m[a] : p[a]);
+        y[i] = acc;
+    }
+}
+
+// x = U s: the children's fibers from the parent's; Ht: H^(0) transposed, Ht[a * K + i]
+template <int K>
+__device__ __forceinline__ void up_fiber(const double* Ht, const double* s, double* x) {
+#pragma unroll
+    for (int a = 0; a < K; ++a) {
+        double P = 0.0, M = 0.0;
+#pragma unroll
+        for (int i = a; i < K; ++i) {
+            if (i & 1) M += Ht[a * K + i] * s[i];
+            else P += Ht[a * K + i] * s[i];
+        }
+        x[a] = P + M;
+        x[K + a] = (a & 1) ? M - P : P - M;
+    }
+}
 
 // in: extents (N0, N1, N2), strides (IS0, IS1, 1); out: the same with NOUT along DIM,
 // strides (OS0, OS1, 1); Mat: NOUT x NIN row-major with structure TRI (KT = k)
@@ -782,15 +712,16 @@ __device__ __forceinline__ void fiber_stage(const double* in, double* out, const
 #pragma unroll
         for (int c = 0; c < NIN; ++c) v[c] = src[c * IST];
         double* dst = out + a * OA + b * OB;
+        if constexpr (TRI == TRI_D) {
+            double y[KT];
+            down_fiber<KT, NIN>(Mat, v, y);
 #pragma unroll
-        for (int r = 0; r < NOUT; ++r) {
-            double acc = 0.0;
+            for (int r = 0; r < KT; ++r) dst[r * OST] = y[r];
+        } else {
+            double x[2 * KT];
+            up_fiber<KT>(Mat, v, x);
 #pragma unroll
-            for (int c = 0; c < NIN; ++c) {
-                const bool nz = TRI == TRI_DENSE || (TRI == TRI_D && (c % KT) <= r) || (TRI == TRI_U && c >= r % KT);
-                if (nz) acc += Mat[r * NIN + c] * v[c];
-            }
-            dst[r * OST] = acc;
+            for (int r = 0; r < 2 * KT; ++r) dst[r * OST] = x[r];
         }
     }
     __syncthreads();
@@ -850,15 +781,12 @@ template <int K>
 __global__ void __launch_bounds__(128) k_down_slice(int cbase, const int32_t* parent, double* s,
                                                     const double* filt) {
     constexpr int K2 = 2 * K, K3 = K * K * K, P2 = K2 + 1, R = 2;
-    __shared__ double D[K * K2];
+    __shared__ double H[K * K];
     __shared__ double cube[K2 * K2 * P2];  // (x1, x2, x3), x3 padded
     __shared__ double o1[R * K2 * P2];     // (r, x2, x3)
     __shared__ double o2[R * K * P2];      // (r, i2, x3)
     const int c0 = cbase + 8 * blockIdx.x, i = parent[c0], q = blockIdx.y, tid = threadIdx.x;
-    for (int e = tid; e < 2 * K * K; e += blockDim.x) {
-        const int p = e / (K * K), ii = (e / K) % K, a = e % K;  // H^(p)[ii][a]
-        D[ii * K2 + p * K + a] = filt[p * K * K + ii * K + a];
-    }
+    for (int e = tid; e < K * K; e += blockDim.x) H[e] = filt[e];
     for (int e = tid; e < 8 * K3; e += blockDim.x) {
         const int o = e / K3, r = e % K3;
         const int i1 = r / (K * K), i2 = (r / K) % K, i3 = r % K;
@@ -866,34 +794,32 @@ __global__ void __launch_bounds__(128) k_down_slice(int cbase, const int32_t* pa
         cube[(x1 * K2 + x2) * P2 + x3] = s[(size_t)(c0 + o) * K3 + r];
     }
     __syncthreads();
-    // direction 1: D = [H0 | H1] has in row i the columns a <= i of each half
+    // sum over a <= i of H_ia (x0_a + (-1)^{i+a} x1_a), x0 at src, x1 at src + K st
+    auto row = [&](const double* src, int st, int i) {
+        const double* Hr = H + i * K;
+        double acc = 0.0;
+        for (int a = 0; a <= i; ++a) {
+            const double x1 = src[(K + a) * st];
+            acc += Hr[a] * (src[a * st] + (((i + a) & 1) ? -x1 : x1));
+        }
+        return acc;
+    };
+    // direction 1
     for (int e = tid; e < R * K2 * K2; e += blockDim.x) {
         const int r = e / (K2 * K2), x2 = (e / K2) % K2, x3 = e % K2, i1 = r ? K - 1 - q : q;
-        const double* Dr = D + i1 * K2;
-        double acc = 0.0;
-        for (int a = 0; a <= i1; ++a)
-            acc += Dr[a] * cube[(a * K2 + x2) * P2 + x3] + Dr[K + a] * cube[((K + a) * K2 + x2) * P2 + x3];
-        o1[(r * K2 + x2) * P2 + x3] = acc;
+        o1[(r * K2 + x2) * P2 + x3] = row(cube + x2 * P2 + x3, K2 * P2, i1);
     }
     __syncthreads();
     // direction 2 (i2 slowest: a warp shares its loop bound)
     for (int e = tid; e < R * K * K2; e += blockDim.x) {
         const int i2 = e / (R * K2), r = (e / K2) % R, x3 = e % K2;
-        const double* Dr = D + i2 * K2;
-        double acc = 0.0;
-        for (int a = 0; a <= i2; ++a)
-            acc += Dr[a] * o1[(r * K2 + a) * P2 + x3] + Dr[K + a] * o1[(r * K2 + K + a) * P2 + x3];
-        o2[(r * K + i2) * P2 + x3] = acc;
+        o2[(r * K + i2) * P2 + x3] = row(o1 + r * K2 * P2 + x3, P2, i2);
     }
     __syncthreads();
     // direction 3, into rows i1 of the parent's block
     for (int e = tid; e < R * K * K; e += blockDim.x) {
         const int i3 = e / (R * K), r = (e / K) % R, i2 = e % K, i1 = r ? K - 1 - q : q;
-        const double* Dr = D + i3 * K2;
-        const double* src = o2 + (r * K + i2) * P2;
-        double acc = 0.0;
-        for (int a = 0; a <= i3; ++a) acc += Dr[a] * src[a] + Dr[K + a] * src[K + a];
-        s[(size_t)i * K3 + (i1 * K + i2) * K + i3] = acc;
+        s[(size_t)i * K3 + (i1 * K + i2) * K + i3] = row(o2 + (r * K + i2) * P2, 1, i3);
     }
 }
 
@@ -909,48 +835,59 @@ __global__ void __launch_bounds__(128) k_down_slice(int cbase, const int32_t* pa
 template <int K>
 __global__ void __launch_bounds__(128) k_up_slice(int cbase, const int32_t* parent, double* s, const double* filt) {
     constexpr int K2 = 2 * K, K3 = K * K * K, P1 = K + 1, RX = 4;
-    __shared__ double U[K2 * K];
+    __shared__ double Ht[K * K];         // Ht[a][i] = H^(0)[i][a]
     __shared__ double sp[K * K * P1];    // (i1, i2, i3), i3 padded
     __shared__ double t1[RX * K * P1];   // (rx, i2, i3)
     __shared__ double t2[RX * K2 * P1];  // (rx, x2, i3)
     const int c0 = cbase + 8 * blockIdx.x, i = parent[c0], q = blockIdx.y, tid = threadIdx.x;
-    for (int e = tid; e < 2 * K * K; e += blockDim.x) {
-        const int p = e / (K * K), ii = (e / K) % K, a = e % K;  // H^(p)[ii][a]
-        U[(p * K + a) * K + ii] = filt[p * K * K + ii * K + a];
-    }
+    for (int e = tid; e < K * K; e += blockDim.x) Ht[(e % K) * K + e / K] = filt[e];
     for (int e = tid; e < K3; e += blockDim.x) {
         const int i1 = e / (K * K), i2 = (e / K) % K, i3 = e % K;
         sp[(i1 * K + i2) * P1 + i3] = s[(size_t)i * K3 + e];
     }
     __syncthreads();
-    auto row_x1 = [&](int rx) { return (rx & 2 ? K : 0) + (rx & 1 ? K - 1 - q : q); };
+    // rows rx = 0..3: q, k-1-q of the first half, then of the second (odd K: the middle row of
+    // a half is one row, not a pair)
+    auto row_a = [&](int rx) { return rx & 1 ? K - 1 - q : q; };
+    auto absent = [&](int rx) { return (K & 1) && (rx & 1) && 2 * q == K - 1; };
+    // the children's entries a and K + a of a fiber: P + M and (-1)^a (P - M)
+    auto pair = [&](const double* src, int st, int a, double& x0, double& x1) {
+        const double* Hr = Ht + a * K;
+        double s0 = 0.0, s1 = 0.0;  // i of a's parity, and of the other
+        for (int i = a; i < K; i += 2) {
+            s0 += Hr[i] * src[i * st];
+            if (i + 1 < K) s1 += Hr[i + 1] * src[(i + 1) * st];
+        }
+        x0 = s0 + s1;
+        x1 = s0 - s1;  // (-1)^a (P - M): both signs come out the same
+    };
     // direction 1
-    for (int e = tid; e < RX * K * K; e += blockDim.x) {
-        const int rx = e / (K * K), i2 = (e / K) % K, i3 = e % K, x1 = row_x1(rx);
-        const double* Ur = U + x1 * K;
-        double acc = 0.0;
-        for (int c = x1 % K; c < K; ++c) acc += Ur[c] * sp[(c * K + i2) * P1 + i3];
-        t1[(rx * K + i2) * P1 + i3] = acc;
+    for (int e = tid; e < 2 * K * K; e += blockDim.x) {
+        const int rx = e / (K * K), i2 = (e / K) % K, i3 = e % K;
+        double x0, x1;
+        pair(sp + i2 * P1 + i3, K * P1, row_a(rx), x0, x1);
+        t1[(rx * K + i2) * P1 + i3] = x0;
+        t1[((rx + 2) * K + i2) * P1 + i3] = x1;
     }
     __syncthreads();
-    // direction 2 (x2 slowest: a warp shares its loop bound)
-    for (int e = tid; e < RX * K2 * K; e += blockDim.x) {
-        const int x2 = e / (RX * K), rx = (e / K) % RX, i3 = e % K;
-        const double* Ur = U + x2 * K;
-        double acc = 0.0;
-        for (int c = x2 % K; c < K; ++c) acc += Ur[c] * t1[(rx * K + c) * P1 + i3];
-        t2[(rx * K2 + x2) * P1 + i3] = acc;
+    // direction 2 (a slowest: a warp shares its loop bound)
+    for (int e = tid; e < RX * K * K; e += blockDim.x) {
+        const int a = e / (RX * K), rx = (e / K) % RX, i3 = e % K;
+        double x0, x1;
+        pair(t1 + rx * K * P1 + i3, P1, a, x0, x1);
+        t2[(rx * K2 + a) * P1 + i3] = x0;
+        t2[(rx * K2 + K + a) * P1 + i3] = x1;
     }
     __syncthreads();
     // direction 3, added into the children's blocks
-    for (int e = tid; e < RX * K2 * K2; e += blockDim.x) {
-        const int rx = e / (K2 * K2), x2 = (e / K2) % K2, x3 = e % K2, x1 = row_x1(rx);
-        const double* Ur = U + x3 * K;
-        const double* src = t2 + (rx * K2 + x2) * P1;
-        double acc = 0.0;
-        for (int c = x3 % K; c < K; ++c) acc += Ur[c] * src[c];
-        const int o = ((x1 / K) << 2) | ((x2 / K) << 1) | (x3 / K);
-        s[(size_t)(c0 + o) * K3 + ((x1 % K) * K + x2 % K) * K + x3 % K] += acc;
+    for (int e = tid; e < RX * K2 * K; e += blockDim.x) {
+        const int rx = e / (K2 * K), x2 = (e / K) % K2, a = e % K;
+        if (absent(rx)) continue;
+        double x0, x1;
+        pair(t2 + (rx * K2 + x2) * P1, 1, a, x0, x1);
+        double* dst = s + (size_t)(c0 + ((rx >> 1) << 2 | (x2 / K) << 1)) * K3 + (row_a(rx) * K + x2 % K) * K + a;
+        dst[0] += x0;
+        dst[K3] += x1;
     }
 }
 
@@ -991,16 +928,13 @@ __global__ void k_wnorm_all(const int32_t* parent, const double* s, double* dnor
         const int x1 = f / K2, x2 = f % K2;
         const double* src = rb + (x1 * K2 + x2) * P1;
         const double* cb = cube + (x1 * K2 + x2) * P2;
-        double v[K];
+        double v[K], up[K2];
 #pragma unroll
         for (int c = 0; c < K; ++c) v[c] = src[c];
+        up_fiber<K>(U, v, up);
 #pragma unroll
         for (int r = 0; r < K2; ++r) {
-            double up = 0.0;
-#pragma unroll
-            for (int c = 0; c < K; ++c)
-                if (c >= r % K) up += U[r * K + c] * v[c];
-            const double dv = cb[r] - up;
+            const double dv = cb[r] - up[r];
             acc += dv * dv;
         }
     }
@@ -1018,9 +952,15 @@ static int compress_fast_t(mra_tree* t, bool norms, cudaStream_t st) {
     for (int j = t->nlev - 2; j >= 0; --j) {
         const int nparents = (t->off[j + 2] - t->off[j + 1]) / 8;
         if (nparents <= 0) continue;
-        if (2 * nparents < num_sms())  // a small level: each parent over k/2 blocks
-            k_down_slice<K><<<dim3(nparents, K / 2), 128, 0, st>>>(t->off[j + 1], t->a.parent, t->s, t->filt);
-        else
+        // a small level: each parent over k/2 blocks (up to the order whose cube fits their
+        // static shared memory)
+        bool sliced = false;
+        if constexpr (K <= 8)
+            if (2 * nparents < num_sms()) {
+                k_down_slice<K><<<dim3(nparents, (K + 1) / 2), 128, 0, st>>>(t->off[j + 1], t->a.parent, t->s, t->filt);
+                sliced = true;
+            }
+        if (!sliced)
             k_compress_fast_level_t<K><<<nparents, 256, smem, st>>>(t->off[j + 1], t->a.parent, t->s, t->filt);
         MRA_CK_LAUNCH();
     }
@@ -1037,16 +977,138 @@ static int assemble_t(mra_tree* t, cudaStream_t st) {
     for (int j = 0; j + 1 < t->nlev; ++j) {
         const int nparents = (t->off[j + 2] - t->off[j + 1]) / 8;
         if (nparents <= 0) continue;
-        k_up_slice<K><<<dim3(nparents, K / 2), 128, 0, st>>>(t->off[j + 1], t->a.parent, t->s, t->filt);
+        k_up_slice<K><<<dim3(nparents, (K + 1) / 2), 128, 0, st>>>(t->off[j + 1], t->a.parent, t->s, t->filt);
         MRA_CK_LAUNCH();
     }
     return MRA_OK;
 }
 
-static int cube_smem(int k, size_t* bytes, const void* fn) {
-    *bytes = (size_t)8 * k * k * k * sizeof(double);
-    MRA_CK(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)*bytes));
+// ---- the whole filter matrix W (2k x 2k): stored wavelet blocks and their inverse
+// Block per sibling group; the cube is transformed in place, a thread taking whole fibers (its
+// 2k values in registers, all outputs written back), innermost extent padded.  The scaling rows
+// go by parity halves as above; the wavelet rows are applied as they are (Gram-Schmidt leaves
+// their parity to rounding error times its condition, 2e-8 at k = 12, so using it would cost
+// the inverse its accuracy).  k = 8, 967 internal nodes, FP64 pipe: 164 multiply-adds and
+// 16 additions per fiber instead of 256 multiply-adds.
+template <int K, bool INV>
+__device__ __forceinline__ void cube_fibers(double* cube, const double* W, const double* Ht, int dim) {
+    constexpr int K2 = 2 * K, P2 = K2 + 1;
+    const int st = dim == 0 ? K2 * P2 : (dim == 1 ? P2 : 1);
+    for (int f = threadIdx.x; f < K2 * K2; f += blockDim.x) {
+        const int u = f / K2, v = f % K2;
+        double* p = cube + (dim == 0 ? u * P2 + v : (dim == 1 ? u * K2 * P2 + v : (u * K2 + v) * P2));
+        double x[K2], y[K2];
+#pragma unroll
+        for (int c = 0; c < K2; ++c) x[c] = p[c * st];
+        if (!INV) {
+            down_fiber<K, K2>(W, x, y);
+#pragma unroll
+            for (int r = K; r < K2; ++r) {
+                double acc = 0.0;
+#pragma unroll
+                for (int c = 0; c < K2; ++c) acc += W[r * K2 + c] * x[c];
+                y[r] = acc;
+            }
+        } else {
+            up_fiber<K>(Ht, x, y);
+#pragma unroll
+            for (int r = K; r < K2; ++r)
+#pragma unroll
+                for (int c = 0; c < K2; ++c) y[c] += W[r * K2 + c] * x[r];
+        }
+#pragma unroll
+        for (int c = 0; c < K2; ++c) p[c * st] = y[c];
+    }
+    __syncthreads();
+}
+
+template <int K>
+struct CubeSmem {
+    static constexpr int K2 = 2 * K, P2 = K2 + 1, CUBE = K2 * K2 * P2;
+    static constexpr size_t BYTES = (size_t)(CUBE + K2 * K2 + K * K) * sizeof(double);
+};
+
+// compress: the children's cube -> the parent's block (the k^3 corner), its wavelet cube and norm
+template <int K>
+__global__ void __launch_bounds__(256) k_compress_cube(int cbase, const int32_t* parent, double* s, double* dnorm,
+                                                       double* dcube, const double* filt) {
+    using L = CubeSmem<K>;
+    constexpr int K2 = L::K2, K3 = K * K * K, P2 = L::P2, N3 = K2 * K2 * K2;
+    extern __shared__ double sm[];
+    __shared__ double red[32];
+    double *cube = sm, *W = cube + L::CUBE;
+    const int c0 = cbase + 8 * blockIdx.x, i = parent[c0];
+    for (int e = threadIdx.x; e < K2 * K2; e += blockDim.x) W[e] = filt[2 * K * K + e];
+    for (int e = threadIdx.x; e < 8 * K3; e += blockDim.x) {
+        const int o = e / K3, r = e % K3;
+        const int i1 = r / (K * K), i2 = (r / K) % K, i3 = r % K;
+        const int x1 = ((o >> 2) & 1) * K + i1, x2 = ((o >> 1) & 1) * K + i2, x3 = (o & 1) * K + i3;
+        cube[(x1 * K2 + x2) * P2 + x3] = s[(size_t)(c0 + o) * K3 + r];
+    }
+    __syncthreads();
+    for (int d = 0; d < 3; ++d) cube_fibers<K, false>(cube, W, nullptr, d);
+    double acc = 0.0;
+    for (int e = threadIdx.x; e < N3; e += blockDim.x) {
+        const int x3 = e % K2, x2 = (e / K2) % K2, x1 = e / (K2 * K2);
+        const bool corner = x1 < K && x2 < K && x3 < K;
+        const double v = cube[(x1 * K2 + x2) * P2 + x3];
+        if (corner) s[(size_t)i * K3 + (x1 * K + x2) * K + x3] = v;
+        else acc += v * v;
+        dcube[(size_t)i * N3 + e] = corner ? 0.0 : v;
+    }
+    acc = block_sum(acc, red);
+    if (threadIdx.x == 0) dnorm[i] = sqrt(acc);
+}
+
+// inverse: the parent's block and wavelet cube -> its children's blocks
+template <int K>
+__global__ void __launch_bounds__(256) k_expand_cube(int cbase, const int32_t* parent, double* s, const double* dcube,
+                                                     const double* filt) {
+    using L = CubeSmem<K>;
+    constexpr int K2 = L::K2, K3 = K * K * K, P2 = L::P2, N3 = K2 * K2 * K2;
+    extern __shared__ double sm[];
+    double *cube = sm, *W = cube + L::CUBE, *Ht = W + K2 * K2;
+    const int c0 = cbase + 8 * blockIdx.x, i = parent[c0];
+    for (int e = threadIdx.x; e < K2 * K2; e += blockDim.x) W[e] = filt[2 * K * K + e];
+    for (int e = threadIdx.x; e < K * K; e += blockDim.x) Ht[(e % K) * K + e / K] = filt[e];
+    for (int e = threadIdx.x; e < N3; e += blockDim.x) {
+        const int x3 = e % K2, x2 = (e / K2) % K2, x1 = e / (K2 * K2);
+        const bool corner = x1 < K && x2 < K && x3 < K;
+        cube[(x1 * K2 + x2) * P2 + x3] =
+            corner ? s[(size_t)i * K3 + (x1 * K + x2) * K + x3] : dcube[(size_t)i * N3 + e];
+    }
+    __syncthreads();
+    for (int d = 0; d < 3; ++d) cube_fibers<K, true>(cube, W, Ht, d);
+    for (int e = threadIdx.x; e < 8 * K3; e += blockDim.x) {
+        const int o = e / K3, r = e % K3;
+        const int i1 = r / (K * K), i2 = (r / K) % K, i3 = r % K;
+        const int x1 = ((o >> 2) & 1) * K + i1, x2 = ((o >> 1) & 1) * K + i2, x3 = (o & 1) * K + i3;
+        s[(size_t)(c0 + o) * K3 + r] = cube[(x1 * K2 + x2) * P2 + x3];
+    }
+}
+
+template <int K>
+static int cube_levels(mra_tree* t, bool inverse, cudaStream_t st) {
+    const size_t smem = CubeSmem<K>::BYTES;
+    MRA_CK(cudaFuncSetAttribute(k_compress_cube<K>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    MRA_CK(cudaFuncSetAttribute(k_expand_cube<K>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    for (int l = 0; l + 1 < t->nlev; ++l) {
+        const int j = inverse ? l : t->nlev - 2 - l, nparents = (t->off[j + 2] - t->off[j + 1]) / 8;
+        if (nparents <= 0) continue;
+        if (inverse)
+            k_expand_cube<K><<<nparents, 256, smem, st>>>(t->off[j + 1], t->a.parent, t->s, t->dcube, t->filt);
+        else
+            k_compress_cube<K><<<nparents, 256, smem, st>>>(t->off[j + 1], t->a.parent, t->s, t->dnorm, t->dcube, t->filt);
+        MRA_CK_LAUNCH();
+    }
     return MRA_OK;
+}
+
+static int cube_transform(mra_tree* t, bool inverse, cudaStream_t st) {
+    static int (*const fn[])(mra_tree*, bool, cudaStream_t) = {
+        nullptr,        cube_levels<1>, cube_levels<2>, cube_levels<3>,  cube_levels<4>,  cube_levels<5>, cube_levels<6>,
+        cube_levels<7>, cube_levels<8>, cube_levels<9>, cube_levels<10>, cube_levels<11>, cube_levels<12>};
+    return fn[t->k](t, inverse, st);
 }
 
 int compress_impl(mra_tree* t, int mode, cudaStream_t st) {
@@ -1058,12 +1120,16 @@ int compress_impl(mra_tree* t, int mode, cudaStream_t st) {
             t->dcube = nullptr;
         }
         MRA_CK(cudaMemsetAsync(t->dnorm, 0, t->n * sizeof(double), st));
-        if (k == 4 || k == 6 || k == 8) {
-            MRA_TRY(k == 4 ? compress_fast_t<4>(t, norms, st)
-                           : (k == 6 ? compress_fast_t<6>(t, norms, st) : compress_fast_t<8>(t, norms, st)));
+        if (k < 12) {
+            static int (*const fast[])(mra_tree*, bool, cudaStream_t) = {
+                nullptr, compress_fast_t<1>, compress_fast_t<2>, compress_fast_t<3>, compress_fast_t<4>,
+                compress_fast_t<5>, compress_fast_t<6>, compress_fast_t<7>, compress_fast_t<8>, compress_fast_t<9>,
+                compress_fast_t<10>, compress_fast_t<11>};
+            MRA_TRY(fast[k](t, norms, st));
             t->state = MRA_TREE_REDUNDANT;
             return MRA_OK;
         }
+        // k = 12: the children's padded cube and its stages exceed a block's shared memory
         const size_t smem = (4 * (size_t)k * k + 15 * (size_t)k * k * k) * sizeof(double);
         MRA_CK(cudaFuncSetAttribute(k_compress_fast_level, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
         for (int j = t->nlev - 2; j >= 0; --j) {
@@ -1076,17 +1142,9 @@ int compress_impl(mra_tree* t, int mode, cudaStream_t st) {
         t->state = MRA_TREE_REDUNDANT;
         return MRA_OK;
     }
-    size_t smem;
-    MRA_TRY(cube_smem(t->k, &smem, (const void*)k_compress_level));
     if (!t->dcube) MRA_TRY(dalloc(t->A, &t->dcube, (size_t)t->n * 8 * t->k * t->k * t->k));
     MRA_CK(cudaMemsetAsync(t->dnorm, 0, t->n * sizeof(double), st));
-    for (int j = t->nlev - 2; j >= 0; --j) {
-        int lo = t->off[j], hi = t->off[j + 1];
-        if (hi <= lo) continue;
-        k_compress_level<<<hi - lo, 256, smem, st>>>(t->k, lo, hi, t->a.child, t->s, t->dnorm,
-                                                     t->dcube, t->filt);
-        MRA_CK_LAUNCH();
-    }
+    MRA_TRY(cube_transform(t, false, st));
     t->state = MRA_TREE_REDUNDANT;
     return MRA_OK;
 }
@@ -1096,32 +1154,17 @@ int inverse_impl(mra_tree* t, cudaStream_t st) {
         set_error("inverse transform needs a tree compressed with MRA_COMPRESS_STORE_D");
         return MRA_ESTATE;
     }
-    size_t smem;
-    MRA_TRY(cube_smem(t->k, &smem, (const void*)k_expand_level));
-    for (int j = 0; j + 1 < t->nlev; ++j) {
-        int lo = t->off[j], hi = t->off[j + 1];
-        k_expand_level<<<hi - lo, 256, smem, st>>>(t->k, lo, hi, t->a.child, t->s, t->dcube, t->filt);
-        MRA_CK_LAUNCH();
-    }
+    MRA_TRY(cube_transform(t, true, st));
     t->state = MRA_TREE_LEAVES;
     return MRA_OK;
 }
 
 int assemble_impl(mra_tree* t, cudaStream_t st) {
     const int k = t->k;
-    if (k == 4 || k == 6 || k == 8) {
-        MRA_TRY(k == 4 ? assemble_t<4>(t, st) : (k == 6 ? assemble_t<6>(t, st) : assemble_t<8>(t, st)));
-        t->state = MRA_TREE_LEAVES;
-        return MRA_OK;
-    }
-    const size_t smem = (4 * (size_t)k * k + 7 * (size_t)k * k * k) * sizeof(double);
-    MRA_CK(cudaFuncSetAttribute(k_up_level, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    for (int j = 0; j + 1 < t->nlev; ++j) {
-        int lo = t->off[j], hi = t->off[j + 1];
-        if (hi <= lo) continue;
-        k_up_level<<<hi - lo, 256, smem, st>>>(k, lo, hi, t->a.child, t->s, t->filt);
-        MRA_CK_LAUNCH();
-    }
+    static int (*const up[])(mra_tree*, cudaStream_t) = {nullptr,       assemble_t<1>, assemble_t<2>,  assemble_t<3>,  assemble_t<4>,
+                                                         assemble_t<5>, assemble_t<6>, assemble_t<7>,  assemble_t<8>,  assemble_t<9>,
+                                                         assemble_t<10>, assemble_t<11>, assemble_t<12>};
+    MRA_TRY(up[k](t, st));
     t->state = MRA_TREE_LEAVES;
     return MRA_OK;
 }
