@@ -47,82 +47,245 @@ struct mra_mlp {
 
 namespace mra {
 
-// out[r][o] for a block of MLP_RB rows; in: float or half [n][din];
-// Wio: half [din][dout] (element (i, o) at i * dout + o).
-//   mode 0: relu(in W + b) -> half     (hidden layer, forward)
-//   mode 1: in W + b       -> float    (output layer, forward)
-//   mode 2: (in W) * [mask > 0] -> float  (backward data pass; mask half [n][dout])
-template <class TI, int MODE>
-__global__ void k_dense(int64_t n, int din, int dout, const TI* in, const __half* Wio, const float* b,
-                        const __half* mask, void* out) {
-    extern __shared__ float xs[];  // [MLP_RB][din]
-    const int64_t r0 = (int64_t)blockIdx.x * MLP_RB;
-    const int rows = (int)min((int64_t)MLP_RB, n - r0);
-    for (int e = threadIdx.x; e < rows * din; e += blockDim.x)
-        xs[e] = (float)in[r0 * din + e];
-    __syncthreads();
-    for (int o = threadIdx.x; o < dout; o += blockDim.x) {
-        float acc[MLP_RB];
-        const float bo = b ? b[o] : 0.0f;
+// Rows are independent of each other through the whole network, the loss and the backward
+// data pass, so one block carries MLP_RB rows through all of it with the activations in
+// shared memory; what bounds it is then the multiply-adds (2 din dout per row and layer) and
+// the shared-memory reads that feed them.  A thread's tile is 4 rows x 4 outputs: per input i
+// one 16-byte broadcast of activations and one 8-byte weight read for 16 multiply-adds.
+// (One output x 32 rows per thread, a launch per layer: one shared read per multiply-add,
+// 67 us per 128 x 128 layer at 4,096 rows.)  Each output sums its bias, then the products in
+// increasing i, as a chain of fused multiply-adds.
+#define MLP_NT 256
+#define MLP_XS 36   // activations [i][row], rows padded to a multiple of 4
+#define MLP_WI 64   // weight rows staged at a time
+
+struct MlpTile {
+    float v[4][4];  // [row][output]
+};
+
+// rows 4 warp.., outputs o0 + 4 lane..: bias + sum_i xs[i][row] Wio[i][o]; Wio half [din][dout]
+// in global memory (dout a multiple of 4 or read element by element)
+__device__ void mlp_layer(const float* xs, int din, const __half* Wio, int dout, int o0, const float* bias, __half* ws,
+                          MlpTile& t) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
-        for (int r = 0; r < MLP_RB; ++r) acc[r] = bo;
-        for (int i = 0; i < din; ++i) {
-            const float w = __half2float(Wio[(size_t)i * dout + o]);
+    for (int q = 0; q < 4; ++q) {
+        const int o = o0 + 4 * lane + q;
+        const float b = bias && o < dout ? bias[o] : 0.0f;
 #pragma unroll
-            for (int r = 0; r < MLP_RB; ++r) acc[r] += w * xs[r * din + i];
+        for (int r = 0; r < 4; ++r) t.v[r][q] = b;
+    }
+    for (int i0 = 0; i0 < din; i0 += MLP_WI) {
+        const int ni = min(MLP_WI, din - i0);
+        __syncthreads();
+        for (int e = threadIdx.x; e < ni * 128; e += MLP_NT) {
+            const int i = e >> 7, o = o0 + (e & 127);
+            ws[e] = o < dout ? Wio[(size_t)(i0 + i) * dout + o] : __half(0.0f);
         }
+        __syncthreads();
+        if (o0 + 4 * lane < dout)
+#pragma unroll 4
+            for (int i = 0; i < ni; ++i) {
+                const float4 x = *(const float4*)(xs + (size_t)(i0 + i) * MLP_XS + 4 * warp);
+                const uint2 w2 = *(const uint2*)(ws + i * 128 + 4 * lane);
+                const float2 wa = __half22float2(*(const __half2*)&w2.x), wb = __half22float2(*(const __half2*)&w2.y);
+                const float xr[4] = {x.x, x.y, x.z, x.w}, w[4] = {wa.x, wa.y, wb.x, wb.y};
 #pragma unroll
-        for (int r = 0; r < MLP_RB; ++r) {
-            if (r >= rows) break;
-            const size_t idx = (size_t)(r0 + r) * dout + o;
-            if (MODE == 0) ((__half*)out)[idx] = __float2half_rn(fmaxf(acc[r], 0.0f));
-            else if (MODE == 1) ((float*)out)[idx] = acc[r];
-            else ((float*)out)[idx] = __half2float(mask[idx]) > 0.0f ? acc[r] : 0.0f;
-        }
+                for (int r = 0; r < 4; ++r)
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) t.v[r][q] = fmaf(w[q], xr[r], t.v[r][q]);
+            }
     }
 }
 
-// loss and dL/dy (divided by n); loss accumulated in FP64
-__global__ void k_mlp_loss(int64_t n, const float* y, const float* t, float* dy, double* loss) {
-    __shared__ double red[32];
-    double acc = 0.0;
-    const double inv = 1.0 / (double)n;
-    for (int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; r < n; r += (int64_t)gridDim.x * blockDim.x) {
-        for (int S = 0; S < 4; ++S) {
-            const float e = y[r * 12 + 3 * S], lo = y[r * 12 + 3 * S + 1], hi = y[r * 12 + 3 * S + 2];
-            const float E = t[r * 12 + 3 * S], LO = t[r * 12 + 3 * S + 1], HI = t[r * 12 + 3 * S + 2];
-            const double sp = e > 0.0f ? (double)e + log1p(exp(-(double)e)) : log1p(exp((double)e));
-            acc += sp - (double)E * e + (1.0 - E) * ((double)(lo - LO) * (lo - LO) + (double)(hi - HI) * (hi - HI));
-            const double sg = 1.0 / (1.0 + exp(-(double)e));
-            dy[r * 12 + 3 * S] = (float)((sg - E) * inv);
-            dy[r * 12 + 3 * S + 1] = (float)(2.0 * (1.0 - E) * (lo - LO) * inv);
-            dy[r * 12 + 3 * S + 2] = (float)(2.0 * (1.0 - E) * (hi - HI) * inv);
+struct MlpArgs {
+    int64_t n;
+    int n_in, n_out;
+    const float* x;
+    const __half *wt[4], *wr[4];  // [in][out] and [out][in] copies
+    const float* b[4];
+    float* y;
+    __half* h[3];                 // activations kept for the gradient (NULL: not kept)
+    // training: targets, dL/dy, the data gradients of the hidden layers, the loss
+    const float* target;
+    float *dy, *d[3];
+    double* loss;
+};
+
+template <bool TRAIN>
+__global__ void __launch_bounds__(MLP_NT) k_mlp_rows(MlpArgs A) {
+    extern __shared__ __align__(16) float mlp_sm[];
+    __shared__ __align__(8) __half ws[MLP_WI * 128];
+    __shared__ double red[MLP_NT / 32];
+    float* xa = mlp_sm;                                     // [max(n_in, 128)][MLP_XS]
+    float* xb = xa + (size_t)max(A.n_in, MLP_H) * MLP_XS;   // [128][MLP_XS]
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int64_t r0 = (int64_t)blockIdx.x * MLP_RB;
+    const int rows = (int)min((int64_t)MLP_RB, A.n - r0);
+    for (int e = tid; e < MLP_RB * A.n_in; e += MLP_NT) {
+        const int r = e / A.n_in, i = e - r * A.n_in;
+        xa[i * MLP_XS + r] = r < rows ? A.x[(r0 + r) * A.n_in + i] : 0.0f;
+    }
+    MlpTile t;
+    unsigned on[3] = {0, 0, 0};  // hidden units of this thread's tile above zero
+    float *in = xa, *out = xb;
+    for (int l = 0; l < 3; ++l) {
+        mlp_layer(in, l ? MLP_H : A.n_in, A.wt[l], MLP_H, 0, A.b[l], ws, t);
+        __syncthreads();
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+            __align__(8) __half hv[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                hv[q] = __float2half_rn(fmaxf(t.v[r][q], 0.0f));
+                const float f = __half2float(hv[q]);
+                out[(4 * lane + q) * MLP_XS + 4 * warp + r] = f;
+                on[l] |= (unsigned)(f > 0.0f) << (4 * r + q);
+            }
+            if (TRAIN && 4 * warp + r < rows)
+                *(uint2*)(A.h[l] + (r0 + 4 * warp + r) * MLP_H + 4 * lane) = *(const uint2*)hv;
         }
+        float* s = in;
+        in = out;
+        out = s;
+    }
+    for (int o0 = 0; o0 < A.n_out; o0 += 128) {
+        mlp_layer(in, MLP_H, A.wt[3], A.n_out, o0, A.b[3], ws, t);
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const int o = o0 + 4 * lane + q;
+                if (o < A.n_out && 4 * warp + r < rows) A.y[(r0 + 4 * warp + r) * A.n_out + o] = t.v[r][q];
+                if (TRAIN && o < 12) out[o * MLP_XS + 4 * warp + r] = t.v[r][q];
+            }
+    }
+    if (!TRAIN) return;
+    // loss and dL/dy (divided by n), FP64: thread (row, class)
+    __syncthreads();
+    double acc = 0.0;
+    if (tid < MLP_RB * 4) {
+        const int r = tid >> 2, S = tid & 3;
+        float g[3] = {0.0f, 0.0f, 0.0f};
+        if (r < rows) {
+            const double inv = 1.0 / (double)A.n;
+            const float e = out[(3 * S) * MLP_XS + r], lo = out[(3 * S + 1) * MLP_XS + r], hi = out[(3 * S + 2) * MLP_XS + r];
+            const float* T = A.target + (r0 + r) * 12 + 3 * S;
+            const float E = T[0], LO = T[1], HI = T[2];
+            const double z = exp(-fabs((double)e));  // softplus and sigmoid from one exponential
+            const double sp = fmax((double)e, 0.0) + log1p(z);
+            const double sg = (e > 0.0f ? 1.0 : z) / (1.0 + z);
+            acc = sp - (double)E * e + (1.0 - E) * ((double)(lo - LO) * (lo - LO) + (double)(hi - HI) * (hi - HI));
+            g[0] = (float)((sg - E) * inv);
+            g[1] = (float)(2.0 * (1.0 - E) * (lo - LO) * inv);
+            g[2] = (float)(2.0 * (1.0 - E) * (hi - HI) * inv);
+            for (int q = 0; q < 3; ++q) A.dy[(r0 + r) * 12 + 3 * S + q] = g[q];
+        }
+        for (int q = 0; q < 3; ++q) out[(3 * S + q) * MLP_XS + r] = g[q];
     }
     for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
+    if (lane == 0) red[warp] = acc;
     __syncthreads();
-    if (threadIdx.x == 0) {
+    if (tid == 0) {
         double s = 0.0;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) s += red[w];
-        atomicAdd(loss, s * inv);
+        for (int w = 0; w < MLP_RB * 4 / 32; ++w) s += red[w];
+        atomicAdd(A.loss, s / (double)A.n);
+    }
+    // back through the layers: d_l = (d_{l+1} W) where the unit was on
+    float* g = out;
+    float* nx = in;
+    for (int l = 2; l >= 0; --l) {
+        mlp_layer(g, l == 2 ? A.n_out : MLP_H, A.wr[l + 1], MLP_H, 0, nullptr, ws, t);
+        __syncthreads();
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+            float v[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                v[q] = ((on[l] >> (4 * r + q)) & 1u) ? t.v[r][q] : 0.0f;
+                nx[(4 * lane + q) * MLP_XS + 4 * warp + r] = v[q];
+            }
+            if (4 * warp + r < rows)
+                *(float4*)(A.d[l] + (r0 + 4 * warp + r) * MLP_H + 4 * lane) = make_float4(v[0], v[1], v[2], v[3]);
+        }
+        float* s = g;
+        g = nx;
+        nx = s;
     }
 }
 
-// gW[o][i] = sum_r d[r][o] h[r][i], gb[o] = sum_r d[r][o]; thread per (o, i)
-// (i == din: the bias)
-template <class TI>
-__global__ void k_wgrad(int64_t n, int din, int dout, const float* d, const TI* h, float* gW, float* gb) {
-    const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (e >= (int64_t)dout * (din + 1)) return;
-    const int o = (int)(e / (din + 1)), i = (int)(e % (din + 1));
-    float acc = 0.0f;
-    if (i < din) {
-        for (int64_t r = 0; r < n; ++r) acc += d[r * dout + o] * (float)h[r * din + i];
-        gW[(size_t)o * din + i] = acc;
-    } else {
-        for (int64_t r = 0; r < n; ++r) acc += d[r * dout + o];
-        gb[o] = acc;
+// Weight gradients gW[o][i] = sum_r d[r][o] h[r][i], gb[o] = sum_r d[r][o] of all layers in one
+// launch: block (row slice, layer, tile of 128 x 128), 8 x 8 outputs per thread, 32 rows at a
+// time in shared memory; the slices' sums are added in order afterwards, so the result does
+// not depend on scheduling.  (A thread per weight walking all rows by itself: 2.7 ms for the
+// four layers at 4,096 rows, a serial chain of 4,096 loads.)
+struct WgradArgs {
+    int64_t n, np;
+    int rows;  // rows per slice
+    const float* d[4];
+    const void* h[4];   // layer 0: float x, else half
+    int din[4], dout[4], ti[4];   // ti: tiles along i
+    int tile0[5];       // first tile of each layer
+    int64_t off_w[4], off_b[4];
+    float* part;        // [slices][np]
+};
+
+__global__ void __launch_bounds__(256) k_mlp_wgrad(WgradArgs A) {
+    __shared__ __align__(16) float ds[32][128], hs[32][128];
+    int l = 0;
+    while (l < 3 && (int)blockIdx.y >= A.tile0[l + 1]) ++l;
+    const int tile = blockIdx.y - A.tile0[l], o0 = tile / A.ti[l] * 128, i0 = tile % A.ti[l] * 128;
+    const int din = A.din[l], dout = A.dout[l], tid = threadIdx.x, to = tid >> 4, ti = tid & 15;
+    const int64_t r0 = (int64_t)blockIdx.x * A.rows, r1 = min(A.n, r0 + A.rows);
+    float acc[8][8], gb = 0.0f;
+#pragma unroll
+    for (int a = 0; a < 8; ++a)
+#pragma unroll
+        for (int b = 0; b < 8; ++b) acc[a][b] = 0.0f;
+    const bool busy = o0 + 4 * to < dout && i0 + 4 * ti < din;
+    for (int64_t r = r0; r < r1; r += 32) {
+        __syncthreads();
+        for (int e = tid; e < 32 * 128; e += 256) {
+            const int rr = e >> 7, c = e & 127;
+            const int64_t row = r + rr;
+            ds[rr][c] = row < r1 && o0 + c < dout ? A.d[l][row * dout + o0 + c] : 0.0f;
+            hs[rr][c] = row < r1 && i0 + c < din
+                            ? (l ? __half2float(((const __half*)A.h[l])[row * din + i0 + c]) : ((const float*)A.h[l])[row * din + i0 + c])
+                            : 0.0f;
+        }
+        __syncthreads();
+        if (busy)
+#pragma unroll 4
+            for (int rr = 0; rr < 32; ++rr) {
+                // outputs 4 to + {0..3, 64..67}, inputs 4 ti + {0..3, 64..67}
+                const float4 da = *(const float4*)&ds[rr][4 * to], db = *(const float4*)&ds[rr][64 + 4 * to];
+                const float4 ha = *(const float4*)&hs[rr][4 * ti], hb = *(const float4*)&hs[rr][64 + 4 * ti];
+                const float dv[8] = {da.x, da.y, da.z, da.w, db.x, db.y, db.z, db.w};
+                const float hv[8] = {ha.x, ha.y, ha.z, ha.w, hb.x, hb.y, hb.z, hb.w};
+#pragma unroll
+                for (int a = 0; a < 8; ++a)
+#pragma unroll
+                    for (int b = 0; b < 8; ++b) acc[a][b] = fmaf(dv[a], hv[b], acc[a][b]);
+            }
+        if (i0 == 0 && tid < 128)
+            for (int rr = 0; rr < 32; ++rr) gb += ds[rr][tid];
+    }
+    float* part = A.part + (size_t)blockIdx.x * A.np;
+#pragma unroll
+    for (int a = 0; a < 8; ++a)
+#pragma unroll
+        for (int b = 0; b < 8; ++b) {
+            const int o = o0 + 4 * to + (a & 3) + (a >> 2) * 64, i = i0 + 4 * ti + (b & 3) + (b >> 2) * 64;
+            if (o < dout && i < din) part[A.off_w[l] + (size_t)o * din + i] = acc[a][b];
+        }
+    if (i0 == 0 && tid < 128 && o0 + tid < dout) part[A.off_b[l] + o0 + tid] = gb;
+}
+
+__global__ void k_mlp_wsum(int64_t np, int slices, const float* part, float* g) {
+    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < np; e += (int64_t)gridDim.x * blockDim.x) {
+        float s = 0.0f;
+        for (int q = 0; q < slices; ++q) s += part[(size_t)q * np + e];
+        g[e] = s;
     }
 }
 
@@ -199,32 +362,28 @@ static int ensure_cap(mra_mlp* M, int64_t n) {
     return MRA_OK;
 }
 
-template <class TI, int MODE>
-static int dense(int64_t n, int din, int dout, const TI* in, const __half* Wio, const float* b, const __half* mask,
-                 void* out, cudaStream_t st) {
-    if (n <= 0) return MRA_OK;
-    const int64_t blocks = (n + MLP_RB - 1) / MLP_RB;
-    k_dense<TI, MODE><<<(unsigned)blocks, 128, (size_t)MLP_RB * din * sizeof(float), st>>>(n, din, dout, in, Wio, b,
-                                                                                          mask, out);
-    MRA_CK_LAUNCH();
-    return MRA_OK;
+static MlpArgs mlp_args(const mra_mlp* M, const float* x, int64_t n, float* y) {
+    MlpArgs A{};
+    A.n = n;
+    A.n_in = M->n_in;
+    A.n_out = M->n_out;
+    A.x = x;
+    for (int l = 0; l < 4; ++l) {
+        A.wt[l] = w_trans(M, l);
+        A.wr[l] = w_rowmajor(M, l);
+        A.b[l] = M->master + M->off_b[l];
+    }
+    A.y = y;
+    return A;
 }
 
-// forward with the activations kept (h1, h2, h3 in M's buffers), output y
-int mlp_forward_impl(const mra_mlp* M, const float* x, int64_t n, float* y, __half* h1, __half* h2, __half* h3,
-                     cudaStream_t st) {
-    const float* p = M->master;
-    MRA_TRY((dense<float, 0>(n, M->n_in, MLP_H, x, w_trans(M, 0), p + M->off_b[0], nullptr, h1, st)));
-    MRA_TRY((dense<__half, 0>(n, MLP_H, MLP_H, h1, w_trans(M, 1), p + M->off_b[1], nullptr, h2, st)));
-    MRA_TRY((dense<__half, 0>(n, MLP_H, MLP_H, h2, w_trans(M, 2), p + M->off_b[2], nullptr, h3, st)));
-    MRA_TRY((dense<__half, 1>(n, MLP_H, M->n_out, h3, w_trans(M, 3), p + M->off_b[3], nullptr, y, st)));
-    return MRA_OK;
-}
-
-template <class TI>
-static int wgrad(int64_t n, int din, int dout, const float* d, const TI* h, float* gW, float* gb, cudaStream_t st) {
-    const int64_t tot = (int64_t)dout * (din + 1);
-    k_wgrad<TI><<<(unsigned)((tot + 127) / 128), 128, 0, st>>>(n, din, dout, d, h, gW, gb);
+template <bool TRAIN>
+static int mlp_rows(const MlpArgs& A, cudaStream_t st) {
+    if (A.n <= 0) return MRA_OK;
+    const int64_t blocks = (A.n + MLP_RB - 1) / MLP_RB;
+    const size_t smem = (size_t)(std::max(A.n_in, MLP_H) + MLP_H) * MLP_XS * sizeof(float);
+    MRA_CK(cudaFuncSetAttribute(k_mlp_rows<TRAIN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    k_mlp_rows<TRAIN><<<(unsigned)blocks, MLP_NT, smem, st>>>(A);
     MRA_CK_LAUNCH();
     return MRA_OK;
 }
@@ -232,19 +391,38 @@ static int wgrad(int64_t n, int din, int dout, const float* d, const TI* h, floa
 // forward, loss and gradients of the batch into M->grad (loss into M->loss)
 static int mlp_loss_grad_impl(mra_mlp* M, const float* x, const float* t, int64_t n, cudaStream_t st) {
     MRA_TRY(ensure_cap(M, n));
-    MRA_TRY(mlp_forward_impl(M, x, n, M->y, M->h1, M->h2, M->h3, st));
+    MlpArgs A = mlp_args(M, x, n, M->y);
+    A.h[0] = M->h1; A.h[1] = M->h2; A.h[2] = M->h3;
+    A.target = t;
+    A.dy = M->dy;
+    A.d[0] = M->d1; A.d[1] = M->d2; A.d[2] = M->d3;
+    A.loss = M->loss;
     MRA_CK(cudaMemsetAsync(M->loss, 0, sizeof(double), st));
-    k_mlp_loss<<<(unsigned)std::min<int64_t>(1024, (n + 255) / 256), 256, 0, st>>>(n, M->y, t, M->dy, M->loss);
+    MRA_TRY(mlp_rows<true>(A, st));
+    // row slices: about an SM each for a 128 x 128 layer, at least 32 rows, at most 64 slices
+    WgradArgs W{};
+    W.n = n;
+    W.np = M->np;
+    W.rows = (int)std::max<int64_t>(32, ((n + 63) / 64 + 31) / 32 * 32);
+    const int slices = (int)((n + W.rows - 1) / W.rows);
+    const float* d[4] = {M->d1, M->d2, M->d3, M->dy};
+    const void* h[4] = {x, M->h1, M->h2, M->h3};
+    for (int l = 0; l < 4; ++l) {
+        W.d[l] = d[l];
+        W.h[l] = h[l];
+        W.din[l] = M->din[l];
+        W.dout[l] = M->dout[l];
+        W.off_w[l] = M->off_w[l];
+        W.off_b[l] = M->off_b[l];
+        W.ti[l] = (M->din[l] + 127) / 128;
+        W.tile0[l + 1] = W.tile0[l] + W.ti[l] * ((M->dout[l] + 127) / 128);
+    }
+    Scratch tmp(M->A);
+    MRA_TRY(tmp.get(&W.part, (size_t)slices * M->np));
+    k_mlp_wgrad<<<dim3(slices, W.tile0[4]), 256, 0, st>>>(W);
     MRA_CK_LAUNCH();
-    float* g = M->grad;
-    // layer 4 (linear), then back through the ReLU layers
-    MRA_TRY(wgrad<__half>(n, MLP_H, M->n_out, M->dy, M->h3, g + M->off_w[3], g + M->off_b[3], st));
-    MRA_TRY((dense<float, 2>(n, M->n_out, MLP_H, M->dy, w_rowmajor(M, 3), nullptr, M->h3, M->d3, st)));
-    MRA_TRY(wgrad<__half>(n, MLP_H, MLP_H, M->d3, M->h2, g + M->off_w[2], g + M->off_b[2], st));
-    MRA_TRY((dense<float, 2>(n, MLP_H, MLP_H, M->d3, w_rowmajor(M, 2), nullptr, M->h2, M->d2, st)));
-    MRA_TRY(wgrad<__half>(n, MLP_H, MLP_H, M->d2, M->h1, g + M->off_w[1], g + M->off_b[1], st));
-    MRA_TRY((dense<float, 2>(n, MLP_H, MLP_H, M->d2, w_rowmajor(M, 1), nullptr, M->h1, M->d1, st)));
-    MRA_TRY(wgrad<float>(n, M->n_in, MLP_H, M->d1, x, g + M->off_w[0], g + M->off_b[0], st));
+    k_mlp_wsum<<<(unsigned)std::min<int64_t>(num_sms() * 4, (M->np + 255) / 256), 256, 0, st>>>(M->np, slices, W.part, M->grad);
+    MRA_CK_LAUNCH();
     return MRA_OK;
 }
 
@@ -260,12 +438,8 @@ const mra_mlp* mlp_checked(const void* h) {
     return mlp_ok(M) ? M : nullptr;
 }
 int mlp_forward(const mra_mlp* M, const float* x, int64_t n, float* y, const Alloc& A, cudaStream_t st) {
-    Scratch tmp(A);
-    __half *h1, *h2, *h3;
-    MRA_TRY(tmp.get(&h1, (size_t)std::max<int64_t>(n, 1) * MLP_H));
-    MRA_TRY(tmp.get(&h2, (size_t)std::max<int64_t>(n, 1) * MLP_H));
-    MRA_TRY(tmp.get(&h3, (size_t)std::max<int64_t>(n, 1) * MLP_H));
-    return mlp_forward_impl(M, x, n, y, h1, h2, h3, st);
+    (void)A;
+    return mlp_rows<false>(mlp_args(M, x, n, y), st);
 }
 int mlp_n_in(const mra_mlp* M) { return M->n_in; }
 int mlp_n_out(const mra_mlp* M) { return M->n_out; }
