@@ -17,13 +17,19 @@
 // descriptor (constant strides) covers both outputs and both boxes; a piece's excluded
 // translations are zero tiles.
 //
-// One CTA per SM (202 KB of shared memory, all 512 TMEM columns), 15 warps with roles, so
-// that loading, MMAs and conversions run beside each other: warps 0-7 convert accumulators to
-// the next stage's operands (warps 0-3 the chunk's first half of the pieces, 4-7 the second),
-// 8-11 load X (two buffers; the blocks' power-of-two scales are made equal on the way),
-// 12 issues stage I into one of two accumulators, 13 and 14 issue stages II and III of a half
-// each.  Every wait is bounded: one that reaches its limit makes all roles stop, the error
-// word is set to 4 and the kernel frees its tensor memory.
+// One persistent CTA per SM (216 KB of shared memory, all 512 TMEM columns), 19 warps with roles
+// that meet at mbarriers only, so that setting up units, loading, MMAs and conversions overlap:
+//   0-7    convert accumulators to the next stage's operands, half of the pieces per four warps,
+//          two pieces ("a pair") at a time, so that a pair's MMAs run while the next is converted;
+//   8-11   load X (two buffers; the blocks' power-of-two scales are made equal on the way);
+//   12     issues stage I into one of two accumulators;
+//   13, 14 issue stages II and III of a half each;
+//   15-18  set up the next unit (pieces, inputs, scales, F tiles) in the other of two slots.
+// What bounds it is the shared-memory side of the tensor core: an MMA of stage II or III reads
+// 4 KB of A for 16 columns of output (23 % of the launch's cycles in the version whose units
+// were set up and finished by the whole CTA between barriers: 1.38 ms on 3-D Poisson k = 8).
+// Every wait is bounded: one that reaches its limit makes all roles stop, the error word is set
+// to 4 and the kernel frees its tensor memory.
 #include <cfloat>
 #include <climits>
 
@@ -33,7 +39,7 @@
 
 namespace mra {
 
-#define OTC_THREADS 480
+#define OTC_THREADS 608
 #define OTC_WAIT_LIMIT (1u << 24)
 #define OTC_WAIT_MIN 4096u
 #define OTC_P 8  // pieces per chunk
@@ -45,31 +51,41 @@ struct OtcSmem {
     static constexpr int A2_PIECE = 4 * A2_LBO;        // stage II: hi, lo (2 K groups each); stage III: a2' = 0, 1
     static constexpr int A2 = X + 2 * XBUF;
     static constexpr int TAB = 7 * OTC_P * 128;        // tiles [u 0..6][piece]
-    static constexpr int T = A2 + OTC_P * A2_PIECE;    // [direction][hi, lo]
-    static constexpr int Z = T + 6 * TAB;              // zeros: two tiles a tile row apart
-    static constexpr int TIN = Z + OTC_P * 128 + 128;  // 216 int
-    static constexpr int TG = TIN + 864;               // 216 float
-    static constexpr int LIST = TG + 864;              // pieces
+    static constexpr int T = A2 + OTC_P * A2_PIECE;    // per slot [direction][hi, lo]
+    static constexpr int Z = T + 12 * TAB;             // zeros: two tiles a tile row apart
+    static constexpr int TIN = Z + OTC_P * 128 + 128;  // per slot 216 int
+    static constexpr int TG = TIN + 2 * 864;           // per slot 216 float
+    static constexpr int LIST = TG + 2 * 864;          // pieces of the group being set up
     static size_t bytes(int M) { return LIST + 4 * (size_t)M * sizeof(uint32_t); }
 };
-static_assert(OtcSmem::LIST + 4 * MRA_MAX_TERMS * 4 + 1024 <= 232448, "shared memory of one CTA");
+static_assert(OtcSmem::LIST + 4 * MRA_MAX_TERMS * 4 + 2048 <= 232448, "shared memory of one CTA");
+
+// a unit as its roles see it
+struct OtcUnit {
+    int unit;            // -1: no more units
+    int npc, ps;         // pieces; tile stride (4 or 8 pieces)
+    unsigned m1, m2, m3; // boxes the pieces read, per direction
+    int nout;
+    unsigned leaf;       // leaf outputs
+    uint32_t piece[OTC_P];
+    float c2[OTC_P], c3[OTC_P], fin[OTC_P];
+};
 
 __global__ void __launch_bounds__(OTC_THREADS, 1) k_apply_oct_tc(OctTcArgs Q) {
     using L = OtcSmem;
     extern __shared__ __align__(1024) unsigned char sm[];
     __shared__ uint32_t s_tmem;
-    __shared__ __align__(8) uint64_t b_xf[2], b_xe[2], b_df[2], b_de[2], b_af[2], b_ae[2], b_vf[2];
+    // X full / empty, D_I full / empty; per half and pair: operands full, MMAs done; per slot: set up, done with;
+    // the second half's sums written, read
+    __shared__ __align__(8) uint64_t b_xf[2], b_xe[2], b_df[2], b_de[2], b_af[4], b_ae[4], b_sf[2], b_se[2], b_y, b_yr;
     __shared__ volatile int s_abort;
     __shared__ int s_unit, s_emin;
-    __shared__ unsigned s_leaf, s_xmax;
-    __shared__ float s_c2[OTC_P], s_c3[OTC_P], s_fin[OTC_P];
+    __shared__ unsigned s_xmax;
+    __shared__ OtcUnit s_u[2];
     const OctArgs& P = Q.P;
     if (P.skip && *P.skip != P.run_if) return;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const uint32_t sbase = tc::smem_u32(sm);
-    int* tin = (int*)(sm + L::TIN);
-    float* tg = (float*)(sm + L::TG);
-    uint32_t* list = (uint32_t*)(sm + L::LIST);
     for (int e = tid; e < L::TIN / 16; e += OTC_THREADS) ((uint4*)sm)[e] = make_uint4(0, 0, 0, 0);
     if (warp == 0) tc::tmem_alloc(&s_tmem, 512);
     if (tid == 0) {
@@ -78,9 +94,14 @@ __global__ void __launch_bounds__(OTC_THREADS, 1) k_apply_oct_tc(OctTcArgs Q) {
             tc::mbar_init(&b_xe[i], 1);
             tc::mbar_init(&b_df[i], 1);
             tc::mbar_init(&b_de[i], 256);
+            tc::mbar_init(&b_sf[i], 128);
+            tc::mbar_init(&b_se[i], 128 + 256 + 3);
+        }
+        tc::mbar_init(&b_y, 128);
+        tc::mbar_init(&b_yr, 128);
+        for (int i = 0; i < 4; ++i) {
             tc::mbar_init(&b_af[i], 128);
             tc::mbar_init(&b_ae[i], 1);
-            tc::mbar_init(&b_vf[i], 1);
         }
         s_abort = 0;
     }
@@ -89,411 +110,493 @@ __global__ void __launch_bounds__(OTC_THREADS, 1) k_apply_oct_tc(OctTcArgs Q) {
     __syncthreads();
     tc::fence_after();
     const uint32_t tbase = s_tmem;
-    // TMEM columns: D_I 2 x 128; per half D_II 4 pieces x 16 at 256 + 64 half, and D_III 4 pieces
-    // x 2 a2' x 16: the first two pieces' at 384 + 64 half, the others' over D_II, which stage III
-    // has no more use for
+    // TMEM columns: D_I 2 x 128; D_II 16 per piece at 256 + 64 half; D_III 2 a2' x 16 per piece: a
+    // pair's first piece at 384 + 64 half, its second over the pair's D_II, which stage III no longer
+    // needs
     auto cII = [&](int h, int lp) { return tbase + 256u + (uint32_t)(h * 64 + lp * 16); };
-    auto cIII = [&](int h, int lp, int a) { return tbase + (lp < 2 ? 384u : 256u) + (uint32_t)(h * 64 + (lp & 1) * 32 + a * 16); };
-    // running counts of lines, stage II / III batches and planes: every role counts the same
-    uint32_t line0 = 0, batch0 = 0, plane0 = 0;
-    bool stop = false;
+    auto cIII = [&](int h, int lp, int a) { return tbase + ((lp & 1) ? 256u : 384u) + (uint32_t)(h * 64 + (lp >> 1) * 32 + a * 16); };
 #define OTC_WAIT(bar, parity) tc::mbar_wait_or(bar, parity, Q.wait_limit, &s_abort)
     // the same by a whole warp, whose lanes go on or give up together (what follows is warp-collective)
 #define OTC_WAITW(bar, parity) __all_sync(0xffffffffu, OTC_WAIT(bar, parity))
+    // barriers complete once per use; a use's parity is its running number's lowest bit
+    uint32_t ln = 0;  // lines (pairs of boxes b2) so far
 
-    while (!stop) {
-        if (tid == 0) s_unit = atomicAdd(Q.counter, 1);
-        __syncthreads();
-        const int unit = s_unit;
-        if (unit >= Q.nunits) break;
-        const int g = P.g0 + unit / P.ns, sl = unit % P.ns, np = P.np[g], q0 = sl * OTC_P;
-        if (q0 >= np) {
-            __syncthreads();
-            continue;
-        }
-        const int npc = min(OTC_P, np - q0), ps = npc <= 4 ? 4 : 8, ph = ps / 2;
-        const int i0 = P.first[g], tree = P.node_tree ? P.node_tree[i0] : 0;
-        const int j = P.coord[4 * i0], nout = j ? 8 : 1;
-        if (tid == 0) {
-            s_emin = INT_MAX;
-            s_xmax = 0u;
-        }
-        if (warp == 14) {
-            const unsigned lf = __ballot_sync(0xffffffffu, lane < nout && P.leaf[i0 + (lane < nout ? lane : 0)]);
-            if (lane == 0) s_leaf = lf;
-            oct_pieces(P.sched + (size_t)tree * P.sl, P.M, P.lm, j, lf != 0, lf != (1u << nout) - 1u, list);
-        }
-        __syncthreads();
-        // the inputs: the neighbourhood's smallest scale and largest value
-        int in = -1;
-        float sxb = 0.0f;
-        if (tid < 216) {
-            in = P.in[(size_t)g * 216 + tid];
-            tin[tid] = in;
-            if (in >= 0) {
-                sxb = Q.sx[in];
-                int e;
-                frexpf(sxb, &e);
-                atomicMin(&s_emin, e);
-                atomicMax(&s_xmax, __float_as_uint(Q.xmax[in]));  // non-negative floats order as ints
-            }
-        } else {
-            // F tiles of the chunk, masked by the pieces' sets
-            for (int e = tid - 216; e < 7 * ps * 8 * 6; e += OTC_THREADS - 216) {
-                const int v = e & 7, pc = (e >> 3) % ps, r = (e >> 3) / ps, u = r % 7, dh = r / 7;
-                const int d = dh >> 1, hl = dh & 1;
-                uint4 x = make_uint4(0, 0, 0, 0);
-                if (pc < npc) {
-                    const uint32_t p = list[q0 + pc];
-                    const int set = (p >> (20 - 2 * d)) & 3;
-                    if (set & ((u >= 2 && u <= 4) ? 1 : 2))
-                        x = ((const uint4*)(hl ? Q.Fl : Q.Fh))[(((size_t)j * P.M + (p & 0xffff)) * 7 + 6 - u) * 8 + v];
+    if (warp >= 15) {
+        // ================= set up units
+        const int t = tid - 480;
+        uint32_t* list = (uint32_t*)(sm + L::LIST);
+        auto sync = [] { asm volatile("bar.sync 2, 128;" ::: "memory"); };
+        for (uint32_t k = 0;; ++k) {
+            const int slot = k & 1;
+            bool ok = k < 2 || OTC_WAIT(&b_se[slot], ((k >> 1) - 1) & 1);
+            OtcUnit& U = s_u[slot];
+            int* tin = (int*)(sm + L::TIN + slot * 864);
+            float* tg = (float*)(sm + L::TG + slot * 864);
+            int unit, g, np, q0;
+            for (;;) {  // the next unit that has pieces and inputs (one without inputs is zero)
+                if (t == 0) {
+                    int u = ok ? atomicAdd(Q.counter, 1) : Q.nunits;
+                    while (u < Q.nunits && (u % P.ns) * OTC_P >= P.np[P.g0 + u / P.ns]) u = atomicAdd(Q.counter, 1);
+                    s_unit = u;
+                    s_emin = INT_MAX;
+                    s_xmax = 0u;
                 }
-                ((uint4*)(sm + L::T + dh * L::TAB))[(u * ps + pc) * 8 + v] = x;
-            }
-        }
-        __syncthreads();
-        const float xmax = __uint_as_float(s_xmax);
-        const int es = s_emin - 1;  // the common scale 2^es
-        if (!(xmax <= FLT_MAX) && tid == 0) atomicExch(Q.err, 5);  // input values beyond FP32's range
-        const bool live = xmax > 0.0f && xmax <= FLT_MAX;
-        if (tid < 216) tg[tid] = in < 0 ? 0.0f : ldexpf(1.0f, es) / sxb;
-        if (warp == 14 && live) {
-            // power-of-two scales as in apply_tc.cu: sW = 2^eW, the largest power of two <=
-            // 8192 / (48 max|F| max|x|), and sV = 2^eV <= 8192 / (48^2 max|F|^2 max|x|)
-            if (lane < OTC_P) {
-                float c2 = 0.0f, c3 = 0.0f, fin = 0.0f;
-                if (lane < npc) {
-                    const int m = list[q0 + lane] & 0xffff;
-                    const size_t jm = (size_t)j * P.M + m;
-                    const float mf = Q.maxF[jm], sf = Q.sF[jm];
-                    if (mf > 0.0f) {
-                        int em, ex, ef, e1, e2;
-                        const float fm = frexpf(mf, &em), fx = frexpf(xmax, &ex);
-                        frexpf(sf, &ef);
-                        ef -= 1;
-                        frexpf(8192.0f / (48.0f * fm * fx), &e1);
-                        frexpf(8192.0f / (2304.0f * fm * fm * fx), &e2);
-                        const int eW = min(e1 - 1 - em - ex, 126), eV = min(e2 - 1 - 2 * em - ex, 126);
-                        if (eW >= -126 && eV >= -126) {
-                            c2 = ldexpf(1.0f, eW - ef - es);            // sW / (sF sx)
-                            c3 = ldexpf(1.0f, eV - eW - ef);            // sV / (sW sF)
-                            fin = ldexpf((float)P.w[m], -(eV + ef));    // w_m / (sV sF)
-                            if (!(fin <= FLT_MAX)) {  // outputs beyond the FP32 range: refuse
-                                atomicExch(Q.err, 5);
-                                fin = 0.0f;
-                            }
-                        }
+                sync();
+                unit = s_unit;
+                if (unit >= Q.nunits) break;
+                g = P.g0 + unit / P.ns;
+                q0 = (unit % P.ns) * OTC_P;
+                np = P.np[g];
+                const int i0 = P.first[g], j = P.coord[4 * i0], nout = j ? 8 : 1;
+                const size_t fb = (size_t)j * P.M;
+                int in[2] = {-1, -1};
+                float sx[2] = {1.0f, 1.0f};
+#pragma unroll
+                for (int r = 0; r < 2; ++r)
+                    if (t + 128 * r < 216) in[r] = P.in[(size_t)g * 216 + t + 128 * r];
+#pragma unroll
+                for (int r = 0; r < 2; ++r)
+                    if (in[r] >= 0) {
+                        sx[r] = Q.sx[in[r]];
+                        int e;
+                        frexpf(sx[r], &e);
+                        atomicMin(&s_emin, e);
+                        atomicMax(&s_xmax, __float_as_uint(Q.xmax[in[r]]));  // non-negative floats order as ints
+                    }
+                if (warp == 15) {
+                    const unsigned lf = __ballot_sync(0xffffffffu, lane < nout && P.leaf[i0 + (lane < nout ? lane : 0)]);
+                    const int tree = P.node_tree ? P.node_tree[i0] : 0;
+                    oct_pieces(P.sched + (size_t)tree * P.sl, P.M, P.lm, j, lf != 0, lf != (1u << nout) - 1u, list);
+                    __syncwarp();
+                    const int npc = min(OTC_P, np - q0);
+                    unsigned m1 = 0, m2 = 0, m3 = 0;
+                    for (int pc = 0; pc < npc; ++pc) {
+                        const uint32_t p = list[q0 + pc];
+                        m1 |= set_boxes((p >> 20) & 3);
+                        m2 |= set_boxes((p >> 18) & 3);
+                        m3 |= set_boxes((p >> 16) & 3);
+                    }
+                    if (lane < OTC_P) U.piece[lane] = lane < npc ? list[q0 + lane] : 0u;
+                    if (lane == 0) {
+                        U.unit = unit;
+                        U.npc = npc;
+                        U.ps = npc <= 4 ? 4 : 8;
+                        U.m1 = m1;
+                        U.m2 = m2;
+                        U.m3 = m3;
+                        U.nout = nout;
+                        U.leaf = lf;
                     }
                 }
-                s_c2[lane] = c2;
-                s_c3[lane] = c3;
-                s_fin[lane] = fin;
-            }
-        }
-        // boxes any piece reads, per direction
-        unsigned m1 = 0, m2 = 0, m3 = 0;
-        for (int pc = 0; pc < npc; ++pc) {
-            const uint32_t p = list[q0 + pc];
-            m1 |= set_boxes((p >> 20) & 3);
-            m2 |= set_boxes((p >> 18) & 3);
-            m3 |= set_boxes((p >> 16) & 3);
-        }
-        const int s1 = m1 == 0x1e ? 1 : 0, s2 = m2 == 0x1e ? 1 : 0;   // first box of the first pair
-        const int n1 = m1 == 0x1e ? 2 : 3, n2 = m2 == 0x1e ? 2 : 3;   // pairs
-        tc::fence_async_smem();
-        __syncthreads();
-        float* part = (float*)Q.part + (size_t)unit * 8 * P.k * P.k * P.k;
-        uint32_t nline = 0, nplane = 0;  // lines and planes of this unit
-        if (live) {
-            for (int b3 = 0; b3 < 6; ++b3) nplane += (m3 >> b3) & 1u;
-            for (int q = 0; q < n2; ++q) nline += ((m2 >> (s2 + 2 * q)) & 3u) != 0;
-            const uint32_t lpp = nline;  // lines (pairs) per plane
-            nline *= nplane;
-            float* ysum = (float*)(sm + L::A2 + ph * L::A2_PIECE);  // 32 x 128
-            if (warp >= 8 && warp < 12) {
-                // ---- X of a pair of lines into a buffer
-                const int lt = tid - 256, hl = lt >> 6, v = lt & 63;
-                const __half* src0 = hl ? Q.xl : Q.xh;
-                uint32_t ln = line0;
-                bool ok = true;
-                for (int b3 = 0; b3 < 6 && ok; ++b3) {
-                    if (!((m3 >> b3) & 1u)) continue;
-                    for (int q = 0; q < n2 && ok; ++q) {
-                        const int b2 = s2 + 2 * q;
-                        if (!((m2 >> b2) & 3u)) continue;
-                        const int buf = ln & 1;
-                        uint4 x[12];
-                        float gs[12];
+                sync();
+                const float xmax = __uint_as_float(s_xmax);
+                const int es = s_emin - 1;  // the common scale 2^es
+                if (!(xmax <= FLT_MAX) && t == 0) atomicExch(Q.err, 5);  // input values beyond FP32's range
+                if (!(xmax > 0.0f && xmax <= FLT_MAX)) {
+                    const int k3 = P.k * P.k * P.k;
+                    for (int e = t; e < nout * k3; e += 128) ((float*)Q.part)[(size_t)unit * 8 * k3 + e] = 0.0f;
+                    sync();
+                    continue;
+                }
 #pragma unroll
-                        for (int r = 0; r < 12; ++r) {  // r = (b1, line)
-                            const int b1 = s1 + (r >> 1), qq = b1 * 36 + (b2 + (r & 1)) * 6 + b3;
-                            gs[r] = 0.0f;
-                            x[r] = make_uint4(0, 0, 0, 0);
-                            if ((r >> 1) < 2 * n1 && ((m1 >> b1) & 1u)) {
-                                const int b = tin[qq];
-                                if (b >= 0) {
-                                    gs[r] = tg[qq];
-                                    x[r] = __ldg((const uint4*)(src0 + (size_t)b * 512) + v);
+                for (int r = 0; r < 2; ++r)
+                    if (t + 128 * r < 216) {
+                        tin[t + 128 * r] = in[r];
+                        tg[t + 128 * r] = in[r] < 0 ? 0.0f : ldexpf(1.0f, es) / sx[r];
+                    }
+                // F tiles, masked by the pieces' sets
+                const int ps = U.ps, lp = ps == 8 ? 3 : 2;
+                for (int e = t; e < 7 * 6 * 8 * ps; e += 128) {
+                    const int v = e & 7, pc = (e >> 3) & (ps - 1), r = e >> (3 + lp), u = r % 7, dh = r / 7;
+                    uint4 x = make_uint4(0, 0, 0, 0);
+                    if (pc < U.npc) {
+                        const uint32_t p = U.piece[pc];
+                        const int set = (p >> (20 - 2 * (dh >> 1))) & 3;
+                        if (set & ((u >= 2 && u <= 4) ? 1 : 2))
+                            x = __ldg((const uint4*)((dh & 1) ? Q.Fl : Q.Fh) + ((fb + (p & 0xffff)) * 7 + 6 - u) * 8 + v);
+                    }
+                    ((uint4*)(sm + L::T + (slot * 6 + dh) * L::TAB))[(u * ps + pc) * 8 + v] = x;
+                }
+                // power-of-two scales as in apply_tc.cu: sW = 2^eW, the largest power of two <=
+                // 8192 / (48 max|F| max|x|), and sV = 2^eV <= 8192 / (48^2 max|F|^2 max|x|)
+                if (t < OTC_P) {
+                    float c2 = 0.0f, c3 = 0.0f, fin = 0.0f;
+                    if (t < U.npc) {
+                        const int m = U.piece[t] & 0xffff;
+                        const float mf = Q.maxF[fb + m], sf = Q.sF[fb + m];
+                        if (mf > 0.0f) {
+                            int em, ex, ef, e1, e2;
+                            const float fm = frexpf(mf, &em), fx = frexpf(xmax, &ex);
+                            frexpf(sf, &ef);
+                            ef -= 1;
+                            frexpf(8192.0f / (48.0f * fm * fx), &e1);
+                            frexpf(8192.0f / (2304.0f * fm * fm * fx), &e2);
+                            const int eW = min(e1 - 1 - em - ex, 126), eV = min(e2 - 1 - 2 * em - ex, 126);
+                            if (eW >= -126 && eV >= -126) {
+                                c2 = ldexpf(1.0f, eW - ef - es);            // sW / (sF sx)
+                                c3 = ldexpf(1.0f, eV - eW - ef);            // sV / (sW sF)
+                                fin = ldexpf((float)P.w[m], -(eV + ef));    // w_m / (sV sF)
+                                if (!(fin <= FLT_MAX)) {  // outputs beyond the FP32 range: refuse
+                                    atomicExch(Q.err, 5);
+                                    fin = 0.0f;
                                 }
                             }
                         }
-                        if (ln >= 2) ok = OTC_WAIT(&b_xe[buf], ((ln >> 1) - 1) & 1);
-                        if (!ok) break;
-                        unsigned char* dst = sm + L::X + buf * L::XBUF + hl * (L::XBUF / 2) + v * 16;
-#pragma unroll
-                        for (int r = 0; r < 12; ++r) {
-                            if ((r >> 1) >= 2 * n1) break;
-                            const __half2 g2 = __float2half2_rn(gs[r]);
-                            __half2* h = (__half2*)&x[r];
-#pragma unroll
-                            for (int i = 0; i < 4; ++i) h[i] = __hmul2(h[i], g2);
-                            *(uint4*)(dst + r * 1024) = x[r];
-                        }
-                        tc::fence_async_smem();
-                        tc::mbar_arrive(&b_xf[buf]);
-                        ++ln;
                     }
+                    U.c2[t] = c2;
+                    U.c3[t] = c3;
+                    U.fin[t] = fin;
                 }
-            } else if (warp == 12) {
-                // ---- stage I
-                if (lane == 0 && !Q.withhold) {
-                    const uint32_t id = tc::idesc_f16(128, 16 * ps);
-                    uint32_t ln = line0;
-                    for (uint32_t l = 0; l < nline; ++l, ++ln) {
-                        const int buf = ln & 1;
-                        if (!OTC_WAIT(&b_xf[buf], (ln >> 1) & 1)) break;
-                        if (ln >= 2 && !OTC_WAIT(&b_de[buf], ((ln >> 1) - 1) & 1)) break;
-                        tc::fence_after();
-                        const uint32_t d = tbase + buf * 128;
-                        const uint64_t xh = tc::sdesc(sbase + L::X + buf * L::XBUF, 2048, 128);
-                        const uint64_t th = tc::sdesc(sbase + L::T + s1 * ps * 128, ps * 128, 128);
-                        for (int s = 0; s < n1; ++s) {  // boxes s1 + 2 s, + 1
-                            const uint64_t ah = xh + (uint64_t)(s * (4096 / 16)), al = ah + L::XBUF / 32;
-                            const uint64_t bh = th + (uint64_t)(s * 2 * ps * 8), bl = bh + L::TAB / 16;
-                            tc::mma_f16(d, ah, bh, id, s > 0);
-                            tc::mma_f16(d, ah, bl, id, 1);
-                            tc::mma_f16(d, al, bh, id, 1);
+                break;
+            }
+            if (unit >= Q.nunits && t == 0) U.unit = -1;
+            tc::fence_async_smem();
+            tc::mbar_arrive(&b_sf[slot]);
+            if (unit >= Q.nunits) break;
+            sync();  // s_unit and the scale words are free again
+        }
+    } else if (warp >= 8 && warp < 12) {
+        // ================= X of a pair of lines into a buffer
+        const int lt = tid - 256, hl = lt >> 6, v = lt & 63;
+        const uint4* src0 = (const uint4*)(hl ? Q.xl : Q.xh) + v;
+        bool ok = true;
+        for (uint32_t k = 0; ok; ++k) {
+            const int slot = k & 1;
+            ok = OTC_WAIT(&b_sf[slot], (k >> 1) & 1);
+            if (!ok || s_u[slot].unit < 0) break;
+            const unsigned m1 = s_u[slot].m1, m2 = s_u[slot].m2, m3 = s_u[slot].m3;
+            const int s1 = m1 == 0x1e, s2 = m2 == 0x1e, n1 = 3 - s1, n2 = 3 - s2;
+            const int* tin = (const int*)(sm + L::TIN + slot * 864);
+            const float* tg = (const float*)(sm + L::TG + slot * 864);
+            for (int b3 = 0; b3 < 6 && ok; ++b3) {
+                if (!((m3 >> b3) & 1u)) continue;
+                for (int q = 0; q < n2 && ok; ++q) {
+                    const int b2 = s2 + 2 * q, buf = ln & 1;
+                    if (!((m2 >> b2) & 3u)) continue;
+                    uint4 x[12];
+                    float gs[12];
+#pragma unroll
+                    for (int r = 0; r < 12; ++r) {  // r = (b1, line)
+                        const int b1 = s1 + (r >> 1), qq = b1 * 36 + (b2 + (r & 1)) * 6 + b3;
+                        gs[r] = 0.0f;
+                        x[r] = make_uint4(0, 0, 0, 0);
+                        if ((r >> 1) < 2 * n1 && ((m1 >> b1) & 1u)) {
+                            const int b = tin[qq];
+                            if (b >= 0) {
+                                gs[r] = tg[qq];
+                                x[r] = __ldg(src0 + (size_t)b * 64);
+                            }
                         }
-                        tc::commit(&b_xe[buf]);
-                        tc::commit(&b_df[buf]);
                     }
+                    if (ln >= 2) ok = OTC_WAIT(&b_xe[buf], ((ln >> 1) - 1) & 1);
+                    if (!ok) break;
+                    unsigned char* dst = sm + L::X + buf * L::XBUF + hl * (L::XBUF / 2) + v * 16;
+#pragma unroll
+                    for (int r = 0; r < 12; ++r) {
+                        if ((r >> 1) >= 2 * n1) break;
+                        const __half2 g2 = __float2half2_rn(gs[r]);
+                        __half2* hv = (__half2*)&x[r];
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) hv[i] = __hmul2(hv[i], g2);
+                        *(uint4*)(dst + r * 1024) = x[r];
+                    }
+                    tc::fence_async_smem();
+                    tc::mbar_arrive(&b_xf[buf]);
+                    ++ln;
                 }
-            } else if (warp >= 13) {
-                // ---- stages II and III of one half of the pieces
-                if (lane == 0) {
-                    const int h = warp - 13, pl = min(npc, h * ph), pe = min(npc, h * ph + ph);
-                    const uint32_t id = tc::idesc_f16(128, 16);
-                    uint32_t bt = batch0;
-                    bool ok = true;
-                    for (int b3 = 0; b3 < 6 && ok; ++b3) {
-                        if (!((m3 >> b3) & 1u)) continue;
-                        bool first = true;
-                        for (int q = 0; q < n2 && ok; ++q) {
-                            const int b2 = s2 + 2 * q;
-                            if (!((m2 >> b2) & 3u)) continue;
-                            ok = OTC_WAIT(&b_af[h], bt & 1);
+            }
+            tc::mbar_arrive(&b_se[slot]);
+        }
+    } else if (warp == 12) {
+        // ================= stage I
+        if (lane == 0 && !Q.withhold) {
+            bool ok = true;
+            for (uint32_t k = 0; ok; ++k) {
+                const int slot = k & 1;
+                ok = OTC_WAIT(&b_sf[slot], (k >> 1) & 1);
+                if (!ok || s_u[slot].unit < 0) break;
+                const unsigned m1 = s_u[slot].m1, m2 = s_u[slot].m2, m3 = s_u[slot].m3;
+                const int s1 = m1 == 0x1e, s2 = m2 == 0x1e, n1 = 3 - s1, n2 = 3 - s2, ps = s_u[slot].ps;
+                const uint32_t id = tc::idesc_f16(128, 16 * ps);
+                const uint64_t th = tc::sdesc(sbase + L::T + slot * 6 * L::TAB + s1 * ps * 128, ps * 128, 128);
+                int lines = 0;
+                for (int q = 0; q < n2; ++q) lines += ((m2 >> (s2 + 2 * q)) & 3u) != 0;
+                lines *= __popc(m3);
+                for (int l = 0; l < lines && ok; ++l, ++ln) {
+                    const int buf = ln & 1;
+                    ok = OTC_WAIT(&b_xf[buf], (ln >> 1) & 1) && (ln < 2 || OTC_WAIT(&b_de[buf], ((ln >> 1) - 1) & 1));
+                    if (!ok) break;
+                    tc::fence_after();
+                    const uint32_t d = tbase + buf * 128;
+                    const uint64_t xh = tc::sdesc(sbase + L::X + buf * L::XBUF, 2048, 128);
+#pragma unroll
+                    for (int s = 0; s < 3; ++s) {  // boxes s1 + 2 s, + 1
+                        if (s >= n1) break;
+                        const uint64_t ah = xh + (uint64_t)(s * (4096 / 16)), al = ah + L::XBUF / 32;
+                        const uint64_t bh = th + (uint64_t)(s * 2 * ps * 8), bl = bh + L::TAB / 16;
+                        tc::mma_f16(d, ah, bh, id, s > 0);
+                        tc::mma_f16(d, ah, bl, id, 1);
+                        tc::mma_f16(d, al, bh, id, 1);
+                    }
+                    tc::commit(&b_xe[buf]);
+                    tc::commit(&b_df[buf]);
+                }
+                tc::commit(&b_se[slot]);
+            }
+        }
+    } else if (warp >= 13) {
+        // ================= stages II and III of one half of the pieces
+        if (lane == 0) {
+            const int h = warp - 13;
+            uint32_t bt[2] = {0, 0};  // batches so far, per pair
+            bool ok = true;
+            const uint32_t id = tc::idesc_f16(128, 16);
+            for (uint32_t k = 0; ok; ++k) {
+                const int slot = k & 1;
+                ok = OTC_WAIT(&b_sf[slot], (k >> 1) & 1);
+                if (!ok || s_u[slot].unit < 0) break;
+                const unsigned m2 = s_u[slot].m2, m3 = s_u[slot].m3;
+                const int s2 = m2 == 0x1e, n2 = 3 - s2, ps = s_u[slot].ps, ph = ps / 2;
+                const int pl = min(s_u[slot].npc, h * ph), n = min(s_u[slot].npc, h * ph + ph) - pl;
+                const uint32_t tab = sbase + L::T + slot * 6 * L::TAB;
+                for (int b3 = 0; b3 < 6 && ok; ++b3) {
+                    if (!((m3 >> b3) & 1u)) continue;
+                    bool first = true;
+                    for (int q = 0; q < n2 && ok; ++q) {
+                        const int b2 = s2 + 2 * q;
+                        if (!((m2 >> b2) & 3u)) continue;
+#pragma unroll
+                        for (int pp = 0; pp < 2; ++pp) {
+                            if (2 * pp >= n) break;
+                            ok = OTC_WAIT(&b_af[2 * h + pp], bt[pp] & 1);
                             if (!ok) break;
                             tc::fence_after();
-                            for (int pc = pl; pc < pe; ++pc) {
-                                const uint32_t d = cII(h, pc - pl);
+#pragma unroll
+                            for (int r = 0; r < 2; ++r) {
+                                const int lp = 2 * pp + r, pc = pl + lp;
+                                if (lp >= n) break;
+                                const uint32_t d = cII(h, lp);
                                 const uint64_t ah = tc::sdesc(sbase + L::A2 + pc * L::A2_PIECE, L::A2_LBO, L::A2_SBO);
                                 const uint64_t al = ah + 2 * L::A2_LBO / 16;
-                                const uint64_t bh = tc::sdesc(sbase + L::T + 2 * L::TAB + (b2 * ps + pc) * 128, ps * 128,
-                                                              ps * 128);
+                                const uint64_t bh = tc::sdesc(tab + 2 * L::TAB + (b2 * ps + pc) * 128, ps * 128, ps * 128);
                                 const uint64_t bl = bh + L::TAB / 16;
                                 tc::mma_f16(d, ah, bh, id, first ? 0u : 1u);
                                 tc::mma_f16(d, ah, bl, id, 1);
                                 tc::mma_f16(d, al, bh, id, 1);
                             }
-                            first = false;
-                            tc::commit(&b_ae[h]);
-                            ++bt;
+                            tc::commit(&b_ae[2 * h + pp]);
+                            ++bt[pp];
                         }
-                        if (!ok) break;
-                        tc::commit(&b_vf[h]);
-                        ok = OTC_WAIT(&b_af[h], bt & 1);
+                        first = false;
+                    }
+                    if (!ok) break;
+#pragma unroll
+                    for (int pp = 0; pp < 2; ++pp) {
+                        if (2 * pp >= n) break;
+                        ok = OTC_WAIT(&b_af[2 * h + pp], bt[pp] & 1);
                         if (!ok) break;
                         tc::fence_after();
-                        for (int pc = pl; pc < pe; ++pc) {
-                            const uint32_t tile = sbase + L::T + 4 * L::TAB + (b3 * ps + pc) * 128;
+#pragma unroll
+                        for (int r = 0; r < 2; ++r) {
+                            const int lp = 2 * pp + r, pc = pl + lp;
+                            if (lp >= n) break;
+                            const uint32_t tile = tab + 4 * L::TAB + (b3 * ps + pc) * 128;
                             const uint64_t bh = tc::sdesc(tile, 0, ps * 128);  // [F_hi ; F_hi]
                             const uint64_t bl = tc::sdesc(tile + L::TAB, sbase + L::Z - tile - L::TAB, ps * 128);  // [F_lo ; 0]
+#pragma unroll
                             for (int a = 0; a < 2; ++a) {
-                                const uint32_t d = cIII(h, pc - pl, a);
-                                const uint64_t av = tc::sdesc(sbase + L::A2 + pc * L::A2_PIECE + a * 2 * L::A2_LBO,
-                                                              L::A2_LBO, L::A2_SBO);
-                                tc::mma_f16(d, av, bh, id, 0);
-                                tc::mma_f16(d, av, bl, id, 1);
+                                const uint64_t av = tc::sdesc(sbase + L::A2 + pc * L::A2_PIECE + a * 2 * L::A2_LBO, L::A2_LBO,
+                                                              L::A2_SBO);
+                                tc::mma_f16(cIII(h, lp, a), av, bh, id, 0);
+                                tc::mma_f16(cIII(h, lp, a), av, bl, id, 1);
                             }
                         }
-                        tc::commit(&b_ae[h]);
-                        ++bt;
+                        tc::commit(&b_ae[2 * h + pp]);
+                        ++bt[pp];
                     }
                 }
-            } else if (warp < 8) {
-                // ---- conversions of one half of the pieces
-                const int h = warp >> 2, w4 = warp & 3, pl = min(npc, h * ph), n = min(npc, h * ph + ph) - pl;
-                const uint32_t lane_off = (uint32_t)(w4 * 32) << 16;
-                const int mi = lane >> 3, mr = lane & 7;  // this lane's matrix and row of a stmatrix
-                // D_I: lanes (line, i3, i2) -> rows (a1', c1 | i3), K = (line, i2); matrices hi, lo of two i3
-                const uint32_t rowI = sbase + L::A2 + (mi & 1) * 2 * L::A2_LBO + (w4 >> 1) * L::A2_LBO + mr * L::A2_SBO +
-                                      ((w4 & 1) * 4 + (mi >> 1)) * 16;
-                // D_II: lanes (a1', c1, i3) -> rows (a1' c1 | c2), K = hi | lo; matrices hi, lo of two (a1', c1)
-                const uint32_t rowII = sbase + L::A2 + (mi & 1) * L::A2_LBO + (w4 * 4 + (mi >> 1)) * L::A2_SBO + mr * 16;
-                uint32_t ln = line0, bt = batch0, pn = plane0;
-                bool ok = true;
-                float y[2][16];  // [a2'][(a3', c3)] of lane (a1', c1, c2), this half's pieces
+                tc::commit(&b_se[slot]);
+            }
+        }
+    } else {
+        // ================= conversions of one half of the pieces, and the outputs
+        const int h = warp >> 2, w4 = warp & 3;
+        const uint32_t lane_off = (uint32_t)(w4 * 32) << 16;
+        const int mi = lane >> 3, mr = lane & 7;  // this lane's matrix and row of a stmatrix
+        // D_I: lanes (line, i3, i2) -> rows (a1', c1 | i3), K = (line, i2); matrices hi, lo of two i3
+        const uint32_t rowI = sbase + L::A2 + (mi & 1) * 2 * L::A2_LBO + (w4 >> 1) * L::A2_LBO + mr * L::A2_SBO +
+                              ((w4 & 1) * 4 + (mi >> 1)) * 16;
+        // D_II: lanes (a1', c1, i3) -> rows (a1' c1 | c2), K = hi | lo; matrices hi, lo of two (a1', c1)
+        const uint32_t rowII = sbase + L::A2 + (mi & 1) * L::A2_LBO + (w4 * 4 + (mi >> 1)) * L::A2_SBO + mr * 16;
+        uint32_t bt[2] = {0, 0}, ny = 0;
+        bool ok = true;
+        for (uint32_t k = 0; ok; ++k) {
+            const int slot = k & 1;
+            ok = OTC_WAITW(&b_sf[slot], (k >> 1) & 1);
+            const OtcUnit& U = s_u[slot];
+            if (!ok || U.unit < 0) break;
+            const unsigned m2 = U.m2;
+            const int ps = U.ps, ph = ps / 2, npc = U.npc, nplane = __popc(U.m3);
+            const int pl = min(npc, h * ph), n = min(npc, h * ph + ph) - pl;
+            const int s2 = m2 == 0x1e, n2 = 3 - s2;
+            int lpp = 0;  // lines per plane
+            for (int q = 0; q < n2; ++q) lpp += ((m2 >> (s2 + 2 * q)) & 3u) != 0;
+            float y[2][16];  // [a2'][(a3', c3)] of lane (a1', c1, c2), this half's pieces
 #pragma unroll
-                for (int c = 0; c < 16; ++c) y[0][c] = y[1][c] = 0.0f;
-                // outputs a2', a3' of this lane that are leaves: bit 2 a2' + a3'
-                unsigned lf = 0;
-                for (int q = 0; q < 4; ++q) lf |= ((s_leaf >> ((1 - (w4 >> 1)) * 4 + (1 - (q >> 1)) * 2 + 1 - (q & 1))) & 1u) << q;
-                // y += fin Y of the plane whose stage III has completed
-                auto add_plane = [&]() {
+            for (int c = 0; c < 16; ++c) y[0][c] = y[1][c] = 0.0f;
+            // outputs a2', a3' of this lane that are leaves: bit 2 a2' + a3'
+            unsigned lf = 0;
+            for (int q = 0; q < 4; ++q) lf |= ((U.leaf >> ((1 - (w4 >> 1)) * 4 + (1 - (q >> 1)) * 2 + 1 - (q & 1))) & 1u) << q;
+            // y += fin Y of a pair whose stage III of a plane has completed
+            auto add_pair = [&](int pp) {
 #pragma unroll
-                    for (int pc = 0; pc < 4; ++pc) {
-                        if (pc >= n) break;
-                        const float fin = s_fin[pl + pc];
-                        const bool leaf_only = (list[q0 + pl + pc] >> 24) != 0;
+                for (int r = 0; r < 2; ++r) {
+                    const int lp = 2 * pp + r;
+                    if (lp >= n) break;
+                    const float fin = U.fin[pl + lp];
+                    const bool leaf_only = (U.piece[pl + lp] >> 24) != 0;
 #pragma unroll
-                        for (int a = 0; a < 2; ++a) {
-                            float t[16];
-                            tc::tmem_ld32x16(cIII(h, pc, a) + lane_off, t);
+                    for (int a = 0; a < 2; ++a) {
+                        float t[16];
+                        tc::tmem_ld32x16(cIII(h, lp, a) + lane_off, t);
 #pragma unroll
-                            for (int c = 0; c < 16; ++c) {
-                                const float f = leaf_only && !((lf >> (2 * a + (c >> 3))) & 1u) ? 0.0f : fin;
-                                y[a][c] = fmaf(f, t[c], y[a][c]);
-                            }
+                        for (int c = 0; c < 16; ++c) {
+                            const float f = leaf_only && !((lf >> (2 * a + (c >> 3))) & 1u) ? 0.0f : fin;
+                            y[a][c] = fmaf(f, t[c], y[a][c]);
                         }
                     }
-                };
-                for (uint32_t p = 0; p < nplane && ok; ++p, ++pn) {
-                    for (uint32_t q = 0; q < lpp && ok; ++q, ++ln, ++bt) {
-                        const int buf = ln & 1;
-                        // the last batch is complete: the operands are free, and after a stage III
-                        // its result is whole
-                        if (bt > 0) ok = OTC_WAITW(&b_ae[h], (bt - 1) & 1);
-                        if (ok && p > 0 && q == 0) {
-                            tc::fence_after();
-                            add_plane();
+                }
+            };
+            for (int p = 0; p < nplane && ok; ++p) {
+                for (int q = 0; q < lpp && ok; ++q, ++ln) {
+                    const int buf = ln & 1;
+                    bool dwait = true;
+#pragma unroll
+                    for (int pp = 0; pp < 2; ++pp) {
+                        if (2 * pp >= n) break;
+                        // the pair's last batch is complete: its operands are free, and after a
+                        // stage III its result is whole
+                        if (bt[pp] > 0) ok = OTC_WAITW(&b_ae[2 * h + pp], (bt[pp] - 1) & 1);
+                        if (ok && dwait) {
+                            ok = OTC_WAITW(&b_df[buf], (ln >> 1) & 1);
+                            dwait = false;
                         }
-                        ok = ok && OTC_WAITW(&b_df[buf], (ln >> 1) & 1);
                         if (!ok) break;
                         tc::fence_after();
+                        if (p > 0 && q == 0) add_pair(pp);
+                        uint32_t ad[4];
 #pragma unroll
-                        for (int lh = 0; lh < 2; ++lh) {
-                            float v[2][4][4];  // [a1'][piece][.]
-                            if (n > 0) {
+                        for (int i = 0; i < 4; ++i)  // (lane half, a1')
+                            ad[i] = tbase + buf * 128 + (uint32_t)((i & 1) * ps * 8 + (pl + 2 * pp) * 8) + lane_off + ((uint32_t)((i >> 1) * 16) << 16);
+                        float v[4][2][4];
+                        tc::tmem_ld16x256_x2x4(ad, v);
+                        tc::fence_before();
+                        if (2 * pp + 2 >= n) tc::mbar_arrive(&b_de[buf]);  // D_I read
 #pragma unroll
-                                for (int a = 0; a < 2; ++a) {
-                                    const uint32_t ad = tbase + buf * 128 + (uint32_t)(a * ps * 8 + pl * 8) + lane_off + ((uint32_t)(lh * 16) << 16);
-                                    if (ps == 8) tc::tmem_ld16x256_rep<4>(ad, v[a]);
-                                    else tc::tmem_ld16x256_rep<2>(ad, v[a]);
-                                }
-                            }
-                            if (lh == 1) {
-                                tc::fence_before();
-                                tc::mbar_arrive(&b_de[buf]);
-                            }
+                        for (int r = 0; r < 2; ++r) {
+                            const int pc = pl + 2 * pp + r;
+                            if (2 * pp + r >= n) break;
+                            const float c2 = U.c2[pc];
 #pragma unroll
-                            for (int pc = 0; pc < 4; ++pc) {
-                                if (pc >= n) break;
-                                const float c2 = s_c2[pl + pc];
-#pragma unroll
-                                for (int a = 0; a < 2; ++a) {
-                                    const float* x = v[a][pc];
-                                    uint32_t h0, l0, h1, l1;
-                                    tc::split_h2(x[0] * c2, x[1] * c2, h0, l0);
-                                    tc::split_h2(x[2] * c2, x[3] * c2, h1, l1);
-                                    tc::stmatrix_x4_trans(rowI + (pl + pc) * L::A2_PIECE + a * 8 * L::A2_SBO + lh * 32, h0,
-                                                          l0, h1, l1);
-                                }
+                            for (int i = 0; i < 4; ++i) {
+                                const float* x = v[i][r];
+                                uint32_t h0, l0, h1, l1;
+                                tc::split_h2(x[0] * c2, x[1] * c2, h0, l0);
+                                tc::split_h2(x[2] * c2, x[3] * c2, h1, l1);
+                                tc::stmatrix_x4_trans(rowI + pc * L::A2_PIECE + (i & 1) * 8 * L::A2_SBO + (i >> 1) * 32, h0, l0, h1, l1);
                             }
                         }
-                        tc::fence_before();
                         tc::fence_async_smem();
-                        tc::mbar_arrive(&b_af[h]);
+                        tc::mbar_arrive(&b_af[2 * h + pp]);
+                        ++bt[pp];
                     }
-                    if (!ok) break;
-                    // the plane's stage II is complete: D_II is whole and the operands are free
-                    ok = OTC_WAITW(&b_vf[h], pn & 1) && OTC_WAITW(&b_ae[h], (bt - 1) & 1);
+                    if (ok && n == 0) {  // nothing to convert: only keep step
+                        ok = OTC_WAITW(&b_df[buf], (ln >> 1) & 1);
+                        if (ok) tc::mbar_arrive(&b_de[buf]);
+                    }
+                }
+                // the plane's V
+#pragma unroll
+                for (int pp = 0; pp < 2; ++pp) {
+                    if (!ok || 2 * pp >= n) break;
+                    ok = OTC_WAITW(&b_ae[2 * h + pp], (bt[pp] - 1) & 1);
                     if (!ok) break;
                     tc::fence_after();
-                    if (n > 0) {
+                    uint32_t ad[4];
 #pragma unroll
-                        for (int lh = 0; lh < 2; ++lh) {
-                            float v[2][4][4];  // [piece pair][2 piece' + a2'][.]
+                    for (int i = 0; i < 4; ++i)  // (lane half, piece)
+                        ad[i] = cII(h, 2 * pp + (i & 1)) + lane_off + ((uint32_t)((i >> 1) * 16) << 16);
+                    float v[4][2][4];  // [.][a2'][.]
+                    tc::tmem_ld16x256_x2x4(ad, v);
 #pragma unroll
-                            for (int pp = 0; pp < 2; ++pp)
-                                if (2 * pp < n) tc::tmem_ld16x256_rep<4>(cII(h, 2 * pp) + lane_off + ((uint32_t)(lh * 16) << 16), v[pp]);
+                    for (int r = 0; r < 2; ++r) {
+                        const int pc = pl + 2 * pp + r;
+                        if (2 * pp + r >= n) break;
+                        const float c3 = U.c3[pc];
 #pragma unroll
-                            for (int pc = 0; pc < 4; ++pc) {
-                                if (pc >= n) break;
-                                const float c3 = s_c3[pl + pc];
-#pragma unroll
-                                for (int a = 0; a < 2; ++a) {
-                                    const float* x = v[pc >> 1][2 * (pc & 1) + a];
-                                    uint32_t h0, l0, h1, l1;
-                                    tc::split_h2(x[0] * c3, x[1] * c3, h0, l0);
-                                    tc::split_h2(x[2] * c3, x[3] * c3, h1, l1);
-                                    tc::stmatrix_x4_trans(rowII + (pl + pc) * L::A2_PIECE + a * 2 * L::A2_LBO + lh * 2 * L::A2_SBO,
-                                                          h0, l0, h1, l1);
-                                }
-                            }
+                        for (int i = 0; i < 4; ++i) {  // (lane half, a2')
+                            const float* x = v[(i & 2) + r][i & 1];
+                            uint32_t h0, l0, h1, l1;
+                            tc::split_h2(x[0] * c3, x[1] * c3, h0, l0);
+                            tc::split_h2(x[2] * c3, x[3] * c3, h1, l1);
+                            tc::stmatrix_x4_trans(rowII + pc * L::A2_PIECE + (i & 1) * 2 * L::A2_LBO + (i >> 1) * 2 * L::A2_SBO, h0, l0, h1, l1);
                         }
                     }
                     tc::fence_before();
                     tc::fence_async_smem();
-                    tc::mbar_arrive(&b_af[h]);
-                    ++bt;
+                    tc::mbar_arrive(&b_af[2 * h + pp]);
+                    ++bt[pp];
                 }
-                if (ok) ok = OTC_WAITW(&b_ae[h], (bt - 1) & 1);
-                if (ok) {
-                    tc::fence_after();
-                    add_plane();
-                    tc::fence_before();
-                    // the second half's sum waits in its operand space for the first half's
-                    if (h == 1 && n > 0)
+            }
 #pragma unroll
-                        for (int c = 0; c < 32; ++c) ysum[c * 128 + w4 * 32 + lane] = y[c >> 4][c & 15];
+            for (int pp = 0; pp < 2; ++pp) {
+                if (!ok || 2 * pp >= n) break;
+                ok = OTC_WAITW(&b_ae[2 * h + pp], (bt[pp] - 1) & 1);
+                if (!ok) break;
+                tc::fence_after();
+                add_pair(pp);
+                tc::fence_before();
+            }
+            // the halves' sums meet in the second half's operand space, free until its next batch
+            float* ysum = (float*)(sm + L::A2 + ph * L::A2_PIECE);  // 32 x 128
+            const int r = w4 * 32 + lane;
+            if (ok && npc > ph) {
+                if (h == 1) {
+#pragma unroll
+                    for (int c = 0; c < 32; ++c) ysum[c * 128 + r] = y[c >> 4][c & 15];
+                    tc::mbar_arrive(&b_y);
+                    ok = OTC_WAITW(&b_yr, ny & 1);
+                } else {
+                    ok = OTC_WAITW(&b_y, ny & 1);
+                    if (ok)
+#pragma unroll
+                        for (int c = 0; c < 32; ++c) y[c >> 4][c & 15] += ysum[c * 128 + r];
+                    tc::mbar_arrive(&b_yr);
                 }
-                // (after the barrier every thread of the first half writes the sums out)
-                __syncthreads();
-                if (h == 0 && ok && !s_abort) {
-                    const int r = w4 * 32 + lane, a1 = 1 - (r >> 6), c1 = (r >> 3) & 7, c2 = r & 7, k = P.k;
+                ++ny;
+            }
+            if (h == 0 && ok) {
+                const int a1 = 1 - (r >> 6), c1 = (r >> 3) & 7, c2 = r & 7, kk = P.k;
+                float* part = (float*)Q.part + (size_t)U.unit * 8 * kk * kk * kk;
 #pragma unroll
-                    for (int q = 0; q < 4; ++q) {
-                        const int o = a1 * 4 + (1 - (q >> 1)) * 2 + 1 - (q & 1);
-                        if (o < nout && c1 < k && c2 < k) {
-                            float* dst = part + (size_t)o * k * k * k + (c1 * k + c2) * k;
+                for (int q = 0; q < 4; ++q) {
+                    const int o = a1 * 4 + (1 - (q >> 1)) * 2 + 1 - (q & 1);
+                    if (o < U.nout && c1 < kk && c2 < kk) {
+                        float* dst = part + (size_t)o * kk * kk * kk + (c1 * kk + c2) * kk;
 #pragma unroll
-                            for (int c3 = 0; c3 < 8; ++c3) {
-                                const int c = q * 8 + c3;
-                                if (c3 < k) dst[c3] = y[c >> 4][c & 15] + (npc > ph ? ysum[c * 128 + r] : 0.0f);
-                            }
-                        }
+                        for (int c3 = 0; c3 < 8; ++c3)
+                            if (c3 < kk) dst[c3] = y[q >> 1][(q & 1) * 8 + c3];
                     }
                 }
             }
-            if (warp >= 8) __syncthreads();
-            line0 += nline;
-            batch0 += nline + nplane;
-            plane0 += nplane;
-        } else {
-            for (int e = tid; e < nout * P.k * P.k * P.k; e += OTC_THREADS) part[e] = 0.0f;
-        }
-        __syncthreads();
-        tc::fence_after();
-        if (s_abort) {
-            stop = true;
-            if (tid == 0) atomicExch(Q.err, 4);
+            tc::mbar_arrive(&b_se[slot]);
         }
     }
 #undef OTC_WAIT
 #undef OTC_WAITW
     tc::fence_before();
     __syncthreads();
+    if (s_abort && tid == 0) atomicExch(Q.err, 4);
     if (warp == 0) tc::tmem_dealloc(tbase, 512);
 }
 

@@ -150,6 +150,28 @@ __device__ __forceinline__ void tmem_ld32x16(uint32_t taddr, float* v) {
     for (int q = 0; q < 16; ++q) v[q] = __uint_as_float(r[q]);
 }
 
+// four loads of 16 lanes x 16 columns (16x256b.x2: v[i][r][0..3] as tmem_ld16x256_rep<2> of
+// taddr[i]) in flight together, one wait
+__device__ __forceinline__ void tmem_ld16x256_x2x4(const uint32_t* taddr, float (*v)[2][4]) {
+    uint32_t r[32];
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+        asm volatile("tcgen05.ld.sync.aligned.16x256b.x2.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                     : "=r"(r[8 * i]), "=r"(r[8 * i + 1]), "=r"(r[8 * i + 2]), "=r"(r[8 * i + 3]), "=r"(r[8 * i + 4]),
+                       "=r"(r[8 * i + 5]), "=r"(r[8 * i + 6]), "=r"(r[8 * i + 7])
+                     : "r"(taddr[i]));
+    asm volatile("tcgen05.wait::ld.sync.aligned;"
+                 : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]),
+                   "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15]),
+                   "+r"(r[16]), "+r"(r[17]), "+r"(r[18]), "+r"(r[19]), "+r"(r[20]), "+r"(r[21]), "+r"(r[22]), "+r"(r[23]),
+                   "+r"(r[24]), "+r"(r[25]), "+r"(r[26]), "+r"(r[27]), "+r"(r[28])
+                 :
+                 : "memory");
+    asm volatile("" : "+r"(r[29]), "+r"(r[30]), "+r"(r[31]) : : "memory");
+#pragma unroll
+    for (int q = 0; q < 32; ++q) v[q >> 3][(q >> 2) & 1][q & 3] = __uint_as_float(r[q]);
+}
+
 // one arrival of the calling thread
 __device__ __forceinline__ void mbar_arrive(uint64_t* mbar) {
     asm volatile("{\n.reg .b64 t;\nmbarrier.arrive.shared::cta.b64 t, [%0];\n}\n" ::"r"(smem_u32(mbar)) : "memory");
