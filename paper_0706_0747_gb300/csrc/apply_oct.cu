@@ -446,17 +446,32 @@ __global__ void __launch_bounds__(OctCfg<T, K>::NT) k_apply_oct(OctArgs P) {
     }
 }
 
-// ghat of a group's outputs: its slices' sums in order
+// ghat of a group's outputs: its slices' sums in order.  FP32 slices are added in two floats
+// (Knuth's two-sum, as exact as FP64 for so few terms) and converted once: on this part FP64
+// additions and conversions run at 1/64 of the FP32 rate (120 us on 3-D Poisson k = 8 with an FP64
+// conversion and addition per slice).
 template <typename TP>
 __global__ void k_oct_reduce(OctArgs P, int slice, int k3, const TP* part, double* out) {
     if (P.skip && *P.skip != P.run_if) return;
     const int g = P.g0 + blockIdx.x, np = P.np[g], n = (np + slice - 1) / slice;
     const int i0 = P.first[g], total = (P.coord[4 * i0] ? 8 : 1) * k3;
     const TP* src = part + (size_t)blockIdx.x * P.ns * 8 * k3;
+    double* dst = out + (size_t)i0 * k3;
     for (int e = threadIdx.x; e < total; e += blockDim.x) {
-        double v = 0.0;
-        for (int s = 0; s < n; ++s) v += (double)src[(size_t)s * 8 * k3 + e];
-        out[(size_t)i0 * k3 + e] = v;
+        if (sizeof(TP) == 8) {
+            double v = 0.0;
+            for (int s = 0; s < n; ++s) v += (double)src[(size_t)s * 8 * k3 + e];
+            dst[e] = v;
+        } else {
+            float hi = 0.0f, lo = 0.0f;
+#pragma unroll 4
+            for (int s = 0; s < n; ++s) {
+                const float x = (float)src[(size_t)s * 8 * k3 + e], t = __fadd_rn(hi, x), b = __fsub_rn(t, hi);
+                lo += __fadd_rn(__fsub_rn(hi, __fsub_rn(t, b)), __fsub_rn(x, b));
+                hi = t;
+            }
+            dst[e] = (double)hi + (double)lo;
+        }
     }
 }
 

@@ -17,14 +17,13 @@
 // descriptor (constant strides) covers both outputs and both boxes; a piece's excluded
 // translations are zero tiles.
 //
-// One persistent CTA per SM (216 KB of shared memory, all 512 TMEM columns), 19 warps with roles
+// One persistent CTA per SM (216 KB of shared memory, all 512 TMEM columns), 28 warps with roles
 // that meet at mbarriers only, so that setting up units, loading, MMAs and conversions overlap:
-//   0-7    convert accumulators to the next stage's operands, half of the pieces per four warps,
-//          two pieces ("a pair") at a time, so that a pair's MMAs run while the next is converted;
-//   8-11   load X (two buffers; the blocks' power-of-two scales are made equal on the way);
-//   12     issues stage I into one of two accumulators;
-//   13, 14 issue stages II and III of a half each;
-//   15-18  set up the next unit (pieces, inputs, scales, F tiles) in the other of two slots.
+//   0-15   convert accumulators to the next stage's operands, a pair of pieces per four warps;
+//   16-19  load X (two buffers; the blocks' power-of-two scales are made equal on the way);
+//   20-23  issue stages II and III of a pair each;
+//   24     issues stage I into one of two accumulators;
+//   25-27  set up the next unit (pieces, inputs, scales, F tiles) in the other of two slots.
 // What bounds it is the shared-memory side of the tensor core: an MMA of stage II or III reads
 // 4 KB of A for 16 columns of output (23 % of the launch's cycles in the version whose units
 // were set up and finished by the whole CTA between barriers: 1.38 ms on 3-D Poisson k = 8).
@@ -39,8 +38,10 @@
 
 namespace mra {
 
-#define OTC_THREADS 608
-#define OTC_WAIT_LIMIT (1u << 24)
+#define OTC_THREADS 896
+#define OTC_SETUP 96  // threads that set up units
+// polls of one completion wait (TC_SUSPEND_NS each at most)
+#define OTC_WAIT_LIMIT (1u << 20)
 #define OTC_WAIT_MIN 4096u
 #define OTC_P 8  // pieces per chunk
 
@@ -71,12 +72,18 @@ struct OtcUnit {
     float c2[OTC_P], c3[OTC_P], fin[OTC_P];
 };
 
+// c x[0..3] (c a power of two) as FP16 hi and lo pairs: hi01, lo01, hi23, lo23
+__device__ __forceinline__ void split_scaled(const float* x, float c, uint32_t* w) {
+    tc::split_h2(x[0] * c, x[1] * c, w[0], w[1]);
+    tc::split_h2(x[2] * c, x[3] * c, w[2], w[3]);
+}
+
 __global__ void __launch_bounds__(OTC_THREADS, 1) k_apply_oct_tc(OctTcArgs Q) {
     using L = OtcSmem;
     extern __shared__ __align__(1024) unsigned char sm[];
     __shared__ uint32_t s_tmem;
-    // X full / empty, D_I full / empty; per half and pair: operands full, MMAs done; per slot: set up, done with;
-    // the second half's sums written, read
+    // X full / empty, D_I full / empty; per pair: operands full, MMAs done; per slot: set up, done with;
+    // the pairs' sums written, read
     __shared__ __align__(8) uint64_t b_xf[2], b_xe[2], b_df[2], b_de[2], b_af[4], b_ae[4], b_sf[2], b_se[2], b_y, b_yr;
     __shared__ volatile int s_abort;
     __shared__ int s_unit, s_emin;
@@ -90,17 +97,17 @@ __global__ void __launch_bounds__(OTC_THREADS, 1) k_apply_oct_tc(OctTcArgs Q) {
     if (warp == 0) tc::tmem_alloc(&s_tmem, 512);
     if (tid == 0) {
         for (int i = 0; i < 2; ++i) {
-            tc::mbar_init(&b_xf[i], 128);
+            tc::mbar_init(&b_xf[i], 4);
             tc::mbar_init(&b_xe[i], 1);
             tc::mbar_init(&b_df[i], 1);
-            tc::mbar_init(&b_de[i], 256);
-            tc::mbar_init(&b_sf[i], 128);
-            tc::mbar_init(&b_se[i], 128 + 256 + 3);
+            tc::mbar_init(&b_de[i], 16);
+            tc::mbar_init(&b_sf[i], OTC_SETUP / 32);
+            tc::mbar_init(&b_se[i], 4 + 16 + 5);
         }
-        tc::mbar_init(&b_y, 128);
-        tc::mbar_init(&b_yr, 128);
+        tc::mbar_init(&b_y, 16);
+        tc::mbar_init(&b_yr, 16);
         for (int i = 0; i < 4; ++i) {
-            tc::mbar_init(&b_af[i], 128);
+            tc::mbar_init(&b_af[i], 4);
             tc::mbar_init(&b_ae[i], 1);
         }
         s_abort = 0;
@@ -109,26 +116,31 @@ __global__ void __launch_bounds__(OTC_THREADS, 1) k_apply_oct_tc(OctTcArgs Q) {
     tc::fence_before();
     __syncthreads();
     tc::fence_after();
-    const uint32_t tbase = s_tmem;
-    // TMEM columns: D_I 2 x 128; D_II 16 per piece at 256 + 64 half; D_III 2 a2' x 16 per piece: a
-    // pair's first piece at 384 + 64 half, its second over the pair's D_II, which stage III no longer
+    const uint32_t tbase = (uint32_t)tc::uniform((int)s_tmem);
+    // TMEM columns: D_I 2 x 128; D_II 16 per piece at 256 + 32 pair; D_III 2 a2' x 16 per piece: a
+    // pair's first piece at 384 + 32 pair, its second over the pair's D_II, which stage III no longer
     // needs
-    auto cII = [&](int h, int lp) { return tbase + 256u + (uint32_t)(h * 64 + lp * 16); };
-    auto cIII = [&](int h, int lp, int a) { return tbase + ((lp & 1) ? 256u : 384u) + (uint32_t)(h * 64 + (lp >> 1) * 32 + a * 16); };
+    auto cII = [&](int g, int r) { return tbase + 256u + (uint32_t)(g * 32 + r * 16); };
+    auto cIII = [&](int g, int r, int a) { return tbase + (r ? 256u : 384u) + (uint32_t)(g * 32 + a * 16); };
 #define OTC_WAIT(bar, parity) tc::mbar_wait_or(bar, parity, Q.wait_limit, &s_abort)
     // the same by a whole warp, whose lanes go on or give up together (what follows is warp-collective)
 #define OTC_WAITW(bar, parity) __all_sync(0xffffffffu, OTC_WAIT(bar, parity))
+    // by 128 threads of named barrier `id`: the leading warp polls, the others sleep at the barrier
+#define OTC_WAITG(id, lead, expr) tc::group_all(id, !(lead) || (expr))
     // barriers complete once per use; a use's parity is its running number's lowest bit
     uint32_t ln = 0;  // lines (pairs of boxes b2) so far
 
-    if (warp >= 15) {
+    // registers by warpgroup: 896 threads x 72 at launch = 512 x 80 + 128 x (72 + 48 + 64)
+    if (warp >= 24) {
+        tc::reg_dec<64>();
+        if (warp > 24) {
         // ================= set up units
-        const int t = tid - 480;
+        const int t = tid - 800;
         uint32_t* list = (uint32_t*)(sm + L::LIST);
-        auto sync = [] { asm volatile("bar.sync 2, 128;" ::: "memory"); };
+        auto sync = [] { asm volatile("bar.sync 6, 96;" ::: "memory"); };  // (1-5: the groups of OTC_WAITG)
         for (uint32_t k = 0;; ++k) {
             const int slot = k & 1;
-            bool ok = k < 2 || OTC_WAIT(&b_se[slot], ((k >> 1) - 1) & 1);
+            const bool ok = k < 2 || t != 0 || tc::mbar_wait_or(&b_se[slot], ((k >> 1) - 1) & 1, Q.wait_limit, &s_abort, 500);
             OtcUnit& U = s_u[slot];
             int* tin = (int*)(sm + L::TIN + slot * 864);
             float* tg = (float*)(sm + L::TG + slot * 864);
@@ -149,13 +161,13 @@ __global__ void __launch_bounds__(OTC_THREADS, 1) k_apply_oct_tc(OctTcArgs Q) {
                 np = P.np[g];
                 const int i0 = P.first[g], j = P.coord[4 * i0], nout = j ? 8 : 1;
                 const size_t fb = (size_t)j * P.M;
-                int in[2] = {-1, -1};
-                float sx[2] = {1.0f, 1.0f};
+                int in[3] = {-1, -1, -1};
+                float sx[3] = {1.0f, 1.0f, 1.0f};
 #pragma unroll
-                for (int r = 0; r < 2; ++r)
-                    if (t + 128 * r < 216) in[r] = P.in[(size_t)g * 216 + t + 128 * r];
+                for (int r = 0; r < 3; ++r)
+                    if (t + OTC_SETUP * r < 216) in[r] = P.in[(size_t)g * 216 + t + OTC_SETUP * r];
 #pragma unroll
-                for (int r = 0; r < 2; ++r)
+                for (int r = 0; r < 3; ++r)
                     if (in[r] >= 0) {
                         sx[r] = Q.sx[in[r]];
                         int e;
@@ -163,7 +175,7 @@ __global__ void __launch_bounds__(OTC_THREADS, 1) k_apply_oct_tc(OctTcArgs Q) {
                         atomicMin(&s_emin, e);
                         atomicMax(&s_xmax, __float_as_uint(Q.xmax[in[r]]));  // non-negative floats order as ints
                     }
-                if (warp == 15) {
+                if (warp == 25) {
                     const unsigned lf = __ballot_sync(0xffffffffu, lane < nout && P.leaf[i0 + (lane < nout ? lane : 0)]);
                     const int tree = P.node_tree ? P.node_tree[i0] : 0;
                     oct_pieces(P.sched + (size_t)tree * P.sl, P.M, P.lm, j, lf != 0, lf != (1u << nout) - 1u, list);
@@ -194,19 +206,19 @@ __global__ void __launch_bounds__(OTC_THREADS, 1) k_apply_oct_tc(OctTcArgs Q) {
                 if (!(xmax <= FLT_MAX) && t == 0) atomicExch(Q.err, 5);  // input values beyond FP32's range
                 if (!(xmax > 0.0f && xmax <= FLT_MAX)) {
                     const int k3 = P.k * P.k * P.k;
-                    for (int e = t; e < nout * k3; e += 128) ((float*)Q.part)[(size_t)unit * 8 * k3 + e] = 0.0f;
+                    for (int e = t; e < nout * k3; e += OTC_SETUP) ((float*)Q.part)[(size_t)unit * 8 * k3 + e] = 0.0f;
                     sync();
                     continue;
                 }
 #pragma unroll
-                for (int r = 0; r < 2; ++r)
-                    if (t + 128 * r < 216) {
-                        tin[t + 128 * r] = in[r];
-                        tg[t + 128 * r] = in[r] < 0 ? 0.0f : ldexpf(1.0f, es) / sx[r];
+                for (int r = 0; r < 3; ++r)
+                    if (t + OTC_SETUP * r < 216) {
+                        tin[t + OTC_SETUP * r] = in[r];
+                        tg[t + OTC_SETUP * r] = in[r] < 0 ? 0.0f : ldexpf(1.0f, es) / sx[r];
                     }
                 // F tiles, masked by the pieces' sets
                 const int ps = U.ps, lp = ps == 8 ? 3 : 2;
-                for (int e = t; e < 7 * 6 * 8 * ps; e += 128) {
+                for (int e = t; e < 7 * 6 * 8 * ps; e += OTC_SETUP) {
                     const int v = e & 7, pc = (e >> 3) & (ps - 1), r = e >> (3 + lp), u = r % 7, dh = r / 7;
                     uint4 x = make_uint4(0, 0, 0, 0);
                     if (pc < U.npc) {
@@ -251,18 +263,56 @@ __global__ void __launch_bounds__(OTC_THREADS, 1) k_apply_oct_tc(OctTcArgs Q) {
             }
             if (unit >= Q.nunits && t == 0) U.unit = -1;
             tc::fence_async_smem();
-            tc::mbar_arrive(&b_sf[slot]);
+            tc::mbar_arrive_warp(&b_sf[slot]);
             if (unit >= Q.nunits) break;
             sync();  // s_unit and the scale words are free again
         }
-    } else if (warp >= 8 && warp < 12) {
+        } else {
+        // ================= stage I
+        if (!Q.withhold) {
+            bool ok = true;
+            for (uint32_t k = 0; ok; ++k) {
+                const int slot = k & 1;
+                ok = OTC_WAITW(&b_sf[slot], (k >> 1) & 1);
+                if (!ok || tc::uniform(s_u[slot].unit) < 0) break;
+                const unsigned m1 = tc::uniform(s_u[slot].m1), m2 = tc::uniform(s_u[slot].m2), m3 = tc::uniform(s_u[slot].m3);
+                const int s1 = m1 == 0x1e, s2 = m2 == 0x1e, n1 = 3 - s1, n2 = 3 - s2, ps = tc::uniform(s_u[slot].ps);
+                const uint32_t id = tc::idesc_f16(128, 16 * ps);
+                const uint64_t th = tc::sdesc(sbase + L::T + slot * 6 * L::TAB + s1 * ps * 128, ps * 128, 128);
+                int lines = 0;
+                for (int q = 0; q < n2; ++q) lines += ((m2 >> (s2 + 2 * q)) & 3u) != 0;
+                lines *= __popc(m3);
+                for (int l = 0; l < lines && ok; ++l, ++ln) {
+                    const int buf = ln & 1;
+                    ok = OTC_WAITW(&b_xf[buf], (ln >> 1) & 1) && (ln < 2 || OTC_WAITW(&b_de[buf], ((ln >> 1) - 1) & 1));
+                    if (!ok) break;
+                    tc::fence_after();
+                    const uint32_t d = tbase + buf * 128;
+                    const uint64_t xh = tc::sdesc(sbase + L::X + buf * L::XBUF, 2048, 128);
+#pragma unroll
+                    for (int s = 0; s < 3; ++s) {  // boxes s1 + 2 s, + 1
+                        if (s >= n1) break;
+                        const uint64_t ah = xh + (uint64_t)(s * (4096 / 16)), al = ah + L::XBUF / 32;
+                        const uint64_t bh = th + (uint64_t)(s * 2 * ps * 8), bl = bh + L::TAB / 16;
+                        tc::mma_f16_warp(d, ah, bh, id, s > 0);
+                        tc::mma_f16_warp(d, ah, bl, id, 1);
+                        tc::mma_f16_warp(d, al, bh, id, 1);
+                    }
+                    tc::commit_warp(&b_xe[buf]);
+                    tc::commit_warp(&b_df[buf]);
+                }
+                tc::commit_warp(&b_se[slot]);
+            }
+        }
+        }
+    } else if (warp >= 16 && warp < 20) {
         // ================= X of a pair of lines into a buffer
-        const int lt = tid - 256, hl = lt >> 6, v = lt & 63;
+        const int lt = tid - 512, hl = lt >> 6, v = lt & 63;
         const uint4* src0 = (const uint4*)(hl ? Q.xl : Q.xh) + v;
         bool ok = true;
         for (uint32_t k = 0; ok; ++k) {
             const int slot = k & 1;
-            ok = OTC_WAIT(&b_sf[slot], (k >> 1) & 1);
+            ok = OTC_WAITG(5, warp == 16, OTC_WAIT(&b_sf[slot], (k >> 1) & 1));
             if (!ok || s_u[slot].unit < 0) break;
             const unsigned m1 = s_u[slot].m1, m2 = s_u[slot].m2, m3 = s_u[slot].m3;
             const int s1 = m1 == 0x1e, s2 = m2 == 0x1e, n1 = 3 - s1, n2 = 3 - s2;
@@ -288,7 +338,7 @@ __global__ void __launch_bounds__(OTC_THREADS, 1) k_apply_oct_tc(OctTcArgs Q) {
                             }
                         }
                     }
-                    if (ln >= 2) ok = OTC_WAIT(&b_xe[buf], ((ln >> 1) - 1) & 1);
+                    if (ln >= 2) ok = OTC_WAITG(5, warp == 16, OTC_WAIT(&b_xe[buf], ((ln >> 1) - 1) & 1));
                     if (!ok) break;
                     unsigned char* dst = sm + L::X + buf * L::XBUF + hl * (L::XBUF / 2) + v * 16;
 #pragma unroll
@@ -301,299 +351,241 @@ __global__ void __launch_bounds__(OTC_THREADS, 1) k_apply_oct_tc(OctTcArgs Q) {
                         *(uint4*)(dst + r * 1024) = x[r];
                     }
                     tc::fence_async_smem();
-                    tc::mbar_arrive(&b_xf[buf]);
+                    tc::mbar_arrive_warp(&b_xf[buf]);
                     ++ln;
                 }
             }
-            tc::mbar_arrive(&b_se[slot]);
+            tc::mbar_arrive_warp(&b_se[slot]);
         }
-    } else if (warp == 12) {
-        // ================= stage I
-        if (lane == 0 && !Q.withhold) {
-            bool ok = true;
-            for (uint32_t k = 0; ok; ++k) {
-                const int slot = k & 1;
-                ok = OTC_WAIT(&b_sf[slot], (k >> 1) & 1);
-                if (!ok || s_u[slot].unit < 0) break;
-                const unsigned m1 = s_u[slot].m1, m2 = s_u[slot].m2, m3 = s_u[slot].m3;
-                const int s1 = m1 == 0x1e, s2 = m2 == 0x1e, n1 = 3 - s1, n2 = 3 - s2, ps = s_u[slot].ps;
-                const uint32_t id = tc::idesc_f16(128, 16 * ps);
-                const uint64_t th = tc::sdesc(sbase + L::T + slot * 6 * L::TAB + s1 * ps * 128, ps * 128, 128);
-                int lines = 0;
-                for (int q = 0; q < n2; ++q) lines += ((m2 >> (s2 + 2 * q)) & 3u) != 0;
-                lines *= __popc(m3);
-                for (int l = 0; l < lines && ok; ++l, ++ln) {
-                    const int buf = ln & 1;
-                    ok = OTC_WAIT(&b_xf[buf], (ln >> 1) & 1) && (ln < 2 || OTC_WAIT(&b_de[buf], ((ln >> 1) - 1) & 1));
-                    if (!ok) break;
-                    tc::fence_after();
-                    const uint32_t d = tbase + buf * 128;
-                    const uint64_t xh = tc::sdesc(sbase + L::X + buf * L::XBUF, 2048, 128);
-#pragma unroll
-                    for (int s = 0; s < 3; ++s) {  // boxes s1 + 2 s, + 1
-                        if (s >= n1) break;
-                        const uint64_t ah = xh + (uint64_t)(s * (4096 / 16)), al = ah + L::XBUF / 32;
-                        const uint64_t bh = th + (uint64_t)(s * 2 * ps * 8), bl = bh + L::TAB / 16;
-                        tc::mma_f16(d, ah, bh, id, s > 0);
-                        tc::mma_f16(d, ah, bl, id, 1);
-                        tc::mma_f16(d, al, bh, id, 1);
-                    }
-                    tc::commit(&b_xe[buf]);
-                    tc::commit(&b_df[buf]);
-                }
-                tc::commit(&b_se[slot]);
-            }
-        }
-    } else if (warp >= 13) {
-        // ================= stages II and III of one half of the pieces
-        if (lane == 0) {
-            const int h = warp - 13;
-            uint32_t bt[2] = {0, 0};  // batches so far, per pair
-            bool ok = true;
-            const uint32_t id = tc::idesc_f16(128, 16);
-            for (uint32_t k = 0; ok; ++k) {
-                const int slot = k & 1;
-                ok = OTC_WAIT(&b_sf[slot], (k >> 1) & 1);
-                if (!ok || s_u[slot].unit < 0) break;
-                const unsigned m2 = s_u[slot].m2, m3 = s_u[slot].m3;
-                const int s2 = m2 == 0x1e, n2 = 3 - s2, ps = s_u[slot].ps, ph = ps / 2;
-                const int pl = min(s_u[slot].npc, h * ph), n = min(s_u[slot].npc, h * ph + ph) - pl;
-                const uint32_t tab = sbase + L::T + slot * 6 * L::TAB;
-                for (int b3 = 0; b3 < 6 && ok; ++b3) {
-                    if (!((m3 >> b3) & 1u)) continue;
-                    bool first = true;
-                    for (int q = 0; q < n2 && ok; ++q) {
-                        const int b2 = s2 + 2 * q;
-                        if (!((m2 >> b2) & 3u)) continue;
-#pragma unroll
-                        for (int pp = 0; pp < 2; ++pp) {
-                            if (2 * pp >= n) break;
-                            ok = OTC_WAIT(&b_af[2 * h + pp], bt[pp] & 1);
-                            if (!ok) break;
-                            tc::fence_after();
-#pragma unroll
-                            for (int r = 0; r < 2; ++r) {
-                                const int lp = 2 * pp + r, pc = pl + lp;
-                                if (lp >= n) break;
-                                const uint32_t d = cII(h, lp);
-                                const uint64_t ah = tc::sdesc(sbase + L::A2 + pc * L::A2_PIECE, L::A2_LBO, L::A2_SBO);
-                                const uint64_t al = ah + 2 * L::A2_LBO / 16;
-                                const uint64_t bh = tc::sdesc(tab + 2 * L::TAB + (b2 * ps + pc) * 128, ps * 128, ps * 128);
-                                const uint64_t bl = bh + L::TAB / 16;
-                                tc::mma_f16(d, ah, bh, id, first ? 0u : 1u);
-                                tc::mma_f16(d, ah, bl, id, 1);
-                                tc::mma_f16(d, al, bh, id, 1);
-                            }
-                            tc::commit(&b_ae[2 * h + pp]);
-                            ++bt[pp];
-                        }
-                        first = false;
-                    }
-                    if (!ok) break;
-#pragma unroll
-                    for (int pp = 0; pp < 2; ++pp) {
-                        if (2 * pp >= n) break;
-                        ok = OTC_WAIT(&b_af[2 * h + pp], bt[pp] & 1);
-                        if (!ok) break;
-                        tc::fence_after();
-#pragma unroll
-                        for (int r = 0; r < 2; ++r) {
-                            const int lp = 2 * pp + r, pc = pl + lp;
-                            if (lp >= n) break;
-                            const uint32_t tile = tab + 4 * L::TAB + (b3 * ps + pc) * 128;
-                            const uint64_t bh = tc::sdesc(tile, 0, ps * 128);  // [F_hi ; F_hi]
-                            const uint64_t bl = tc::sdesc(tile + L::TAB, sbase + L::Z - tile - L::TAB, ps * 128);  // [F_lo ; 0]
-#pragma unroll
-                            for (int a = 0; a < 2; ++a) {
-                                const uint64_t av = tc::sdesc(sbase + L::A2 + pc * L::A2_PIECE + a * 2 * L::A2_LBO, L::A2_LBO,
-                                                              L::A2_SBO);
-                                tc::mma_f16(cIII(h, lp, a), av, bh, id, 0);
-                                tc::mma_f16(cIII(h, lp, a), av, bl, id, 1);
-                            }
-                        }
-                        tc::commit(&b_ae[2 * h + pp]);
-                        ++bt[pp];
-                    }
-                }
-                tc::commit(&b_se[slot]);
-            }
-        }
-    } else {
-        // ================= conversions of one half of the pieces, and the outputs
-        const int h = warp >> 2, w4 = warp & 3;
-        const uint32_t lane_off = (uint32_t)(w4 * 32) << 16;
-        const int mi = lane >> 3, mr = lane & 7;  // this lane's matrix and row of a stmatrix
-        // D_I: lanes (line, i3, i2) -> rows (a1', c1 | i3), K = (line, i2); matrices hi, lo of two i3
-        const uint32_t rowI = sbase + L::A2 + (mi & 1) * 2 * L::A2_LBO + (w4 >> 1) * L::A2_LBO + mr * L::A2_SBO +
-                              ((w4 & 1) * 4 + (mi >> 1)) * 16;
-        // D_II: lanes (a1', c1, i3) -> rows (a1' c1 | c2), K = hi | lo; matrices hi, lo of two (a1', c1)
-        const uint32_t rowII = sbase + L::A2 + (mi & 1) * L::A2_LBO + (w4 * 4 + (mi >> 1)) * L::A2_SBO + mr * 16;
-        uint32_t bt[2] = {0, 0}, ny = 0;
+    } else if (warp >= 20) {
+        // ================= stages II and III of one pair of pieces
+        tc::reg_dec<48>();
+        const int g = tc::uniform(warp - 20);
+        uint32_t bt = 0;  // batches so far
         bool ok = true;
+        const uint32_t id = tc::idesc_f16(128, 16);
+        const uint64_t a0 = tc::sdesc(sbase + L::A2 + 2 * g * L::A2_PIECE, L::A2_LBO, L::A2_SBO);
         for (uint32_t k = 0; ok; ++k) {
             const int slot = k & 1;
             ok = OTC_WAITW(&b_sf[slot], (k >> 1) & 1);
+            if (!ok || tc::uniform(s_u[slot].unit) < 0) break;
+            const unsigned m2 = tc::uniform(s_u[slot].m2), m3 = tc::uniform(s_u[slot].m3);
+            const int ps = tc::uniform(s_u[slot].ps), n = min(2, tc::uniform(s_u[slot].npc) - 2 * g);
+            const int s2 = m2 == 0x1e, n2 = 3 - s2;
+            const uint32_t tab = sbase + L::T + slot * 6 * L::TAB;
+            for (int b3 = 0; b3 < 6 && ok && n > 0; ++b3) {
+                if (!((m3 >> b3) & 1u)) continue;
+                uint32_t acc = 0;
+                for (int q = 0; q < n2 && ok; ++q) {
+                    const int b2 = s2 + 2 * q;
+                    if (!((m2 >> b2) & 3u)) continue;
+                    ok = OTC_WAITW(&b_af[g], bt & 1);
+                    if (!ok) break;
+                    tc::fence_after();
+                    const uint64_t b0 = tc::sdesc(tab + 2 * L::TAB + (b2 * ps + 2 * g) * 128, ps * 128, ps * 128);
+#pragma unroll
+                    for (int r = 0; r < 2; ++r) {
+                        if (r >= n) break;
+                        const uint64_t ah = a0 + (uint64_t)(r * (L::A2_PIECE / 16)), al = ah + 2 * L::A2_LBO / 16;
+                        const uint64_t bh = b0 + (uint64_t)(r * 8), bl = bh + L::TAB / 16;
+                        tc::mma_f16_warp(cII(g, r), ah, bh, id, acc);
+                        tc::mma_f16_warp(cII(g, r), ah, bl, id, 1);
+                        tc::mma_f16_warp(cII(g, r), al, bh, id, 1);
+                    }
+                    tc::commit_warp(&b_ae[g]);
+                    ++bt;
+                    acc = 1;
+                }
+                if (!ok) break;
+                // B operands of stage III: [F_hi ; F_hi], and [F_lo ; 0] (a tile further on the zeros
+                // are a tile nearer)
+                const uint32_t tile = tab + 4 * L::TAB + (b3 * ps + 2 * g) * 128;
+                const uint64_t h0 = tc::sdesc(tile, 0, ps * 128);
+                const uint64_t l0 = tc::sdesc(tile + L::TAB, sbase + L::Z - tile - L::TAB, ps * 128);
+                ok = OTC_WAITW(&b_af[g], bt & 1);
+                if (!ok) break;
+                tc::fence_after();
+#pragma unroll
+                for (int r = 0; r < 2; ++r) {
+                    if (r >= n) break;
+                    const uint64_t bh = h0 + (uint64_t)(r * 8), bl = l0 + (uint64_t)(r * 8) - ((uint64_t)(r * 8) << 16);
+#pragma unroll
+                    for (int a = 0; a < 2; ++a) {
+                        const uint64_t av = a0 + (uint64_t)((r * L::A2_PIECE + a * 2 * L::A2_LBO) / 16);
+                        tc::mma_f16_warp(cIII(g, r, a), av, bh, id, 0);
+                        tc::mma_f16_warp(cIII(g, r, a), av, bl, id, 1);
+                    }
+                }
+                tc::commit_warp(&b_ae[g]);
+                ++bt;
+            }
+            tc::commit_warp(&b_se[slot]);
+        }
+    } else {
+        // ================= conversions of one pair of pieces, and the outputs
+        tc::reg_inc<80>();
+        const int g = warp >> 2, w4 = warp & 3;
+        const uint32_t lane_off = (uint32_t)(w4 * 32) << 16;
+        const int mi = lane >> 3, mr = lane & 7;  // this lane's matrix and row of a stmatrix
+        const uint32_t mine = sbase + L::A2 + 2 * g * L::A2_PIECE;
+        // D_I: lanes (line, i3, i2) -> rows (a1', c1 | i3), K = (line, i2); matrices hi, lo of two i3
+        const uint32_t rowI = mine + (mi & 1) * 2 * L::A2_LBO + (w4 >> 1) * L::A2_LBO + mr * L::A2_SBO +
+                              ((w4 & 1) * 4 + (mi >> 1)) * 16;
+        // D_II: lanes (a1', c1, i3) -> rows (a1' c1 | c2), K = hi | lo; matrices hi, lo of two (a1', c1)
+        const uint32_t rowII = mine + (mi & 1) * L::A2_LBO + (w4 * 4 + (mi >> 1)) * L::A2_SBO + mr * 16;
+        uint32_t bt = 0, units = 0;
+        const bool lead = w4 == 0;
+#define OTC_WAITC(expr) OTC_WAITG(1 + g, lead, expr)
+        bool ok = true;
+        for (uint32_t k = 0; ok; ++k) {
+            const int slot = k & 1;
+            ok = OTC_WAITC(OTC_WAIT(&b_sf[slot], (k >> 1) & 1));
             const OtcUnit& U = s_u[slot];
             if (!ok || U.unit < 0) break;
             const unsigned m2 = U.m2;
-            const int ps = U.ps, ph = ps / 2, npc = U.npc, nplane = __popc(U.m3);
-            const int pl = min(npc, h * ph), n = min(npc, h * ph + ph) - pl;
+            const int ps = U.ps, npc = U.npc, nplane = __popc(U.m3), n = min(2, npc - 2 * g);
             const int s2 = m2 == 0x1e, n2 = 3 - s2;
             int lpp = 0;  // lines per plane
             for (int q = 0; q < n2; ++q) lpp += ((m2 >> (s2 + 2 * q)) & 3u) != 0;
-            float y[2][16];  // [a2'][(a3', c3)] of lane (a1', c1, c2), this half's pieces
+            float y[2][16];  // [a2'][(a3', c3)] of lane (a1', c1, c2), this pair's pieces
 #pragma unroll
             for (int c = 0; c < 16; ++c) y[0][c] = y[1][c] = 0.0f;
-            // outputs a2', a3' of this lane that are leaves: bit 2 a2' + a3'
-            unsigned lf = 0;
-            for (int q = 0; q < 4; ++q) lf |= ((U.leaf >> ((1 - (w4 >> 1)) * 4 + (1 - (q >> 1)) * 2 + 1 - (q & 1))) & 1u) << q;
-            // y += fin Y of a pair whose stage III of a plane has completed
-            auto add_pair = [&](int pp) {
+            // y += fin Y after a plane's stage III
+            auto add_plane = [&]() {
 #pragma unroll
                 for (int r = 0; r < 2; ++r) {
-                    const int lp = 2 * pp + r;
-                    if (lp >= n) break;
-                    const float fin = U.fin[pl + lp];
-                    const bool leaf_only = (U.piece[pl + lp] >> 24) != 0;
+                    if (r >= n) break;
+                    const float fin = U.fin[2 * g + r];
+                    const bool leaf_only = (U.piece[2 * g + r] >> 24) != 0;
 #pragma unroll
                     for (int a = 0; a < 2; ++a) {
                         float t[16];
-                        tc::tmem_ld32x16(cIII(h, lp, a) + lane_off, t);
+                        tc::tmem_ld32x16(cIII(g, r, a) + lane_off, t);
 #pragma unroll
-                        for (int c = 0; c < 16; ++c) {
-                            const float f = leaf_only && !((lf >> (2 * a + (c >> 3))) & 1u) ? 0.0f : fin;
-                            y[a][c] = fmaf(f, t[c], y[a][c]);
+                        for (int a3 = 0; a3 < 2; ++a3) {
+                            const int o = (1 - (w4 >> 1)) * 4 + (1 - a) * 2 + 1 - a3;
+                            const float f = leaf_only && !((U.leaf >> o) & 1u) ? 0.0f : fin;
+#pragma unroll
+                            for (int c = 0; c < 8; ++c) y[a][8 * a3 + c] = fmaf(f, t[8 * a3 + c], y[a][8 * a3 + c]);
                         }
                     }
                 }
             };
+            // the pairs' sums of the unit before have been read out of the operand space
+            if (units > 0) ok = OTC_WAITC(OTC_WAIT(&b_yr, (units - 1) & 1));
             for (int p = 0; p < nplane && ok; ++p) {
                 for (int q = 0; q < lpp && ok; ++q, ++ln) {
                     const int buf = ln & 1;
-                    bool dwait = true;
-#pragma unroll
-                    for (int pp = 0; pp < 2; ++pp) {
-                        if (2 * pp >= n) break;
-                        // the pair's last batch is complete: its operands are free, and after a
-                        // stage III its result is whole
-                        if (bt[pp] > 0) ok = OTC_WAITW(&b_ae[2 * h + pp], (bt[pp] - 1) & 1);
-                        if (ok && dwait) {
-                            ok = OTC_WAITW(&b_df[buf], (ln >> 1) & 1);
-                            dwait = false;
-                        }
+                    // the last batch is complete: the operands are free, and after a stage III its result
+                    // is whole; D_I of the line is there
+                    if (n > 0 && p > 0 && q == 0) {
+                        ok = OTC_WAITC(OTC_WAIT(&b_ae[g], (bt - 1) & 1));
                         if (!ok) break;
                         tc::fence_after();
-                        if (p > 0 && q == 0) add_pair(pp);
-                        uint32_t ad[4];
+                        add_plane();
+                    }
+                    ok = OTC_WAITC((n <= 0 || bt == 0 || OTC_WAIT(&b_ae[g], (bt - 1) & 1)) && OTC_WAIT(&b_df[buf], (ln >> 1) & 1));
+                    if (!ok) break;
+                    if (n <= 0) {  // nothing to convert: only keep step
+                        tc::mbar_arrive_warp(&b_de[buf]);
+                        continue;
+                    }
+                    tc::fence_after();
+                    const float c20 = U.c2[2 * g], c21 = n > 1 ? U.c2[2 * g + 1] : 0.0f;
+                    const uint32_t ad = tbase + buf * 128 + (uint32_t)(2 * g * 8) + lane_off;
 #pragma unroll
-                        for (int i = 0; i < 4; ++i)  // (lane half, a1')
-                            ad[i] = tbase + buf * 128 + (uint32_t)((i & 1) * ps * 8 + (pl + 2 * pp) * 8) + lane_off + ((uint32_t)((i >> 1) * 16) << 16);
-                        float v[4][2][4];
-                        tc::tmem_ld16x256_x2x4(ad, v);
-                        tc::fence_before();
-                        if (2 * pp + 2 >= n) tc::mbar_arrive(&b_de[buf]);  // D_I read
+                    for (int lh = 0; lh < 2; ++lh) {
+                        float v[2][2][4];  // [a1'][piece][.]
+                        tc::tmem_ld16x256_x2x2(ad + ((uint32_t)(lh * 16) << 16), ad + (uint32_t)(ps * 8) + ((uint32_t)(lh * 16) << 16), v);
+                        if (lh) {
+                            tc::fence_before();
+                            tc::mbar_arrive_warp(&b_de[buf]);  // D_I read
+                        }
+                        uint32_t w[2][2][4];
+#pragma unroll
+                        for (int a = 0; a < 2; ++a)
+#pragma unroll
+                            for (int r = 0; r < 2; ++r) split_scaled(v[a][r], r ? c21 : c20, w[r][a]);
 #pragma unroll
                         for (int r = 0; r < 2; ++r) {
-                            const int pc = pl + 2 * pp + r;
-                            if (2 * pp + r >= n) break;
-                            const float c2 = U.c2[pc];
+                            if (r >= n) break;
 #pragma unroll
-                            for (int i = 0; i < 4; ++i) {
-                                const float* x = v[i][r];
-                                uint32_t h0, l0, h1, l1;
-                                tc::split_h2(x[0] * c2, x[1] * c2, h0, l0);
-                                tc::split_h2(x[2] * c2, x[3] * c2, h1, l1);
-                                tc::stmatrix_x4_trans(rowI + pc * L::A2_PIECE + (i & 1) * 8 * L::A2_SBO + (i >> 1) * 32, h0, l0, h1, l1);
-                            }
-                        }
-                        tc::fence_async_smem();
-                        tc::mbar_arrive(&b_af[2 * h + pp]);
-                        ++bt[pp];
-                    }
-                    if (ok && n == 0) {  // nothing to convert: only keep step
-                        ok = OTC_WAITW(&b_df[buf], (ln >> 1) & 1);
-                        if (ok) tc::mbar_arrive(&b_de[buf]);
-                    }
-                }
-                // the plane's V
-#pragma unroll
-                for (int pp = 0; pp < 2; ++pp) {
-                    if (!ok || 2 * pp >= n) break;
-                    ok = OTC_WAITW(&b_ae[2 * h + pp], (bt[pp] - 1) & 1);
-                    if (!ok) break;
-                    tc::fence_after();
-                    uint32_t ad[4];
-#pragma unroll
-                    for (int i = 0; i < 4; ++i)  // (lane half, piece)
-                        ad[i] = cII(h, 2 * pp + (i & 1)) + lane_off + ((uint32_t)((i >> 1) * 16) << 16);
-                    float v[4][2][4];  // [.][a2'][.]
-                    tc::tmem_ld16x256_x2x4(ad, v);
-#pragma unroll
-                    for (int r = 0; r < 2; ++r) {
-                        const int pc = pl + 2 * pp + r;
-                        if (2 * pp + r >= n) break;
-                        const float c3 = U.c3[pc];
-#pragma unroll
-                        for (int i = 0; i < 4; ++i) {  // (lane half, a2')
-                            const float* x = v[(i & 2) + r][i & 1];
-                            uint32_t h0, l0, h1, l1;
-                            tc::split_h2(x[0] * c3, x[1] * c3, h0, l0);
-                            tc::split_h2(x[2] * c3, x[3] * c3, h1, l1);
-                            tc::stmatrix_x4_trans(rowII + pc * L::A2_PIECE + (i & 1) * 2 * L::A2_LBO + (i >> 1) * 2 * L::A2_SBO, h0, l0, h1, l1);
+                            for (int a = 0; a < 2; ++a)
+                                tc::stmatrix_x4_trans(rowI + r * L::A2_PIECE + a * 8 * L::A2_SBO + lh * 32, w[r][a][0], w[r][a][1],
+                                                      w[r][a][2], w[r][a][3]);
                         }
                     }
-                    tc::fence_before();
                     tc::fence_async_smem();
-                    tc::mbar_arrive(&b_af[2 * h + pp]);
-                    ++bt[pp];
+                    tc::mbar_arrive_warp(&b_af[g]);
+                    ++bt;
                 }
-            }
-#pragma unroll
-            for (int pp = 0; pp < 2; ++pp) {
-                if (!ok || 2 * pp >= n) break;
-                ok = OTC_WAITW(&b_ae[2 * h + pp], (bt[pp] - 1) & 1);
+                if (!ok || n <= 0) continue;
+                // the plane's V
+                ok = OTC_WAITC(OTC_WAIT(&b_ae[g], (bt - 1) & 1));
                 if (!ok) break;
                 tc::fence_after();
-                add_pair(pp);
-                tc::fence_before();
-            }
-            // the halves' sums meet in the second half's operand space, free until its next batch
-            float* ysum = (float*)(sm + L::A2 + ph * L::A2_PIECE);  // 32 x 128
-            const int r = w4 * 32 + lane;
-            if (ok && npc > ph) {
-                if (h == 1) {
+                const float c30 = U.c3[2 * g], c31 = n > 1 ? U.c3[2 * g + 1] : 0.0f;
 #pragma unroll
-                    for (int c = 0; c < 32; ++c) ysum[c * 128 + r] = y[c >> 4][c & 15];
-                    tc::mbar_arrive(&b_y);
-                    ok = OTC_WAITW(&b_yr, ny & 1);
-                } else {
-                    ok = OTC_WAITW(&b_y, ny & 1);
-                    if (ok)
+                for (int lh = 0; lh < 2; ++lh) {
+                    float v[2][2][4];  // [piece][a2'][.]
+                    tc::tmem_ld16x256_x2x2(cII(g, 0) + lane_off + ((uint32_t)(lh * 16) << 16), cII(g, 1) + lane_off + ((uint32_t)(lh * 16) << 16), v);
+                    uint32_t w[2][2][4];
 #pragma unroll
-                        for (int c = 0; c < 32; ++c) y[c >> 4][c & 15] += ysum[c * 128 + r];
-                    tc::mbar_arrive(&b_yr);
+                    for (int r = 0; r < 2; ++r)
+#pragma unroll
+                        for (int a = 0; a < 2; ++a) split_scaled(v[r][a], r ? c31 : c30, w[r][a]);
+#pragma unroll
+                    for (int r = 0; r < 2; ++r) {
+                        if (r >= n) break;
+#pragma unroll
+                        for (int a = 0; a < 2; ++a)
+                            tc::stmatrix_x4_trans(rowII + r * L::A2_PIECE + a * 2 * L::A2_LBO + lh * 2 * L::A2_SBO, w[r][a][0], w[r][a][1],
+                                                  w[r][a][2], w[r][a][3]);
+                    }
                 }
-                ++ny;
+                tc::fence_before();
+                tc::fence_async_smem();
+                tc::mbar_arrive_warp(&b_af[g]);
+                ++bt;
             }
-            if (h == 0 && ok) {
+            float* ysum = (float*)(sm + L::A2);  // per pair, in its operand space: 32 x 128
+            constexpr int YS = 2 * L::A2_PIECE / 4;
+            const int r = w4 * 32 + lane;
+            if (ok && n > 0) {
+                ok = OTC_WAITC(OTC_WAIT(&b_ae[g], (bt - 1) & 1));
+                if (ok) {
+                    tc::fence_after();
+                    add_plane();
+                    tc::fence_before();
+#pragma unroll
+                    for (int c = 0; c < 32; ++c) ysum[g * YS + c * 128 + r] = y[c >> 4][c & 15];
+                }
+            }
+            tc::mbar_arrive_warp(&b_y);
+            ok = OTC_WAITC(ok && OTC_WAIT(&b_y, units & 1));
+            if (ok) {  // four warps per (a2', a3') add the pairs' sums in order
                 const int a1 = 1 - (r >> 6), c1 = (r >> 3) & 7, c2 = r & 7, kk = P.k;
-                float* part = (float*)Q.part + (size_t)U.unit * 8 * kk * kk * kk;
+                const int o = a1 * 4 + (1 - (g >> 1)) * 2 + 1 - (g & 1);
+                if (o < U.nout && c1 < kk && c2 < kk) {
+                    float* dst = (float*)Q.part + (size_t)U.unit * 8 * kk * kk * kk + (size_t)o * kk * kk * kk + (c1 * kk + c2) * kk;
 #pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    const int o = a1 * 4 + (1 - (q >> 1)) * 2 + 1 - (q & 1);
-                    if (o < U.nout && c1 < kk && c2 < kk) {
-                        float* dst = part + (size_t)o * kk * kk * kk + (c1 * kk + c2) * kk;
-#pragma unroll
-                        for (int c3 = 0; c3 < 8; ++c3)
-                            if (c3 < kk) dst[c3] = y[q >> 1][(q & 1) * 8 + c3];
+                    for (int c3 = 0; c3 < 8; ++c3) {
+                        if (c3 >= kk) break;
+                        float s = 0.0f;
+                        for (int gg = 0; 2 * gg < npc; ++gg) s += ysum[gg * YS + (g * 8 + c3) * 128 + r];
+                        dst[c3] = s;
                     }
                 }
             }
-            tc::mbar_arrive(&b_se[slot]);
+            tc::mbar_arrive_warp(&b_yr);
+            tc::mbar_arrive_warp(&b_se[slot]);
+            ++units;
         }
     }
 #undef OTC_WAIT
 #undef OTC_WAITW
+#undef OTC_WAITG
+#undef OTC_WAITC
     tc::fence_before();
     __syncthreads();
     if (s_abort && tid == 0) atomicExch(Q.err, 4);

@@ -150,52 +150,98 @@ __device__ __forceinline__ void tmem_ld32x16(uint32_t taddr, float* v) {
     for (int q = 0; q < 16; ++q) v[q] = __uint_as_float(r[q]);
 }
 
-// four loads of 16 lanes x 16 columns (16x256b.x2: v[i][r][0..3] as tmem_ld16x256_rep<2> of
+// two loads of 16 lanes x 16 columns (16x256b.x2: v[i][r][0..3] as tmem_ld16x256_rep<2> of
 // taddr[i]) in flight together, one wait
-__device__ __forceinline__ void tmem_ld16x256_x2x4(const uint32_t* taddr, float (*v)[2][4]) {
-    uint32_t r[32];
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-        asm volatile("tcgen05.ld.sync.aligned.16x256b.x2.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-                     : "=r"(r[8 * i]), "=r"(r[8 * i + 1]), "=r"(r[8 * i + 2]), "=r"(r[8 * i + 3]), "=r"(r[8 * i + 4]),
-                       "=r"(r[8 * i + 5]), "=r"(r[8 * i + 6]), "=r"(r[8 * i + 7])
-                     : "r"(taddr[i]));
+__device__ __forceinline__ void tmem_ld16x256_x2x2(uint32_t ta0, uint32_t ta1, float (*v)[2][4]) {
+    uint32_t r[16];
+    asm volatile("tcgen05.ld.sync.aligned.16x256b.x2.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+                 : "r"(ta0));
+    asm volatile("tcgen05.ld.sync.aligned.16x256b.x2.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                 : "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+                 : "r"(ta1));
     asm volatile("tcgen05.wait::ld.sync.aligned;"
                  : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]),
-                   "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15]),
-                   "+r"(r[16]), "+r"(r[17]), "+r"(r[18]), "+r"(r[19]), "+r"(r[20]), "+r"(r[21]), "+r"(r[22]), "+r"(r[23]),
-                   "+r"(r[24]), "+r"(r[25]), "+r"(r[26]), "+r"(r[27]), "+r"(r[28])
+                   "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15])
                  :
                  : "memory");
-    asm volatile("" : "+r"(r[29]), "+r"(r[30]), "+r"(r[31]) : : "memory");
 #pragma unroll
-    for (int q = 0; q < 32; ++q) v[q >> 3][(q >> 2) & 1][q & 3] = __uint_as_float(r[q]);
+    for (int q = 0; q < 16; ++q) v[q >> 3][(q >> 2) & 1][q & 3] = __uint_as_float(r[q]);
 }
+
+// one arrival of a warp whose lanes have all got here
+__device__ __forceinline__ void mbar_arrive_warp(uint64_t* mbar);
+
+// move registers between the warpgroups of a CTA (every warp of the warpgroup; N a multiple of 8)
+template <int N>
+__device__ __forceinline__ void reg_dec() { asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(N)); }
+template <int N>
+__device__ __forceinline__ void reg_inc() { asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(N)); }
 
 // one arrival of the calling thread
 __device__ __forceinline__ void mbar_arrive(uint64_t* mbar) {
     asm volatile("{\n.reg .b64 t;\nmbarrier.arrive.shared::cta.b64 t, [%0];\n}\n" ::"r"(smem_u32(mbar)) : "memory");
 }
 
-// As mbar_wait, but also gives up once *abort (shared memory) is set by another waiter;
-// a wait that reaches its limit sets it.
-__device__ __forceinline__ bool mbar_wait_or(uint64_t* mbar, uint32_t phase, uint32_t limit, volatile int* abort) {
+__device__ __forceinline__ void mbar_arrive_warp(uint64_t* mbar) {
+    __syncwarp();
+    if ((threadIdx.x & 31) == 0) mbar_arrive(mbar);
+}
+
+// the same predicate for the 128 threads of named barrier `id`: true when it is for all of them
+__device__ __forceinline__ bool group_all(int id, bool v) {
+    uint32_t r;
+    asm volatile("{\n.reg .pred p, q;\nsetp.ne.u32 q, %2, 0;\nbarrier.cta.red.and.pred p, %1, 128, q;\nselp.u32 %0, 1, 0, p;\n}\n"
+                 : "=r"(r)
+                 : "r"(id), "r"((uint32_t)v)
+                 : "memory");
+    return r != 0;
+}
+
+// As mbar_wait, but also gives up once *abort (shared memory) is set by another waiter; a wait
+// that reaches its limit sets it.  A poll suspends the thread in hardware until the phase completes
+// or TC_SUSPEND_NS have passed, so that waiting warps leave the issue slots to the others.
+#define TC_SUSPEND_NS 1000
+__device__ __forceinline__ bool mbar_wait_or(uint64_t* mbar, uint32_t phase, uint32_t limit, volatile int* abort,
+                                             uint32_t nap = TC_POLL_NS) {
+    uint32_t done;
+    asm volatile(
+        "{\n.reg .pred p;\nmbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}\n"
+        : "=r"(done)
+        : "r"(smem_u32(mbar)), "r"(phase)
+        : "memory");
+    if (done) return true;
     for (uint32_t it = 0; it < limit; ++it) {
-        uint32_t done;
         asm volatile(
-            "{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}\n"
+            "{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\nselp.u32 %0, 1, 0, p;\n}\n"
             : "=r"(done)
-            : "r"(smem_u32(mbar)), "r"(phase)
+            : "r"(smem_u32(mbar)), "r"(phase), "r"((uint32_t)TC_SUSPEND_NS)
             : "memory");
         if (done) return true;
-        if ((it & 15) == 15) {
-            if (*abort) return false;
-            __nanosleep(TC_POLL_NS);
-        }
+        if (*abort) return false;
+        __nanosleep(nap);
     }
     *abort = 1;
     return false;
 }
+
+// MMA and commit by one elected lane of a converged warp: called by all lanes with the same
+// operands, which then stay in uniform registers (a lone lane's operands are moved there for every
+// instruction)
+__device__ __forceinline__ void mma_f16_warp(uint32_t dtmem, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
+    asm volatile(
+        "{\n.reg .pred p, e;\nsetp.ne.b32 p, %4, 0;\nelect.sync _|e, 0xffffffff;\n"
+        "@e tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(dtmem),
+        "l"(a), "l"(b), "r"(idesc), "r"(acc));
+}
+
+__device__ __forceinline__ void commit_warp(uint64_t* mbar) {
+    asm volatile(
+        "{\n.reg .pred e;\nelect.sync _|e, 0xffffffff;\n"
+        "@e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n}\n" ::"r"(smem_u32(mbar)));
+}
+
+__device__ __forceinline__ int uniform(int v) { return __shfl_sync(0xffffffffu, v, 0); }
 
 // 16-byte asynchronous global -> shared copies (completion by wait_all)
 __device__ __forceinline__ void cp_async16(void* smem_dst, const void* gsrc) {
