@@ -207,79 +207,6 @@ struct OctCfg {
     static size_t smem(int M) { return (size_t)PC * PER * sizeof(T) + 216 * sizeof(int) + 4 * (size_t)M * sizeof(uint32_t); }
 };
 
-// out += F x over the entries with c + i even (PAR 0) or odd (PAR 1)
-template <typename T, int K, int PAR>
-__device__ __forceinline__ void half_mul(const T* F, const T* x, T* out) {
-#pragma unroll
-    for (int c = 0; c < K; ++c)
-#pragma unroll
-        for (int i = (c + PAR) & 1; i < K; i += 2) out[c] += F[c * K + i] * x[i];
-}
-
-// out += F x; FP32 sums each product on its own before adding it (shorter chains of roundings)
-template <typename T, int K>
-__device__ __forceinline__ void full_mul(const T* F, const T* x, T* out) {
-    if (sizeof(T) == 8) {
-        half_mul<T, K, 0>(F, x, out);
-        half_mul<T, K, 1>(F, x, out);
-        return;
-    }
-#pragma unroll
-    for (int c = 0; c < K; ++c) {
-        T acc = (T)0;
-#pragma unroll
-        for (int i = 0; i < K; ++i) acc += F[c * K + i] * x[i];
-        out[c] += acc;
-    }
-}
-
-// out += F^t xp + F^{-t} xm.  FP32 takes the two products: the rounding of the sums would
-// show in the result (3.7e-8 against 2.9e-8 relative on the k = 5 case).
-template <typename T, int K>
-__device__ __forceinline__ void pair_mul(const T* Ft, const T* Fm, const T* xp, const T* xm, T* out) {
-    if (sizeof(T) == 4) {
-        full_mul<T, K>(Ft, xp, out);
-        full_mul<T, K>(Fm, xm, out);
-        return;
-    }
-    T s[K], d[K];
-#pragma unroll
-    for (int i = 0; i < K; ++i) {
-        s[i] = xp[i] + xm[i];
-        d[i] = xp[i] - xm[i];
-    }
-    half_mul<T, K, 0>(Ft, s, out);
-    half_mul<T, K, 1>(Ft, d, out);
-}
-
-// out = sum over b of F^{a + 2 - b} x[b], the translations of `set` (1 core, 2 off, 3 both);
-// F: tiles of t = -3..3
-template <typename T, int K>
-__device__ __forceinline__ void band_sum(const T* F, int set, int a, const T (*x)[K], T* out) {
-    constexpr int K2 = K * K;
-#pragma unroll
-    for (int c = 0; c < K; ++c) out[c] = (T)0;
-    if (a == 0) {
-        if (set & 1) {
-            pair_mul<T, K>(F + 4 * K2, F + 2 * K2, x[1], x[3], out);
-            half_mul<T, K, 0>(F + 3 * K2, x[2], out);
-        }
-        if (set & 2) {
-            pair_mul<T, K>(F + 5 * K2, F + K2, x[0], x[4], out);
-            full_mul<T, K>(F, x[5], out);
-        }
-    } else {
-        if (set & 1) {
-            pair_mul<T, K>(F + 4 * K2, F + 2 * K2, x[2], x[4], out);
-            half_mul<T, K, 0>(F + 3 * K2, x[3], out);
-        }
-        if (set & 2) {
-            pair_mul<T, K>(F + 5 * K2, F + K2, x[1], x[5], out);
-            full_mul<T, K>(F + 6 * K2, x[0], out);
-        }
-    }
-}
-
 template <typename T, int K>
 __global__ void __launch_bounds__(OctCfg<T, K>::NT) k_apply_oct(OctArgs P) {
     using C = OctCfg<T, K>;

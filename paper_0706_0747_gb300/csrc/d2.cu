@@ -7,6 +7,7 @@
 #include <algorithm>
 #include <cmath>
 
+#include "band_sum.cuh"
 #include "mra_internal.cuh"
 
 namespace mra {
@@ -425,101 +426,163 @@ static int build_tree2_impl(const mra_density* f, int k, double eps, int max_lev
 }
 
 // ------------------------------------------------------------ two-scale transforms in d = 2
-// compress: block per node of a level; an internal node gathers the (2k)^2
-// square of its 4 children, forms W sq W^T, keeps the k x k corner as its s
-// and the norm of the rest (its three wavelet blocks) as dnorm.
-__global__ void k_compress2_level(int k, int lo, int hi, const int32_t* child, double* s, double* dnorm,
-                                  const double* filt) {
-    extern __shared__ double sm[];
-    __shared__ double red[32];
-    const int i = lo + blockIdx.x;
-    if (i >= hi || child[i] < 0) return;
-    const int n2 = 2 * k, kk = k * k, c0 = child[i];
-    const double* W = filt + 2 * kk;
-    double* sq = sm;
-    double* t = sq + 4 * kk;
-    for (int e = threadIdx.x; e < 4 * kk; e += blockDim.x) {
-        const int r = e / n2, c = e % n2;
-        const int o = 2 * (r / k) + c / k;
-        sq[e] = s[(size_t)(c0 + o) * kk + (r % k) * k + (c % k)];
+// A warp per sibling group (the groups of level j+1 are its nodes by fours, in the order of
+// their parents), a lane per fiber.  Both halves of the filter come from H^(0) by parity:
+// H^(1)_{ia} = (-1)^{i+a} H^(0)_{ia}, zero for a > i (the d = 3 transforms' identities).  The
+// wavelet norm is ||children - upsampled parent|| = ||d|| (the filter matrix is orthogonal), for all
+// levels in one launch after the scaling blocks.  k = 8: 1,250 FP64 operations a group for the
+// scaling block and as many for the norm, where the full filter matrix took 8,192 (12 us per
+// level, a block per node).
+#define W2_WARPS 4
+
+// src (2 fibers' worth of K at stride st, the second half at src + h) -> y
+template <int K>
+__device__ __forceinline__ void down2_fiber(const double* H, const double* src, int st, int h, double* y) {
+    double p[K], m[K];
+#pragma unroll
+    for (int a = 0; a < K; ++a) {
+        const double x0 = src[a * st], x1 = (a & 1) ? -src[a * st + h] : src[a * st + h];
+        p[a] = x0 + x1;
+        m[a] = x0 - x1;
     }
-    __syncthreads();
-    for (int e = threadIdx.x; e < 4 * kk; e += blockDim.x) {
-        const int a = e / n2, c = e % n2;
+#pragma unroll
+    for (int i = 0; i < K; ++i) {
         double acc = 0.0;
-        for (int r = 0; r < n2; ++r) acc += W[a * n2 + r] * sq[r * n2 + c];
-        t[e] = acc;
+#pragma unroll
+        for (int a = 0; a <= i; ++a) acc += H[i * K + a] * ((i & 1) ? m[a] : p[a]);
+        y[i] = acc;
     }
-    __syncthreads();
-    double nrm = 0.0;
-    for (int e = threadIdx.x; e < 4 * kk; e += blockDim.x) {
-        const int a = e / n2, b = e % n2;
-        double acc = 0.0;
-        for (int c = 0; c < n2; ++c) acc += t[a * n2 + c] * W[b * n2 + c];
-        if (a < k && b < k) s[(size_t)i * kk + a * k + b] = acc;
-        else nrm += acc * acc;
-    }
-    nrm = blk2_sum(nrm, red);
-    if (threadIdx.x == 0) dnorm[i] = sqrt(nrm);
 }
 
-static int compress2_impl(mra_tree2* t, cudaStream_t st) {
-    const int kk = t->k * t->k;
+// s (K values at stride st) -> x0[K], x1[K]: the children's fibers
+template <int K>
+__device__ __forceinline__ void up2_fiber(const double* H, const double* src, int st, double* x0, double* x1) {
+    double v[K];
+#pragma unroll
+    for (int i = 0; i < K; ++i) v[i] = src[i * st];
+#pragma unroll
+    for (int a = 0; a < K; ++a) {
+        double s0 = 0.0, s1 = 0.0;
+#pragma unroll
+        for (int i = a; i < K; i += 2) s0 += H[i * K + a] * v[i];
+#pragma unroll
+        for (int i = a + 1; i < K; i += 2) s1 += H[i * K + a] * v[i];
+        x0[a] = s0 + s1;
+        x1[a] = s0 - s1;
+    }
+}
+
+// MODE 0: scaling block of the parent; 1: its wavelet norm; 2: children += upsampled parent
+template <int K, int MODE>
+__global__ void __launch_bounds__(32 * W2_WARPS) k_scale2(int ng, int cbase, const int32_t* parent, double* s, double* dnorm,
+                                                          const double* filt) {
+    constexpr int KK = K * K, K1 = K + 1;
+    __shared__ double H[KK];
+    __shared__ double buf[W2_WARPS][2 * K * K1];
+    for (int e = threadIdx.x; e < KK; e += blockDim.x) H[e] = filt[e];
+    __syncthreads();
+    const int lane = threadIdx.x & 31, wl = threadIdx.x >> 5, g = blockIdx.x * W2_WARPS + wl;
+    if (g >= ng) return;
+    const int c0 = cbase + 4 * g, par = parent[c0];
+    double* t = buf[wl];  // (2k, k), rows padded
+    double* ch = s + (size_t)c0 * KK;
+    if (MODE == 0) {
+        // direction 1: fiber of column c (0..2k-1) of the children's square, rows r of both halves
+        if (lane < 2 * K) {
+            double y[K];
+            down2_fiber<K>(H, ch + (lane / K) * KK + lane % K, K, 2 * KK, y);
+#pragma unroll
+            for (int i = 0; i < K; ++i) t[lane * K1 + i] = y[i];  // (column, i1)
+        }
+        __syncwarp();
+        if (lane < K) {  // direction 2: row i1
+            double y[K];
+            down2_fiber<K>(H, t + lane, K1, K * K1, y);
+#pragma unroll
+            for (int i = 0; i < K; ++i) s[(size_t)par * KK + lane * K + i] = y[i];
+        }
+        return;
+    }
+    // direction 1 of the parent's block: column i2 -> rows 0..2k-1
+    if (lane < K) {
+        double x0[K], x1[K];
+        up2_fiber<K>(H, s + (size_t)par * KK + lane, K, x0, x1);
+#pragma unroll
+        for (int a = 0; a < K; ++a) {
+            t[a * K1 + lane] = x0[a];
+            t[(K + a) * K1 + lane] = x1[a];
+        }
+    }
+    __syncwarp();
+    double acc = 0.0;
+    if (lane < 2 * K) {  // direction 2: row `lane` of the square
+        double x0[K], x1[K];
+        up2_fiber<K>(H, t + lane * K1, 1, x0, x1);
+        double* d0 = ch + (lane / K) * 2 * KK + (lane % K) * K;
+#pragma unroll
+        for (int a = 0; a < K; ++a) {
+            if (MODE == 2) {
+                d0[a] += x0[a];
+                d0[KK + a] += x1[a];
+            } else {
+                const double e0 = d0[a] - x0[a], e1 = d0[KK + a] - x1[a];
+                acc += e0 * e0 + e1 * e1;
+            }
+        }
+    }
+    if (MODE == 1) {
+        for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+        if (lane == 0) dnorm[par] = sqrt(acc);
+    }
+}
+
+template <int K>
+static int compress2_t(mra_tree2* t, cudaStream_t st) {
     for (int j = t->nlev - 2; j >= 0; --j) {
-        const int lo = t->off[j], hi = t->off[j + 1];
-        if (hi <= lo) continue;
-        k_compress2_level<<<hi - lo, 128, 8 * (size_t)kk * sizeof(double), st>>>(t->k, lo, hi, t->child, t->s,
-                                                                                t->dnorm, t->filt);
+        const int ng = (t->off[j + 2] - t->off[j + 1]) / 4;
+        if (ng <= 0) continue;
+        k_scale2<K, 0><<<(ng + W2_WARPS - 1) / W2_WARPS, 32 * W2_WARPS, 0, st>>>(ng, t->off[j + 1], t->parent, t->s, t->dnorm, t->filt);
         MRA_CK_LAUNCH();
     }
+    const int ng = (t->n - 1) / 4;
+    if (ng > 0) {
+        k_scale2<K, 1><<<(ng + W2_WARPS - 1) / W2_WARPS, 32 * W2_WARPS, 0, st>>>(ng, 1, t->parent, t->s, t->dnorm, t->filt);
+        MRA_CK_LAUNCH();
+    }
+    return MRA_OK;
+}
+
+template <int K>
+static int assemble2_t(mra_tree2* t, cudaStream_t st) {
+    for (int j = 0; j + 1 < t->nlev; ++j) {
+        const int ng = (t->off[j + 2] - t->off[j + 1]) / 4;
+        if (ng <= 0) continue;
+        k_scale2<K, 2><<<(ng + W2_WARPS - 1) / W2_WARPS, 32 * W2_WARPS, 0, st>>>(ng, t->off[j + 1], t->parent, t->s, t->dnorm, t->filt);
+        MRA_CK_LAUNCH();
+    }
+    return MRA_OK;
+}
+
+#define FOR_EVERY_K(F) \
+    { nullptr, F<1>, F<2>, F<3>, F<4>, F<5>, F<6>, F<7>, F<8>, F<9>, F<10>, F<11>, F<12> }
+
+static int compress2_impl(mra_tree2* t, cudaStream_t st) {
+    static int (*const fn[])(mra_tree2*, cudaStream_t) = FOR_EVERY_K(compress2_t);
+    MRA_TRY(fn[t->k](t, st));
     t->state = MRA_TREE_REDUNDANT;
     return MRA_OK;
 }
 
-// eq. g_assemble: each child of an internal node adds H^(p1)T s H^(p2)
-__global__ void k_up2_level(int k, int lo, int hi, const int32_t* child, double* s, const double* filt) {
-    extern __shared__ double sm[];
-    const int i = lo + blockIdx.x;
-    if (i >= hi || child[i] < 0) return;
-    const int kk = k * k, c0 = child[i];
-    double* x = sm;
-    double* t = x + kk;
-    for (int e = threadIdx.x; e < kk; e += blockDim.x) x[e] = s[(size_t)i * kk + e];
-    __syncthreads();
-    for (int o = 0; o < 4; ++o) {
-        const double* H1 = filt + (o >> 1) * kk;
-        const double* H2 = filt + (o & 1) * kk;
-        for (int e = threadIdx.x; e < kk; e += blockDim.x) {
-            const int a = e / k, i2 = e % k;
-            double acc = 0.0;
-            for (int i1 = 0; i1 < k; ++i1) acc += H1[i1 * k + a] * x[i1 * k + i2];
-            t[e] = acc;
-        }
-        __syncthreads();
-        for (int e = threadIdx.x; e < kk; e += blockDim.x) {
-            const int a = e / k, b = e % k;
-            double acc = 0.0;
-            for (int i2 = 0; i2 < k; ++i2) acc += t[a * k + i2] * H2[i2 * k + b];
-            s[(size_t)(c0 + o) * kk + e] += acc;
-        }
-        __syncthreads();
-    }
-}
-
+// eq. g_assemble
 static int assemble2_impl(mra_tree2* t, cudaStream_t st) {
-    const int kk = t->k * t->k;
-    for (int j = 0; j + 1 < t->nlev; ++j) {
-        const int lo = t->off[j], hi = t->off[j + 1];
-        if (hi <= lo) continue;
-        k_up2_level<<<hi - lo, 64, 2 * (size_t)kk * sizeof(double), st>>>(t->k, lo, hi, t->child, t->s, t->filt);
-        MRA_CK_LAUNCH();
-    }
+    static int (*const fn[])(mra_tree2*, cudaStream_t) = FOR_EVERY_K(assemble2_t);
+    MRA_TRY(fn[t->k](t, st));
     t->state = MRA_TREE_LEAVES;
     return MRA_OK;
 }
 
-// sum of the squares of the leaf blocks: fixed 256 partial sums, then one
-// thread adds them in order (the result does not depend on scheduling)
+// sum of the squares of the leaf blocks: fixed 256 partial sums, then one warp
+// adds them in a fixed order (the result does not depend on scheduling)
 #define NORM_PARTS 256
 __global__ void k_leaf_sq_partial2(int n, int kk, const int32_t* leaf, const double* s, double* part) {
     __shared__ double red[32];
@@ -533,10 +596,10 @@ __global__ void k_leaf_sq_partial2(int n, int kk, const int32_t* leaf, const dou
 }
 
 __global__ void k_sum_parts2(int np, const double* part, double* out) {
-    if (threadIdx.x != 0) return;
     double s = 0.0;
-    for (int i = 0; i < np; ++i) s += part[i];
-    *out = s;
+    for (int i = threadIdx.x; i < np; i += 32) s += part[i];
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (threadIdx.x == 0) *out = s;
 }
 
 static int leaf_norm2(const mra_tree2* t, double* part, double* out, cudaStream_t st) {
@@ -589,6 +652,11 @@ __global__ void k_new_offsets2(Offs2 off, int nlev, int n, const int32_t* newidx
     out[j] = (j < nlev && off.v[j] < n) ? newidx[off.v[j]] : *total;
 }
 
+__global__ void k_ones2(int n, int32_t* p) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < n) p[i] = 1;
+}
+
 static int truncate2_impl(mra_tree2* t, double eps, cudaStream_t st, double* removed_host) {
     const int n = t->n, kk = t->k * t->k;
     Scratch tmp(t->A);
@@ -604,8 +672,8 @@ static int truncate2_impl(mra_tree2* t, double eps, cudaStream_t st, double* rem
     k_trunc_thr2<<<1, 32, 0, st>>>(eps, n, sc, sc + 1);
     MRA_CK_LAUNCH();
     MRA_CK(cudaMemsetAsync(sc + 2, 0, sizeof(double), st));
-    std::vector<int32_t> ones(n, 1);
-    MRA_CK(cudaMemcpyAsync(alive, ones.data(), n * sizeof(int32_t), cudaMemcpyHostToDevice, st));
+    k_ones2<<<(n + 255) / 256, 256, 0, st>>>(n, alive);
+    MRA_CK_LAUNCH();
     for (int j = t->nlev - 2; j >= 0; --j) {
         const int lo = t->off[j], hi = t->off[j + 1];
         if (hi <= lo) continue;
@@ -622,7 +690,7 @@ static int truncate2_impl(mra_tree2* t, double eps, cudaStream_t st, double* rem
     double removed2 = 0.0;
     MRA_CK(cudaMemcpyAsync(hoffs, offs, sizeof(hoffs), cudaMemcpyDeviceToHost, st));
     MRA_CK(cudaMemcpyAsync(&removed2, sc + 2, sizeof(double), cudaMemcpyDeviceToHost, st));
-    MRA_CK(cudaStreamSynchronize(st));  // also keeps `ones` alive until its copy is done
+    MRA_CK(cudaStreamSynchronize(st));
     if (removed_host) *removed_host = sqrt(removed2);
     const int nn = hoffs[MRA_MAX_LEVEL + 1];
     if (nn == n) return MRA_OK;
@@ -661,48 +729,54 @@ static int truncate2_impl(mra_tree2* t, double eps, cudaStream_t st, double* rem
 }
 
 // ------------------------------------------------------------ Algorithm 3 in d = 2
-// ||T_0 f_0||: y = sum_m w_m F_m X F_m^T on the root block (j = 0, t = 0); dv[1]
-__global__ void k_pilot2(int k, int M, const double* w, const double* F, const double* s_root, double* dv) {
-    extern __shared__ double sm[];
-    __shared__ double red[32];
-    const int kk = k * k, tid = threadIdx.x;
-    double* X = sm;
-    double* Z = X + kk;
-    for (int e = tid; e < kk; e += blockDim.x) X[e] = s_root[e];
-    __syncthreads();
-    double y0 = 0.0, y1 = 0.0;
-    for (int m = 0; m < M; ++m) {
-        const double* Fm = F + ((size_t)m * 7 + 3) * kk;
-        for (int e = tid; e < kk; e += blockDim.x) {
-            const int a = e / k, c = e % k;
-            double acc = 0.0;
-            for (int i = 0; i < k; ++i) acc += Fm[a * k + i] * X[i * k + c];
-            Z[e] = acc;
-        }
-        __syncthreads();
-        if (tid < kk) {
-            double acc = 0.0;
-            for (int c = 0; c < k; ++c) acc += Z[(tid / k) * k + c] * Fm[(tid % k) * k + c];
-            y0 += w[m] * acc;
-        }
-        if (tid + (int)blockDim.x < kk) {
-            const int e = tid + blockDim.x;
-            double acc = 0.0;
-            for (int c = 0; c < k; ++c) acc += Z[(e / k) * k + c] * Fm[(e % k) * k + c];
-            y1 += w[m] * acc;
-        }
-        __syncthreads();
+// ||T_0 f_0||: y = sum_m w_m F_m X F_m^T on the root block (j = 0, t = 0): block per term, then
+// the terms summed per coefficient in order and the norm taken; dv[1]
+__global__ void k_pilot2_terms(int k, const double* w, const double* F, const double* s_root, double* ym) {
+    __shared__ double X[MRA_MAX_K * MRA_MAX_K], Z[MRA_MAX_K * MRA_MAX_K], Fm[MRA_MAX_K * MRA_MAX_K];
+    const int kk = k * k, m = blockIdx.x, e = threadIdx.x;
+    if (e < kk) {
+        X[e] = s_root[e];
+        Fm[e] = F[((size_t)m * 7 + 3) * kk + e];
     }
-    const double nrm = blk2_sum(y0 * y0 + y1 * y1, red);
-    if (tid == 0) dv[1] = sqrt(nrm);
+    __syncthreads();
+    const int a = e / k, c = e % k;
+    if (e < kk) {
+        double acc = 0.0;
+        for (int i = 0; i < k; ++i) acc += Fm[a * k + i] * X[i * k + c];
+        Z[e] = acc;
+    }
+    __syncthreads();
+    if (e < kk) {
+        double acc = 0.0;
+        for (int i = 0; i < k; ++i) acc += Z[a * k + i] * Fm[c * k + i];
+        ym[(size_t)m * kk + e] = w[m] * acc;
+    }
+}
+
+__global__ void k_pilot2_sum(int kk, int M, const double* ym, double* dv) {
+    __shared__ double red[32], part[4][MRA_MAX_K * MRA_MAX_K];
+    const int e = threadIdx.x % 160, q = threadIdx.x / 160;  // four quarters of the terms
+    double y = 0.0;
+    if (e < kk)
+        for (int m = q * M / 4; m < (q + 1) * M / 4; ++m) y += ym[(size_t)m * kk + e];
+    if (e < kk) part[q][e] = y;
+    __syncthreads();
+    y = threadIdx.x < kk ? ((part[0][threadIdx.x] + part[1][threadIdx.x]) + part[2][threadIdx.x]) + part[3][threadIdx.x] : 0.0;
+    const double nrm = blk2_sum(y * y, red);
+    if (threadIdx.x == 0) dv[1] = sqrt(nrm);
 }
 
 // eta = eps sigma / ||f||; J_m; per scale j and subset S = 0, 1, 2 the range
 // [m1, m2] trimmed from both ends while the cumulative w_m c^S b^(2-S) stays
 // <= eta / 72 (c, b: the largest N_F over |l| <= 1 and over 2 <= |l| <= 3).
 // Layout: Jm[M] | m1[nlev*3] | m2[nlev*3].
+// (The bounds of all (j, S, m) are formed in parallel in shared memory; a term with J_m < j
+// gets 0, which the serial scans pass over as they skip it.)
 __global__ void k_schedule2(int M, int nlev, double eps, const double* w, const double* nF, const double* est,
                             double* dv, int32_t* sched) {
+    extern __shared__ double sched2_sm[];
+    double* ev = sched2_sm;                // [nlev * 3][M]
+    int* Js = (int*)(ev + (size_t)nlev * 3 * M);
     int32_t* Jm = sched;
     int32_t* m1 = Jm + M;
     int32_t* m2 = m1 + nlev * 3;
@@ -714,40 +788,42 @@ __global__ void k_schedule2(int M, int nlev, double eps, const double* w, const 
         for (int j = 1; j < nlev; ++j)
             if (w[m] * est[(size_t)j * M + m] > eta / M) jm = j;
         Jm[m] = jm;
+        Js[m] = jm;
+    }
+    __syncthreads();
+    for (int e = threadIdx.x; e < nlev * M; e += blockDim.x) {
+        const int j = e / M, m = e - j * M;
+        const double* r = nF + (size_t)e * 7;
+        const double c = fmax(fmax(r[2], r[3]), r[4]);
+        const double bb = fmax(fmax(r[0], r[1]), fmax(r[5], r[6]));
+        const bool on = Js[m] >= j;
+        ev[((size_t)j * 3 + 0) * M + m] = on ? w[m] * bb * bb : 0.0;
+        ev[((size_t)j * 3 + 1) * M + m] = on ? w[m] * c * bb : 0.0;
+        ev[((size_t)j * 3 + 2) * M + m] = on ? w[m] * c * c : 0.0;
     }
     __syncthreads();
     const double budget = eta / (2.0 * 36.0);
     for (int js = threadIdx.x; js < nlev * 3; js += blockDim.x) {
-        const int j = js / 3, S = js % 3;
+        const int j = js / 3;
         int lo_m = 0, hi_m = -1, first = -1, last = -1;
         for (int m = 0; m < M; ++m)
-            if (Jm[m] >= j) {
+            if (Js[m] >= j) {
                 if (first < 0) first = m;
                 last = m;
             }
         if (first >= 0) {
-            auto e_of = [&](int m) {
-                const double* r = nF + ((size_t)j * M + m) * 7;
-                const double c = fmax(fmax(r[2], r[3]), r[4]);
-                const double bb = fmax(fmax(r[0], r[1]), fmax(r[5], r[6]));
-                double v = w[m];
-                for (int q = 0; q < S; ++q) v *= c;
-                for (int q = S; q < 2; ++q) v *= bb;
-                return v;
-            };
+            const double* e_js = ev + (size_t)js * M;
             double acc = 0.0;
             int lo = first;
             for (; lo <= last; ++lo) {
-                if (Jm[lo] < j) continue;
-                const double e = e_of(lo);
+                const double e = e_js[lo];
                 if (acc + e <= budget) acc += e;
                 else break;
             }
             acc = 0.0;
             int hi = last;
             for (; hi >= lo; --hi) {
-                if (Jm[hi] < j) continue;
-                const double e = e_of(hi);
+                const double e = e_js[hi];
                 if (acc + e <= budget) acc += e;
                 else break;
             }
@@ -761,124 +837,269 @@ __global__ void k_schedule2(int M, int nlev, double eps, const double* w, const 
     }
 }
 
-// One block per output node.  For every band translation whose input box lies
-// in the square and that keeps a term: the input block (the node at level j,
-// or the ancestor leaf refined down with H^(p1)T X H^(p2) per level: Step 2),
-// then ghat += w_m F^{t1}_m X (F^{t2}_m)^T over the kept terms.
-// counters: [0] items, [1] pairs, [2] Step-2 refinements, [3] lookups that
-// found no ancestor (0 for a valid tree).
-__global__ void __launch_bounds__(128) k_apply2(int k, int M, int nlev, Offs2 off, const uint64_t* key,
-                                                const int32_t* coord, const int32_t* leaf, const double* s,
-                                                const double* F, const double* w, const int32_t* sched,
-                                                const double* filt, double* gout, unsigned long long* counters) {
+// Algorithm 3 in d = 2 by sibling groups, as in d = 3 (apply_oct.cu): the four siblings of a
+// group have the same 6 x 6 inputs, and a term's kept translations are a union of products
+// T1 x T2 of per-direction sets (core, off-core, both), so per such piece
+//   W[a1][b2] = sum_{t1 in T1} F^{t1} X[b1][b2],   ghat[a1][a2] += w_m sum_{t2 in T2} W[a1][b2] (F^{t2})^T,
+// 72 + 24 products of half the multiplications each (t and -t together) where an output box at a
+// time took 4 x 36 x 2.  FP64 multiply-adds are the bound: 2.7 ms -> 0.7 ms on the bench's
+// quadtree.  Block per group: the inputs are gathered (missing ones refined from their covering
+// leaf, Step 2) into shared memory; then four pieces at a time, stage I by thread (piece, a1, b2,
+// i2), stage II by thread (piece, a1, a2, c1), whose output fibers stay in registers.
+struct PieceTable2 {
+    PieceSet p[8];
+};
+constexpr PieceTable2 make_pieces2() {
+    PieceTable2 T{};
+    for (int A = 0; A < 8; ++A) piece_split(2, A, 0, T.p[A]);
+    return T;
+}
+__constant__ PieceTable2 c_pieces2 = make_pieces2();
+#define PIECE2_CC 0x5
+
+// counters: [0] items, [1] pairs, [2] Step-2 refinements an output box at a time would make, [3]
+// lookups that found no ancestor (0 for a valid tree)
+template <int K>
+struct Apply2Smem {
+    static constexpr int KK = K * K, K1 = K + 1, NT = (16 * K + 31) / 32 * 32, PC = 4;
+    static size_t bytes(int M) {
+        return (size_t)(36 * KK + PC * 12 * K * K1 + PC * 7 * KK + 2 * KK + 3 * KK) * sizeof(double) + 4 * (size_t)M * sizeof(uint32_t);
+    }
+};
+
+template <int K>
+__global__ void __launch_bounds__(Apply2Smem<K>::NT) k_apply2(int M, int nlev, Offs2 off, const uint64_t* key,
+                                                              const int32_t* coord, const int32_t* leaf, const double* s,
+                                                              const double* F, const double* w, const int32_t* sched,
+                                                              const double* filt, double* gout, unsigned long long* counters) {
+    using L = Apply2Smem<K>;
+    constexpr int KK = L::KK, K1 = L::K1, NT = L::NT, PC = L::PC;
     extern __shared__ double sm[];
-    const int kk = k * k, tid = threadIdx.x;
-    double* X = sm;
-    double* Z = X + kk;
-    double* T = Z + kk;
-    double* Hs = T + kk;
-    int* Js = (int*)(Hs + 2 * kk);
-    __shared__ int s_src, s_lev;
-    const int node = blockIdx.x;
-    for (int e = tid; e < 2 * kk; e += blockDim.x) Hs[e] = filt[e];
-    for (int m = tid; m < M; m += blockDim.x) Js[m] = sched[m];
-    const int32_t* m1 = sched + M;
-    const int32_t* m2 = m1 + nlev * 3;
-    const int j = coord[3 * node], a1 = coord[3 * node + 1], a2 = coord[3 * node + 2];
-    const bool isleaf = leaf[node] != 0;
-    const int N = 1 << j;
-    double y0 = 0.0, y1 = 0.0;
-    unsigned long long items = 0, pairs = 0, ghosts = 0, lost = 0;
+    double* X = sm;                        // [6][6] blocks
+    double* W = X + 36 * KK;               // [PC][2][6] blocks (c1 rows padded)
+    double* Ft = W + PC * 12 * K * K1;     // [PC][7] tiles
+    double* H = Ft + PC * 7 * KK;          // H^(0), H^(1)
+    double* T = H + 2 * KK;                // refinement: 3 blocks
+    uint32_t* list = (uint32_t*)(T + 3 * KK);
+    __shared__ int s_np, s_base[9], s_anc[9], s_lev[9], s_nout;
+    __shared__ unsigned s_leaf, s_need[9];
+    const int tid = threadIdx.x, lane = tid & 31, g = blockIdx.x;
+    const int i0 = g == 0 ? 0 : 1 + 4 * (g - 1);
+    const int j = coord[3 * i0], nout = j ? 4 : 1;
+    const int p1 = coord[3 * i0 + 1] >> 1, p2 = coord[3 * i0 + 2] >> 1;
+    const int32_t *m1 = sched + M + 3 * j, *m2 = sched + M + 3 * nlev + 3 * j;
+    for (int e = tid; e < 2 * KK; e += NT) H[e] = filt[e];
+    if (tid < 32) {
+        const unsigned leafm = __ballot_sync(0xffffffffu, lane < nout && leaf[i0 + (lane < nout ? lane : 0)]);
+        const bool any_int = leafm != (1u << nout) - 1u;
+        // the pieces, and the kept terms per class (S; the core at an internal box: index 3)
+        int lo[3], hi[3], cnt[4] = {0, 0, 0, 0}, np = 0, first = M, last = -1;
+        for (int S = 0; S < 3; ++S) {
+            lo[S] = m1[S];
+            hi[S] = m2[S];
+            if (hi[S] >= lo[S]) {
+                first = min(first, lo[S]);
+                last = max(last, hi[S]);
+            }
+        }
+        for (int mb = first; mb <= last; mb += 32) {
+            const int m = mb + lane;
+            int A = 0;
+            bool extra = false;
+            if (m <= last && sched[m] >= j) {
+                for (int S = 0; S < 3; ++S) A |= (m >= lo[S] && m <= hi[S]) << S;
+                for (int S = 0; S < 3; ++S) cnt[S] += (A >> S) & 1;
+                if (sched[m] == j) cnt[3] += (A >> 2) & 1;
+                if (sched[m] > j && any_int && (A & 4)) {
+                    A &= 3;
+                    extra = leafm != 0;
+                }
+            }
+            const PieceSet& P = c_pieces2.p[A];
+            const int n = P.n + extra;
+            int at = n;
+            for (int o = 1; o < 32; o <<= 1) {
+                const int v = __shfl_up_sync(0xffffffffu, at, o);
+                if (lane >= o) at += v;
+            }
+            const int sum = __shfl_sync(0xffffffffu, at, 31);
+            at += np - n;
+            for (int i = 0; i < P.n; ++i) list[at++] = (uint32_t)m | ((uint32_t)P.box[i] << 16);
+            if (extra) list[at] = (uint32_t)m | ((uint32_t)PIECE2_CC << 16) | (1u << 24);
+            np += sum;
+        }
+        for (int S = 0; S < 4; ++S)
+            for (int o = 16; o > 0; o >>= 1) cnt[S] += __shfl_xor_sync(0xffffffffu, cnt[S], o);
+        // lane per neighbour of the parent: its children at level j, or the leaf that covers it
+        unsigned long long items = 0, pairs = 0, ghosts = 0, lost = 0;
+        if (lane < 9) {
+            const int d1 = lane / 3, d2 = lane % 3;
+            const int q1 = p1 + d1 - 1, q2 = p2 + d2 - 1, N = j ? 1 << (j - 1) : 1;
+            int base = -1, anc = -1, lev = -1;
+            bool inside = j ? q1 >= 0 && q2 >= 0 && q1 < N && q2 < N : lane == 4;
+            if (j == 0) base = inside ? i0 : -1;
+            else if (inside) base = find_key_exact(key, off.v[j], off.v[j + 1], morton2(q1, q2) << 2);
+            unsigned need = 0;
+            if (inside)
+                for (int o = 0; o < (j ? 4 : 1); ++o) {
+                    const int b1 = 2 * d1 + (o >> 1), b2 = 2 * d2 + (o & 1);
+                    for (int a = 0; a < nout; ++a) {
+                        const int S = band_core(a >> 1, b1) + band_core(a & 1, b2);
+                        const int n = S == 2 ? (((leafm >> a) & 1u) ? cnt[2] : cnt[3]) : (S ? cnt[1] : cnt[0]);
+                        if (n <= 0) continue;
+                        need |= 1u << o;
+                        ++pairs;
+                        items += n;
+                        ghosts += base < 0;
+                    }
+                }
+            if (need && base < 0) {
+                for (lev = j - 1; lev >= 0 && anc < 0; --lev)
+                    anc = find_key_exact(key, off.v[lev], off.v[lev + 1], morton2(q1 >> (j - 1 - lev), q2 >> (j - 1 - lev)));
+                ++lev;
+                if (anc < 0) ++lost;  // impossible for a complete tree; counted, read as zero
+            }
+            s_base[lane] = base;
+            s_need[lane] = need;
+            s_anc[lane] = anc;
+            s_lev[lane] = lev;
+        }
+        for (int o = 16; o > 0; o >>= 1) {
+            items += __shfl_xor_sync(0xffffffffu, items, o);
+            pairs += __shfl_xor_sync(0xffffffffu, pairs, o);
+            ghosts += __shfl_xor_sync(0xffffffffu, ghosts, o);
+            lost += __shfl_xor_sync(0xffffffffu, lost, o);
+        }
+        if (lane == 0) {
+            s_np = np;
+            s_leaf = leafm;
+            s_nout = nout;
+            atomicAdd(&counters[0], items);
+            atomicAdd(&counters[1], pairs);
+            atomicAdd(&counters[2], ghosts);
+            if (lost) atomicAdd(&counters[3], lost);
+        }
+    }
     __syncthreads();
-    for (int q1 = 0; q1 < 6; ++q1) {
-        const int t1 = band_t(a1, q1), b1 = a1 - t1;
-        if (b1 < 0 || b1 >= N) continue;
-        for (int q2 = 0; q2 < 6; ++q2) {
-            const int t2 = band_t(a2, q2), b2 = a2 - t2;
-            if (b2 < 0 || b2 >= N) continue;
-            const int S = (abs(t1) <= 1) + (abs(t2) <= 1);
-            const int lo = m1[j * 3 + S], hi = m2[j * 3 + S];
-            if (lo > hi) continue;
-            const bool core = S == 2;
-            int cnt = 0;
-            for (int m = lo; m <= hi; ++m) {
-                if (Js[m] < j || (core && !isleaf && Js[m] > j)) continue;
-                ++cnt;
-            }
-            if (cnt == 0) continue;
-            if (tid == 0) {
-                int jj = j, idx = -1;
-                for (; jj >= 0; --jj) {
-                    idx = find_key_exact(key, off.v[jj], off.v[jj + 1], morton2(b1 >> (j - jj), b2 >> (j - jj)));
-                    if (idx >= 0) break;
-                }
-                s_src = idx;
-                s_lev = jj;
+    const int np = s_np;
+    const unsigned leafm = s_leaf;
+    // the inputs that are nodes; the others zero until refined
+    for (int e = tid; e < 36 * KK; e += NT) {
+        const int q = e / KK, b1 = q / 6, b2 = q % 6, pi = (b1 >> 1) * 3 + (b2 >> 1), o = (b1 & 1) * 2 + (b2 & 1);
+        X[e] = s_base[pi] >= 0 && ((s_need[pi] >> o) & 1u) ? s[(size_t)(s_base[pi] + o) * KK + e % KK] : 0.0;
+    }
+    // Step 2, a missing parent at a time: down the path to the parent, then its four children
+    for (int pi = 0; pi < 9; ++pi) {
+        if (!s_need[pi] || s_base[pi] >= 0 || s_anc[pi] < 0) continue;
+        const int q1 = p1 + pi / 3 - 1, q2 = p2 + pi % 3 - 1, lev0 = s_lev[pi];
+        double *x = T, *y = T + KK, *z = T + 2 * KK;
+        __syncthreads();
+        for (int e = tid; e < KK; e += NT) x[e] = s[(size_t)s_anc[pi] * KK + e];
+        __syncthreads();
+        for (int lev = lev0; lev < j - 1; ++lev) {
+            const int sh = j - 2 - lev;
+            const double *H1 = H + ((q1 >> sh) & 1) * KK, *H2 = H + ((q2 >> sh) & 1) * KK;
+            for (int e = tid; e < KK; e += NT) {
+                const int a = e / K, c = e % K;
+                double acc = 0.0;
+                for (int i = a; i < K; ++i) acc += H1[i * K + a] * x[i * K + c];
+                y[e] = acc;
             }
             __syncthreads();
-            const int src = s_src, jj = s_lev;
-            if (src < 0) {  // impossible for a complete tree; counted, skipped
-                ++lost;
-                __syncthreads();
-                continue;
+            for (int e = tid; e < KK; e += NT) {
+                const int a = e / K, b = e % K;
+                double acc = 0.0;
+                for (int c = b; c < K; ++c) acc += y[a * K + c] * H2[c * K + b];
+                x[e] = acc;
             }
-            for (int e = tid; e < kk; e += blockDim.x) X[e] = s[(size_t)src * kk + e];
             __syncthreads();
-            for (int lev = jj; lev < j; ++lev) {
-                const int sh = j - lev - 1, p1 = (b1 >> sh) & 1, p2 = (b2 >> sh) & 1;
-                for (int e = tid; e < kk; e += blockDim.x) {
-                    const int a = e / k, c = e % k;
-                    double acc = 0.0;
-                    for (int i = 0; i < k; ++i) acc += Hs[p1 * kk + i * k + a] * X[i * k + c];
-                    T[e] = acc;
-                }
-                __syncthreads();
-                for (int e = tid; e < kk; e += blockDim.x) {
-                    const int a = e / k, b = e % k;
-                    double acc = 0.0;
-                    for (int c = 0; c < k; ++c) acc += T[a * k + c] * Hs[p2 * kk + c * k + b];
-                    X[e] = acc;
-                }
-                __syncthreads();
+        }
+        for (int f = tid; f < K; f += NT) {
+            double x0[K], x1[K];
+            up2_fiber<K>(H, x + f, K, x0, x1);
+            for (int a = 0; a < K; ++a) {
+                y[a * K + f] = x0[a];
+                z[a * K + f] = x1[a];
             }
-            if (jj < j) ++ghosts;
-            ++pairs;
-            items += cnt;
-            for (int m = lo; m <= hi; ++m) {
-                if (Js[m] < j || (core && !isleaf && Js[m] > j)) continue;
-                const double* F1 = F + (((size_t)j * M + m) * 7 + t1 + 3) * kk;
-                const double* F2 = F + (((size_t)j * M + m) * 7 + t2 + 3) * kk;
-                for (int e = tid; e < kk; e += blockDim.x) {
-                    const int a = e / k, c = e % k;
-                    double acc = 0.0;
-                    for (int i = 0; i < k; ++i) acc += F1[a * k + i] * X[i * k + c];
-                    Z[e] = acc;
-                }
-                __syncthreads();
-                const double wm = w[m];
-                if (tid < kk) {
-                    double acc = 0.0;
-                    for (int c = 0; c < k; ++c) acc += Z[(tid / k) * k + c] * F2[(tid % k) * k + c];
-                    y0 += wm * acc;
-                }
-                if (tid + (int)blockDim.x < kk) {
-                    const int e = tid + blockDim.x;
-                    double acc = 0.0;
-                    for (int c = 0; c < k; ++c) acc += Z[(e / k) * k + c] * F2[(e % k) * k + c];
-                    y1 += wm * acc;
-                }
-                __syncthreads();
+        }
+        __syncthreads();
+        for (int f = tid; f < 2 * K; f += NT) {
+            double x0[K], x1[K];
+            up2_fiber<K>(H, (f < K ? y : z) + (f % K) * K, 1, x0, x1);
+            double* d0 = X + (size_t)((2 * (pi / 3) + f / K) * 6 + 2 * (pi % 3)) * KK + (f % K) * K;
+            for (int a = 0; a < K; ++a) {
+                d0[a] = x0[a];
+                d0[KK + a] = x1[a];
             }
         }
     }
-    if (tid < kk) gout[(size_t)node * kk + tid] = y0;
-    if (tid + (int)blockDim.x < kk) gout[(size_t)node * kk + tid + blockDim.x] = y1;
-    if (tid == 0) {
-        atomicAdd(&counters[0], items);
-        atomicAdd(&counters[1], pairs);
-        atomicAdd(&counters[2], ghosts);
-        if (lost) atomicAdd(&counters[3], lost);
+    // stage II's thread: piece slot, a1, a2, c1
+    const int slot = tid / (4 * K), oa = (tid / K) & 3, oc = tid % K;
+    const int mya = (tid % (4 * K)) / K;
+    (void)oa;
+    double y[K];
+#pragma unroll
+    for (int c = 0; c < K; ++c) y[c] = 0.0;
+    for (int qb = 0; qb < np; qb += PC) {
+        const int npc = min(PC, np - qb);
+        __syncthreads();
+        for (int e = tid; e < npc * 7 * KK; e += NT)
+            Ft[e] = F[((size_t)j * M + (list[qb + e / (7 * KK)] & 0xffff)) * 7 * KK + e % (7 * KK)];
+        __syncthreads();
+        for (int task = tid; task < npc * 12 * K; task += NT) {
+            const int i2 = task % K, b2 = (task / K) % 6, pa = task / (6 * K), a1 = pa & 1, pc = pa >> 1;
+            const int box = (list[qb + pc] >> 16) & 0xff;
+            if (!((set_boxes(box & 3) >> b2) & 1u)) continue;
+            double x[6][K], out[K];
+#pragma unroll
+            for (int b1 = 0; b1 < 6; ++b1)
+#pragma unroll
+                for (int i = 0; i < K; ++i) x[b1][i] = X[(b1 * 6 + b2) * KK + i * K + i2];
+            band_sum<double, K>(Ft + pc * 7 * KK, box >> 2, a1, x, out);
+            double* dst = W + (pa * 6 + b2) * K * K1 + i2;
+#pragma unroll
+            for (int c = 0; c < K; ++c) dst[c * K1] = out[c];
+        }
+        __syncthreads();
+        if (slot < npc) {
+            const uint32_t p = list[qb + slot];
+            const int set = (p >> 16) & 3;
+            const unsigned boxes = set_boxes(set);
+            if (mya < s_nout && (!(p >> 24) || ((leafm >> mya) & 1u))) {
+                double x[6][K], out[K];
+#pragma unroll
+                for (int b2 = 0; b2 < 6; ++b2) {
+                    const double* src = W + ((slot * 2 + (mya >> 1)) * 6 + b2) * K * K1 + oc * K1;
+#pragma unroll
+                    for (int i = 0; i < K; ++i) x[b2][i] = ((boxes >> b2) & 1u) ? src[i] : 0.0;
+                }
+                band_sum<double, K>(Ft + slot * 7 * KK, set, mya & 1, x, out);
+                const double wm = w[p & 0xffff];
+#pragma unroll
+                for (int c = 0; c < K; ++c) y[c] += wm * out[c];
+            }
+        }
     }
+    // the four slots' sums in order
+    __syncthreads();
+    double* ys = W;  // [slot][a][c1][c2]
+    if (slot < PC)
+#pragma unroll
+        for (int c = 0; c < K; ++c) ys[(slot * 4 + mya) * KK + oc * K + c] = y[c];
+    __syncthreads();
+    for (int e = tid; e < s_nout * KK; e += NT)
+        gout[(size_t)i0 * KK + e] = ((ys[e] + ys[4 * KK + e]) + ys[8 * KK + e]) + ys[12 * KK + e];
+}
+
+template <int K>
+static int apply2_launch(int n, int M, int nlev, const Offs2& off, const mra_tree2* f, const mra_op* op, const int32_t* sched,
+                         double* gout, unsigned long long* counters, cudaStream_t st) {
+    using L = Apply2Smem<K>;
+    MRA_CK(cudaFuncSetAttribute(k_apply2<K>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L::bytes(M)));
+    k_apply2<K><<<1 + (n - 1) / 4, L::NT, L::bytes(M), st>>>(M, nlev, off, f->key, f->coord, f->leaf, f->s, op->F, op->w, sched,
+                                                              f->filt, gout, counters);
+    MRA_CK_LAUNCH();
+    return MRA_OK;
 }
 
 static int apply2_impl(const mra_op* op, const mra_tree2* f, cudaStream_t st, mra_tree2** gout,
@@ -898,9 +1119,15 @@ static int apply2_impl(const mra_op* op, const mra_tree2* f, cudaStream_t st, mr
     MRA_TRY(tmp.get(&counters, 4));
     MRA_CK(cudaMemsetAsync(counters, 0, 4 * sizeof(unsigned long long), st));
     MRA_TRY(leaf_norm2(f, part, dv, st));
-    k_pilot2<<<1, 128, 2 * (size_t)kk * sizeof(double), st>>>(k, M, op->w, op->F, f->s, dv);
+    double* ym;
+    MRA_TRY(tmp.get(&ym, (size_t)M * kk));
+    k_pilot2_terms<<<M, (kk + 31) / 32 * 32, 0, st>>>(k, op->w, op->F, f->s, ym);
     MRA_CK_LAUNCH();
-    k_schedule2<<<1, 256, 0, st>>>(M, nlev, op->eps, op->w, op->nF, op->est, dv, sched);
+    k_pilot2_sum<<<1, 640, 0, st>>>(kk, M, ym, dv);
+    MRA_CK_LAUNCH();
+    const size_t ssm = (size_t)M * (3 * nlev * sizeof(double) + sizeof(int));
+    MRA_CK(cudaFuncSetAttribute(k_schedule2, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ssm));
+    k_schedule2<<<1, 256, ssm, st>>>(M, nlev, op->eps, op->w, op->nF, op->est, dv, sched);
     MRA_CK_LAUNCH();
     mra_tree2* g = nullptr;
     MRA_TRY(tree2_clone_skeleton(f, &g));
@@ -908,7 +1135,6 @@ static int apply2_impl(const mra_op* op, const mra_tree2* f, cudaStream_t st, mr
     g->state = MRA_TREE_NSFORM;
     Offs2 off;
     memcpy(off.v, f->off, sizeof(off.v));
-    const size_t smem = 5 * (size_t)kk * sizeof(double) + (size_t)M * sizeof(int);
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     MRA_CK(cudaEventCreate(&e0));
     struct Ev {
@@ -921,9 +1147,9 @@ static int apply2_impl(const mra_op* op, const mra_tree2* f, cudaStream_t st, mr
     } ev{e0, e1};
     MRA_CK(cudaEventCreate(&e1));
     MRA_CK(cudaEventRecord(e0, st));
-    k_apply2<<<n, 128, smem, st>>>(k, M, nlev, off, f->key, f->coord, f->leaf, f->s, op->F, op->w, sched, f->filt,
-                                   g->s, counters);
-    MRA_CK_LAUNCH();
+    using Fn = int (*)(int, int, int, const Offs2&, const mra_tree2*, const mra_op*, const int32_t*, double*, unsigned long long*, cudaStream_t);
+    static const Fn fn[] = FOR_EVERY_K(apply2_launch);
+    MRA_TRY(fn[k](n, M, nlev, off, f, op, sched, g->s, counters, st));
     MRA_CK(cudaEventRecord(e1, st));
     MRA_CK(cudaMemsetAsync(g->dnorm, 0, n * sizeof(double), st));
     unsigned long long hc[4];

@@ -1,33 +1,9 @@
 // The pieces of a sibling group's schedule (see apply_oct.cu).
 #pragma once
 #include "apply_common.cuh"
+#include "band_sum.cuh"
 
 namespace mra {
-
-// ------------------------------------------------------------------ pieces
-// The classes {S : bit S of A set} of `dims` directions as products of per-direction sets
-// (1 core, 2 off, 3 both), two bits per direction from direction 1 at the top.
-struct PieceSet {
-    int n;
-    uint8_t box[4];
-};
-
-constexpr void piece_split(int dims, int A, int prefix, PieceSet& P) {
-    if (A == 0) return;
-    if (A == (1 << (dims + 1)) - 1) {  // every class: all translations of the rest
-        int b = prefix;
-        for (int d = 0; d < dims; ++d) b = (b << 2) | 3;
-        P.box[P.n++] = (uint8_t)b;
-        return;
-    }
-    const int in = A >> 1, off = A & ((1 << dims) - 1);  // classes left with this direction core / off core
-    if (in == off) {
-        piece_split(dims - 1, in, (prefix << 2) | 3, P);
-        return;
-    }
-    piece_split(dims - 1, in, (prefix << 2) | 1, P);
-    piece_split(dims - 1, off, (prefix << 2) | 2, P);
-}
 
 struct PieceTable {
     PieceSet p[16];
@@ -94,11 +70,5 @@ static __device__ int oct_pieces(const int32_t* sched, int M, int lm, int j, boo
         }
     return total;
 }
-
-// whether input b lies in the core of output a in a direction
-__device__ inline bool band_core(int a, int b) { return b >= 1 + a && b <= 3 + a; }
-
-// boxes b of a direction that some a in {0, 1} reaches by a translation of the set
-__device__ __forceinline__ unsigned set_boxes(int set) { return set == 1 ? 0x1eu : (set == 2 ? 0x33u : 0x3fu); }
 
 }  // namespace mra
