@@ -563,8 +563,6 @@ static int assemble2_t(mra_tree2* t, cudaStream_t st) {
     return MRA_OK;
 }
 
-#define FOR_EVERY_K(F) \
-    { nullptr, F<1>, F<2>, F<3>, F<4>, F<5>, F<6>, F<7>, F<8>, F<9>, F<10>, F<11>, F<12> }
 
 static int compress2_impl(mra_tree2* t, cudaStream_t st) {
     static int (*const fn[])(mra_tree2*, cudaStream_t) = FOR_EVERY_K(compress2_t);
@@ -837,51 +835,110 @@ __global__ void k_schedule2(int M, int nlev, double eps, const double* w, const 
     }
 }
 
-// Algorithm 3 in d = 2 by sibling groups, as in d = 3 (apply_oct.cu): the four siblings of a
-// group have the same 6 x 6 inputs, and a term's kept translations are a union of products
-// T1 x T2 of per-direction sets (core, off-core, both), so per such piece
-//   W[a1][b2] = sum_{t1 in T1} F^{t1} X[b1][b2],   ghat[a1][a2] += w_m sum_{t2 in T2} W[a1][b2] (F^{t2})^T,
-// 72 + 24 products of half the multiplications each (t and -t together) where an output box at a
-// time took 4 x 36 x 2.  FP64 multiply-adds are the bound: 2.7 ms -> 0.7 ms on the bench's
-// quadtree.  Block per group: the inputs are gathered (missing ones refined from their covering
-// leaf, Step 2) into shared memory; then four pieces at a time, stage I by thread (piece, a1, b2,
-// i2), stage II by thread (piece, a1, a2, c1), whose output fibers stay in registers.
-struct PieceTable2 {
-    PieceSet p[8];
-};
-constexpr PieceTable2 make_pieces2() {
-    PieceTable2 T{};
-    for (int A = 0; A < 8; ++A) piece_split(2, A, 0, T.p[A]);
-    return T;
-}
-__constant__ PieceTable2 c_pieces2 = make_pieces2();
-#define PIECE2_CC 0x5
+// Algorithm 3 in d = 2.  The four siblings of a group have the same 6 x 6 inputs (b = 0..5 a
+// direction, t = a + 2 - b), and whether a translation is core depends on |t1| and |t2| alone.
+// So the kept terms of a level sum to one k^2 x k^2 matrix per translation,
+//   D^t[c][i] = sum_m w_m F^{t1}[c1][i1] F^{t2}[c2][i2],
+// and with F^{-t}[c][i] = (-1)^{c+i} F^t[c][i] the matrices of |t1|, |t2| = 0..3 suffice: output c takes
+// from input i the sum of the (up to four) inputs at +-t1, +-t2 with signs (-1)^{c1+i1}, (-1)^{c2+i2}.
+// FP64 multiply-adds are the bound: a group takes 4 x 12.25 k^4 of them whatever the number of
+// terms (k = 8: 0.2 M; the terms one at a time, by separable sums shared by the four siblings, took
+// 33 K each, 1.1 M on the bench's quadtree: apply 1.69 ms, 2.7 ms an output box at a time).
+//
+// Planes of a level: 4 |t1| + |t2|, the core x core ones (|t| <= 1) with the terms that a leaf
+// keeps (J_m >= j); 16 + 2 |t1| + |t2| those ones with the terms an internal box keeps (J_m = j).
+#define D2_PLANES 20
+#define D2_Q 16   // entries of F^{t1} a block
+#define D2_MB 8   // terms staged at a time
 
+// One block per (level, plane |t1| <= |t2|, 16 entries (c1, i1)); thread (i2, c2), the 16 sums in
+// registers.  The plane with |t1| and |t2| exchanged is the same matrix with directions exchanged.
+// Layout [i][c]: the apply's threads read consecutive c.
+template <int K>
+__global__ void __launch_bounds__((K * K + 31) / 32 * 32) k_dense2(int M, int nlev, const double* F, const double* w,
+                                                                  const int32_t* sched, double* D) {
+    constexpr int KK = K * K;
+    constexpr int U1[13] = {0, 0, 0, 0, 1, 1, 1, 2, 2, 3, 0, 0, 1}, U2[13] = {0, 1, 2, 3, 1, 2, 3, 2, 3, 3, 0, 1, 1};
+    __shared__ double f1[D2_MB][D2_Q], f2[D2_MB][KK];
+    const int j = blockIdx.x, q0 = blockIdx.z * D2_Q, tid = threadIdx.x, lane = tid & 31;
+    int u1 = 0, u2 = 0;
+#pragma unroll
+    for (int p = 0; p < 13; ++p)
+        if ((int)blockIdx.y == p) u1 = U1[p], u2 = U2[p];
+    const bool inner = blockIdx.y >= 10;
+    const int S = (u1 <= 1) + (u2 <= 1);
+    const int lo = sched[M + 3 * j + S], hi = sched[M + 3 * nlev + 3 * j + S];
+    unsigned use = 0;  // entries that are not zero by parity (|t1| = 0: c1 + i1 even)
+    for (int q = 0; q < D2_Q; ++q)
+        if (q0 + q < KK && (u1 || !(((q0 + q) / K + (q0 + q) % K) & 1))) use |= 1u << q;
+    double acc[D2_Q];
+#pragma unroll
+    for (int q = 0; q < D2_Q; ++q) acc[q] = 0.0;
+    for (int mb = lo; mb <= hi; mb += 32) {
+        const int ml = mb + lane;
+        unsigned mask = __ballot_sync(0xffffffffu, ml <= hi && (inner ? sched[ml] == j : sched[ml] >= j));
+        while (mask) {  // the same in every warp
+            unsigned take = 0;
+            for (int n = 0; n < D2_MB && mask; ++n) {
+                take |= mask & -mask;
+                mask &= mask - 1;
+            }
+            const int nb = __popc(take);
+            __syncthreads();
+            for (int n = 0; n < nb; ++n, take &= take - 1) {
+                const int m = mb + __ffs(take) - 1;
+                const double* Fm = F + ((size_t)j * M + m) * 7 * KK;
+                if (tid < D2_Q && q0 + tid < KK) f1[n][tid] = w[m] * Fm[(3 + u1) * KK + q0 + tid];
+                if (tid < KK) f2[n][tid] = Fm[(3 + u2) * KK + (tid % K) * K + tid / K];
+            }
+            __syncthreads();
+            if (tid < KK)
+                for (int n = 0; n < nb; ++n) {
+                    const double y = f2[n][tid];
+#pragma unroll
+                    for (int q = 0; q < D2_Q; ++q)
+                        if ((use >> q) & 1u) acc[q] += f1[n][q] * y;
+                }
+        }
+    }
+    if (tid >= KK) return;
+    const int i2 = tid / K, c2 = tid % K;
+    double* D0 = D + ((size_t)j * D2_PLANES + (inner ? 16 + 2 * u1 + u2 : 4 * u1 + u2)) * KK * KK;
+    double* D1 = D + ((size_t)j * D2_PLANES + (inner ? 16 + 2 * u2 + u1 : 4 * u2 + u1)) * KK * KK;
+#pragma unroll
+    for (int q = 0; q < D2_Q; ++q) {
+        if (q0 + q >= KK) break;
+        const int c1 = (q0 + q) / K, i1 = (q0 + q) % K;
+        D0[(size_t)(i1 * K + i2) * KK + c1 * K + c2] = acc[q];
+        if (u1 != u2) D1[(size_t)(i2 * K + i1) * KK + c2 * K + c1] = acc[q];
+    }
+}
+
+// The apply.  Block per sibling group: the 36 inputs are gathered into shared memory, missing ones
+// refined from their covering leaf (Step 2, a warp per missing parent); then per |t1| the sums Y of
+// inputs at +-t1, per |t2| those of Y at +-t2, and the plane's product: thread (c, part of the i)
+// for the four outputs, a matrix entry read once per group (k = 8: 0.5 MB a group out of L2).
 // counters: [0] items, [1] pairs, [2] Step-2 refinements an output box at a time would make, [3]
 // lookups that found no ancestor (0 for a valid tree)
+#define A2_NT 256
 template <int K>
 struct Apply2Smem {
-    static constexpr int KK = K * K, K1 = K + 1, NT = (16 * K + 31) / 32 * 32, PC = 4;
-    static size_t bytes(int M) {
-        return (size_t)(36 * KK + PC * 12 * K * K1 + PC * 7 * KK + 2 * KK + 3 * KK) * sizeof(double) + 4 * (size_t)M * sizeof(uint32_t);
-    }
+    static constexpr int KK = K * K, PARTS = A2_NT / KK < KK ? A2_NT / KK : KK;
+    static constexpr size_t bytes = (size_t)(36 + 24 + 16) * KK * sizeof(double);
 };
 
 template <int K>
-__global__ void __launch_bounds__(Apply2Smem<K>::NT) k_apply2(int M, int nlev, Offs2 off, const uint64_t* key,
+__global__ void __launch_bounds__(A2_NT) k_apply2(int M, int nlev, Offs2 off, const uint64_t* key,
                                                               const int32_t* coord, const int32_t* leaf, const double* s,
-                                                              const double* F, const double* w, const int32_t* sched,
+                                                              const double* D, const int32_t* sched,
                                                               const double* filt, double* gout, unsigned long long* counters) {
-    using L = Apply2Smem<K>;
-    constexpr int KK = L::KK, K1 = L::K1, NT = L::NT, PC = L::PC;
-    extern __shared__ double sm[];
-    double* X = sm;                        // [6][6] blocks
-    double* W = X + 36 * KK;               // [PC][2][6] blocks (c1 rows padded)
-    double* Ft = W + PC * 12 * K * K1;     // [PC][7] tiles
-    double* H = Ft + PC * 7 * KK;          // H^(0), H^(1)
-    double* T = H + 2 * KK;                // refinement: 3 blocks
-    uint32_t* list = (uint32_t*)(T + 3 * KK);
-    __shared__ int s_np, s_base[9], s_anc[9], s_lev[9], s_nout;
+    constexpr int KK = K * K, NT = A2_NT, PARTS = Apply2Smem<K>::PARTS;
+    extern __shared__ __align__(16) double sm[];
+    double* X = sm;            // [6][6] blocks
+    double* Y = X + 36 * KK;   // [parity of c1 + i1][a1][6] blocks
+    double* Z = Y + 24 * KK;   // [parities][i][a]
+    double* H = Z;             // H^(0), H^(1) while inputs are refined
+    __shared__ int s_cnt[4], s_base[9], s_anc[9], s_lev[9], s_nout;
     __shared__ unsigned s_leaf, s_need[9];
     const int tid = threadIdx.x, lane = tid & 31, g = blockIdx.x;
     const int i0 = g == 0 ? 0 : 1 + 4 * (g - 1);
@@ -891,43 +948,13 @@ __global__ void __launch_bounds__(Apply2Smem<K>::NT) k_apply2(int M, int nlev, O
     for (int e = tid; e < 2 * KK; e += NT) H[e] = filt[e];
     if (tid < 32) {
         const unsigned leafm = __ballot_sync(0xffffffffu, lane < nout && leaf[i0 + (lane < nout ? lane : 0)]);
-        const bool any_int = leafm != (1u << nout) - 1u;
-        // the pieces, and the kept terms per class (S; the core at an internal box: index 3)
-        int lo[3], hi[3], cnt[4] = {0, 0, 0, 0}, np = 0, first = M, last = -1;
-        for (int S = 0; S < 3; ++S) {
-            lo[S] = m1[S];
-            hi[S] = m2[S];
-            if (hi[S] >= lo[S]) {
-                first = min(first, lo[S]);
-                last = max(last, hi[S]);
+        // the kept terms per class (S; the core at an internal box: index 3)
+        int cnt[4] = {0, 0, 0, 0};
+        for (int S = 0; S < 3; ++S)
+            for (int m = m1[S] + lane; m <= m2[S]; m += 32) {
+                cnt[S] += sched[m] >= j;
+                if (S == 2) cnt[3] += sched[m] == j;
             }
-        }
-        for (int mb = first; mb <= last; mb += 32) {
-            const int m = mb + lane;
-            int A = 0;
-            bool extra = false;
-            if (m <= last && sched[m] >= j) {
-                for (int S = 0; S < 3; ++S) A |= (m >= lo[S] && m <= hi[S]) << S;
-                for (int S = 0; S < 3; ++S) cnt[S] += (A >> S) & 1;
-                if (sched[m] == j) cnt[3] += (A >> 2) & 1;
-                if (sched[m] > j && any_int && (A & 4)) {
-                    A &= 3;
-                    extra = leafm != 0;
-                }
-            }
-            const PieceSet& P = c_pieces2.p[A];
-            const int n = P.n + extra;
-            int at = n;
-            for (int o = 1; o < 32; o <<= 1) {
-                const int v = __shfl_up_sync(0xffffffffu, at, o);
-                if (lane >= o) at += v;
-            }
-            const int sum = __shfl_sync(0xffffffffu, at, 31);
-            at += np - n;
-            for (int i = 0; i < P.n; ++i) list[at++] = (uint32_t)m | ((uint32_t)P.box[i] << 16);
-            if (extra) list[at] = (uint32_t)m | ((uint32_t)PIECE2_CC << 16) | (1u << 24);
-            np += sum;
-        }
         for (int S = 0; S < 4; ++S)
             for (int o = 16; o > 0; o >>= 1) cnt[S] += __shfl_xor_sync(0xffffffffu, cnt[S], o);
         // lane per neighbour of the parent: its children at level j, or the leaf that covers it
@@ -971,7 +998,7 @@ __global__ void __launch_bounds__(Apply2Smem<K>::NT) k_apply2(int M, int nlev, O
             lost += __shfl_xor_sync(0xffffffffu, lost, o);
         }
         if (lane == 0) {
-            s_np = np;
+            for (int S = 0; S < 4; ++S) s_cnt[S] = cnt[S];
             s_leaf = leafm;
             s_nout = nout;
             atomicAdd(&counters[0], items);
@@ -981,123 +1008,148 @@ __global__ void __launch_bounds__(Apply2Smem<K>::NT) k_apply2(int M, int nlev, O
         }
     }
     __syncthreads();
-    const int np = s_np;
     const unsigned leafm = s_leaf;
     // the inputs that are nodes; the others zero until refined
     for (int e = tid; e < 36 * KK; e += NT) {
         const int q = e / KK, b1 = q / 6, b2 = q % 6, pi = (b1 >> 1) * 3 + (b2 >> 1), o = (b1 & 1) * 2 + (b2 & 1);
         X[e] = s_base[pi] >= 0 && ((s_need[pi] >> o) & 1u) ? s[(size_t)(s_base[pi] + o) * KK + e % KK] : 0.0;
     }
-    // Step 2, a missing parent at a time: down the path to the parent, then its four children
-    for (int pi = 0; pi < 9; ++pi) {
+    __syncthreads();
+    // Step 2, a warp per missing parent: down the path to the parent, then its four children
+    for (int pi = tid >> 5; pi < 9; pi += NT / 32) {
         if (!s_need[pi] || s_base[pi] >= 0 || s_anc[pi] < 0) continue;
         const int q1 = p1 + pi / 3 - 1, q2 = p2 + pi % 3 - 1, lev0 = s_lev[pi];
-        double *x = T, *y = T + KK, *z = T + 2 * KK;
-        __syncthreads();
-        for (int e = tid; e < KK; e += NT) x[e] = s[(size_t)s_anc[pi] * KK + e];
-        __syncthreads();
+        double *x = Y + (tid >> 5) * 3 * KK, *y = x + KK, *z = y + KK;
+        __syncwarp();
+        for (int e = lane; e < KK; e += 32) x[e] = s[(size_t)s_anc[pi] * KK + e];
+        __syncwarp();
         for (int lev = lev0; lev < j - 1; ++lev) {
             const int sh = j - 2 - lev;
             const double *H1 = H + ((q1 >> sh) & 1) * KK, *H2 = H + ((q2 >> sh) & 1) * KK;
-            for (int e = tid; e < KK; e += NT) {
+            for (int e = lane; e < KK; e += 32) {
                 const int a = e / K, c = e % K;
                 double acc = 0.0;
                 for (int i = a; i < K; ++i) acc += H1[i * K + a] * x[i * K + c];
                 y[e] = acc;
             }
-            __syncthreads();
-            for (int e = tid; e < KK; e += NT) {
+            __syncwarp();
+            for (int e = lane; e < KK; e += 32) {
                 const int a = e / K, b = e % K;
                 double acc = 0.0;
                 for (int c = b; c < K; ++c) acc += y[a * K + c] * H2[c * K + b];
                 x[e] = acc;
             }
-            __syncthreads();
+            __syncwarp();
         }
-        for (int f = tid; f < K; f += NT) {
+        if (lane < K) {
             double x0[K], x1[K];
-            up2_fiber<K>(H, x + f, K, x0, x1);
+            up2_fiber<K>(H, x + lane, K, x0, x1);
+#pragma unroll
             for (int a = 0; a < K; ++a) {
-                y[a * K + f] = x0[a];
-                z[a * K + f] = x1[a];
+                y[a * K + lane] = x0[a];
+                z[a * K + lane] = x1[a];
             }
         }
-        __syncthreads();
-        for (int f = tid; f < 2 * K; f += NT) {
+        __syncwarp();
+        if (lane < 2 * K) {
             double x0[K], x1[K];
-            up2_fiber<K>(H, (f < K ? y : z) + (f % K) * K, 1, x0, x1);
-            double* d0 = X + (size_t)((2 * (pi / 3) + f / K) * 6 + 2 * (pi % 3)) * KK + (f % K) * K;
+            up2_fiber<K>(H, (lane < K ? y : z) + (lane % K) * K, 1, x0, x1);
+            double* d0 = X + (size_t)((2 * (pi / 3) + lane / K) * 6 + 2 * (pi % 3)) * KK + (lane % K) * K;
+#pragma unroll
             for (int a = 0; a < K; ++a) {
                 d0[a] = x0[a];
                 d0[KK + a] = x1[a];
             }
         }
     }
-    // stage II's thread: piece slot, a1, a2, c1
-    const int slot = tid / (4 * K), oa = (tid / K) & 3, oc = tid % K;
-    const int mya = (tid % (4 * K)) / K;
-    (void)oa;
-    double y[K];
-#pragma unroll
-    for (int c = 0; c < K; ++c) y[c] = 0.0;
-    for (int qb = 0; qb < np; qb += PC) {
-        const int npc = min(PC, np - qb);
+    const int c = tid % KK, part = tid / KK, pc1 = (c / K) & 1, pc2 = (c % K) & 1;
+    const double* Dj = D + (size_t)j * D2_PLANES * KK * KK;
+    const bool inner = s_cnt[3] > 0 && leafm != 0xfu;  // some internal output keeps core terms
+    double y[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll 1
+    for (int u1 = 0; u1 < 4; ++u1) {
         __syncthreads();
-        for (int e = tid; e < npc * 7 * KK; e += NT)
-            Ft[e] = F[((size_t)j * M + (list[qb + e / (7 * KK)] & 0xffff)) * 7 * KK + e % (7 * KK)];
-        __syncthreads();
-        for (int task = tid; task < npc * 12 * K; task += NT) {
-            const int i2 = task % K, b2 = (task / K) % 6, pa = task / (6 * K), a1 = pa & 1, pc = pa >> 1;
-            const int box = (list[qb + pc] >> 16) & 0xff;
-            if (!((set_boxes(box & 3) >> b2) & 1u)) continue;
-            double x[6][K], out[K];
-#pragma unroll
-            for (int b1 = 0; b1 < 6; ++b1)
-#pragma unroll
-                for (int i = 0; i < K; ++i) x[b1][i] = X[(b1 * 6 + b2) * KK + i * K + i2];
-            band_sum<double, K>(Ft + pc * 7 * KK, box >> 2, a1, x, out);
-            double* dst = W + (pa * 6 + b2) * K * K1 + i2;
-#pragma unroll
-            for (int c = 0; c < K; ++c) dst[c * K1] = out[c];
+        for (int e = tid; e < 12 * KK; e += NT) {  // (a1, b2, i)
+            const int a1 = e / (6 * KK), r = e % (6 * KK);
+            const double xp = a1 + 2 - u1 >= 0 ? X[(a1 + 2 - u1) * 6 * KK + r] : 0.0;
+            const double xm = u1 && a1 + 2 + u1 < 6 ? X[(a1 + 2 + u1) * 6 * KK + r] : 0.0;
+            Y[e] = xp + xm;
+            Y[12 * KK + e] = xp - xm;
         }
-        __syncthreads();
-        if (slot < npc) {
-            const uint32_t p = list[qb + slot];
-            const int set = (p >> 16) & 3;
-            const unsigned boxes = set_boxes(set);
-            if (mya < s_nout && (!(p >> 24) || ((leafm >> mya) & 1u))) {
-                double x[6][K], out[K];
-#pragma unroll
-                for (int b2 = 0; b2 < 6; ++b2) {
-                    const double* src = W + ((slot * 2 + (mya >> 1)) * 6 + b2) * K * K1 + oc * K1;
-#pragma unroll
-                    for (int i = 0; i < K; ++i) x[b2][i] = ((boxes >> b2) & 1u) ? src[i] : 0.0;
+#pragma unroll 1
+        for (int u2 = 0; u2 < 4; ++u2) {
+            const int S = (u1 <= 1) + (u2 <= 1);
+            if (!s_cnt[S]) continue;
+            __syncthreads();
+            for (int e = tid; e < 8 * KK; e += NT) {  // (p1, i, a)
+                const int a = e & 3, i = (e >> 2) % KK, p = e / (4 * KK), a2 = a & 1;
+                const double* Yr = Y + (p * 2 + (a >> 1)) * 6 * KK + i;
+                // (an internal output without core terms reads zeros)
+                const bool on = S < 2 || ((leafm >> a) & 1u) || inner;
+                const double yp = on && a2 + 2 - u2 >= 0 ? Yr[(a2 + 2 - u2) * KK] : 0.0;
+                const double ym = on && u2 && a2 + 2 + u2 < 6 ? Yr[(a2 + 2 + u2) * KK] : 0.0;
+                Z[((2 * p) * KK + i) * 4 + a] = yp + ym;
+                Z[((2 * p + 1) * KK + i) * 4 + a] = yp - ym;
+            }
+            __syncthreads();
+            if (part < PARTS) {
+                const double* Dp = Dj + (size_t)(4 * u1 + u2) * KK * KK + c;
+                // F^0 has no entries with c + i odd
+                const int s1 = u1 ? 1 : 2, s2 = u2 ? 1 : 2, o1 = u1 ? 0 : pc1, o2 = u2 ? 0 : pc2;
+                const int n2 = (K - o2 + s2 - 1) / s2, nq = ((K - o1 + s1 - 1) / s1) * n2;
+                if (S < 2 || !inner) {
+#pragma unroll 4
+                    for (int q = part; q < nq; q += PARTS) {
+                        const int i1 = (q / n2) * s1 + o1, i2 = (q % n2) * s2 + o2, i = i1 * K + i2;
+                        const double d = Dp[(size_t)i * KK];
+                        const double2* z = (const double2*)(Z + ((2 * ((i1 + pc1) & 1) + ((i2 + pc2) & 1)) * KK + i) * 4);
+                        const double2 z0 = z[0], z1 = z[1];
+                        y[0] += d * z0.x;
+                        y[1] += d * z0.y;
+                        y[2] += d * z1.x;
+                        y[3] += d * z1.y;
+                    }
+                } else {
+                    const double* Di = Dj + (size_t)(16 + 2 * u1 + u2) * KK * KK + c;
+#pragma unroll 4
+                    for (int q = part; q < nq; q += PARTS) {
+                        const int i1 = (q / n2) * s1 + o1, i2 = (q % n2) * s2 + o2, i = i1 * K + i2;
+                        const double dl = Dp[(size_t)i * KK], di = Di[(size_t)i * KK];
+                        const double2* z = (const double2*)(Z + ((2 * ((i1 + pc1) & 1) + ((i2 + pc2) & 1)) * KK + i) * 4);
+                        const double2 z0 = z[0], z1 = z[1];
+                        y[0] += ((leafm & 1u) ? dl : di) * z0.x;
+                        y[1] += ((leafm & 2u) ? dl : di) * z0.y;
+                        y[2] += ((leafm & 4u) ? dl : di) * z1.x;
+                        y[3] += ((leafm & 8u) ? dl : di) * z1.y;
+                    }
                 }
-                band_sum<double, K>(Ft + slot * 7 * KK, set, mya & 1, x, out);
-                const double wm = w[p & 0xffff];
-#pragma unroll
-                for (int c = 0; c < K; ++c) y[c] += wm * out[c];
             }
         }
     }
-    // the four slots' sums in order
+    // the parts' sums in order
     __syncthreads();
-    double* ys = W;  // [slot][a][c1][c2]
-    if (slot < PC)
+    double* ys = X;  // [part][a][c]
+    if (part < PARTS)
 #pragma unroll
-        for (int c = 0; c < K; ++c) ys[(slot * 4 + mya) * KK + oc * K + c] = y[c];
+        for (int a = 0; a < 4; ++a) ys[(part * 4 + a) * KK + c] = y[a];
     __syncthreads();
-    for (int e = tid; e < s_nout * KK; e += NT)
-        gout[(size_t)i0 * KK + e] = ((ys[e] + ys[4 * KK + e]) + ys[8 * KK + e]) + ys[12 * KK + e];
+    for (int e = tid; e < s_nout * KK; e += NT) {
+        double v = ys[e];
+        for (int p = 1; p < PARTS; ++p) v += ys[p * 4 * KK + e];
+        gout[(size_t)i0 * KK + e] = v;
+    }
 }
 
 template <int K>
 static int apply2_launch(int n, int M, int nlev, const Offs2& off, const mra_tree2* f, const mra_op* op, const int32_t* sched,
-                         double* gout, unsigned long long* counters, cudaStream_t st) {
-    using L = Apply2Smem<K>;
-    MRA_CK(cudaFuncSetAttribute(k_apply2<K>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L::bytes(M)));
-    k_apply2<K><<<1 + (n - 1) / 4, L::NT, L::bytes(M), st>>>(M, nlev, off, f->key, f->coord, f->leaf, f->s, op->F, op->w, sched,
-                                                              f->filt, gout, counters);
+                         double* D, double* gout, unsigned long long* counters, cudaStream_t st) {
+    constexpr int KK = K * K;
+    constexpr size_t bytes = Apply2Smem<K>::bytes;
+    k_dense2<K><<<dim3(nlev, 13, (KK + D2_Q - 1) / D2_Q), (KK + 31) / 32 * 32, 0, st>>>(M, nlev, op->F, op->w, sched, D);
+    MRA_CK_LAUNCH();
+    MRA_CK(cudaFuncSetAttribute(k_apply2<K>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
+    k_apply2<K><<<1 + (n - 1) / 4, A2_NT, bytes, st>>>(M, nlev, off, f->key, f->coord, f->leaf, f->s, D, sched, f->filt, gout,
+                                                     counters);
     MRA_CK_LAUNCH();
     return MRA_OK;
 }
@@ -1121,6 +1173,8 @@ static int apply2_impl(const mra_op* op, const mra_tree2* f, cudaStream_t st, mr
     MRA_TRY(leaf_norm2(f, part, dv, st));
     double* ym;
     MRA_TRY(tmp.get(&ym, (size_t)M * kk));
+    double* D;
+    MRA_TRY(tmp.get(&D, (size_t)nlev * D2_PLANES * kk * kk));
     k_pilot2_terms<<<M, (kk + 31) / 32 * 32, 0, st>>>(k, op->w, op->F, f->s, ym);
     MRA_CK_LAUNCH();
     k_pilot2_sum<<<1, 640, 0, st>>>(kk, M, ym, dv);
@@ -1147,9 +1201,9 @@ static int apply2_impl(const mra_op* op, const mra_tree2* f, cudaStream_t st, mr
     } ev{e0, e1};
     MRA_CK(cudaEventCreate(&e1));
     MRA_CK(cudaEventRecord(e0, st));
-    using Fn = int (*)(int, int, int, const Offs2&, const mra_tree2*, const mra_op*, const int32_t*, double*, unsigned long long*, cudaStream_t);
+    using Fn = int (*)(int, int, int, const Offs2&, const mra_tree2*, const mra_op*, const int32_t*, double*, double*, unsigned long long*, cudaStream_t);
     static const Fn fn[] = FOR_EVERY_K(apply2_launch);
-    MRA_TRY(fn[k](n, M, nlev, off, f, op, sched, g->s, counters, st));
+    MRA_TRY(fn[k](n, M, nlev, off, f, op, sched, D, g->s, counters, st));
     MRA_CK(cudaEventRecord(e1, st));
     MRA_CK(cudaMemsetAsync(g->dnorm, 0, n * sizeof(double), st));
     unsigned long long hc[4];

@@ -31,6 +31,10 @@ void set_error(const char* fmt, ...);
         }                                                                         \
     } while (0)
 
+// the instances of a template for the orders 0 (none) .. MRA_MAX_K
+#define FOR_EVERY_K(F) \
+    { nullptr, F<1>, F<2>, F<3>, F<4>, F<5>, F<6>, F<7>, F<8>, F<9>, F<10>, F<11>, F<12> }
+
 // streaming multiprocessors of the current device (queried once per device;
 // grids of persistent and grid-stride kernels are sized in multiples of it)
 int num_sms();
