@@ -772,13 +772,18 @@ __global__ void k_compress_fast_level_t(int cbase, const int32_t* parent, double
     }
 }
 
+// threads of a slice's block on a small level: its time is the chain of loads and FP64 latencies,
+// one output element per thread and stage (k = 8, a level of 8 parents: 13.6 us with 128 threads,
+// 8.9 with 512)
+#define SLICE_NT 512
+
 // ---- the scaling blocks of a small level: one parent over k/2 blocks
 // Block (b, q) computes rows i1 in {q, K-1-q} of the parent's block (the contractions
 // along directions 2 and 3 never mix rows of direction 1), one output element per
 // thread and step.  It pays where a level has fewer parents than SMs: each parent then
 // runs on k/2 SMs; on the large levels the per-parent kernel below is faster.
 template <int K>
-__global__ void __launch_bounds__(128) k_down_slice(int cbase, const int32_t* parent, double* s,
+__global__ void __launch_bounds__(SLICE_NT) k_down_slice(int cbase, const int32_t* parent, double* s,
                                                     const double* filt) {
     constexpr int K2 = 2 * K, K3 = K * K * K, P2 = K2 + 1, R = 2;
     __shared__ double H[K * K];
@@ -786,8 +791,11 @@ __global__ void __launch_bounds__(128) k_down_slice(int cbase, const int32_t* pa
     __shared__ double o1[R * K2 * P2];     // (r, x2, x3)
     __shared__ double o2[R * K * P2];      // (r, i2, x3)
     const int c0 = cbase + 8 * blockIdx.x, i = parent[c0], q = blockIdx.y, tid = threadIdx.x;
-    for (int e = tid; e < K * K; e += blockDim.x) H[e] = filt[e];
-    for (int e = tid; e < 8 * K3; e += blockDim.x) {
+    for (int e = tid; e < K * K; e += SLICE_NT) H[e] = filt[e];
+#pragma unroll
+    for (int it = 0; it < (8 * K3 + SLICE_NT - 1) / SLICE_NT; ++it) {
+        const int e = tid + it * SLICE_NT;
+        if (e >= 8 * K3) break;
         const int o = e / K3, r = e % K3;
         const int i1 = r / (K * K), i2 = (r / K) % K, i3 = r % K;
         const int x1 = ((o >> 2) & 1) * K + i1, x2 = ((o >> 1) & 1) * K + i2, x3 = (o & 1) * K + i3;
@@ -833,7 +841,7 @@ __global__ void __launch_bounds__(128) k_down_slice(int cbase, const int32_t* pa
 // Assembly (eq. g_assemble, d = 0): children += (U x U x U) s_parent, U = D^T (row
 // p K + r has the columns c >= r), rows x1 in {q, K-1-q, K+q, 2K-1-q} of the cube.
 template <int K>
-__global__ void __launch_bounds__(128) k_up_slice(int cbase, const int32_t* parent, double* s, const double* filt) {
+__global__ void __launch_bounds__(SLICE_NT) k_up_slice(int cbase, const int32_t* parent, double* s, const double* filt) {
     constexpr int K2 = 2 * K, K3 = K * K * K, P1 = K + 1, RX = 4;
     __shared__ double Ht[K * K];         // Ht[a][i] = H^(0)[i][a]
     __shared__ double sp[K * K * P1];    // (i1, i2, i3), i3 padded
@@ -957,7 +965,7 @@ static int compress_fast_t(mra_tree* t, bool norms, cudaStream_t st) {
         bool sliced = false;
         if constexpr (K <= 8)
             if (2 * nparents < num_sms()) {
-                k_down_slice<K><<<dim3(nparents, (K + 1) / 2), 128, 0, st>>>(t->off[j + 1], t->a.parent, t->s, t->filt);
+                k_down_slice<K><<<dim3(nparents, (K + 1) / 2), SLICE_NT, 0, st>>>(t->off[j + 1], t->a.parent, t->s, t->filt);
                 sliced = true;
             }
         if (!sliced)
@@ -977,7 +985,7 @@ static int assemble_t(mra_tree* t, cudaStream_t st) {
     for (int j = 0; j + 1 < t->nlev; ++j) {
         const int nparents = (t->off[j + 2] - t->off[j + 1]) / 8;
         if (nparents <= 0) continue;
-        k_up_slice<K><<<dim3(nparents, (K + 1) / 2), 128, 0, st>>>(t->off[j + 1], t->a.parent, t->s, t->filt);
+        k_up_slice<K><<<dim3(nparents, (K + 1) / 2), 2 * nparents < num_sms() ? SLICE_NT : 128, 0, st>>>(t->off[j + 1], t->a.parent, t->s, t->filt);
         MRA_CK_LAUNCH();
     }
     return MRA_OK;
