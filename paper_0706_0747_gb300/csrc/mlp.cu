@@ -78,9 +78,17 @@ __device__ void mlp_layer(const float* xs, int din, const __half* Wio, int dout,
     for (int i0 = 0; i0 < din; i0 += MLP_WI) {
         const int ni = min(MLP_WI, din - i0);
         __syncthreads();
-        for (int e = threadIdx.x; e < ni * 128; e += MLP_NT) {
-            const int i = e >> 7, o = o0 + (e & 127);
-            ws[e] = o < dout ? Wio[(size_t)(i0 + i) * dout + o] : __half(0.0f);
+        if (dout % 8 == 0 && o0 + 128 <= dout) {  // whole rows of 16-byte words
+#pragma unroll
+            for (int q = 0; q < MLP_WI * 16 / MLP_NT; ++q) {
+                const int e = threadIdx.x + q * MLP_NT, i = e >> 4;
+                if (i < ni) ((uint4*)ws)[e] = *(const uint4*)(Wio + (size_t)(i0 + i) * dout + o0 + (e & 15) * 8);
+            }
+        } else {
+            for (int e = threadIdx.x; e < ni * 128; e += MLP_NT) {
+                const int i = e >> 7, o = o0 + (e & 127);
+                ws[e] = o < dout ? Wio[(size_t)(i0 + i) * dout + o] : __half(0.0f);
+            }
         }
         __syncthreads();
         if (o0 + 4 * lane < dout)
@@ -115,7 +123,7 @@ struct MlpArgs {
 template <bool TRAIN>
 __global__ void __launch_bounds__(MLP_NT) k_mlp_rows(MlpArgs A) {
     extern __shared__ __align__(16) float mlp_sm[];
-    __shared__ __align__(8) __half ws[MLP_WI * 128];
+    __shared__ __align__(16) __half ws[MLP_WI * 128];
     __shared__ double red[MLP_NT / 32];
     float* xa = mlp_sm;                                     // [max(n_in, 128)][MLP_XS]
     float* xb = xa + (size_t)max(A.n_in, MLP_H) * MLP_XS;   // [128][MLP_XS]
@@ -129,6 +137,7 @@ __global__ void __launch_bounds__(MLP_NT) k_mlp_rows(MlpArgs A) {
     MlpTile t;
     unsigned on[3] = {0, 0, 0};  // hidden units of this thread's tile above zero
     float *in = xa, *out = xb;
+#pragma unroll
     for (int l = 0; l < 3; ++l) {
         mlp_layer(in, l ? MLP_H : A.n_in, A.wt[l], MLP_H, 0, A.b[l], ws, t);
         __syncthreads();
@@ -138,13 +147,15 @@ __global__ void __launch_bounds__(MLP_NT) k_mlp_rows(MlpArgs A) {
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
                 hv[q] = __float2half_rn(fmaxf(t.v[r][q], 0.0f));
-                const float f = __half2float(hv[q]);
-                out[(4 * lane + q) * MLP_XS + 4 * warp + r] = f;
-                on[l] |= (unsigned)(f > 0.0f) << (4 * r + q);
+                t.v[r][q] = __half2float(hv[q]);
+                on[l] |= (unsigned)(t.v[r][q] > 0.0f) << (4 * r + q);
             }
             if (TRAIN && 4 * warp + r < rows)
                 *(uint2*)(A.h[l] + (r0 + 4 * warp + r) * MLP_H + 4 * lane) = *(const uint2*)hv;
         }
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+            *(float4*)(out + (4 * lane + q) * MLP_XS + 4 * warp) = make_float4(t.v[0][q], t.v[1][q], t.v[2][q], t.v[3][q]);
         float* s = in;
         in = out;
         out = s;
@@ -194,20 +205,20 @@ __global__ void __launch_bounds__(MLP_NT) k_mlp_rows(MlpArgs A) {
     // back through the layers: d_l = (d_{l+1} W) where the unit was on
     float* g = out;
     float* nx = in;
+#pragma unroll
     for (int l = 2; l >= 0; --l) {
         mlp_layer(g, l == 2 ? A.n_out : MLP_H, A.wr[l + 1], MLP_H, 0, nullptr, ws, t);
         __syncthreads();
 #pragma unroll
         for (int r = 0; r < 4; ++r) {
-            float v[4];
 #pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                v[q] = ((on[l] >> (4 * r + q)) & 1u) ? t.v[r][q] : 0.0f;
-                nx[(4 * lane + q) * MLP_XS + 4 * warp + r] = v[q];
-            }
+            for (int q = 0; q < 4; ++q) t.v[r][q] = ((on[l] >> (4 * r + q)) & 1u) ? t.v[r][q] : 0.0f;
             if (4 * warp + r < rows)
-                *(float4*)(A.d[l] + (r0 + 4 * warp + r) * MLP_H + 4 * lane) = make_float4(v[0], v[1], v[2], v[3]);
+                *(float4*)(A.d[l] + (r0 + 4 * warp + r) * MLP_H + 4 * lane) = make_float4(t.v[r][0], t.v[r][1], t.v[r][2], t.v[r][3]);
         }
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+            *(float4*)(nx + (4 * lane + q) * MLP_XS + 4 * warp) = make_float4(t.v[0][q], t.v[1][q], t.v[2][q], t.v[3][q]);
         float* s = g;
         g = nx;
         nx = s;
@@ -228,6 +239,7 @@ struct WgradArgs {
     int tile0[5];       // first tile of each layer
     int64_t off_w[4], off_b[4];
     float* part;        // [slices][np]
+    bool x16;           // x starts on a 16-byte boundary
 };
 
 __global__ void __launch_bounds__(256) k_mlp_wgrad(WgradArgs A) {
@@ -245,13 +257,39 @@ __global__ void __launch_bounds__(256) k_mlp_wgrad(WgradArgs A) {
     const bool busy = o0 + 4 * to < dout && i0 + 4 * ti < din;
     for (int64_t r = r0; r < r1; r += 32) {
         __syncthreads();
-        for (int e = tid; e < 32 * 128; e += 256) {
-            const int rr = e >> 7, c = e & 127;
+        // four columns at a time (every row starts on a 16-byte boundary when the width is a multiple of 4)
+        const bool vd = dout % 4 == 0, vh = din % 4 == 0;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int e = tid + q * 256, rr = e >> 5, c = (e & 31) * 4;
             const int64_t row = r + rr;
-            ds[rr][c] = row < r1 && o0 + c < dout ? A.d[l][row * dout + o0 + c] : 0.0f;
-            hs[rr][c] = row < r1 && i0 + c < din
-                            ? (l ? __half2float(((const __half*)A.h[l])[row * din + i0 + c]) : ((const float*)A.h[l])[row * din + i0 + c])
-                            : 0.0f;
+            float4 dv = make_float4(0.0f, 0.0f, 0.0f, 0.0f), hv = dv;
+            if (row < r1) {
+                const float* dp = A.d[l] + row * dout + o0 + c;
+                if (vd && o0 + c < dout) dv = *(const float4*)dp;
+                else if (!vd) {
+                    float* v = (float*)&dv;
+                    for (int z = 0; z < 4; ++z)
+                        if (o0 + c + z < dout) v[z] = dp[z];
+                }
+                if (vh && i0 + c < din) {
+                    if (l) {
+                        const uint2 h2 = *(const uint2*)((const __half*)A.h[l] + row * din + i0 + c);
+                        const float2 a = __half22float2(*(const __half2*)&h2.x), b = __half22float2(*(const __half2*)&h2.y);
+                        hv = make_float4(a.x, a.y, b.x, b.y);
+                    } else if (A.x16) {
+                        hv = *(const float4*)((const float*)A.h[0] + row * din + i0 + c);
+                    }
+                }
+                if (!vh || (l == 0 && !A.x16)) {
+                    float* v = (float*)&hv;
+                    for (int z = 0; z < 4; ++z)
+                        if (i0 + c + z < din)
+                            v[z] = l ? __half2float(((const __half*)A.h[l])[row * din + i0 + c + z]) : ((const float*)A.h[0])[row * din + i0 + c + z];
+                }
+            }
+            *(float4*)&ds[rr][c] = dv;
+            *(float4*)&hs[rr][c] = hv;
         }
         __syncthreads();
         if (busy)
@@ -417,6 +455,7 @@ static int mlp_loss_grad_impl(mra_mlp* M, const float* x, const float* t, int64_
         W.ti[l] = (M->din[l] + 127) / 128;
         W.tile0[l + 1] = W.tile0[l] + W.ti[l] * ((M->dout[l] + 127) / 128);
     }
+    W.x16 = ((uintptr_t)x & 15) == 0;
     Scratch tmp(M->A);
     MRA_TRY(tmp.get(&W.part, (size_t)slices * M->np));
     k_mlp_wgrad<<<dim3(slices, W.tile0[4]), 256, 0, st>>>(W);
