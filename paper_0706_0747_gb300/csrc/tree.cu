@@ -53,22 +53,6 @@ int scan_exclusive(const int32_t* in, int32_t* out, int n, int32_t* total, cudaS
     return MRA_OK;
 }
 
-// out[along dim] = Mat * in[along dim] for a k^3 array in shared memory;
-// Mat is k x k row-major (out index, in index).  All threads of the block.
-__device__ void mode_product(const double* in, double* out, const double* Mat, int dim, int k) {
-    const int n = k * k * k;
-    for (int idx = threadIdx.x; idx < n; idx += blockDim.x) {
-        int i3 = idx % k, i2 = (idx / k) % k, i1 = idx / (k * k);
-        int r = dim == 0 ? i1 : (dim == 1 ? i2 : i3);
-        int stride = dim == 0 ? k * k : (dim == 1 ? k : 1);
-        const double* src = in + idx - r * stride;
-        double acc = 0.0;
-        for (int c = 0; c < k; ++c) acc += Mat[r * k + c] * src[c * stride];
-        out[idx] = acc;
-    }
-    __syncthreads();
-}
-
 __device__ double block_sum(double v, double* red) {
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     const int w = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
@@ -243,168 +227,301 @@ struct DensDev {
     const double *coef, *r2, *expo, *cen;
 };
 
-__device__ double dens_eval(const DensDev& D, double x, double y, double z) {
-    double f = 0.0;
-    for (int g = 0; g < D.n; ++g) {
-        double dx = x - D.cen[3 * g], dy = y - D.cen[3 * g + 1], dz = z - D.cen[3 * g + 2];
-        double r2 = dx * dx + dy * dy + dz * dz;
-        f += (D.coef[g] + D.r2[g] * r2) * exp(-D.expo[g] * r2);
-    }
-    return f;
-}
+// Tables of the build, for one order: nodes and weights of [0, 1], the projection's rows of the first
+// half of the nodes and the interpolation to the children's nodes of the lower half box.  The rest
+// follows by parity: phi_i(g_{k-1-q}) = (-1)^i phi_i(g_q), phi_i((g_{k-1-q} + 1)/2) = (-1)^i phi_i(g_q/2).
+struct BuildTables {
+    double g[MRA_MAX_K], w[MRA_MAX_K];
+    double P[MRA_MAX_K / 2 * MRA_MAX_K];  // [q < (k+1)/2][i] phi_i(g_q) w_q
+    double Q[MRA_MAX_K * MRA_MAX_K];      // [q][i] phi_i(g_q / 2)
+};
 
-__global__ void k_dens_scale(DensDev D, double eps, double* tol) {
-    __shared__ double red[32];
+// max |f| over the centres as the bits of a non-negative double; the last block fills the tables
+__global__ void k_dens_scale(DensDev D, unsigned long long* maxbits, int k, BuildTables* T) {
+    if (blockIdx.x == gridDim.x - 1) {
+        __shared__ double g[MRA_MAX_K], w[MRA_MAX_K];
+        const int q = threadIdx.x;
+        if (q < k) gauss_legendre01_root(k, q, g, w);
+        __syncthreads();
+        if (q >= k) return;
+        double ph[MRA_MAX_K];
+        T->g[q] = g[q];
+        T->w[q] = w[q];
+        phi_all(k, g[q], ph);
+        if (q < (k + 1) / 2)
+            for (int i = 0; i < k; ++i) T->P[q * k + i] = ph[i] * w[q];
+        phi_all(k, 0.5 * g[q], ph);
+        for (int i = 0; i < k; ++i) T->Q[q * k + i] = ph[i];
+        return;
+    }
+    const int lane = threadIdx.x & 31, nw = (gridDim.x - 1) * (blockDim.x / 32);
     double m = 0.0;
-    for (int g = threadIdx.x; g < D.n; g += blockDim.x)
-        m = fmax(m, fabs(dens_eval(D, D.cen[3 * g], D.cen[3 * g + 1], D.cen[3 * g + 2])));
-    m = block_max(m, red);
-    if (threadIdx.x == 0) {
-        tol[0] = eps * m;
-        tol[1] = 1e-18 * m;  // terms below this on a box are skipped (rounding level)
+    for (int c = blockIdx.x * (blockDim.x / 32) + (threadIdx.x >> 5); c < D.n; c += nw) {
+        double f = 0.0;
+        for (int g = lane; g < D.n; g += 32) {
+            double r2 = 0.0;
+            for (int d = 0; d < 3; ++d) {
+                const double dx = D.cen[3 * c + d] - D.cen[3 * g + d];
+                r2 += dx * dx;
+            }
+            f += (D.coef[g] + D.r2[g] * r2) * exp(-D.expo[g] * r2);
+        }
+        for (int o = 16; o > 0; o >>= 1) f += __shfl_xor_sync(0xffffffffu, f, o);
+        m = fmax(m, fabs(f));
     }
+    if (lane == 0) atomicMax(maxbits, (unsigned long long)__double_as_longlong(m));
 }
 
-// Values of the density on the tensor grid X[0][q1] x X[1][q2] x X[2][q3]
-// (k increasing points per direction) added into v[(q1 k + q2) k + q3],
-// block-cooperatively.  Each term factors by direction,
-// exp(-a|x - c|^2) = prod_d exp(-a (x_d - c_d)^2) and |x - c|^2 = sum_d (x_d - c_d)^2,
-// so per term the block forms 3k one-dimensional factors (in shared memory,
-// DG_CHUNK terms at a time) and each grid point costs a few products instead
-// of an exponential.  A term whose bound on the grid's box,
-// (|c| + |b| dmax^2) exp(-a dmin^2), is below `cut` is skipped.
+// One block per box.  FP64 operations bound it: per term and box 9 k one-dimensional factors
+// exp(-a (x_d - c_d)^2) and one or two multiply-adds per grid point, and the mode products.  A thread
+// takes a fiber of the grid along direction 1: the factors of the other two directions are one
+// product per term, the fiber's values stay in registers, and the children's 8 grids are one
+// (2k)^3 grid whose one-dimensional factors are shared.  Projection and interpolation halve by
+// parity (see BuildTables).  (A block-wide pass per grid and term chunk, six operations a point, full
+// matrices: 4.5 ms on the 32-Gaussian k = 8 build.)
 #define DG_CHUNK 32
-__device__ void dens_grid(const DensDev& D, int k, const double* X, double* v, double* E, double* R,
-                          double* cb, int* act, double cut) {
-    const int k3 = k * k * k, kk = k * k, k3d = 3 * k;
-    __shared__ int nact;
-    for (int g0 = 0; g0 < D.n; g0 += DG_CHUNK) {
-        const int ng = min(DG_CHUNK, D.n - g0);
-        if (threadIdx.x < 32) {  // warp 0: which terms of the chunk reach the box
-            const int g = g0 + threadIdx.x;
-            bool on = false;
-            if ((int)threadIdx.x < ng) {
-                double dmin2 = 0.0, dmax2 = 0.0;
-                for (int d = 0; d < 3; ++d) {
-                    const double lo = X[d * k] - D.cen[3 * g + d], hi = X[d * k + k - 1] - D.cen[3 * g + d];
-                    const double dn = lo > 0.0 ? lo : (hi < 0.0 ? -hi : 0.0);
-                    const double dx = fmax(fabs(lo), fabs(hi));
-                    dmin2 += dn * dn;
-                    dmax2 += dx * dx;
-                }
-                on = (fabs(D.coef[g]) + fabs(D.r2[g]) * dmax2) * exp(-D.expo[g] * dmin2) >= cut;
+template <int K>
+struct BuildSmem {
+    static constexpr int K2 = 2 * K, KK = K * K, K3 = KK * K, P2 = K2 + 1;
+    static constexpr int NT = (4 * KK + 31) / 32 * 32;  // a thread per fiber of the children's grid
+    static constexpr int GR = 4;                        // term groups of the box's own grid
+    static constexpr int T2 = GR * K3, T3 = KK * P2;    // (the children's: 4 k^3)
+    static constexpr size_t bytes = (K3 + T2 + T3 + 3 * K2 + 6 * K2 * DG_CHUNK) * sizeof(double);
+};
+
+// The terms of a chunk that reach the grid X[3][H k] or, for H = 2, one of its 8 octants (bits of
+// mask), by the bound (|c| + |b| dmax^2) exp(-a dmin^2) >= cut; their one-dimensional factors in E
+// ([term][d][q]) and squared distances in R (direction 1: times the factor).
+template <int K, int H>
+__device__ int dens_factors(const DensDev& D, int g0, const double* X, double cut, double* E, double* R, int* act,
+                            unsigned* mask, double2* cb) {
+    constexpr int N = H * K, OCT = H == 2 ? 8 : 1;
+    __shared__ int s_na;
+    const int tid = threadIdx.x, lane = tid & 31;
+    __syncthreads();
+    for (int e = tid; e < DG_CHUNK * OCT; e += BuildSmem<K>::NT) {  // (a multiple of 32: whole warps)
+        const int g = g0 + e / OCT, o = e % OCT;
+        bool on = false;
+        if (g < D.n) {
+            double dmin2 = 0.0, dmax2 = 0.0;
+#pragma unroll
+            for (int d = 0; d < 3; ++d) {
+                const double* Xd = X + d * N + ((o >> (2 - d)) & 1) * K;
+                const double lo = Xd[0] - D.cen[3 * g + d], hi = Xd[K - 1] - D.cen[3 * g + d];
+                const double dn = lo > 0.0 ? lo : (hi < 0.0 ? -hi : 0.0);
+                const double dx = fmax(fabs(lo), fabs(hi));
+                dmin2 += dn * dn;
+                dmax2 += dx * dx;
             }
-            const unsigned mask = __ballot_sync(0xffffffffu, on);
-            if (on) {
-                const int slot = __popc(mask & ((1u << threadIdx.x) - 1u));
-                act[slot] = g;
-                cb[2 * slot] = D.coef[g];
-                cb[2 * slot + 1] = D.r2[g];
-            }
-            if (threadIdx.x == 0) nact = __popc(mask);
+            on = (fabs(D.coef[g]) + fabs(D.r2[g]) * dmax2) * exp(-D.expo[g] * dmin2) >= cut;
         }
-        __syncthreads();
-        const int na = nact;
-        for (int e = threadIdx.x; e < na * k3d; e += blockDim.x) {
-            const int a = e / k3d, d = (e / k) % 3, q = e % k, g = act[a];
-            const double dx = X[d * k + q] - D.cen[3 * g + d];
-            R[e] = dx * dx;
-            E[e] = exp(-D.expo[g] * dx * dx);
-        }
-        __syncthreads();
-        for (int idx = threadIdx.x; idx < k3; idx += blockDim.x) {
-            const int q1 = idx / kk, q2 = (idx / k) % k, q3 = idx % k;
-            double acc = v[idx];
-            for (int g = 0; g < na; ++g) {
-                const double* Eg = E + g * k3d;
-                const double* Rg = R + g * k3d;
-                const double prod = Eg[q1] * Eg[k + q2] * Eg[2 * k + q3];
-                acc += (cb[2 * g] + cb[2 * g + 1] * (Rg[q1] + Rg[k + q2] + Rg[2 * k + q3])) * prod;
-            }
-            v[idx] = acc;
-        }
-        __syncthreads();
+        const unsigned b = __ballot_sync(0xffffffffu, on);
+        if (o == 0) mask[e / OCT] = OCT == 1 ? (b >> lane) & 1u : (b >> lane) & 0xffu;
     }
+    __syncthreads();
+    if (tid < 32) {
+        const unsigned mk = mask[lane], any = __ballot_sync(0xffffffffu, mk != 0);
+        if (mk) {
+            const int slot = __popc(any & ((1u << lane) - 1u));
+            act[slot] = g0 + lane;
+            mask[slot] = mk;  // (slot <= lane: read above by this lane's ballot)
+            cb[slot] = make_double2(D.coef[g0 + lane], D.r2[g0 + lane]);
+        }
+        if (lane == 0) s_na = __popc(any);
+    }
+    __syncthreads();
+    const int na = s_na;
+    for (int e = tid; e < na * 3 * N; e += BuildSmem<K>::NT) {
+        const int a = e / (3 * N), d = (e / N) % 3, g = act[a];
+        const double dx = X[e % (3 * N)] - D.cen[3 * g + d], f = exp(-D.expo[g] * dx * dx);
+        E[e] = f;
+        R[e] = d == 0 ? dx * dx * f : dx * dx;
+    }
+    __syncthreads();
+    return na;
 }
 
-// One block per box of level j.  mode: 0 adaptive test, 1 refine, 2 leaf.
-__global__ void k_build_level(int k, int j, DensDev D, const int32_t* boxes, const double* tolp, int mode,
-                              int at_max, double* s_out, int32_t* refine, int32_t* depth_hit) {
-    extern __shared__ double sm[];
-    const int k3 = k * k * k, kk = k * k;
-    double* g = sm;             // k nodes
-    double* gw = g + k;         // k weights
-    double* P = gw + k;         // [i][q] phi_i(g_q) w_q
-    double* Q = P + kk;         // [p][q][i] phi_i((g_q + p)/2): (q, i) as a k x k matrix per p
-    double* v = Q + 2 * kk;     // k^3 values
-    double* t1 = v + k3;
-    double* t2 = t1 + k3;
-    double* s = t2 + k3;
-    double* X = s + k3;          // 3k grid coordinates
-    double* E = X + 3 * k;       // DG_CHUNK * 3k factors
-    double* R = E + DG_CHUNK * 3 * k;
-    double* cb = R + DG_CHUNK * 3 * k;  // (coef, r2coef) per term of a chunk
-    __shared__ double red[32];
+template <int K>
+__global__ void __launch_bounds__(BuildSmem<K>::NT) k_build_level(int j, DensDev D, const int32_t* boxes,
+                                                                  const unsigned long long* maxbits, double eps,
+                                                                  const BuildTables* T, int mode, int at_max, double* s_out,
+                                                                  int32_t* refine, int32_t* depth_hit) {
+    using L = BuildSmem<K>;
+    constexpr int K2 = 2 * K, KK = K * K, K3 = L::K3, P2 = L::P2, NT = L::NT, GR = L::GR, HQ = (K + 1) / 2;
+    extern __shared__ __align__(16) double sm[];
+    double* s = sm;
+    double* t2 = s + K3;
+    double* t3 = t2 + L::T2;
+    double* X = t3 + L::T3;  // [3][2k] grid coordinates
+    double* E = X + 3 * K2;
+    double* R = E + 3 * K2 * DG_CHUNK;
+    __shared__ double gq[K], P[HQ * K], Q[KK], red[32];
+    __shared__ double2 cb[DG_CHUNK];
     __shared__ int act[DG_CHUNK];
-    const double cut = tolp[1];
+    __shared__ unsigned mask[DG_CHUNK];
     const int b = blockIdx.x, tid = threadIdx.x;
-    const int a1 = boxes[3 * b], a2 = boxes[3 * b + 1], a3 = boxes[3 * b + 2];
-    if (tid < k) gauss_legendre01_root(k, tid, g, gw);
+    const double fm = __longlong_as_double((long long)*maxbits);
+    const double cut = 1e-18 * fm;  // terms below this on a grid are skipped (rounding level)
+    const int32_t* a = boxes + 3 * b;
+    for (int e = tid; e < K; e += NT) gq[e] = T->g[e];
+    for (int e = tid; e < HQ * K; e += NT) P[e] = T->P[e];
+    for (int e = tid; e < KK; e += NT) Q[e] = T->Q[e];
     __syncthreads();
-    if (tid < k) {
-        double tmp[MRA_MAX_K];
-        phi_all(k, g[tid], tmp);
-        for (int i = 0; i < k; ++i) P[i * k + tid] = tmp[i] * gw[tid];
-        for (int p = 0; p < 2; ++p) {
-            phi_all(k, 0.5 * (g[tid] + p), tmp);
-            for (int i = 0; i < k; ++i) Q[p * kk + tid * k + i] = tmp[i];
-        }
-    }
     const double h = exp2(-(double)j);
-    for (int e = tid; e < 3 * k; e += blockDim.x) {
-        const int d = e / k, q = e % k;
-        X[e] = (g[q] + (d == 0 ? a1 : (d == 1 ? a2 : a3))) * h;
+    for (int e = tid; e < 3 * K; e += NT) X[e] = (gq[e % K] + a[e / K]) * h;
+    // the density on the box's grid; thread group r takes every GR-th term
+    {
+        const int f = tid % KK, r = tid / KK, q2 = f / K, q3 = f % K;
+        double v[K];
+#pragma unroll
+        for (int q = 0; q < K; ++q) v[q] = 0.0;
+        for (int g0 = 0; g0 < D.n; g0 += DG_CHUNK) {
+            const int na = dens_factors<K, 1>(D, g0, X, cut, E, R, act, mask, cb);
+            if (r < GR)
+                for (int t = r; t < na; t += GR) {
+                    const double *Et = E + t * 3 * K, *Rt = R + t * 3 * K;
+                    const double2 c = cb[t];
+                    const double p = Et[K + q2] * Et[2 * K + q3];
+                    const double u = c.y == 0.0 ? p * c.x : p * (c.x + c.y * (Rt[K + q2] + Rt[2 * K + q3]));
+#pragma unroll
+                    for (int q = 0; q < K; ++q) v[q] += u * Et[q];
+                    if (c.y != 0.0) {
+                        const double u2 = p * c.y;
+#pragma unroll
+                        for (int q = 0; q < K; ++q) v[q] += u2 * Rt[q];
+                    }
+                }
+        }
+        if (r < GR)
+#pragma unroll
+            for (int q = 0; q < K; ++q) t2[r * K3 + q * KK + f] = v[q];
     }
-    for (int idx = tid; idx < k3; idx += blockDim.x) v[idx] = 0.0;
     __syncthreads();
-    dens_grid(D, k, X, v, E, R, cb, act, cut);
-    // s = 2^{-3j/2} (P x P x P) v  (eq. fvals2coefs in tensor form)
-    mode_product(v, t1, P, 2, k);
-    mode_product(t1, t2, P, 1, k);
-    mode_product(t2, s, P, 0, k);
+    // s = 2^{-3j/2} (P x P x P) v  (eq. fvals2coefs in tensor form), directions 1, 2, 3
     const double sc = exp2(-1.5 * j);
-    for (int idx = tid; idx < k3; idx += blockDim.x) s[idx] *= sc;
-    __syncthreads();
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+        const double* src = d == 0 ? t2 : (d == 1 ? s : t3);
+        double* dst = d == 1 ? t3 : s;
+        const int sf = d == 0 ? KK : (d == 1 ? K : 1), sa = d == 0 ? K : KK, sb = d == 2 ? K : 1;
+        for (int e = tid; e < 2 * KK; e += NT) {  // (parity of i, fiber)
+            const int par = e / KK, f = e % KK, at = (f / K) * sa + (f % K) * sb;
+            double v[K], p[HQ];
+#pragma unroll
+            for (int q = 0; q < K; ++q) {
+                v[q] = src[at + q * sf];
+                if (d == 0)
+#pragma unroll
+                    for (int r = 1; r < GR; ++r) v[q] += src[r * K3 + at + q * sf];
+            }
+#pragma unroll
+            for (int q = 0; q < HQ; ++q) p[q] = 2 * q == K - 1 ? v[q] : (par ? v[q] - v[K - 1 - q] : v[q] + v[K - 1 - q]);
+#pragma unroll
+            for (int i2 = 0; i2 < HQ; ++i2) {
+                const int i = 2 * i2 + par;
+                if (i >= K) break;
+                double acc = 0.0;
+#pragma unroll
+                for (int q = 0; q < HQ; ++q) acc += P[q * K + i] * p[q];
+                dst[at + i * sf] = d == 2 ? acc * sc : acc;
+            }
+        }
+        __syncthreads();
+    }
     int ref = (mode == 1);
     if (mode == 0) {
-        double err = 0.0;
-        const double hc = 0.5 * h, up = exp2(1.5 * j);
-        for (int o = 0; o < 8; ++o) {
-            int p1 = (o >> 2) & 1, p2 = (o >> 1) & 1, p3 = o & 1;
-            // interpolate: f~ = 2^{3j/2} sum_i s_i prod_d phi_{i_d}((g_q + p_d)/2)
-            mode_product(s, t1, Q + p3 * kk, 2, k);
-            mode_product(t1, t2, Q + p2 * kk, 1, k);
-            mode_product(t2, t1, Q + p1 * kk, 0, k);
-            // the child's GL grid, its density values into v
-            for (int e = tid; e < 3 * k; e += blockDim.x) {
-                const int d = e / k, q = e % k;
-                X[e] = (g[q] + (d == 0 ? 2 * a1 + p1 : (d == 1 ? 2 * a2 + p2 : 2 * a3 + p3))) * hc;
+        // f~ = 2^{3j/2} sum_i s_i prod_d phi_{i_d}((g_q + p_d)/2) at the points x = p k + q of a
+        // direction: directions 3 and 2 into shared memory, direction 1 in registers
+        for (int e = tid; e < 3 * K2; e += NT) X[e] = (gq[e % K] + 2 * a[e / K2] + (e / K) % 2) * (0.5 * h);
+#pragma unroll
+        for (int d = 0; d < 2; ++d) {
+            const int nf = d == 0 ? KK : KK * 2;
+            for (int f = tid; f < nf; f += NT) {
+                const double* src = d == 0 ? s + f * K : t3 + (f / K2) * K * P2 + f % K2;
+                const int st = d == 0 ? 1 : P2;
+                double* dst = d == 0 ? t3 + f * P2 : t2 + (f / K2) * K2 * K2 + f % K2;
+                const int ds = d == 0 ? 1 : K2;
+                double v[K];
+#pragma unroll
+                for (int i = 0; i < K; ++i) v[i] = src[i * st];
+#pragma unroll
+                for (int q = 0; q < K; ++q) {
+                    double ev = 0.0, od = 0.0;
+#pragma unroll
+                    for (int i = 0; i < K; i += 2) ev += Q[q * K + i] * v[i];
+#pragma unroll
+                    for (int i = 1; i < K; i += 2) od += Q[q * K + i] * v[i];
+                    dst[q * ds] = ev + od;
+                    dst[(K2 - 1 - q) * ds] = ev - od;
+                }
             }
-            for (int idx = tid; idx < k3; idx += blockDim.x) v[idx] = 0.0;
-            __syncthreads();
-            dens_grid(D, k, X, v, E, R, cb, act, cut);
-            for (int idx = tid; idx < k3; idx += blockDim.x) err = fmax(err, fabs(v[idx] - up * t1[idx]));
             __syncthreads();
         }
+        const double up = exp2(1.5 * j);
+        double err = 0.0;
+        const int po = tid / KK, fq = tid % KK;  // (p2, p3), (q2, q3)
+        const int x2 = (po >> 1) * K + fq / K, x3 = (po & 1) * K + fq % K;
+        const bool have = tid < 4 * KK;
+        double v[K2];
+#pragma unroll
+        for (int q = 0; q < K2; ++q) v[q] = 0.0;
+        for (int g0 = 0; g0 < D.n; g0 += DG_CHUNK) {
+            const int na = dens_factors<K, 2>(D, g0, X, cut, E, R, act, mask, cb);
+            if (have)
+                for (int t = 0; t < na; ++t) {
+                    const unsigned m = mask[t] >> po;
+                    if (!(m & 0x11u)) continue;
+                    const double *Et = E + t * 3 * K2, *Rt = R + t * 3 * K2;
+                    const double2 c = cb[t];
+                    const double p = Et[K2 + x2] * Et[2 * K2 + x3];
+                    const double u = c.y == 0.0 ? p * c.x : p * (c.x + c.y * (Rt[K2 + x2] + Rt[2 * K2 + x3]));
+                    const double u2 = p * c.y;
+#pragma unroll
+                    for (int hf = 0; hf < 2; ++hf)
+                        if ((m >> (4 * hf)) & 1u) {
+#pragma unroll
+                            for (int q = 0; q < K; ++q) v[hf * K + q] += u * Et[hf * K + q];
+                            if (c.y != 0.0)
+#pragma unroll
+                                for (int q = 0; q < K; ++q) v[hf * K + q] += u2 * Rt[hf * K + q];
+                        }
+                }
+        }
+        if (have) {
+            double w[K];
+#pragma unroll
+            for (int i = 0; i < K; ++i) w[i] = t2[(i * K2 + x2) * K2 + x3];
+#pragma unroll
+            for (int q = 0; q < K; ++q) {
+                double ev = 0.0, od = 0.0;
+#pragma unroll
+                for (int i = 0; i < K; i += 2) ev += Q[q * K + i] * w[i];
+#pragma unroll
+                for (int i = 1; i < K; i += 2) od += Q[q * K + i] * w[i];
+                err = fmax(err, fabs(v[q] - up * (ev + od)));
+                err = fmax(err, fabs(v[K2 - 1 - q] - up * (ev - od)));
+            }
+        }
         err = block_max(err, red);
-        ref = err > *tolp;
+        ref = err > eps * fm;
         if (ref && at_max) {
             ref = 0;
             if (tid == 0) atomicExch(depth_hit, 1);
         }
     }
-    for (int idx = tid; idx < k3; idx += blockDim.x) s_out[(size_t)b * k3 + idx] = s[idx];
+    for (int idx = tid; idx < K3; idx += NT) s_out[(size_t)b * K3 + idx] = s[idx];
     if (tid == 0) refine[b] = ref;
+}
+
+template <int K>
+static int build_level_launch(int nb, int j, const DensDev& D, const int32_t* boxes, const unsigned long long* maxbits, double eps,
+                              const BuildTables* T, int mode, int at_max, double* s, int32_t* refine, int32_t* flags,
+                              cudaStream_t st) {
+    constexpr size_t bytes = BuildSmem<K>::bytes;
+    MRA_CK(cudaFuncSetAttribute(k_build_level<K>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
+    k_build_level<K><<<nb, BuildSmem<K>::NT, bytes, st>>>(j, D, boxes, maxbits, eps, T, mode, at_max, s, refine, flags);
+    MRA_CK_LAUNCH();
+    return MRA_OK;
 }
 
 // children of refined boxes (octant order) and the refined-parent list
@@ -460,13 +577,17 @@ int build_tree_impl(const mra_density* f, int k, double eps, int max_level, int 
         MRA_CK(cudaStreamSynchronize(st));
     }
     DensDev D{ng, dd, dd + ng, dd + 2 * ng, dd + 3 * ng};
-    double* tol;
-    int32_t *flags;  // [0] depth_hit, [1] total
-    MRA_TRY(tmp.get(&tol, 2));
+    int32_t *flags;  // [0] depth_hit, [1] total, [2..3] max |f| over the centres (a double's bits)
+    BuildTables* tab;
     MRA_TRY(tmp.get(&flags, 4));
+    MRA_TRY(tmp.get(&tab, 1));
     MRA_CK(cudaMemsetAsync(flags, 0, 4 * sizeof(int32_t), st));
-    k_dens_scale<<<1, 256, 0, st>>>(D, eps, tol);
+    auto* maxbits = (unsigned long long*)(flags + 2);
+    k_dens_scale<<<std::min((ng + 7) / 8, num_sms()) + 1, 256, 0, st>>>(D, maxbits, k, tab);
     MRA_CK_LAUNCH();
+    using LevelFn = int (*)(int, int, const DensDev&, const int32_t*, const unsigned long long*, double, const BuildTables*, int,
+                            int, double*, int32_t*, int32_t*, cudaStream_t);
+    static const LevelFn level_fn[] = FOR_EVERY_K(build_level_launch);
 
     struct Level {
         int n;
@@ -480,9 +601,6 @@ int build_tree_impl(const mra_density* f, int k, double eps, int max_level, int 
     int nb = 1;
     int32_t* cur = boxes0;
     int32_t* plocal_prev = nullptr;
-    const size_t smem =
-        (2 * k + 3 * k * k + 4 * (size_t)k3 + 3 * k + 2 * DG_CHUNK * 3 * (size_t)k + 2 * DG_CHUNK) * sizeof(double);
-    MRA_CK(cudaFuncSetAttribute(k_build_level, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     for (int j = 0; j <= max_level; ++j) {
         Level lv{nb, cur, nullptr, nullptr, plocal_prev, nullptr};
         MRA_TRY(tmp.get(&lv.refine, nb));
@@ -492,8 +610,7 @@ int build_tree_impl(const mra_density* f, int k, double eps, int max_level, int 
         if (uniform_level >= 0) mode = (j < uniform_level) ? 1 : 2;
         else mode = (j < init_level) ? 1 : 0;
         if (j == max_level && mode == 1) mode = 2;
-        k_build_level<<<nb, 128, smem, st>>>(k, j, D, cur, tol, mode, j >= max_level, lv.s, lv.refine, flags);
-        MRA_CK_LAUNCH();
+        MRA_TRY(level_fn[k](nb, j, D, cur, maxbits, eps, tab, mode, j >= max_level, lv.s, lv.refine, flags, st));
         MRA_TRY(scan_exclusive(lv.refine, lv.pos, nb, flags + 1, st));
         int32_t nref = 0;
         MRA_CK(cudaMemcpyAsync(&nref, flags + 1, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
