@@ -220,56 +220,97 @@ __device__ inline int find_key_exact(const uint64_t* keys, int lo, int hi, uint6
     return (l < hi && keys[l] == k) ? l : -1;
 }
 
-// phi_i(u) = sqrt(2i+1) P_i(2u-1), i < n, written to out[0..n)
+// Constants of the Legendre basis, evaluated at compile time: a kernel that built the rule by Newton
+// steps and divided in every recurrence spent 20 to 60 us of serial FP64 latency on it before its
+// work began.  GL_MAX is the longest rule (2 k, and 32 by the largest caller).
+#define GL_MAX 32
+struct LegendreTable {
+    double x[GL_MAX * (GL_MAX + 1) / 2], w[GL_MAX * (GL_MAX + 1) / 2];  // rule n at n (n - 1) / 2
+    double ra[GL_MAX], rb[GL_MAX], nrm[GL_MAX];  // P_i = ra_i v P_{i-1} - rb_i P_{i-2}; sqrt(2i + 1)
+};
+
+constexpr double const_sqrt(double a) {
+    double z = a > 1.0 ? a : 1.0;
+    for (int it = 0; it < 100; ++it) {
+        const double y = 0.5 * (z + a / z);
+        if (y >= z) break;
+        z = y;
+    }
+    return z;
+}
+
+constexpr double const_cos(double t) {  // Taylor series, 0 <= t <= pi
+    double term = 1.0, sum = 1.0;
+    for (int i = 1; i < 30; ++i) {
+        term *= -t * t / ((2 * i - 1) * (2 * i));
+        sum += term;
+    }
+    return sum;
+}
+
+// Root i of P_n by Newton from the asymptotic start cos(pi (i + 3/4) / (n + 1/2)) and its weight; the
+// nodes increase with the index n - 1 - i, the second half of the rule mirrors the first.
+constexpr LegendreTable make_legendre() {
+    LegendreTable T{};
+    for (int i = 0; i < GL_MAX; ++i) {
+        T.ra[i] = i ? (2.0 * i - 1.0) / i : 0.0;
+        T.rb[i] = i ? (i - 1.0) / i : 0.0;
+        T.nrm[i] = const_sqrt(2.0 * i + 1.0);
+    }
+    for (int n = 1; n <= GL_MAX; ++n) {
+        const int at = n * (n - 1) / 2;
+        for (int i = 0; i < (n + 1) / 2; ++i) {
+            double z = 2 * i + 1 == n ? 0.0 : const_cos(3.14159265358979323846 * (i + 0.75) / (n + 0.5));
+            double pn = 0.0, pm = 0.0, dp = 0.0;
+            for (int it = 0; it < 6; ++it) {
+                double p0 = 1.0, p1 = z;
+                for (int q = 2; q <= n; ++q) {
+                    const double p2 = ((2.0 * q - 1.0) * z * p1 - (q - 1.0) * p0) / q;
+                    p0 = p1;
+                    p1 = p2;
+                }
+                pn = p1;
+                pm = p0;
+                dp = n * (z * pn - pm) / (z * z - 1.0);
+                if (it == 5 || 2 * i + 1 == n) break;
+                z -= pn / dp;
+            }
+            const double w = 1.0 / ((1.0 - z * z) * dp * dp);
+            T.x[at + n - 1 - i] = 0.5 * (1.0 + z);
+            T.x[at + i] = 0.5 * (1.0 - z);
+            T.w[at + n - 1 - i] = T.w[at + i] = w;
+        }
+    }
+    return T;
+}
+static __constant__ LegendreTable c_legendre = make_legendre();
+static constexpr LegendreTable h_legendre = make_legendre();
+#ifdef __CUDA_ARCH__
+#define LEGENDRE ::mra::c_legendre
+#else
+#define LEGENDRE ::mra::h_legendre
+#endif
+
+// phi_i(u) = sqrt(2i+1) P_i(2u-1), i < n <= GL_MAX, written to out[0..n)
 __host__ __device__ inline void phi_all(int n, double u, double* out) {
-    double v = 2.0 * u - 1.0;
+    const double v = 2.0 * u - 1.0;
     double p0 = 1.0, p1 = v;
     for (int i = 0; i < n; ++i) {
-        double p;
-        if (i == 0) p = 1.0;
-        else if (i == 1) p = v;
-        else {
-            p = ((2.0 * i - 1.0) * v * p1 - (i - 1.0) * p0) / i;
+        double p = i ? v : 1.0;
+        if (i > 1) {
+            p = LEGENDRE.ra[i] * v * p1 - LEGENDRE.rb[i] * p0;
             p0 = p1;
             p1 = p;
         }
-        out[i] = sqrt(2.0 * i + 1.0) * p;
+        out[i] = LEGENDRE.nrm[i] * p;
     }
 }
 
-// Root i of the n-point Gauss-Legendre rule on [0, 1] (n <= 32) by Newton on
-// P_n from the asymptotic start cos(pi (i + 3/4) / (n + 1/2)): stops once the
-// step is below 1e-15 (quadratic convergence leaves the root at rounding
-// level), then refreshes the derivative for the weight.  Node index
-// n - 1 - i (nodes increase with the index).
+// node and weight n - 1 - i of the n-point Gauss-Legendre rule on [0, 1], n <= GL_MAX
 __host__ __device__ inline void gauss_legendre01_root(int n, int i, double* x, double* w) {
-    double z = cos(3.14159265358979323846 * (i + 0.75) / (n + 0.5));
-    double pn = 0.0, pm = 0.0;
-    for (int it = 0; it < 100; ++it) {
-        double p0 = 1.0, p1 = z;
-        for (int q = 2; q <= n; ++q) {
-            double p2 = ((2.0 * q - 1.0) * z * p1 - (q - 1.0) * p0) / q;
-            p0 = p1;
-            p1 = p2;
-        }
-        pn = (n == 1) ? z : p1;
-        pm = (n == 1) ? 1.0 : p0;
-        const double dz = pn / (n * (z * pn - pm) / (z * z - 1.0));
-        z -= dz;
-        if (fabs(dz) < 1e-15) break;
-    }
-    double p0 = 1.0, p1 = z;
-    for (int q = 2; q <= n; ++q) {
-        double p2 = ((2.0 * q - 1.0) * z * p1 - (q - 1.0) * p0) / q;
-        p0 = p1;
-        p1 = p2;
-    }
-    pn = (n == 1) ? z : p1;
-    pm = (n == 1) ? 1.0 : p0;
-    const double dp = n * (z * pn - pm) / (z * z - 1.0);
-    const int idx = n - 1 - i;  // cos(.) decreases with i
-    x[idx] = 0.5 * (z + 1.0);
-    w[idx] = 1.0 / ((1.0 - z * z) * dp * dp);
+    const int idx = n - 1 - i, at = n * (n - 1) / 2 + idx;
+    x[idx] = LEGENDRE.x[at];
+    w[idx] = LEGENDRE.w[at];
 }
 
 // all n nodes and weights, by one thread

@@ -290,30 +290,41 @@ struct BuildSmem {
 };
 
 // The terms of a chunk that reach the grid X[3][H k] or, for H = 2, one of its 8 octants (bits of
-// mask), by the bound (|c| + |b| dmax^2) exp(-a dmin^2) >= cut; their one-dimensional factors in E
+// mask), by the bound (|c| + |b| dmax^2) exp(-a dmin^2) >= cut (in 32 bits with room for their
+// rounding: a term too many costs its products only); their one-dimensional factors in E
 // ([term][d][q]) and squared distances in R (direction 1: times the factor).
 template <int K, int H>
-__device__ int dens_factors(const DensDev& D, int g0, const double* X, double cut, double* E, double* R, int* act,
+__device__ int dens_factors(const DensDev& D, int g0, const double* X, double rcut, double* E, double* R, int* act,
                             unsigned* mask, double2* cb) {
     constexpr int N = H * K, OCT = H == 2 ? 8 : 1;
     __shared__ int s_na;
-    const int tid = threadIdx.x, lane = tid & 31;
+    __shared__ float2 span[DG_CHUNK][3 * H];  // smallest and largest distance squared per direction and half
+    __shared__ float3 size[DG_CHUNK];         // |c| / cut, |b| / cut, a
+    const int tid = threadIdx.x, lane = tid & 31, ng = min(DG_CHUNK, D.n - g0);
+    __syncthreads();
+    for (int e = tid; e < ng * 3 * H; e += BuildSmem<K>::NT) {
+        const int g = e / (3 * H), r = e % (3 * H), d = r / H;
+        const double c = D.cen[3 * (g0 + g) + d], *Xd = X + d * N + (r % H) * K;
+        const float lo = (float)(Xd[0] - c), hi = (float)(Xd[K - 1] - c);
+        const float dn = lo > 0.0f ? lo : (hi < 0.0f ? -hi : 0.0f), dx = fmaxf(fabsf(lo), fabsf(hi));
+        span[g][r] = make_float2(dn * dn, dx * dx);
+    }
+    for (int g = tid; g < ng; g += BuildSmem<K>::NT) {
+        const double c = fabs(D.coef[g0 + g]), r2 = fabs(D.r2[g0 + g]);
+        // (a term that is not a number reaches nothing)
+        size[g] = c == c && r2 == r2 ? make_float3((float)(c * rcut), (float)(r2 * rcut), (float)D.expo[g0 + g])
+                                     : make_float3(0.0f, 0.0f, 1.0f);
+    }
     __syncthreads();
     for (int e = tid; e < DG_CHUNK * OCT; e += BuildSmem<K>::NT) {  // (a multiple of 32: whole warps)
-        const int g = g0 + e / OCT, o = e % OCT;
+        const int g = e / OCT, o = e % OCT;
         bool on = false;
-        if (g < D.n) {
-            double dmin2 = 0.0, dmax2 = 0.0;
-#pragma unroll
-            for (int d = 0; d < 3; ++d) {
-                const double* Xd = X + d * N + ((o >> (2 - d)) & 1) * K;
-                const double lo = Xd[0] - D.cen[3 * g + d], hi = Xd[K - 1] - D.cen[3 * g + d];
-                const double dn = lo > 0.0 ? lo : (hi < 0.0 ? -hi : 0.0);
-                const double dx = fmax(fabs(lo), fabs(hi));
-                dmin2 += dn * dn;
-                dmax2 += dx * dx;
-            }
-            on = (fabs(D.coef[g]) + fabs(D.r2[g]) * dmax2) * exp(-D.expo[g] * dmin2) >= cut;
+        if (g < ng) {
+            const float2 s1 = span[g][H == 2 ? o >> 2 : 0], s2 = span[g][H == 2 ? 2 + ((o >> 1) & 1) : 1],
+                         s3 = span[g][H == 2 ? 4 + (o & 1) : 2];
+            const float3 z = size[g];
+            // a dmin^2 <= log of the rest over the cut
+            on = !(z.z * (s1.x + s2.x + s3.x) > __logf(z.x + z.y * (s1.y + s2.y + s3.y)) + 1e-2f);
         }
         const unsigned b = __ballot_sync(0xffffffffu, on);
         if (o == 0) mask[e / OCT] = OCT == 1 ? (b >> lane) & 1u : (b >> lane) & 0xffu;
@@ -361,7 +372,7 @@ __global__ void __launch_bounds__(BuildSmem<K>::NT) k_build_level(int j, DensDev
     __shared__ unsigned mask[DG_CHUNK];
     const int b = blockIdx.x, tid = threadIdx.x;
     const double fm = __longlong_as_double((long long)*maxbits);
-    const double cut = 1e-18 * fm;  // terms below this on a grid are skipped (rounding level)
+    const double rcut = 1e18 / fm;  // terms below fm / 1e18 on a grid are skipped (rounding level)
     const int32_t* a = boxes + 3 * b;
     for (int e = tid; e < K; e += NT) gq[e] = T->g[e];
     for (int e = tid; e < HQ * K; e += NT) P[e] = T->P[e];
@@ -376,7 +387,7 @@ __global__ void __launch_bounds__(BuildSmem<K>::NT) k_build_level(int j, DensDev
 #pragma unroll
         for (int q = 0; q < K; ++q) v[q] = 0.0;
         for (int g0 = 0; g0 < D.n; g0 += DG_CHUNK) {
-            const int na = dens_factors<K, 1>(D, g0, X, cut, E, R, act, mask, cb);
+            const int na = dens_factors<K, 1>(D, g0, X, rcut, E, R, act, mask, cb);
             if (r < GR)
                 for (int t = r; t < na; t += GR) {
                     const double *Et = E + t * 3 * K, *Rt = R + t * 3 * K;
@@ -466,7 +477,7 @@ __global__ void __launch_bounds__(BuildSmem<K>::NT) k_build_level(int j, DensDev
 #pragma unroll
         for (int q = 0; q < K2; ++q) v[q] = 0.0;
         for (int g0 = 0; g0 < D.n; g0 += DG_CHUNK) {
-            const int na = dens_factors<K, 2>(D, g0, X, cut, E, R, act, mask, cb);
+            const int na = dens_factors<K, 2>(D, g0, X, rcut, E, R, act, mask, cb);
             if (have)
                 for (int t = 0; t < na; ++t) {
                     const unsigned m = mask[t] >> po;
