@@ -149,7 +149,7 @@ __global__ void k_pilot_terms(Forest F, int M, const double* w, const double* Ft
 
 // Block (b, q) sums the terms of the 32 coefficients e = 32 q + lane of tree b's
 // pilot, eight warps taking every eighth term, and writes the sum of their squares
-// to part[b][q]; k_pilot_reduce then adds a tree's parts in order (deterministic).
+// to part[b][q]; k_schedule then adds a tree's parts in order (deterministic).
 __global__ void k_pilot_partial(int k3, int M, const double* ym, double* part) {
     __shared__ double sl[8][33];
     const int b = blockIdx.x, q = blockIdx.y, lane = threadIdx.x & 31, wq = threadIdx.x >> 5;
@@ -169,22 +169,18 @@ __global__ void k_pilot_partial(int k3, int M, const double* ym, double* part) {
     }
 }
 
-__global__ void k_pilot_reduce(int nq, const double* part, double* dv) {
-    const int b = blockIdx.x, lane = threadIdx.x;
-    double acc = 0.0;
-    for (int q = lane; q < nq; q += 32) acc += part[(size_t)b * nq + q];
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    if (lane == 0) dv[4 * b + 1] = sqrt(acc);
-}
-
 // ------------------------------------------------------------------ schedule
-// Block per tree.  dv[4b]: ||f_b||^2, dv[4b+1]: sigma_b; writes eta_b to
-// dv[4b+2] and the tree's schedule at sched + b * sl, laid out (int32)
+// Block per tree.  dv[4b]: ||f_b||^2; sigma_b (dv[4b+1]) from the pilot's nq parts (NULL: as
+// given); writes eta_b to dv[4b+2] and the tree's schedule at sched + b * sl, laid out (int32)
 //   Jm[M] | m1[lm*4] | m2[lm*4] | cnt[lm*4*2]   (sl = M + 16 lm)
-// Levels at or beyond the tree's own depth get empty ranges.
-__global__ void k_schedule(int M, int lm, const int32_t* nlev_tab, int unscreened, double eps, const double* w,
-                           const double* nF, const double* est, double* dv, int32_t* sched_all, int sl) {
-    const int b = blockIdx.x;
+// Levels at or beyond the tree's own depth get empty ranges.  Latency bounds it, and an FP64
+// instruction occupies the SM as long for one lane as for 32: the scans from below and from above
+// of every (j, S) are lanes of a few warps, candidates and counts are a warp per (j, S).
+#define SCHED_NT 512
+__global__ void __launch_bounds__(SCHED_NT) k_schedule(int M, int lm, const int32_t* nlev_tab, int unscreened, double eps,
+                                                       const double* w, const double* nF, const double* est, int nq,
+                                                       const double* part, double* dv, int32_t* sched_all, int sl) {
+    const int b = blockIdx.x, lane = threadIdx.x & 31;
     const int nlev = nlev_tab ? nlev_tab[b] : lm;
     int32_t* Jm = sched_all + (size_t)b * sl;
     int32_t* m1 = Jm + M;
@@ -193,15 +189,36 @@ __global__ void k_schedule(int M, int lm, const int32_t* nlev_tab, int unscreene
     // shared copies of J_m, w_m and, per level, the core / off-core maxima of
     // the 1-D block norms, so the serial range scans below read shared memory
     extern __shared__ double sched_sm[];
+    __shared__ double s_sigma;
+    __shared__ int s_first[MRA_MAX_LEVEL + 2], s_last[MRA_MAX_LEVEL + 2], s_cut[8 * (MRA_MAX_LEVEL + 2)];
     double* ws = sched_sm;                        // M
     double* cmax = ws + M;                        // lm * M: max over |l| <= 1
     double* bmax = cmax + (size_t)lm * M;         // lm * M: max over |l| >= 2
     double* ev = bmax + (size_t)lm * M;           // lm * 4 * M: the bound e_m per (j, S)
     int* Js = (int*)(ev + (size_t)lm * 4 * M);    // M
+    if (threadIdx.x < 32) {
+        double sigma;
+        if (part) {
+            double acc = 0.0;
+            for (int q = lane; q < nq; q += 32) acc += part[(size_t)b * nq + q];
+            for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+            sigma = sqrt(acc);
+            if (lane == 0) dv[4 * b + 1] = sigma;
+        } else {
+            sigma = dv[4 * b + 1];
+        }
+        if (lane == 0) s_sigma = sigma;
+    }
+    for (int e = threadIdx.x; e < nlev * M; e += SCHED_NT) {
+        const double* r = nF + (size_t)e * 7;  // e = j * M + m
+        cmax[e] = fmax(fmax(r[2], r[3]), r[4]);
+        bmax[e] = fmax(fmax(r[0], r[1]), fmax(r[5], r[6]));
+    }
+    __syncthreads();
     const double fn = sqrt(dv[4 * b]);
-    const double eta = fn > 0.0 ? eps * dv[4 * b + 1] / fn : 0.0;
+    const double eta = fn > 0.0 ? eps * s_sigma / fn : 0.0;
     if (threadIdx.x == 0) dv[4 * b + 2] = eta;
-    for (int m = threadIdx.x; m < M; m += blockDim.x) {
+    for (int m = threadIdx.x; m < M; m += SCHED_NT) {
         int jm = 0;
         if (unscreened) jm = nlev - 1;
         else
@@ -211,16 +228,11 @@ __global__ void k_schedule(int M, int lm, const int32_t* nlev_tab, int unscreene
         Js[m] = jm;
         ws[m] = w[m];
     }
-    for (int e = threadIdx.x; e < nlev * M; e += blockDim.x) {
-        const double* r = nF + (size_t)e * 7;  // e = j * M + m
-        cmax[e] = fmax(fmax(r[2], r[3]), r[4]);
-        bmax[e] = fmax(fmax(r[0], r[1]), fmax(r[5], r[6]));
-    }
     __syncthreads();
     // the bounds e_m = w_m cmax^S bmax^(3-S) of every (j, S, m) at once (the serial
     // scans below then only add); a term with J_m < j gets 0, which the scans pass over
     // exactly as they skip it (acc + 0 <= budget holds while acc <= budget)
-    for (int e = threadIdx.x; e < lm * 4 * M; e += blockDim.x) {
+    for (int e = threadIdx.x; e < lm * 4 * M; e += SCHED_NT) {
         const int js = e / M, m = e - js * M, j = js >> 2, S = js & 3;
         double v = 0.0;
         if (j < nlev && Js[m] >= j) {
@@ -233,54 +245,56 @@ __global__ void k_schedule(int M, int lm, const int32_t* nlev_tab, int unscreene
     }
     __syncthreads();
     const double budget = eta / (2.0 * 216.0);
-    for (int js = threadIdx.x; js < lm * 4; js += blockDim.x) {
+    // candidates: terms with J_m >= j, in increasing m
+    for (int j = threadIdx.x >> 5; j < lm; j += SCHED_NT / 32) {
+        int first = M, last = -1;
+        for (int m0 = 0; m0 < M; m0 += 32) {
+            const unsigned on = __ballot_sync(0xffffffffu, m0 + lane < M && Js[m0 + lane] >= j);
+            if (!on) continue;
+            if (last < 0) first = m0 + __ffs(on) - 1;
+            last = m0 + 31 - __clz(on);
+        }
+        if (lane == 0) {
+            s_first[j] = first;
+            s_last[j] = last;
+        }
+    }
+    __syncthreads();
+    // terms cut below (even threads) and above (odd ones) while their sum keeps the budget
+    for (int e = threadIdx.x; e < 2 * lm * 4; e += SCHED_NT) {
+        const int js = e >> 1, step = e & 1 ? -1 : 1, first = s_first[js >> 2], last = s_last[js >> 2];
+        const double* e_js = ev + (size_t)js * M;
+        int at = e & 1 ? last : first;
+        double acc = 0.0;
+        for (; at >= first && at <= last; at += step) {
+            const double next = acc + e_js[at];
+            if (!(next <= budget)) break;
+            acc = next;
+        }
+        s_cut[e] = at;
+    }
+    __syncthreads();
+    for (int js = threadIdx.x >> 5; js < lm * 4; js += SCHED_NT / 32) {
         const int j = js / 4, S = js % 4;
         int lo_m = 0, hi_m = -1;
-        if (unscreened) {
-            lo_m = 0;
-            hi_m = M - 1;
-        } else {
-            // candidates: terms with J_m >= j, in increasing m
-            int first = -1, last = -1, n = 0;
-            for (int m = 0; m < M; ++m)
-                if (Js[m] >= j) {
-                    if (first < 0) first = m;
-                    last = m;
-                    ++n;
-                }
-            if (n > 0) {
-                const double* e_js = ev + (size_t)js * M;
-                double acc = 0.0;
-                int lo = first;
-                for (; lo <= last; ++lo) {
-                    const double e = e_js[lo];
-                    if (acc + e <= budget) acc += e;
-                    else break;
-                }
-                acc = 0.0;
-                int hi = last;
-                for (; hi >= lo; --hi) {
-                    const double e = e_js[hi];
-                    if (acc + e <= budget) acc += e;
-                    else break;
-                }
-                if (hi >= lo && lo <= last) {
-                    lo_m = lo;
-                    hi_m = hi;
-                }
-            }
+        // (scans that meet or pass each other leave nothing)
+        if (unscreened) hi_m = M - 1;
+        else if (s_last[j] >= 0 && s_cut[2 * js + 1] >= s_cut[2 * js]) {
+            lo_m = s_cut[2 * js];
+            hi_m = s_cut[2 * js + 1];
         }
-        m1[js] = lo_m;
-        m2[js] = hi_m;
         // kept-term counts for (j, S, core-at-internal-node)
-        for (int ci = 0; ci < 2; ++ci) {
-            int c = 0;
-            for (int m = lo_m; m <= hi_m; ++m) {
-                if (Js[m] < j) continue;
-                if (ci && S == 3 && Js[m] > j) continue;
-                ++c;
-            }
-            cnt[js * 2 + ci] = c;
+        int c0 = 0, c1 = 0;
+        for (int m0 = lo_m; m0 <= hi_m; m0 += 32) {
+            const int jm = m0 + lane <= hi_m ? Js[m0 + lane] : -1;
+            c0 += __popc(__ballot_sync(0xffffffffu, jm >= j));
+            c1 += __popc(__ballot_sync(0xffffffffu, S == 3 ? jm == j : jm >= j));
+        }
+        if (lane == 0) {
+            m1[js] = lo_m;
+            m2[js] = hi_m;
+            cnt[js * 2] = c0;
+            cnt[js * 2 + 1] = c1;
         }
     }
 }
@@ -379,9 +393,11 @@ __global__ void k_screen(ScreenArgs A) {
     }
 }
 
-__global__ void k_fill_u64(uint64_t* p, size_t n, uint64_t v) {
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
-        p[i] = v;
+__global__ void k_clear_ghosts(uint64_t* tab, uint32_t* mask, size_t n) {
+    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
+        tab[i] = GH_EMPTY;
+        mask[i] = 0u;
+    }
 }
 
 // ids: each parent slot takes popc(mask) consecutive ids (the order of the slots is
@@ -730,7 +746,7 @@ __global__ void __launch_bounds__(128) k_apply_simt(ApplyArgs A) {
 
 // ------------------------------------------------------------------ driver
 void screen_release(const Alloc& A, ScreenOut* S) {
-    A.put(S->dv); A.put(S->sched); A.put(S->count); A.put(S->pair_off); A.put(S->total); A.put(S->err);
+    A.put(S->dv); A.put(S->sched); A.put(S->count); A.put(S->pair_off);
     A.put(S->gtab); A.put(S->gid); A.put(S->gmask); A.put(S->gkeys); A.put(S->pairs);
     oct_release(A, &S->oct);
     *S = ScreenOut();
@@ -745,7 +761,13 @@ int screen_forest(const mra_op* op, const Forest& F, int unscreened, int what, c
     const int k3 = F.k * F.k * F.k, M = op->M, n = F.n;
     *S = ScreenOut();
     S->sl = M + 16 * F.lm;
-    MRA_TRY(dalloc(A, &S->dv, 4 * (size_t)F.ntrees));
+    const size_t nt = F.ntrees;
+    MRA_TRY(dalloc(A, &S->dv, 6 * nt + 2 + 3));  // the report: see ScreenReport
+    S->oct.pairs = (unsigned long long*)(S->dv + 4 * nt);
+    S->oct.items = S->oct.pairs + nt;
+    S->nitems = S->oct.items + nt;
+    S->total = (int32_t*)(S->nitems + 2);
+    S->err = S->total + 4;
     MRA_TRY(dalloc(A, &S->sched, (size_t)F.ntrees * S->sl));
     const bool pairs = what & SCREEN_PAIRS, groups = what & SCREEN_GROUPS;
     if (pairs) {
@@ -753,10 +775,7 @@ int screen_forest(const mra_op* op, const Forest& F, int unscreened, int what, c
         MRA_TRY(dalloc(A, &S->pair_off, (size_t)n + 1));
     }
     if (groups) MRA_TRY(oct_alloc(F, A, &S->oct));
-    MRA_TRY(dalloc(A, &S->total, 3));
-    MRA_TRY(dalloc(A, &S->err, 2));
-    MRA_CK(cudaMemsetAsync(S->dv, 0, 4 * (size_t)F.ntrees * sizeof(double), st));
-    MRA_CK(cudaMemsetAsync(S->err, 0, 2 * sizeof(int32_t), st));
+    MRA_CK(cudaMemsetAsync(S->dv, 0, (6 * nt + 2 + 3) * sizeof(double), st));
     const int nb_norm = (int)std::max<long>(1, std::min<long>(num_sms() * 16, ((long)n * 32 + 255) / 256));
     k_forest_norm2<<<nb_norm, 256, 0, st>>>(F, S->dv);
     MRA_CK_LAUNCH();
@@ -769,11 +788,9 @@ int screen_forest(const mra_op* op, const Forest& F, int unscreened, int what, c
     MRA_CK_LAUNCH();
     k_pilot_partial<<<dim3(F.ntrees, nq), 256, 0, st>>>(k3, M, ym, part);
     MRA_CK_LAUNCH();
-    k_pilot_reduce<<<F.ntrees, 32, 0, st>>>(nq, part, S->dv);
-    MRA_CK_LAUNCH();
     MRA_TRY(schedule_smem_attr(M, F.lm));
-    k_schedule<<<F.ntrees, 256, schedule_smem(M, F.lm), st>>>(M, F.lm, F.nlev, unscreened, op->eps, op->w, op->nF,
-                                                              op->est, S->dv, S->sched, S->sl);
+    k_schedule<<<F.ntrees, SCHED_NT, schedule_smem(M, F.lm), st>>>(M, F.lm, F.nlev, unscreened, op->eps, op->w, op->nF,
+                                                                   op->est, nq, part, S->dv, S->sched, S->sl);
     MRA_CK_LAUNCH();
 
     ScreenArgs sa;
@@ -787,16 +804,14 @@ int screen_forest(const mra_op* op, const Forest& F, int unscreened, int what, c
     // 27 parent boxes, shared with its neighbours), regrown x4 on a probe overflow
     uint64_t cap = 1024;
     while (cap < (uint64_t)n * 16ull) cap <<= 1;
-    int32_t h[3] = {0, 0, 0}, herr[2] = {0, 0};
+    int32_t h[6];  // total | err
     for (;;) {
         if (cap > (1ull << 30)) { set_error("ghost hash set overflow"); return MRA_ECUDA; }
         S->gcap = (uint32_t)cap;
         MRA_TRY(dalloc(A, &S->gtab, cap));
         MRA_TRY(dalloc(A, &S->gid, cap));
         MRA_TRY(dalloc(A, &S->gmask, cap));
-        MRA_CK(cudaMemsetAsync(S->total, 0, 3 * sizeof(int32_t), st));
-        MRA_CK(cudaMemsetAsync(S->gmask, 0, cap * sizeof(uint32_t), st));
-        k_fill_u64<<<1024, 256, 0, st>>>(S->gtab, cap, GH_EMPTY);
+        k_clear_ghosts<<<1024, 256, 0, st>>>(S->gtab, S->gmask, cap);
         MRA_CK_LAUNCH();
         sa.gtab = S->gtab; sa.gcap = S->gcap; sa.gid = S->gid; sa.gmask = S->gmask;
         if (groups) MRA_TRY(oct_screen(sa, S->oct, S->total + 2, st));
@@ -809,13 +824,12 @@ int screen_forest(const mra_op* op, const Forest& F, int unscreened, int what, c
         k_ghost_ids<<<1024, 256, 0, st>>>(S->gtab, S->gcap, S->gmask, S->gid, S->total + 1);
         MRA_CK_LAUNCH();
         // the one host synchronisation: pair and ghost counts size the worklist
-        MRA_CK(cudaMemcpyAsync(h, S->total, 3 * sizeof(int32_t), cudaMemcpyDeviceToHost, st));
-        MRA_CK(cudaMemcpyAsync(herr, S->err, 2 * sizeof(int32_t), cudaMemcpyDeviceToHost, st));
+        MRA_CK(cudaMemcpyAsync(h, S->total, sizeof(h), cudaMemcpyDeviceToHost, st));
         MRA_CK(cudaStreamSynchronize(st));
-        if (!herr[0]) break;
+        if (!h[4]) break;
         A.put(S->gtab); A.put(S->gid); A.put(S->gmask);
         S->gtab = nullptr; S->gid = nullptr; S->gmask = nullptr;
-        MRA_CK(cudaMemsetAsync(S->err, 0, 2 * sizeof(int32_t), st));
+        MRA_CK(cudaMemsetAsync(S->oct.pairs, 0, (2 * nt + 2 + 3) * sizeof(double), st));  // all counts but dv
         cap <<= 2;
     }
     S->npairs = h[0];
@@ -965,10 +979,7 @@ int apply_impl(const mra_op* op, const mra_tree* f, const mra_apply_opts* o, cud
     MRA_TRY(tree_clone_skeleton(f, &G.g));
     mra_tree* g = G.g;
     g->state = MRA_TREE_NSFORM;
-    unsigned long long* nitems;  // [0] items, [1] items with single FP16 operands
-    MRA_TRY(dalloc(A, &nitems, 2));
-    G.p[2] = nitems;
-    MRA_CK(cudaMemsetAsync(nitems, 0, 2 * sizeof(unsigned long long), st));
+    unsigned long long* nitems = S.nitems;
     double* lpb = nullptr;
 
     ApplyArgs aa;
@@ -1025,33 +1036,23 @@ int apply_impl(const mra_op* op, const mra_tree* f, const mra_apply_opts* o, cud
     MRA_CK(cudaEventRecord(ev[3], st));
 
     if (stats) {
-        unsigned long long ni[2] = {0, 0};
-        double hv[3];
-        int32_t herr[2] = {0, 0};
-        MRA_CK(cudaMemcpyAsync(ni, nitems, sizeof(ni), cudaMemcpyDeviceToHost, st));
-        MRA_CK(cudaMemcpyAsync(hv, S.dv, 3 * sizeof(double), cudaMemcpyDeviceToHost, st));
-        MRA_CK(cudaMemcpyAsync(herr, S.err, 2 * sizeof(int32_t), cudaMemcpyDeviceToHost, st));
-        MRA_CK(cudaStreamSynchronize(st));
-        unsigned long long np64 = (unsigned long long)S.npairs;
-        if (!pairs) {
-            MRA_CK(cudaMemcpyAsync(&np64, S.oct.pairs, sizeof(np64), cudaMemcpyDeviceToHost, st));
-            MRA_CK(cudaStreamSynchronize(st));
-        }
-        stats->n_pairs = (int64_t)np64;
-        stats->n_items = (int64_t)ni[0];
-        stats->n_items_lowp = (int64_t)ni[1];
+        static_assert(sizeof(ScreenReport) == 11 * sizeof(double), "the layout of screen_forest's allocation");
+        ScreenReport R;
         unsigned long long sc[2] = {0, 0};
-        if (scounts) {
-            MRA_CK(cudaMemcpyAsync(sc, scounts, sizeof(sc), cudaMemcpyDeviceToHost, st));
-            MRA_CK(cudaStreamSynchronize(st));
-        }
+        if (scounts) MRA_CK(cudaMemcpyAsync(sc, scounts, sizeof(sc), cudaMemcpyDeviceToHost, st));
+        MRA_CK(cudaMemcpyAsync(&R, S.dv, sizeof(R), cudaMemcpyDeviceToHost, st));
+        MRA_CK(cudaStreamSynchronize(st));
+        const int32_t* herr = R.err;
+        stats->n_pairs = pairs ? (int64_t)S.npairs : (int64_t)R.group_pairs;
+        stats->n_items = (int64_t)R.nitems[0];
+        stats->n_items_lowp = (int64_t)R.nitems[1];
         stats->n_misses = (int64_t)sc[0];
         stats->n_pairs_empty = (int64_t)sc[1];
         stats->n_ghosts = S.nghost;
         stats->n_out_nodes = n;
-        stats->fnorm = sqrt(hv[0]);
-        stats->sigma = hv[1];
-        stats->eta = hv[2];
+        stats->fnorm = sqrt(R.dv[0]);
+        stats->sigma = R.dv[1];
+        stats->eta = R.dv[2];
         cudaEventElapsedTime(&stats->ms_screen, ev[0], ev[1]);
         cudaEventElapsedTime(&stats->ms_ghost, ev[1], ev[2]);
         cudaEventElapsedTime(&stats->ms_apply, ev[2], ev[3]);
@@ -1172,8 +1173,7 @@ int apply_noalloc_impl(const mra_op* op, const mra_tree* f, int precision, doubl
     MRA_CK(cudaMemsetAsync(total, 0, 2 * sizeof(int32_t), st));
     MRA_CK(cudaMemsetAsync(err, 0, 2 * sizeof(int32_t), st));
     MRA_CK(cudaMemsetAsync(nitems, 0, sizeof(unsigned long long), st));
-    MRA_CK(cudaMemsetAsync(gmask, 0, NA_HASH_CAP * sizeof(uint32_t), st));
-    k_fill_u64<<<64, 256, 0, st>>>(gtab, NA_HASH_CAP, GH_EMPTY);
+    k_clear_ghosts<<<64, 256, 0, st>>>(gtab, gmask, NA_HASH_CAP);
     MRA_CK_LAUNCH();
     MRA_TRY(leaf_norm2(f, dv, st));
     const size_t pilot_smem = (4 * (size_t)k3 + k * k) * sizeof(double);
@@ -1181,8 +1181,8 @@ int apply_noalloc_impl(const mra_op* op, const mra_tree* f, int precision, doubl
     MRA_CK_LAUNCH();
     const int sl = M + 16 * nlev;
     MRA_TRY(schedule_smem_attr(M, nlev));
-    k_schedule<<<1, 256, schedule_smem(M, nlev), st>>>(M, nlev, nullptr, 0, op->eps, op->w, op->nF, op->est, dv,
-                                                       sched, sl);
+    k_schedule<<<1, SCHED_NT, schedule_smem(M, nlev), st>>>(M, nlev, nullptr, 0, op->eps, op->w, op->nF, op->est, 0, nullptr,
+                                                            dv, sched, sl);
     MRA_CK_LAUNCH();
     const Forest F = forest_of_tree(f);
     ScreenArgs sa;

@@ -151,7 +151,7 @@ struct OctGroups {
     int32_t* first = nullptr;            // [n] first output node
     int32_t* in = nullptr;               // [n][216] input blocks (node, or node count + Step-2 id; -1 none)
     int32_t* np = nullptr;               // [n] pieces
-    unsigned long long* pairs = nullptr; // [ntrees] static pairs and items
+    unsigned long long* pairs = nullptr; // [ntrees] static pairs and items (in ScreenOut's report)
     unsigned long long* items = nullptr;
 };
 
@@ -159,9 +159,19 @@ struct OctGroups {
 #define SCREEN_PAIRS 1
 #define SCREEN_GROUPS 2
 
+// The host reads what a screen and an apply count in as few copies as it needs the numbers at
+// (each copy is a round trip of about 10 us): all counters lie in one allocation that starts at dv,
+//   dv [ntrees][4] | group pairs [ntrees] | group items [ntrees] | nitems [2] | total [4] | err [2].
+struct ScreenReport {  // of one tree
+    double dv[4];
+    unsigned long long group_pairs, group_items, nitems[2];
+    int32_t total[4], err[2];
+};
+
 // device results of the screen over a forest (screen_forest in apply.cu)
 struct ScreenOut {
-    double* dv = nullptr;         // [ntrees][4]: ||f_b||^2, sigma_b, eta_b, unused
+    double* dv = nullptr;         // [ntrees][4]: ||f_b||^2, sigma_b, eta_b, unused; the report's start
+    unsigned long long* nitems = nullptr;  // [2] for an apply of one tree: items, items with single FP16 operands
     int32_t* sched = nullptr;     // [ntrees][sl]: Jm | m1 | m2 | cnt
     int sl = 0;
     int32_t* count = nullptr;     // [n + 1] pairs per output node

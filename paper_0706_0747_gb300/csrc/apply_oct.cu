@@ -139,19 +139,15 @@ int oct_alloc(const Forest& F, const Alloc& A, OctGroups* O) {
     MRA_TRY(dalloc(A, &O->first, O->n));
     MRA_TRY(dalloc(A, &O->in, (size_t)O->n * 216));
     MRA_TRY(dalloc(A, &O->np, O->n));
-    MRA_TRY(dalloc(A, &O->pairs, F.ntrees));
-    MRA_TRY(dalloc(A, &O->items, F.ntrees));
     return MRA_OK;
 }
 
 void oct_release(const Alloc& A, OctGroups* O) {
-    A.put(O->first); A.put(O->in); A.put(O->np); A.put(O->pairs); A.put(O->items);
+    A.put(O->first); A.put(O->in); A.put(O->np);
     *O = OctGroups();
 }
 
 int oct_screen(const ScreenArgs& sa, const OctGroups& O, int32_t* max_pieces, cudaStream_t st) {
-    MRA_CK(cudaMemsetAsync(O.pairs, 0, sa.F.ntrees * sizeof(unsigned long long), st));
-    MRA_CK(cudaMemsetAsync(O.items, 0, sa.F.ntrees * sizeof(unsigned long long), st));
     const int nb = std::max(1, std::min(num_sms() * 16, (sa.F.n + 255) / 256));
     k_oct_first<<<nb, 256, 0, st>>>(sa.F, O.first);
     MRA_CK_LAUNCH();

@@ -169,9 +169,6 @@ __device__ __forceinline__ void tmem_ld16x256_x2x2(uint32_t ta0, uint32_t ta1, f
     for (int q = 0; q < 16; ++q) v[q >> 3][(q >> 2) & 1][q & 3] = __uint_as_float(r[q]);
 }
 
-// one arrival of a warp whose lanes have all got here
-__device__ __forceinline__ void mbar_arrive_warp(uint64_t* mbar);
-
 // move registers between the warpgroups of a CTA (every warp of the warpgroup; N a multiple of 8)
 template <int N>
 __device__ __forceinline__ void reg_dec() { asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(N)); }
