@@ -6,8 +6,9 @@
 // (b2, b2 + 1):
 //   stage I   D_I[(line, i3, i2)][(a1, piece, c1)] = X F^{t1}: M = 128, N = 128 (64 for at
 //             most 4 pieces), K = 16 per pair of input boxes b1;
-//   stage II  per piece V[(a1, c1, i3)][(a2, c2)] += W F^{t2}: M = 128, N = 16, K = 16 (two
-//             lines of i2), accumulated over the plane's lines;
+//   stage II  per piece V[(a1, c1, i3)][(a2, hi or lo, c2)] += W [F_hi^{t2} | F_lo^{t2}] for W hi and
+//             W lo: M = 128, N = 32, K = 16 (two lines of i2), accumulated over the plane's lines;
+//             the two products are added when V is converted;
 //   stage III per piece, plane and a2, Y[(a1, c1, c2)][(a3, c3)] = V F^{t3}: M = 128, N = 16,
 //             K = 16 (i3 as hi | lo), read out after the plane and summed over the planes and
 //             the chunk's pieces in FP32 registers.  (Summing in the tensor core's accumulator
@@ -24,9 +25,13 @@
 //   20-23  issue stages II and III of a pair each;
 //   24     issues stage I into one of two accumulators;
 //   25-27  set up the next unit (pieces, inputs, scales, F tiles) in the other of two slots.
-// What bounds it is the shared-memory side of the tensor core: an MMA of stage II or III reads
-// 4 KB of A for 16 columns of output (23 % of the launch's cycles in the version whose units
-// were set up and finished by the whole CTA between barriers: 1.38 ms on 3-D Poisson k = 8).
+// A warp waits for itself: meeting at a named barrier behind one polling warp cost a conversion 200
+// to 300 cycles.  What bounds the kernel is shared memory, 76 % busy (half of it the tensor core's: an
+// MMA of stage II or III reads 4 KB of A for 32 or 16 columns), and issue slots, 60 %: the conversions'
+// share of them is why scaling and splitting use two-lane FP32.  3-D Poisson k = 8: 0.79 ms; 0.93 ms
+// with F_hi and F_lo as products of their own and barriers; 1.38 ms in the version whose units were set
+// up and finished by the whole CTA.  Stage I in halves of 4 pieces, or pieces instead of pairs as
+// the grain of conversions and MMAs, lose (0.86 and 1.07 ms): A is read or waited for twice.
 // Every wait is bounded: one that reaches its limit makes all roles stop, the error word is set
 // to 4 and the kernel frees its tensor memory.
 #include <cfloat>
@@ -51,10 +56,11 @@ struct OtcSmem {
     static constexpr int A2_LBO = 2304, A2_SBO = 144;  // 8 x 16-byte core matrices, 16 bytes apart (bank spread)
     static constexpr int A2_PIECE = 4 * A2_LBO;        // stage II: hi, lo (2 K groups each); stage III: a2' = 0, 1
     static constexpr int A2 = X + 2 * XBUF;
-    static constexpr int TAB = 7 * OTC_P * 128;        // tiles [u 0..6][piece]
-    static constexpr int T = A2 + OTC_P * A2_PIECE;    // per slot [direction][hi, lo]
+    static constexpr int TAB = 7 * OTC_P * 128;        // hi or lo tiles of a direction
+    // per slot and direction: tiles [hi, lo][u 0..6][position], direction 2 [u][hi, lo][position]
+    static constexpr int T = A2 + OTC_P * A2_PIECE;
     static constexpr int Z = T + 12 * TAB;             // zeros: two tiles a tile row apart
-    static constexpr int TIN = Z + OTC_P * 128 + 128;  // per slot 216 int
+    static constexpr int TIN = Z + OTC_P * 128 + 128;          // per slot 216 int
     static constexpr int TG = TIN + 2 * 864;           // per slot 216 float
     static constexpr int LIST = TG + 2 * 864;          // pieces of the group being set up
     static size_t bytes(int M) { return LIST + 4 * (size_t)M * sizeof(uint32_t); }
@@ -64,7 +70,7 @@ static_assert(OtcSmem::LIST + 4 * MRA_MAX_TERMS * 4 + 2048 <= 232448, "shared me
 // a unit as its roles see it
 struct OtcUnit {
     int unit;            // -1: no more units
-    int npc, ps;         // pieces; tile stride (4 or 8 pieces)
+    int npc, ps;         // pieces; positions (4 or 8) of a tile row
     unsigned m1, m2, m3; // boxes the pieces read, per direction
     int nout;
     unsigned leaf;       // leaf outputs
@@ -72,10 +78,14 @@ struct OtcUnit {
     float c2[OTC_P], c3[OTC_P], fin[OTC_P];
 };
 
+// Pieces i and i + 4 of a unit are pair i's (up to four pieces are one each for the pairs), neighbours
+// in the tile rows: position 2 i + r of 8, i of 4.
+__device__ __forceinline__ int otc_pieces(int g, int npc) { return (g < npc) + (g + 4 < npc); }
+
 // c x[0..3] (c a power of two) as FP16 hi and lo pairs: hi01, lo01, hi23, lo23
 __device__ __forceinline__ void split_scaled(const float* x, float c, uint32_t* w) {
-    tc::split_h2(x[0] * c, x[1] * c, w[0], w[1]);
-    tc::split_h2(x[2] * c, x[3] * c, w[2], w[3]);
+    tc::split_scaled_h2(x[0], x[1], c, w[0], w[1]);
+    tc::split_scaled_h2(x[2], x[3], c, w[2], w[3]);
 }
 
 __global__ void __launch_bounds__(OTC_THREADS, 1) k_apply_oct_tc(OctTcArgs Q) {
@@ -117,16 +127,13 @@ __global__ void __launch_bounds__(OTC_THREADS, 1) k_apply_oct_tc(OctTcArgs Q) {
     __syncthreads();
     tc::fence_after();
     const uint32_t tbase = (uint32_t)tc::uniform((int)s_tmem);
-    // TMEM columns: D_I 2 x 128; D_II 16 per piece at 256 + 32 pair; D_III 2 a2' x 16 per piece: a
-    // pair's first piece at 384 + 32 pair, its second over the pair's D_II, which stage III no longer
-    // needs
-    auto cII = [&](int g, int r) { return tbase + 256u + (uint32_t)(g * 32 + r * 16); };
-    auto cIII = [&](int g, int r, int a) { return tbase + (r ? 256u : 384u) + (uint32_t)(g * 32 + a * 16); };
+    // TMEM columns: D_I 2 x 128; per piece 32: D_II (a2', product with hi or lo, c2), then D_III 2 a2' x 16
+    auto cII = [&](int g, int r) { return tbase + 256u + (uint32_t)(g * 64 + r * 32); };
+    auto cIII = [&](int g, int r, int a) { return cII(g, r) + (uint32_t)(a * 16); };
 #define OTC_WAIT(bar, parity) tc::mbar_wait_or(bar, parity, Q.wait_limit, &s_abort)
-    // the same by a whole warp, whose lanes go on or give up together (what follows is warp-collective)
-#define OTC_WAITW(bar, parity) __all_sync(0xffffffffu, OTC_WAIT(bar, parity))
-    // by 128 threads of named barrier `id`: the leading warp polls, the others sleep at the barrier
-#define OTC_WAITG(id, lead, expr) tc::group_all(id, !(lead) || (expr))
+    // waits by a whole warp, whose lanes go on or give up together (what follows is warp-collective)
+#define OTC_ALL(expr) __all_sync(0xffffffffu, expr)
+#define OTC_WAITW(bar, parity) OTC_ALL(OTC_WAIT(bar, parity))
     // barriers complete once per use; a use's parity is its running number's lowest bit
     uint32_t ln = 0;  // lines (pairs of boxes b2) so far
 
@@ -137,7 +144,7 @@ __global__ void __launch_bounds__(OTC_THREADS, 1) k_apply_oct_tc(OctTcArgs Q) {
         // ================= set up units
         const int t = tid - 800;
         uint32_t* list = (uint32_t*)(sm + L::LIST);
-        auto sync = [] { asm volatile("bar.sync 6, 96;" ::: "memory"); };  // (1-5: the groups of OTC_WAITG)
+        auto sync = [] { asm volatile("bar.sync 1, 96;" ::: "memory"); };
         for (uint32_t k = 0;; ++k) {
             const int slot = k & 1;
             const bool ok = k < 2 || t != 0 || tc::mbar_wait_or(&b_se[slot], ((k >> 1) - 1) & 1, Q.wait_limit, &s_abort, 500);
@@ -216,18 +223,24 @@ __global__ void __launch_bounds__(OTC_THREADS, 1) k_apply_oct_tc(OctTcArgs Q) {
                         tin[t + OTC_SETUP * r] = in[r];
                         tg[t + OTC_SETUP * r] = in[r] < 0 ? 0.0f : ldexpf(1.0f, es) / sx[r];
                     }
-                // F tiles, masked by the pieces' sets
-                const int ps = U.ps, lp = ps == 8 ? 3 : 2;
-                for (int e = t; e < 7 * 6 * 8 * ps; e += OTC_SETUP) {
-                    const int v = e & 7, pc = (e >> 3) & (ps - 1), r = e >> (3 + lp), u = r % 7, dh = r / 7;
-                    uint4 x = make_uint4(0, 0, 0, 0);
-                    if (pc < U.npc) {
-                        const uint32_t p = U.piece[pc];
-                        const int set = (p >> (20 - 2 * (dh >> 1))) & 3;
-                        if (set & ((u >= 2 && u <= 4) ? 1 : 2))
-                            x = __ldg((const uint4*)((dh & 1) ? Q.Fl : Q.Fh) + ((fb + (p & 0xffff)) * 7 + 6 - u) * 8 + v);
-                    }
-                    ((uint4*)(sm + L::T + (slot * 6 + dh) * L::TAB))[(u * ps + pc) * 8 + v] = x;
+                // F tiles, masked by the pieces' sets; a lane copies 16 bytes of a position, a warp the 7
+                // tiles of 4 positions of a (direction, hi or lo) at once, all loads in flight
+                const int v = lane & 7, ps = U.ps;
+                for (int r = warp - 25; r < 3 * ps / 2; r += OTC_SETUP / 32) {
+                    const int dh = ps == 8 ? r >> 1 : r, pos = (lane >> 3) + (ps == 8 ? 4 * (r & 1) : 0);
+                    const uint32_t p = U.piece[ps == 8 ? (pos >> 1) + 4 * (pos & 1) : pos];  // (0 beyond the last: the empty set)
+                    const int set = (p >> (20 - 2 * (dh >> 1))) & 3;
+                    const uint4* src = (const uint4*)((dh & 1) ? Q.Fl : Q.Fh) + ((fb + (p & 0xffff)) * 7 + 6) * 8 + v;
+                    uint4 x[7];
+#pragma unroll
+                    for (int u = 0; u < 7; ++u)
+                        x[u] = set & ((u >= 2 && u <= 4) ? 1 : 2) ? __ldg(src - u * 8) : make_uint4(0, 0, 0, 0);
+                    const bool mixed = (dh >> 1) == 1;
+                    uint4* dst = (uint4*)(sm + L::T + slot * 6 * L::TAB + (dh >> 1) * 2 * L::TAB) +
+                                 ((dh & 1) * (mixed ? ps : 7 * OTC_P) + pos) * 8 + v;
+                    const int row = (mixed ? 2 : 1) * ps * 8;
+#pragma unroll
+                    for (int u = 0; u < 7; ++u) dst[u * row] = x[u];
                 }
                 // power-of-two scales as in apply_tc.cu: sW = 2^eW, the largest power of two <=
                 // 8192 / (48 max|F| max|x|), and sV = 2^eV <= 8192 / (48^2 max|F|^2 max|x|)
@@ -312,7 +325,7 @@ __global__ void __launch_bounds__(OTC_THREADS, 1) k_apply_oct_tc(OctTcArgs Q) {
         bool ok = true;
         for (uint32_t k = 0; ok; ++k) {
             const int slot = k & 1;
-            ok = OTC_WAITG(5, warp == 16, OTC_WAIT(&b_sf[slot], (k >> 1) & 1));
+            ok = OTC_WAITW(&b_sf[slot], (k >> 1) & 1);
             if (!ok || s_u[slot].unit < 0) break;
             const unsigned m1 = s_u[slot].m1, m2 = s_u[slot].m2, m3 = s_u[slot].m3;
             const int s1 = m1 == 0x1e, s2 = m2 == 0x1e, n1 = 3 - s1, n2 = 3 - s2;
@@ -338,7 +351,7 @@ __global__ void __launch_bounds__(OTC_THREADS, 1) k_apply_oct_tc(OctTcArgs Q) {
                             }
                         }
                     }
-                    if (ln >= 2) ok = OTC_WAITG(5, warp == 16, OTC_WAIT(&b_xe[buf], ((ln >> 1) - 1) & 1));
+                    if (ln >= 2) ok = OTC_WAITW(&b_xe[buf], ((ln >> 1) - 1) & 1);
                     if (!ok) break;
                     unsigned char* dst = sm + L::X + buf * L::XBUF + hl * (L::XBUF / 2) + v * 16;
 #pragma unroll
@@ -363,16 +376,17 @@ __global__ void __launch_bounds__(OTC_THREADS, 1) k_apply_oct_tc(OctTcArgs Q) {
         const int g = tc::uniform(warp - 20);
         uint32_t bt = 0;  // batches so far
         bool ok = true;
-        const uint32_t id = tc::idesc_f16(128, 16);
+        const uint32_t id2 = tc::idesc_f16(128, 32), id = tc::idesc_f16(128, 16);
         const uint64_t a0 = tc::sdesc(sbase + L::A2 + 2 * g * L::A2_PIECE, L::A2_LBO, L::A2_SBO);
         for (uint32_t k = 0; ok; ++k) {
             const int slot = k & 1;
             ok = OTC_WAITW(&b_sf[slot], (k >> 1) & 1);
             if (!ok || tc::uniform(s_u[slot].unit) < 0) break;
             const unsigned m2 = tc::uniform(s_u[slot].m2), m3 = tc::uniform(s_u[slot].m3);
-            const int ps = tc::uniform(s_u[slot].ps), n = min(2, tc::uniform(s_u[slot].npc) - 2 * g);
+            const int npc = tc::uniform(s_u[slot].npc), n = otc_pieces(g, npc);
             const int s2 = m2 == 0x1e, n2 = 3 - s2;
-            const uint32_t tab = sbase + L::T + slot * 6 * L::TAB;
+            const int ps = tc::uniform(s_u[slot].ps);
+            const uint32_t tab = sbase + L::T + slot * 6 * L::TAB + (ps == 8 ? 2 * g : g) * 128;
             for (int b3 = 0; b3 < 6 && ok && n > 0; ++b3) {
                 if (!((m3 >> b3) & 1u)) continue;
                 uint32_t acc = 0;
@@ -382,15 +396,14 @@ __global__ void __launch_bounds__(OTC_THREADS, 1) k_apply_oct_tc(OctTcArgs Q) {
                     ok = OTC_WAITW(&b_af[g], bt & 1);
                     if (!ok) break;
                     tc::fence_after();
-                    const uint64_t b0 = tc::sdesc(tab + 2 * L::TAB + (b2 * ps + 2 * g) * 128, ps * 128, ps * 128);
+                    // B: (a2', hi or lo, c2), so that A is read once for both products
+                    const uint64_t b0 = tc::sdesc(tab + 2 * L::TAB + b2 * 2 * ps * 128, 2 * ps * 128, ps * 128);
 #pragma unroll
                     for (int r = 0; r < 2; ++r) {
                         if (r >= n) break;
-                        const uint64_t ah = a0 + (uint64_t)(r * (L::A2_PIECE / 16)), al = ah + 2 * L::A2_LBO / 16;
-                        const uint64_t bh = b0 + (uint64_t)(r * 8), bl = bh + L::TAB / 16;
-                        tc::mma_f16_warp(cII(g, r), ah, bh, id, acc);
-                        tc::mma_f16_warp(cII(g, r), ah, bl, id, 1);
-                        tc::mma_f16_warp(cII(g, r), al, bh, id, 1);
+                        const uint64_t ah = a0 + (uint64_t)(r * (L::A2_PIECE / 16)), bv = b0 + (uint64_t)(r * 8);
+                        tc::mma_f16_warp(cII(g, r), ah, bv, id2, acc);
+                        tc::mma_f16_warp(cII(g, r), ah + 2 * L::A2_LBO / 16, bv, id2, 1);
                     }
                     tc::commit_warp(&b_ae[g]);
                     ++bt;
@@ -399,7 +412,7 @@ __global__ void __launch_bounds__(OTC_THREADS, 1) k_apply_oct_tc(OctTcArgs Q) {
                 if (!ok) break;
                 // B operands of stage III: [F_hi ; F_hi], and [F_lo ; 0] (a tile further on the zeros
                 // are a tile nearer)
-                const uint32_t tile = tab + 4 * L::TAB + (b3 * ps + 2 * g) * 128;
+                const uint32_t tile = tab + 4 * L::TAB + b3 * ps * 128;
                 const uint64_t h0 = tc::sdesc(tile, 0, ps * 128);
                 const uint64_t l0 = tc::sdesc(tile + L::TAB, sbase + L::Z - tile - L::TAB, ps * 128);
                 ok = OTC_WAITW(&b_af[g], bt & 1);
@@ -434,29 +447,28 @@ __global__ void __launch_bounds__(OTC_THREADS, 1) k_apply_oct_tc(OctTcArgs Q) {
         // D_II: lanes (a1', c1, i3) -> rows (a1' c1 | c2), K = hi | lo; matrices hi, lo of two (a1', c1)
         const uint32_t rowII = mine + (mi & 1) * L::A2_LBO + (w4 * 4 + (mi >> 1)) * L::A2_SBO + mr * 16;
         uint32_t bt = 0, units = 0;
-        const bool lead = w4 == 0;
-#define OTC_WAITC(expr) OTC_WAITG(1 + g, lead, expr)
         bool ok = true;
         for (uint32_t k = 0; ok; ++k) {
             const int slot = k & 1;
-            ok = OTC_WAITC(OTC_WAIT(&b_sf[slot], (k >> 1) & 1));
+            ok = OTC_ALL(OTC_WAIT(&b_sf[slot], (k >> 1) & 1));
             const OtcUnit& U = s_u[slot];
             if (!ok || U.unit < 0) break;
             const unsigned m2 = U.m2;
-            const int ps = U.ps, npc = U.npc, nplane = __popc(U.m3), n = min(2, npc - 2 * g);
+            const int npc = U.npc, nplane = __popc(U.m3), n = otc_pieces(g, npc);
+            const int ps = U.ps;
             const int s2 = m2 == 0x1e, n2 = 3 - s2;
             int lpp = 0;  // lines per plane
             for (int q = 0; q < n2; ++q) lpp += ((m2 >> (s2 + 2 * q)) & 3u) != 0;
-            float y[2][16];  // [a2'][(a3', c3)] of lane (a1', c1, c2), this pair's pieces
+            float2 y[2][8];  // [a2'][(a3', c3)] of lane (a1', c1, c2), this pair's pieces
 #pragma unroll
-            for (int c = 0; c < 16; ++c) y[0][c] = y[1][c] = 0.0f;
+            for (int c = 0; c < 8; ++c) y[0][c] = y[1][c] = make_float2(0.0f, 0.0f);
             // y += fin Y after a plane's stage III
             auto add_plane = [&]() {
 #pragma unroll
                 for (int r = 0; r < 2; ++r) {
                     if (r >= n) break;
-                    const float fin = U.fin[2 * g + r];
-                    const bool leaf_only = (U.piece[2 * g + r] >> 24) != 0;
+                    const float fin = U.fin[g + 4 * r];
+                    const bool leaf_only = (U.piece[g + 4 * r] >> 24) != 0;
 #pragma unroll
                     for (int a = 0; a < 2; ++a) {
                         float t[16];
@@ -466,33 +478,35 @@ __global__ void __launch_bounds__(OTC_THREADS, 1) k_apply_oct_tc(OctTcArgs Q) {
                             const int o = (1 - (w4 >> 1)) * 4 + (1 - a) * 2 + 1 - a3;
                             const float f = leaf_only && !((U.leaf >> o) & 1u) ? 0.0f : fin;
 #pragma unroll
-                            for (int c = 0; c < 8; ++c) y[a][8 * a3 + c] = fmaf(f, t[8 * a3 + c], y[a][8 * a3 + c]);
+                            for (int c = 0; c < 4; ++c)
+                                y[a][4 * a3 + c] = tc::fma2(make_float2(f, f), make_float2(t[8 * a3 + 2 * c], t[8 * a3 + 2 * c + 1]),
+                                                            y[a][4 * a3 + c]);
                         }
                     }
                 }
             };
             // the pairs' sums of the unit before have been read out of the operand space
-            if (units > 0) ok = OTC_WAITC(OTC_WAIT(&b_yr, (units - 1) & 1));
+            if (units > 0) ok = OTC_ALL(OTC_WAIT(&b_yr, (units - 1) & 1));
             for (int p = 0; p < nplane && ok; ++p) {
                 for (int q = 0; q < lpp && ok; ++q, ++ln) {
                     const int buf = ln & 1;
                     // the last batch is complete: the operands are free, and after a stage III its result
                     // is whole; D_I of the line is there
                     if (n > 0 && p > 0 && q == 0) {
-                        ok = OTC_WAITC(OTC_WAIT(&b_ae[g], (bt - 1) & 1));
+                        ok = OTC_ALL(OTC_WAIT(&b_ae[g], (bt - 1) & 1));
                         if (!ok) break;
                         tc::fence_after();
                         add_plane();
                     }
-                    ok = OTC_WAITC((n <= 0 || bt == 0 || OTC_WAIT(&b_ae[g], (bt - 1) & 1)) && OTC_WAIT(&b_df[buf], (ln >> 1) & 1));
+                    ok = OTC_ALL((n <= 0 || bt == 0 || OTC_WAIT(&b_ae[g], (bt - 1) & 1)) && OTC_WAIT(&b_df[buf], (ln >> 1) & 1));
                     if (!ok) break;
                     if (n <= 0) {  // nothing to convert: only keep step
                         tc::mbar_arrive_warp(&b_de[buf]);
                         continue;
                     }
                     tc::fence_after();
-                    const float c20 = U.c2[2 * g], c21 = n > 1 ? U.c2[2 * g + 1] : 0.0f;
-                    const uint32_t ad = tbase + buf * 128 + (uint32_t)(2 * g * 8) + lane_off;
+                    const float c20 = U.c2[g], c21 = n > 1 ? U.c2[g + 4] : 0.0f;
+                    const uint32_t ad = tbase + buf * 128 + (uint32_t)((ps == 8 ? 2 * g : g) * 8) + lane_off;
 #pragma unroll
                     for (int lh = 0; lh < 2; ++lh) {
                         float v[2][2][4];  // [a1'][piece][.]
@@ -521,26 +535,27 @@ __global__ void __launch_bounds__(OTC_THREADS, 1) k_apply_oct_tc(OctTcArgs Q) {
                 }
                 if (!ok || n <= 0) continue;
                 // the plane's V
-                ok = OTC_WAITC(OTC_WAIT(&b_ae[g], (bt - 1) & 1));
+                ok = OTC_ALL(OTC_WAIT(&b_ae[g], (bt - 1) & 1));
                 if (!ok) break;
                 tc::fence_after();
-                const float c30 = U.c3[2 * g], c31 = n > 1 ? U.c3[2 * g + 1] : 0.0f;
+                const float c30 = U.c3[g], c31 = n > 1 ? U.c3[g + 4] : 0.0f;
 #pragma unroll
-                for (int lh = 0; lh < 2; ++lh) {
-                    float v[2][2][4];  // [piece][a2'][.]
-                    tc::tmem_ld16x256_x2x2(cII(g, 0) + lane_off + ((uint32_t)(lh * 16) << 16), cII(g, 1) + lane_off + ((uint32_t)(lh * 16) << 16), v);
-                    uint32_t w[2][2][4];
+                for (int r = 0; r < 2; ++r) {
+                    if (r >= n) break;
 #pragma unroll
-                    for (int r = 0; r < 2; ++r)
+                    for (int lh = 0; lh < 2; ++lh) {
+                        float v[2][2][4];  // [a2'][product with hi or lo][.]
+                        const uint32_t ad = cII(g, r) + lane_off + ((uint32_t)(lh * 16) << 16);
+                        tc::tmem_ld16x256_x2x2(ad, ad + 16u, v);
 #pragma unroll
-                        for (int a = 0; a < 2; ++a) split_scaled(v[r][a], r ? c31 : c30, w[r][a]);
+                        for (int a = 0; a < 2; ++a) {
+                            uint32_t w[4];
 #pragma unroll
-                    for (int r = 0; r < 2; ++r) {
-                        if (r >= n) break;
-#pragma unroll
-                        for (int a = 0; a < 2; ++a)
-                            tc::stmatrix_x4_trans(rowII + r * L::A2_PIECE + a * 2 * L::A2_LBO + lh * 2 * L::A2_SBO, w[r][a][0], w[r][a][1],
-                                                  w[r][a][2], w[r][a][3]);
+                            for (int c = 0; c < 4; ++c) v[a][0][c] += v[a][1][c];
+                            split_scaled(v[a][0], r ? c31 : c30, w);
+                            tc::stmatrix_x4_trans(rowII + r * L::A2_PIECE + a * 2 * L::A2_LBO + lh * 2 * L::A2_SBO, w[0], w[1], w[2],
+                                                  w[3]);
+                        }
                     }
                 }
                 tc::fence_before();
@@ -552,28 +567,40 @@ __global__ void __launch_bounds__(OTC_THREADS, 1) k_apply_oct_tc(OctTcArgs Q) {
             constexpr int YS = 2 * L::A2_PIECE / 4;
             const int r = w4 * 32 + lane;
             if (ok && n > 0) {
-                ok = OTC_WAITC(OTC_WAIT(&b_ae[g], (bt - 1) & 1));
+                ok = OTC_ALL(OTC_WAIT(&b_ae[g], (bt - 1) & 1));
                 if (ok) {
                     tc::fence_after();
                     add_plane();
                     tc::fence_before();
 #pragma unroll
-                    for (int c = 0; c < 32; ++c) ysum[g * YS + c * 128 + r] = y[c >> 4][c & 15];
+                    for (int c = 0; c < 16; ++c) {
+                        ysum[g * YS + (2 * c) * 128 + r] = y[c >> 3][c & 7].x;
+                        ysum[g * YS + (2 * c + 1) * 128 + r] = y[c >> 3][c & 7].y;
+                    }
                 }
             }
             tc::mbar_arrive_warp(&b_y);
-            ok = OTC_WAITC(ok && OTC_WAIT(&b_y, units & 1));
+            ok = OTC_ALL(ok && OTC_WAIT(&b_y, units & 1));
             if (ok) {  // four warps per (a2', a3') add the pairs' sums in order
                 const int a1 = 1 - (r >> 6), c1 = (r >> 3) & 7, c2 = r & 7, kk = P.k;
                 const int o = a1 * 4 + (1 - (g >> 1)) * 2 + 1 - (g & 1);
                 if (o < U.nout && c1 < kk && c2 < kk) {
                     float* dst = (float*)Q.part + (size_t)U.unit * 8 * kk * kk * kk + (size_t)o * kk * kk * kk + (c1 * kk + c2) * kk;
+                    float s[8];
 #pragma unroll
                     for (int c3 = 0; c3 < 8; ++c3) {
-                        if (c3 >= kk) break;
-                        float s = 0.0f;
-                        for (int gg = 0; 2 * gg < npc; ++gg) s += ysum[gg * YS + (g * 8 + c3) * 128 + r];
-                        dst[c3] = s;
+                        s[c3] = 0.0f;
+#pragma unroll
+                        for (int gg = 0; gg < 4; ++gg)
+                            if (otc_pieces(gg, npc) > 0) s[c3] += ysum[gg * YS + (g * 8 + c3) * 128 + r];
+                    }
+                    if (kk == 8) {
+                        ((float4*)dst)[0] = make_float4(s[0], s[1], s[2], s[3]);
+                        ((float4*)dst)[1] = make_float4(s[4], s[5], s[6], s[7]);
+                    } else {
+#pragma unroll
+                        for (int c3 = 0; c3 < 8; ++c3)
+                            if (c3 < kk) dst[c3] = s[c3];
                     }
                 }
             }
@@ -584,8 +611,7 @@ __global__ void __launch_bounds__(OTC_THREADS, 1) k_apply_oct_tc(OctTcArgs Q) {
     }
 #undef OTC_WAIT
 #undef OTC_WAITW
-#undef OTC_WAITG
-#undef OTC_WAITC
+#undef OTC_ALL
     tc::fence_before();
     __syncthreads();
     if (s_abort && tid == 0) atomicExch(Q.err, 4);

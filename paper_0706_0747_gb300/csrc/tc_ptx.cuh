@@ -185,16 +185,6 @@ __device__ __forceinline__ void mbar_arrive_warp(uint64_t* mbar) {
     if ((threadIdx.x & 31) == 0) mbar_arrive(mbar);
 }
 
-// the same predicate for the 128 threads of named barrier `id`: true when it is for all of them
-__device__ __forceinline__ bool group_all(int id, bool v) {
-    uint32_t r;
-    asm volatile("{\n.reg .pred p, q;\nsetp.ne.u32 q, %2, 0;\nbarrier.cta.red.and.pred p, %1, 128, q;\nselp.u32 %0, 1, 0, p;\n}\n"
-                 : "=r"(r)
-                 : "r"(id), "r"((uint32_t)v)
-                 : "memory");
-    return r != 0;
-}
-
 // As mbar_wait, but also gives up once *abort (shared memory) is set by another waiter; a wait
 // that reaches its limit sets it.  A poll suspends the thread in hardware until the phase completes
 // or TC_SUSPEND_NS have passed, so that waiting warps leave the issue slots to the others.
@@ -263,6 +253,32 @@ __device__ __forceinline__ void split_h2(float a, float b, uint32_t& hi, uint32_
     const __half2 l = __floats2half2_rn(a - hf.x, b - hf.y);
     hi = *(const uint32_t*)&h;
     lo = *(const uint32_t*)&l;
+}
+
+// two FP32 lanes an instruction (as many roundings as the two scalar ones)
+__device__ __forceinline__ float2 mul2(float2 a, float2 b) {
+    float2 r;
+    asm("mul.rn.f32x2 %0, %1, %2;"
+        : "=l"(*(unsigned long long*)&r)
+        : "l"(*(const unsigned long long*)&a), "l"(*(const unsigned long long*)&b));
+    return r;
+}
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
+    float2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;"
+        : "=l"(*(unsigned long long*)&r)
+        : "l"(*(const unsigned long long*)&a), "l"(*(const unsigned long long*)&b), "l"(*(const unsigned long long*)&c));
+    return r;
+}
+
+// c (a, b), c a power of two, as split_h2
+__device__ __forceinline__ void split_scaled_h2(float a, float b, float c, uint32_t& hi, uint32_t& lo) {
+    const float2 x = mul2(make_float2(a, b), make_float2(c, c));
+    const __half2 h = __floats2half2_rn(x.x, x.y);
+    const float2 l = fma2(__half22float2(h), make_float2(-1.0f, -1.0f), x);  // exact
+    const __half2 l2 = __floats2half2_rn(l.x, l.y);
+    hi = *(const uint32_t*)&h;
+    lo = *(const uint32_t*)&l2;
 }
 
 // FP32 -> FP16 hi + FP16 lo with v ~= hi + lo to about 2^-22 relative
