@@ -12,6 +12,7 @@
 //              the d = 0 half of eqs. recon_even / recon_odd
 //   apply      per output node: for each pair and kept term,
 //              ghat += w_m (F1 x F2 x F3) f_b as three mode products (Step 3)
+#include <cfloat>
 #include <math.h>
 
 #include <algorithm>
@@ -497,6 +498,34 @@ __global__ void k_ghost_refine(Forest F, const uint64_t* gkeys, double* gblk, in
 }
 
 
+// A number as the unevaluated sum of two floats (about 48 bits), products by fma and sums by Knuth's
+// two-sum: 12 FP32 operations a multiply-add, where an FP64 one costs as much as 64.
+struct F2 {
+    float h, l;
+    F2() = default;
+    __device__ __forceinline__ explicit F2(double x) : h((float)x), l((float)(x - (double)(float)x)) {}
+    __device__ __forceinline__ F2(float a, float b) : h(a), l(b) {}
+    __device__ __forceinline__ explicit operator float() const { return h + l; }
+    __device__ __forceinline__ F2 operator*(const F2& o) const {
+        const float p = __fmul_rn(h, o.h);
+        return F2(p, __fmaf_rn(l, o.h, __fmaf_rn(h, o.l, __fmaf_rn(h, o.h, -p))));
+    }
+    __device__ __forceinline__ F2& operator+=(const F2& o) {
+        const float s = __fadd_rn(h, o.h), b = __fsub_rn(s, h);
+        l = __fadd_rn(l, __fadd_rn(o.l, __fadd_rn(__fsub_rn(h, __fsub_rn(s, b)), __fsub_rn(o.h, b))));
+        h = s;
+        return *this;
+    }
+    __device__ __forceinline__ F2 operator-() const { return F2(-h, -l); }
+    __device__ __forceinline__ F2 operator+(const F2& o) const {  // normalised: |l| at most half an ulp of h
+        F2 r = *this;
+        r += o;
+        const float s = __fadd_rn(r.h, r.l);
+        return F2(s, __fsub_rn(r.l, __fsub_rn(s, r.h)));
+    }
+    __device__ __forceinline__ F2 operator-(const F2& o) const { return *this + -o; }
+};
+
 // out = Mat along dimension `dim` of x (out[c] = sum_i Mat[c][i] x[i]), (K, K, K) arrays whose innermost
 // extent is padded to K + 1 (so that fibers along it, one per thread, hit
 // distinct banks), for upper-triangular Mat: the refinement matrices H^(p)T and
@@ -516,7 +545,7 @@ __device__ __forceinline__ void mode_mul_tri(const T* Mat, const T* x, T* out, i
         T* dst = out + a * sa + b * sb;
 #pragma unroll
         for (int c = 0; c < K; ++c) {
-            T acc = 0;
+            T acc(0.0);
 #pragma unroll
             for (int i = c; i < K; ++i) acc += Mat[c * K + i] * v[i];
             dst[c * sf] = acc;
@@ -529,20 +558,19 @@ __device__ __forceinline__ void mode_mul_tri(const T* Mat, const T* x, T* out, i
 // H^(1)_{ia} = (-1)^{i+a} H^(0)_{ia}, so with the sums s0 over the i >= a of a's parity and s1
 // over the others the children's entries a are s0 + s1 and s0 - s1: half the multiplications
 // of two products.  HT: H^(0) transposed.
-template <int K, typename T, typename TO>
-__device__ __forceinline__ void child_pair(const T* HT, const T* src, int st, TO* d0, TO* d1, int dst, bool n0, bool n1) {
+template <int K, typename T, typename Put>
+__device__ __forceinline__ void child_pair(const T* HT, const T* src, int st, Put put) {
     T v[K];
 #pragma unroll
     for (int i = 0; i < K; ++i) v[i] = src[i * st];
 #pragma unroll
     for (int a = 0; a < K; ++a) {
-        T s0 = 0, s1 = 0;
+        T s0(0.0), s1(0.0);
 #pragma unroll
         for (int i = a; i < K; i += 2) s0 += HT[a * K + i] * v[i];
 #pragma unroll
         for (int i = a + 1; i < K; i += 2) s1 += HT[a * K + i] * v[i];
-        if (n0) d0[a * dst] = (TO)(s0 + s1);
-        if (n1) d1[a * dst] = (TO)(s0 - s1);
+        put(a, s0 + s1, s0 - s1);
     }
 }
 
@@ -552,10 +580,14 @@ __device__ __forceinline__ void child_pair(const T* HT, const T* src, int st, TO
 // multiplied first, then one three-mode product), then every child of the
 // group, sharing the direction-3 and direction-2 partial products among the
 // children (d = 0 half of eqs. recon_even / recon_odd).
-// T = double, or float where the blocks only feed FP16 hi/lo tensor-core operands.
+// Arithmetic T and stored blocks O: double and double; where the blocks only become FP16 hi/lo
+// operands and no screen decision reads them, two floats (F2) and float -- they are rounded to FP32
+// there in any case, and the apply's error against 64 bits stays the same to its digits; or float
+// and float (MRA_PREC_TC_FAST).  3-D Poisson k = 8: 246 us in FP64 (87 % of its rate), 110 us in two
+// floats (issue slots), the operand preparation 59 us and 35 us.
 // k is fixed at compile time: padded arrays and triangular contractions.
-template <int KT, typename T>
-__global__ void k_ghost_refine_groups(Forest F, int ng, const uint64_t* gkeys, double* gblk, int32_t* err) {
+template <int KT, typename T, typename O>
+__global__ void __launch_bounds__(128, sizeof(O) == 4 ? 6 : 1) k_ghost_refine_groups(Forest F, int ng, const uint64_t* gkeys, O* gblk, int32_t* err) {
     extern __shared__ double sm_raw[];
     T* sm = (T*)sm_raw;
     constexpr int k = KT, k3 = k * k * k, kk = k * k;
@@ -570,7 +602,6 @@ __global__ void k_ghost_refine_groups(Forest F, int ng, const uint64_t* gkeys, d
     T* y = x + bs;             // 2 blocks: direction 3 by p3
     T* z = y + 2 * bs;         // 4 blocks: direction 2 by (p2, p3)
     auto at = [&](int e) { return (e / k) * (k + 1) + e % k; };  // element e of a block
-    auto mm = [&](const T* Mat, const T* in, T* out, int dim) { mode_mul_tri<KT, T>(Mat, in, out, dim); };
     const int j = (int)(key0 >> 58);
     const int tree = (int)((key0 >> 36) & ((1ull << GH_TREE_BITS) - 1));
     const uint64_t mk = key0 & ((1ull << 36) - 1);
@@ -583,24 +614,32 @@ __global__ void k_ghost_refine_groups(Forest F, int ng, const uint64_t* gkeys, d
     }
     __shared__ int anc, jj;
     __shared__ unsigned need;  // the octants of the group's ghosts
-    if (threadIdx.x == 0) {
-        unsigned mk8 = 1u << (key0 & 7ull);
-        for (int n = 1; g0 + n < ng && n < 8 && (gkeys[g0 + n] >> 3) == (key0 >> 3); ++n) mk8 |= 1u << (gkeys[g0 + n] & 7ull);
-        need = mk8;
-        anc = -1;
-        for (int lv = jp; lv >= 0 && anc < 0; --lv) {
-            const int sh = jp - lv;
-            const int idx = find_key_exact(F.key, off[lv], off[lv + 1], morton3(b1 >> sh, b2 >> sh, b3 >> sh));
-            if (idx >= 0) {
-                anc = idx;
-                jj = lv;
-            }
+    if (threadIdx.x < 32) {  // a lane per level and per sibling: the searches are chains of loads
+        const int lane = threadIdx.x;
+        const bool sib = lane < 8 && g0 + lane < ng && (gkeys[g0 + lane] >> 3) == (key0 >> 3);
+        const unsigned octs = __reduce_or_sync(0xffffffffu, sib ? 1u << (gkeys[g0 + lane] & 7ull) : 0u);
+        int idx = -1;
+        if (lane <= jp) {
+            const int sh = jp - lane;
+            idx = find_key_exact(F.key, off[lane], off[lane + 1], morton3(b1 >> sh, b2 >> sh, b3 >> sh));
         }
-        if (anc < 0 || !F.leaf[anc]) atomicExch(err, 3);
+        const unsigned found = __ballot_sync(0xffffffffu, idx >= 0);
+        const int lv = found ? 31 - __clz(found) : 0;
+        idx = __shfl_sync(0xffffffffu, idx, lv);
+        if (lane == 0) {
+            need = octs;
+            anc = found ? idx : -1;
+            jj = lv;
+            if (!found || !F.leaf[idx]) atomicExch(err, 3);
+        }
     }
     __syncthreads();
     if (anc < 0) return;
-    for (int e = threadIdx.x; e < k3; e += blockDim.x) x[at(e)] = (T)F.s[(size_t)anc * k3 + e];
+    for (int e = threadIdx.x; e < k3; e += blockDim.x) {
+        const double v = F.s[(size_t)anc * k3 + e];
+        if (sizeof(O) == 4 && fabs(v) > (double)FLT_MAX) atomicExch(err, 5);  // beyond FP32's range: refused
+        x[at(e)] = (T)v;
+    }
     if (jj < jp) {
         // P_d = H^(p_last)T ... H^(p_first)T along the path ancestor -> parent
         const int bd[3] = {b1, b2, b3};
@@ -613,7 +652,7 @@ __global__ void k_ghost_refine_groups(Forest F, int ng, const uint64_t* gkeys, d
             for (int e = threadIdx.x; e < 3 * kk; e += blockDim.x) {
                 const int d = e / kk, a = (e % kk) / k, i = e % k;
                 const T* H = HT + ((bd[d] >> (jp - lv - 1)) & 1) * kk;
-                T acc = 0;
+                T acc(0.0);
                 for (int c = 0; c < k; ++c) acc += H[a * k + c] * P[d * kk + c * k + i];
                 Q[e] = acc;
             }
@@ -621,32 +660,46 @@ __global__ void k_ghost_refine_groups(Forest F, int ng, const uint64_t* gkeys, d
             for (int e = threadIdx.x; e < 3 * kk; e += blockDim.x) P[e] = Q[e];
             __syncthreads();
         }
-        mm(P + 2 * kk, x, y, 2);
-        mm(P + kk, y, z, 1);
-        mm(P, z, x, 0);
+#pragma unroll 1
+        for (int d = 2; d >= 0; --d)  // (one copy of the code: two floats take 12 instructions a multiply-add)
+            mode_mul_tri<KT, T>(P + d * kk, d == 2 ? x : (d == 1 ? y : z), d == 2 ? y : (d == 1 ? z : x), d);
     } else {
         __syncthreads();
     }
     // the children, both of a direction from one set of products (child_pair): direction 3, then
     // 2, then 1 straight into the blocks that are needed
     constexpr int P1 = k + 1, S0 = k * P1;
-    for (int f = threadIdx.x; f < kk; f += blockDim.x) {
-        const int at0 = (f / k) * S0 + (f % k) * P1;
-        child_pair<k, T>(HT, x + at0, 1, y + at0, y + bs + at0, 1, true, true);
-    }
-    __syncthreads();
-    for (int f = threadIdx.x; f < 2 * kk; f += blockDim.x) {
-        const int p3 = f / kk, at0 = (f % kk / k) * S0 + f % k;
-        child_pair<k, T>(HT, y + p3 * bs + at0, P1, z + p3 * bs + at0, z + (2 + p3) * bs + at0, P1, true, true);
-    }
-    __syncthreads();
-    for (int f = threadIdx.x; f < 4 * kk; f += blockDim.x) {
-        const int q = f / kk, r = f % kk;  // q = 2 p2 + p3: octants q and 4 + q
-        const bool n0 = (need >> q) & 1u, n1 = (need >> (4 + q)) & 1u;
-        if (!n0 && !n1) continue;
-        double* d0 = gblk + (size_t)(g0 + __popc(need & ((1u << q) - 1u))) * k3 + r;
-        double* d1 = gblk + (size_t)(g0 + __popc(need & ((16u << q) - 1u))) * k3 + r;
-        child_pair<k, T>(HT, z + q * bs + (r / k) * P1 + r % k, S0, d0, d1, kk, n0, n1);
+#pragma unroll 1
+    for (int d = 0; d < 3; ++d) {
+        if (d) __syncthreads();
+        for (int f = threadIdx.x; f < kk << d; f += blockDim.x) {
+            const int q = f / kk, r = f % kk;  // d = 1: q = p3; d = 2: q = 2 p2 + p3, octants q and 4 + q
+            const T* src = d == 0 ? x + (r / k) * S0 + (r % k) * P1
+                                  : (d == 1 ? y + q * bs + (r / k) * S0 + r % k : z + q * bs + (r / k) * P1 + r % k);
+            const int st = d == 0 ? 1 : (d == 1 ? P1 : S0);
+            T *s0 = nullptr, *s1 = nullptr;
+            O *d0 = nullptr, *d1 = nullptr;
+            if (d == 0) {
+                s0 = y + (r / k) * S0 + (r % k) * P1;
+                s1 = s0 + bs;
+            } else if (d == 1) {
+                s0 = z + q * bs + (r / k) * S0 + r % k;
+                s1 = s0 + 2 * bs;
+            } else {
+                if ((need >> q) & 1u) d0 = gblk + (size_t)(g0 + __popc(need & ((1u << q) - 1u))) * k3 + r;
+                if ((need >> (4 + q)) & 1u) d1 = gblk + (size_t)(g0 + __popc(need & ((16u << q) - 1u))) * k3 + r;
+                if (!d0 && !d1) continue;
+            }
+            child_pair<k, T>(HT, src, st, [&](int a, T v0, T v1) {
+                if (d < 2) {
+                    s0[a * st] = v0;
+                    s1[a * st] = v1;
+                } else {
+                    if (d0) d0[a * kk] = (O)v0;
+                    if (d1) d1[a * kk] = (O)v1;
+                }
+            });
+        }
     }
 }
 
@@ -851,26 +904,28 @@ int screen_forest(const mra_op* op, const Forest& F, int unscreened, int what, c
     return MRA_OK;
 }
 
-template <typename T>
-static int ghost_refine_launch(const Forest& F, const ScreenOut& S, double* gblk, cudaStream_t st) {
-    const int k = F.k;
-    const size_t gsm = (8 * (size_t)k * k + 7 * (size_t)k * k * (k + 1)) * sizeof(T);  // padded blocks
-    using Fn = void (*)(Forest, int, const uint64_t*, double*, int32_t*);
-    static const Fn fns[] = {nullptr,
-                             k_ghost_refine_groups<1, T>, k_ghost_refine_groups<2, T>, k_ghost_refine_groups<3, T>,
-                             k_ghost_refine_groups<4, T>, k_ghost_refine_groups<5, T>, k_ghost_refine_groups<6, T>,
-                             k_ghost_refine_groups<7, T>, k_ghost_refine_groups<8, T>, k_ghost_refine_groups<9, T>,
-                             k_ghost_refine_groups<10, T>, k_ghost_refine_groups<11, T>, k_ghost_refine_groups<12, T>};
-    const Fn fn = fns[k];
-    MRA_CK(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gsm));
-    fn<<<S.nghost, 128, gsm, st>>>(F, S.nghost, S.gkeys, gblk, S.err + 1);
-    MRA_CK_LAUNCH();
-    return MRA_OK;
-}
+template <typename T, typename O>
+struct GhostKernel {
+    template <int K>
+    static int launch(const Forest& F, const ScreenOut& S, void* gblk, cudaStream_t st) {
+        constexpr size_t smem = (8 * (size_t)K * K + 7 * (size_t)K * K * (K + 1)) * sizeof(T);  // padded blocks
+        MRA_CK(cudaFuncSetAttribute(k_ghost_refine_groups<K, T, O>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        k_ghost_refine_groups<K, T, O><<<S.nghost, 128, smem, st>>>(F, S.nghost, S.gkeys, (O*)gblk, S.err + 1);
+        MRA_CK_LAUNCH();
+        return MRA_OK;
+    }
+};
 
-int ghost_refine_forest(const Forest& F, const ScreenOut& S, double* gblk, cudaStream_t st, bool fp32) {
+int ghost_refine_forest(const Forest& F, const ScreenOut& S, double* gblk, cudaStream_t st, GhostBlocks as) {
     if (S.nghost <= 0) return MRA_OK;
-    return fp32 ? ghost_refine_launch<float>(F, S, gblk, st) : ghost_refine_launch<double>(F, S, gblk, st);
+    using Fn = int (*)(const Forest&, const ScreenOut&, void*, cudaStream_t);
+    using G64 = GhostKernel<double, double>;
+    using G2 = GhostKernel<F2, float>;  // (the tensor cores' orders)
+    using G32 = GhostKernel<float, float>;
+#define FOR_TC_K(F) { nullptr, F<1>, F<2>, F<3>, F<4>, F<5>, F<6>, F<7>, F<8> }
+    static const Fn f64[] = FOR_EVERY_K(G64::launch), two[] = FOR_TC_K(G2::launch), f32[] = FOR_TC_K(G32::launch);
+#undef FOR_TC_K
+    return (as == GHOST_FP64 ? f64 : (as == GHOST_TWO_FLOATS ? two : f32))[F.k](F, S, gblk, st);
 }
 
 // Precision ladder budget per tree: single-FP16 terms may add at most
@@ -956,10 +1011,8 @@ int apply_impl(const mra_op* op, const mra_tree* f, const mra_apply_opts* o, cud
     MRA_TRY(dalloc(A, &gblk, (size_t)(S.nghost + 1) * k3));
     G.p[0] = gblk;
     // per-pair term ranges: the exact screen, or the learned one judged by it
-    // Step 2 in FP64 (a two-scale transform); MRA_PREC_TC_FAST refines in FP32 when the
-    // blocks only become FP16 hi/lo operands (rounding 2^-24, below the operands' 2^-22)
-    // and no screen decision reads them
-    MRA_TRY(ghost_refine_forest(F, S, gblk, st, prec == MRA_PREC_TC_FAST && smode == MRA_SCREEN_STATIC));
+    const GhostBlocks ghosts = ghost_blocks_of(prec, smode);
+    MRA_TRY(ghost_refine_forest(F, S, gblk, st, ghosts));
     unsigned long long* scounts = nullptr;
     int32_t* narrowed = nullptr;  // learned: 1 when some pair's range was narrowed
     if (smode != MRA_SCREEN_STATIC) {
@@ -1014,7 +1067,7 @@ int apply_impl(const mra_op* op, const mra_tree* f, const mra_apply_opts* o, cud
             G.p[3] = lpb;
             MRA_TRY(lp_budget(F, S, op->eps, lpb, st));
         }
-        MRA_TRY(launch_apply_tc(aa, S, groups ? &OP : nullptr, part, pairs, op, S.err + 1, lpb, nitems + 1,
+        MRA_TRY(launch_apply_tc(aa, S, ghosts, groups ? &OP : nullptr, part, pairs, op, S.err + 1, lpb, nitems + 1,
                                 o ? (unsigned)o->wait_limit : 0u, o ? (o->test_flags & MRA_TEST_WITHHOLD_MMA) : 0, st));
     } else if (!itemwise) {
         if (groups) MRA_TRY(oct_launch(OP, S, prec, (double*)part, g->s, st));

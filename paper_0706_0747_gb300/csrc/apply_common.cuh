@@ -235,12 +235,20 @@ int screen_forest(const mra_op* op, const Forest& F, int unscreened, int what, c
 void screen_release(const Alloc& A, ScreenOut* S);
 // Step 2 for every missing input block of a forest; fp32: refine in FP32 (for blocks that
 // only feed FP16 hi/lo tensor-core operands), else FP64
-int ghost_refine_forest(const Forest& F, const ScreenOut& S, double* gblk, cudaStream_t st, bool fp32 = false);
+// Step 2's blocks: FP64, or floats from arithmetic in two floats or one, in the same memory
+enum GhostBlocks { GHOST_FP64, GHOST_TWO_FLOATS, GHOST_FP32 };
+// floats where the blocks only become the tensor cores' FP16 operands and no screen reads them
+inline GhostBlocks ghost_blocks_of(int precision, int screen_mode) {
+    if (screen_mode != MRA_SCREEN_STATIC) return GHOST_FP64;
+    return precision == MRA_PREC_TC_SPLIT ? GHOST_TWO_FLOATS : (precision == MRA_PREC_TC_FAST ? GHOST_FP32 : GHOST_FP64);
+}
+int ghost_refine_forest(const Forest& F, const ScreenOut& S, double* gblk, cudaStream_t st, GhostBlocks as = GHOST_FP64);
 Forest forest_of_tree(const mra_tree* f);
 
 int tc_alloc(const mra_op* op, int nb, TcBuffers* B);            // nb: node + Step-2 blocks
 int tc_prep_F(const mra_op* op, const TcBuffers& B, cudaStream_t st);
-int tc_prep_blocks(int nb, int kr, int n, const double* s, const double* gblk, const TcBuffers& B, cudaStream_t st);
+int tc_prep_blocks(int nb, int kr, int n, const double* s, const double* gblk, GhostBlocks ghosts, const TcBuffers& B,
+                   cudaStream_t st);
 void tc_release(const mra_op* op, TcBuffers* B);
 int tc_configure();
 TcArgs tc_args(const ApplyArgs& A, const TcBuffers& B, int* err);
@@ -251,7 +259,7 @@ int tc3_launch(const TcArgs& T, cudaStream_t st);  // counter zeroed by the call
 int launch_apply_fact(const ApplyArgs& A, int precision, cudaStream_t st);
 OctTcArgs oct_tc_args(const OctArgs& P, const TcBuffers& B, int* err);
 // OP: the sibling groups (with their partial sums `part`) and / or the pair lists
-int launch_apply_tc(const ApplyArgs& A, const ScreenOut& S, const OctArgs* OP, void* part, bool pairs,
+int launch_apply_tc(const ApplyArgs& A, const ScreenOut& S, GhostBlocks ghosts, const OctArgs* OP, void* part, bool pairs,
                     const mra_op* op, int* err, const double* lpb, unsigned long long* n_lowp, unsigned wait_limit,
                     int withhold, cudaStream_t st);
 int lp_budget(const Forest& F, const ScreenOut& S, double eps, double* lpb, cudaStream_t st);

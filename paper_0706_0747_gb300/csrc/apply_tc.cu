@@ -61,7 +61,7 @@ namespace mra {
 // of s (b < n) or Step-2 block b - n.
 #define PREP_WARPS 8
 __global__ void __launch_bounds__(32 * PREP_WARPS) k_tc_prep_blocks(int nb, int kr, int n, const double* s,
-                                                                  const double* gblk, __half* xh, __half* xl,
+                                                                  const double* gblk, bool floats, __half* xh, __half* xl,
                                                                   float* sx, float* xmax, float* xnrm) {
     // warp per block: coalesced FP64 reads, each value rounded to FP32 once (the FP16
     // hi/lo pair keeps 22 bits of it; FP32 keeps 24), then FP32 arithmetic only -- the
@@ -73,13 +73,17 @@ __global__ void __launch_bounds__(32 * PREP_WARPS) k_tc_prep_blocks(int nb, int 
     float* x = xs[wl];
     for (int b = blockIdx.x * PREP_WARPS + wl; b < nb; b += gridDim.x * PREP_WARPS) {
         const double* src = b < n ? s + (size_t)b * k3 : gblk + (size_t)(b - n) * k3;
+        const float* src32 = b < n || !floats ? nullptr : (const float*)gblk + (size_t)(b - n) * k3;
         float s2 = 0.0f, m = 0.0f;
-        for (int e = lane; e < k3; e += 32) {
-            const float v = (float)src[e];
+        auto take = [&](int e, float v) {
             x[e] = v;
             m = fmaxf(m, fabsf(v));
             s2 = fmaf(v, v, s2);
-        }
+        };
+        if (src32)  // (apart, so that no conversion is issued for them)
+            for (int e = lane; e < k3; e += 32) take(e, src32[e]);
+        else
+            for (int e = lane; e < k3; e += 32) take(e, (float)src[e]);
         for (int o = 16; o > 0; o >>= 1) {
             m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
             s2 += __shfl_xor_sync(0xffffffffu, s2, o);
@@ -790,10 +794,11 @@ int tc_prep_F(const mra_op* op, const TcBuffers& B, cudaStream_t st) {
     return MRA_OK;
 }
 
-int tc_prep_blocks(int nb, int kr, int n, const double* s, const double* gblk, const TcBuffers& B, cudaStream_t st) {
+int tc_prep_blocks(int nb, int kr, int n, const double* s, const double* gblk, GhostBlocks ghosts, const TcBuffers& B,
+                   cudaStream_t st) {
     if (nb <= 0) return MRA_OK;
     const int grid = std::max(1, std::min(num_sms() * 8, (nb + PREP_WARPS - 1) / PREP_WARPS));
-    k_tc_prep_blocks<<<grid, 32 * PREP_WARPS, 0, st>>>(nb, kr, n, s, gblk, B.xh, B.xl, B.sx, B.xmax, B.xnrm);
+    k_tc_prep_blocks<<<grid, 32 * PREP_WARPS, 0, st>>>(nb, kr, n, s, gblk, ghosts != GHOST_FP64, B.xh, B.xl, B.sx, B.xmax, B.xnrm);
     MRA_CK_LAUNCH();
     return MRA_OK;
 }
@@ -870,7 +875,7 @@ OctTcArgs oct_tc_args(const OctArgs& P, const TcBuffers& B, int* err) {
     return Q;
 }
 
-int launch_apply_tc(const ApplyArgs& A, const ScreenOut& S, const OctArgs* OP, void* part, bool pairs,
+int launch_apply_tc(const ApplyArgs& A, const ScreenOut& S, GhostBlocks ghosts, const OctArgs* OP, void* part, bool pairs,
                     const mra_op* op, int* err, const double* lpb, unsigned long long* n_lowp, unsigned wait_limit,
                     int withhold, cudaStream_t st) {
     if (A.k > 8) {
@@ -886,7 +891,7 @@ int launch_apply_tc(const ApplyArgs& A, const ScreenOut& S, const OctArgs* OP, v
     const int nb = A.n + S.nghost;
     MRA_TRY(tc_alloc(op, nb, &G.B));
     MRA_TRY(tc_prep_F(op, G.B, st));
-    MRA_TRY(tc_prep_blocks(nb, A.k, A.n, A.s, A.gblk, G.B, st));
+    MRA_TRY(tc_prep_blocks(nb, A.k, A.n, A.s, A.gblk, ghosts, G.B, st));
     if (OP) {
         MRA_TRY(oct_tc_configure());
         OctTcArgs Q = oct_tc_args(*OP, G.B, err);
