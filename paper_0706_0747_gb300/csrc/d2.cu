@@ -433,7 +433,7 @@ static int build_tree2_impl(const mra_density* f, int k, double eps, int max_lev
 // levels in one launch after the scaling blocks.  k = 8: 1,250 FP64 operations a group for the
 // scaling block and as many for the norm, where the full filter matrix took 8,192 (12 us per
 // level, a block per node).
-#define W2_WARPS 4
+#define W2_WARPS 1
 
 // src (2 fibers' worth of K at stride st, the second half at src + h) -> y
 template <int K>
@@ -848,10 +848,10 @@ __global__ void k_schedule2(int M, int nlev, double eps, const double* w, const 
 // Planes of a level: 4 |t1| + |t2|, the core x core ones (|t| <= 1) with the terms that a leaf
 // keeps (J_m >= j); 16 + 2 |t1| + |t2| those ones with the terms an internal box keeps (J_m = j).
 #define D2_PLANES 20
-#define D2_Q 16   // entries of F^{t1} a block
-#define D2_MB 8   // terms staged at a time
+#define D2_Q 8     // entries of F^{t1} a block
+#define D2_MB 16   // terms staged at a time
 
-// One block per (level, plane |t1| <= |t2|, 16 entries (c1, i1)); thread (i2, c2), the 16 sums in
+// One block per (level, plane |t1| <= |t2|, D2_Q entries (c1, i1)); thread (i2, c2), the sums in
 // registers.  The plane with |t1| and |t2| exchanged is the same matrix with directions exchanged.
 // Layout [i][c]: the apply's threads read consecutive c.
 template <int K>
