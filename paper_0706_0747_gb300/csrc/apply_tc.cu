@@ -635,8 +635,8 @@ __global__ void __launch_bounds__(TC_THREADS, MC == 4 ? 4 : 3) k_apply_tc(TcArgs
                                 const float* v = vv[mc - mc_lo];
                                 const float c2 = s_c2[mc];
                                 uint32_t h0, l0, h1, l1;
-                                tc::split_h2(v[0] * c2, v[1] * c2, h0, l0);
-                                tc::split_h2(v[2] * c2, v[3] * c2, h1, l1);
+                                tc::split_scaled_h2(v[0], v[1], c2, h0, l0);
+                                tc::split_scaled_h2(v[2], v[3], c2, h1, l1);
                                 tc::stmatrix_x4_trans(a2_row_I + mc * L::A2_TERM, h0, l0, h1, l1);
                             }
                         }
@@ -686,8 +686,8 @@ __global__ void __launch_bounds__(TC_THREADS, MC == 4 ? 4 : 3) k_apply_tc(TcArgs
                                     const float* v = vv[mc - mc_lo];
                                     const float c3 = s_c3[mc];
                                     uint32_t h0, l0, h1, l1;
-                                    tc::split_h2(v[0] * c3, v[1] * c3, h0, l0);
-                                    tc::split_h2(v[2] * c3, v[3] * c3, h1, l1);
+                                    tc::split_scaled_h2(v[0], v[1], c3, h0, l0);
+                                    tc::split_scaled_h2(v[2], v[3], c3, h1, l1);
                                     tc::stmatrix_x4_trans(a2_row_II + mc * L::A2_TERM, h0, l0, h1, l1);
                                 }
                             }
