@@ -15,6 +15,27 @@ constexpr PieceTable make_pieces() {
     return T;
 }
 
+// every translation class (bit d of v: core in direction d) is in exactly one piece of A when A has
+// its number of core directions, in none otherwise
+constexpr bool pieces_cover_classes(int dims) {
+    for (int A = 0; A < 1 << (dims + 1); ++A) {
+        PieceSet P{};
+        piece_split(dims, A, 0, P);
+        for (int v = 0; v < 1 << dims; ++v) {
+            int S = 0, in = 0;
+            for (int d = 0; d < dims; ++d) S += (v >> d) & 1;
+            for (int i = 0; i < P.n; ++i) {
+                bool all = true;
+                for (int d = 0; d < dims; ++d) all = all && ((P.box[i] >> (2 * d)) & (((v >> d) & 1) ? 1 : 2));
+                in += all;
+            }
+            if (in != ((A >> S) & 1)) return false;
+        }
+    }
+    return true;
+}
+static_assert(pieces_cover_classes(3), "a term's pieces are its kept classes");
+
 static __constant__ PieceTable c_pieces = make_pieces();
 
 #define PIECE_CCC 0x15  // core in every direction
