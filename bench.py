@@ -53,9 +53,9 @@ FP64_TFLOPS = 1.25
 # DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) per launch of the
 # apply kernel on this workload, from one ncu capture of the current kernel
 # version; absent where no capture of the current kernel exists.
-TRAFFIC_BYTES = {"tc/static": 141.334272e6, "tc/pair": 97.992448e6}
-# k_apply2 on poisson2d (ncu, one launch): DRAM read + write
-TRAFFIC_D2 = 2.183936e6
+TRAFFIC_BYTES = {"tc/static": 150.528512e6, "tc/pair": 97.199008e6}
+# k_dense2 and k_apply2 on poisson2d (ncu, one launch each): DRAM read + write
+TRAFFIC_D2 = 8.620544e6
 
 
 class Clocks:
@@ -683,9 +683,10 @@ def d2_section(K, Wu, flush, stream, sample_nodes=120):
         ms.append(e0.elapsed_time(e1))
         apl.append(st["ms_apply"])
     k = cfg.k
-    flops_item = 4 * k ** 3
+    # what the sibling-group apply multiplies: 4 outputs x 12.25 k^4 per group, whatever the terms
+    flops_group = 2 * 49 * k ** 4
     ms_step, ms_apply = statistics.median(ms), statistics.median(apl)
-    achieved = st["n_items"] * flops_item / (ms_apply / 1e3) / 1e12
+    achieved = (1 + (t.n - 1) // 4) * flops_group / (ms_apply / 1e3) / 1e12
     # the oracle on a random sample of the same tree's output nodes
     c, l, b, _ = t.export()
     to = {tuple(int(v) for v in cc): OD.Node(bool(ll), bb.copy() if ll else None) for cc, ll, bb in zip(c, l, b)}
@@ -703,7 +704,7 @@ def d2_section(K, Wu, flush, stream, sample_nodes=120):
            "step2_refinements": st["n_ghosts"], "ms_per_step": ms_step, "ms_apply_kernel": ms_apply,
            "value": st["n_items"] / (ms_step / 1e3), "unit": "block-applies/s", "dtype": "f64",
            "roofline": {"bound": "alu", "achieved": achieved, "peak": FP64_TFLOPS, "unit": "TFLOP/s",
-                        "frac": achieved / FP64_TFLOPS, "flops_per_item": flops_item, "traffic": TRAFFIC_D2,
+                        "frac": achieved / FP64_TFLOPS, "flops_per_group": flops_group, "traffic": TRAFFIC_D2,
                         "traffic_unit": "bytes per launch (ncu)",
                         "peak_source": "nominal FP64 rate of the part"},
            "cpu_baseline": {"value": sto["n_items"] / cpu_s, "unit": "block-applies/s", "cores": 1, "kind": "oracle",

@@ -274,7 +274,10 @@ int mra_op_export(const mra_op* op, double* w_host, double* tau_host, double* F_
 #define MRA_PREC_TC_SPLIT 2   /* FP16 hi+lo split products on tcgen05 tensor   */
                               /* cores with FP32 accumulation (TMEM), each    */
                               /* chunk of terms added to the output block in  */
-                              /* FP64; Step-2 blocks refined in FP64          */
+                              /* FP64 (by sibling groups, static screen, in   */
+                              /* two floats); Step-2 blocks refined in FP64,  */
+                              /* under the static screen, where they are only */
+                              /* rounded to FP32, in two floats (48 bits)     */
 #define MRA_PREC_TC_LADDER 3  /* precision ladder on the tensor cores: per     */
                               /* output node and term, single FP16 products    */
                               /* (one MMA instead of three) when the term's    */
@@ -448,7 +451,8 @@ int mra_screen_data(const mra_op* op, const mra_tree* f, float* inputs, float* t
  * a stream the plan owns) and every execute launches that graph; `stream`
  * must not be capturing.  Executes on one plan must not overlap.
  * mra_plan_autotune (synchronous) times the tensor-core kernel variants on
- * the plan's worklist, reps launches each: (terms per chunk, CTAs per SM) in
+ * the plan's worklist (they concern the pair lists; a plan whose screen is static runs
+ * by sibling groups, the same for every variant), reps launches each: (terms per chunk, CTAs per SM) in
  * (8,3) (8,2) (4,3) (4,2) (4,4), node order as screened or heaviest first
  * (most pairs).  The fastest becomes the plan's variant (ms_variant[v],
  * v = pair index + 5 heavy_first); other precisions have one variant.
