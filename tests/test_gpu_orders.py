@@ -59,6 +59,28 @@ def test_multiply_every_order(k):
 
 
 @pytest.mark.parametrize("k", range(1, 13))
+def test_stored_wavelets_every_order(k):
+    """Blocks, norms and the inverse; a tree of one node has neither."""
+    for depth in (0, 3):
+        t, _ = OT.build_tree(OT.Density([1.0, 2.0], [30.0, 300.0], [[0.45, 0.5, 0.55], [0.8, 0.3, 0.2]]), k, 1e-2, depth,
+                             init_level=min(depth, 1))
+        tg = mra.tree_import(k, *oracle_to_arrays(t, k))
+        _, leaf, leaves, _ = tg.export()
+        mra.compress(tg, store_d=True)
+        OT.compress(t, k)
+        _, _, b, dn = tg.export()
+        bo = oracle_to_arrays(t, k)[2]
+        top = np.abs(bo).max()
+        assert np.abs(b - bo).max() <= 1e-12 * top
+        keys = [tuple(int(v) for v in c) for c in tg.export()[0]]
+        for key, d in zip(keys, dn):
+            if not t[key].leaf:
+                assert abs(d - t[key].dnorm) <= 1e-12 * top * k ** 1.5
+        mra.reconstruct(tg, mode="inverse")
+        assert np.abs(tg.export()[2] - leaves)[leaf != 0].max() <= 1e-12 * top
+
+
+@pytest.mark.parametrize("k", range(1, 13))
 def test_apply2_every_order(k):
     """Leaf and internal siblings in a group, inputs refined from one and several levels above."""
     dens = D.Density2([1.0, 0.7], [60.0, 3000.0], [[0.4, 0.55], [0.71, 0.27]])
