@@ -313,11 +313,6 @@ __host__ __device__ inline void gauss_legendre01_root(int n, int i, double* x, d
     w[idx] = LEGENDRE.w[at];
 }
 
-// all n nodes and weights, by one thread
-__host__ __device__ inline void gauss_legendre01(int n, double* x, double* w) {
-    for (int i = 0; i < n; ++i) gauss_legendre01_root(n, i, x, w);
-}
-
 // parity band of the modified ns-form: t_d in [-3, 2] (even a_d) or [-2, 3] (odd)
 __host__ __device__ inline int band_t(int a_d, int q) { return (a_d & 1) ? q - 2 : q - 3; }
 
