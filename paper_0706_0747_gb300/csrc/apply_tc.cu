@@ -89,7 +89,9 @@ __global__ void __launch_bounds__(32 * PREP_WARPS) k_tc_prep_blocks(int nb, int 
             s2 += __shfl_xor_sync(0xffffffffu, s2, o);
         }
         __syncwarp();
-        int e = 0;
+        // (a zero block takes the largest scale: an apply brings the blocks it reads to the smallest
+        // of their scales, and a zero among them must not decide it)
+        int e = -100;
         if (m > 0.0f) frexpf(m, &e);
         // m * scale in [2^9, 2^13): the exponent is rounded up to a multiple of 4,
         // so that neighbouring blocks mostly share a scale (and the stage-I B
