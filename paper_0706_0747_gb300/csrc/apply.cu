@@ -12,7 +12,6 @@
 //              the d = 0 half of eqs. recon_even / recon_odd
 //   apply      per output node: for each pair and kept term,
 //              ghat += w_m (F1 x F2 x F3) f_b as three mode products (Step 3)
-#include <cfloat>
 #include <math.h>
 
 #include <algorithm>
@@ -614,6 +613,7 @@ __global__ void __launch_bounds__(128, sizeof(O) == 4 ? 6 : 1) k_ghost_refine_gr
     }
     __shared__ int anc, jj;
     __shared__ unsigned need;  // the octants of the group's ghosts
+    __shared__ unsigned top;   // largest exponent of the ancestor's values (a double's high word)
     if (threadIdx.x < 32) {  // a lane per level and per sibling: the searches are chains of loads
         const int lane = threadIdx.x;
         const bool sib = lane < 8 && g0 + lane < ng && (gkeys[g0 + lane] >> 3) == (key0 >> 3);
@@ -628,6 +628,7 @@ __global__ void __launch_bounds__(128, sizeof(O) == 4 ? 6 : 1) k_ghost_refine_gr
         idx = __shfl_sync(0xffffffffu, idx, lv);
         if (lane == 0) {
             need = octs;
+            top = 0u;
             anc = found ? idx : -1;
             jj = lv;
             if (!found || !F.leaf[idx]) atomicExch(err, 3);
@@ -635,10 +636,47 @@ __global__ void __launch_bounds__(128, sizeof(O) == 4 ? 6 : 1) k_ghost_refine_gr
     }
     __syncthreads();
     if (anc < 0) return;
-    for (int e = threadIdx.x; e < k3; e += blockDim.x) {
-        const double v = F.s[(size_t)anc * k3 + e];
-        if (sizeof(O) == 4 && fabs(v) > (double)FLT_MAX) atomicExch(err, 5);  // beyond FP32's range: refused
-        x[at(e)] = (T)v;
+    // Float blocks: the arithmetic is on values scaled by a power of two into [0, 2), and a result
+    // takes its scale as it is stored.  So sums beyond FP32's range on the way are as in FP64, a result
+    // beyond it is stored infinite (the apply refuses it where it is read), and small blocks
+    // keep the low halves of their numbers.
+    O up0 = (O)1, up1 = (O)1;
+    {
+        constexpr int NV = (k3 + 127) / 128;
+        double v[NV];
+#pragma unroll
+        for (int r = 0; r < NV; ++r) {
+            const int e = threadIdx.x + 128 * r;
+            v[r] = e < k3 ? F.s[(size_t)anc * k3 + e] : 0.0;
+        }
+        int shift = 0;
+        if (sizeof(O) == 4) {
+            unsigned hi = 0u;
+#pragma unroll
+            for (int r = 0; r < NV; ++r) {
+                const unsigned x = (unsigned)__double2hiint(v[r]) & 0x7ff00000u;
+                if (x < 0x7ff00000u) hi = max(hi, x);
+                // out of FP32's range, as would be what comes of them
+                if (!(fabs(v[r]) < 0x1p252) && v[r] == v[r]) atomicExch(err, 5);
+            }
+            hi = __reduce_max_sync(0xffffffffu, hi);
+            if ((threadIdx.x & 31) == 0) atomicMax(&top, hi);
+            __syncthreads();
+            shift = top ? max((int)(top >> 20) - 1023, -252) : 0;
+            up0 = (O)ldexpf(1.0f, shift / 2);
+            up1 = (O)ldexpf(1.0f, shift - shift / 2);
+        }
+#pragma unroll
+        for (int r = 0; r < NV; ++r) {
+            const int e = threadIdx.x + 128 * r;
+            if (e >= k3) break;
+            if (sizeof(O) == 4) {  // v 2^-shift; what is below 2^-1022 of the largest is zero
+                const int hi = __double2hiint(v[r]), ex = (hi >> 20) & 0x7ff;
+                if (ex < 0x7ff)
+                    v[r] = ex && ex > shift ? __hiloint2double(hi - shift * (1 << 20), __double2loint(v[r])) : 0.0;
+            }
+            x[at(e)] = (T)v[r];
+        }
     }
     if (jj < jp) {
         // P_d = H^(p_last)T ... H^(p_first)T along the path ancestor -> parent
@@ -695,8 +733,8 @@ __global__ void __launch_bounds__(128, sizeof(O) == 4 ? 6 : 1) k_ghost_refine_gr
                     s0[a * st] = v0;
                     s1[a * st] = v1;
                 } else {
-                    if (d0) d0[a * kk] = (O)v0;
-                    if (d1) d1[a * kk] = (O)v1;
+                    if (d0) d0[a * kk] = (O)v0 * up0 * up1;
+                    if (d1) d1[a * kk] = (O)v1 * up0 * up1;
                 }
             });
         }

@@ -51,3 +51,31 @@ def test_zero_blocks_leave_small_inputs_whole(k, precision, screen):
         assert rel(out, one) <= (1e-6 if precision == "tc" else 1e-5), e
         if precision == "tc":
             assert rel(out, ref) <= 2e-6, e
+
+
+@pytest.mark.parametrize("precision", ["tc", "tc_fast"])
+def test_step2_at_the_edge_of_fp32(precision):
+    """A coarse leaf whose refinement (Step 2) passes FP32's range is refused, one close to it is not."""
+    k = 6
+    t, _ = OT.build_tree(OT.Density([1.0], [4000.0], [[0.51, 0.49, 0.26]]), k, 1e-4, 5, init_level=1)
+    c, leaf, b = oracle_to_arrays(t, k)
+    b /= np.abs(b).max()
+    op = mra.make_operator(0.0, 1.0, 1e-5, k, 5)
+    # a coarse leaf: the lowest entry of its children 110 and 111 is (0.71 + 0.61)^2 0.71 = 1.23 of `top`
+    i = int(np.flatnonzero(leaf)[0])
+    assert c[i, 0] < c[:, 0].max() - 1
+    for top, refused in ((1e30, False), (3.2e38, True)):
+        x = b * 1e-3 * top
+        x[i] = 0.0
+        x[i, :2, :2, 0] = top
+        tg = mra.tree_import(k, c, leaf, x)
+        mra.compress(tg)
+        ref, st = mra.apply_ns(op, tg, precision="fp64")
+        assert st["n_ghosts"] > 0
+        if refused:
+            with pytest.raises(mra.MraError) as e:
+                mra.apply_ns(op, tg, precision=precision)
+            assert e.value.code == mra.EINVAL and "FP32" in str(e.value)
+        else:
+            got = mra.apply_ns(op, tg, precision=precision)[0]
+            assert rel(got.export()[2], ref.export()[2]) <= 2e-6
