@@ -257,14 +257,14 @@ __global__ void __launch_bounds__(OTC_THREADS, 1) k_apply_oct_tc(OctTcArgs Q) {
                             frexpf(8192.0f / (48.0f * fm * fx), &e1);
                             frexpf(8192.0f / (2304.0f * fm * fm * fx), &e2);
                             const int eW = min(e1 - 1 - em - ex, 126), eV = min(e2 - 1 - 2 * em - ex, 126);
-                            if (eW >= -126 && eV >= -126) {
-                                c2 = ldexpf(1.0f, eW - ef - es);            // sW / (sF sx)
-                                c3 = ldexpf(1.0f, eV - eW - ef);            // sV / (sW sF)
-                                fin = ldexpf((float)P.w[m], -(eV + ef));    // w_m / (sV sF)
-                                if (!(fin <= FLT_MAX)) {  // outputs beyond the FP32 range: refuse
-                                    atomicExch(Q.err, 5);
-                                    fin = 0.0f;
-                                }
+                            // (sW and sV themselves may pass FP32's range where the factors do not)
+                            const int a2 = eW - ef - es, a3 = eV - eW - ef;
+                            c2 = ldexpf(1.0f, a2);                  // sW / (sF sx)
+                            c3 = ldexpf(1.0f, a3);                  // sV / (sW sF)
+                            fin = ldexpf((float)P.w[m], -(eV + ef));  // w_m / (sV sF)
+                            if (min(a2, a3) < -126 || !(fin <= FLT_MAX)) {  // scales or outputs beyond the FP32 range: refuse
+                                atomicExch(Q.err, 5);
+                                fin = 0.0f;
                             }
                         }
                     }

@@ -288,14 +288,14 @@ __global__ void __launch_bounds__(TC3_THREADS, 2) k_apply_tc3(TcArgs T) {
                             frexpf(8192.0f / (48.0f * fm * fx), &e1);
                             frexpf(8192.0f / (2304.0f * fm * fm * fx), &e2);
                             const int eW = min(e1 - 1 - em - ex, 126), eV = min(e2 - 1 - 2 * em - ex, 126);
-                            if (eW >= -126 && eV >= -126) {
-                                c2 = ldexpf(1.0f, eW - ef - (s_exp_min - 1));  // sW / (sf sx_node)
-                                c3 = ldexpf(1.0f, eV - eW - ef);                // sV / (sW sf)
-                                fin = ldexpf((float)A.w[m], -(eV + ef));        // w_m / (sV sf)
-                                if (!(fin <= FLT_MAX)) {  // outputs beyond the FP32 range: refuse
-                                    atomicExch(T.err, 5);
-                                    fin = 0.0f;
-                                }
+                            // (sW and sV themselves may pass FP32's range where the factors do not)
+                            const int a2 = eW - ef - (s_exp_min - 1), a3 = eV - eW - ef;
+                            c2 = ldexpf(1.0f, a2);                  // sW / (sF sx)
+                            c3 = ldexpf(1.0f, a3);                  // sV / (sW sF)
+                            fin = ldexpf((float)A.w[m], -(eV + ef));  // w_m / (sV sF)
+                            if (min(a2, a3) < -126 || !(fin <= FLT_MAX)) {  // scales or outputs beyond the FP32 range: refuse
+                                atomicExch(T.err, 5);
+                                fin = 0.0f;
                             }
                         }
                     }

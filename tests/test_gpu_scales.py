@@ -79,3 +79,19 @@ def test_step2_at_the_edge_of_fp32(precision):
         else:
             got = mra.apply_ns(op, tg, precision=precision)[0]
             assert rel(got.export()[2], ref.export()[2]) <= 2e-6
+
+
+@pytest.mark.parametrize("precision,screen", [("tc", "static"), ("tc", "pair"), ("tc_ladder", "static")])
+def test_inputs_just_below_the_largest_float(precision, screen):
+    """A root block whose scales leave FP32's exponents while their ratios do not: every term counts."""
+    k = 4
+    op = mra.make_operator(0.0, 1.0, 1e-5, k, 0)
+    x = np.random.default_rng(5).uniform(-1e38, 1e38, (1, k, k, k))
+    for top in (1e37, 1.7e38, 3.39e38):
+        x[0, 0, 0, 0] = top
+        tg = mra.tree_import(k, np.zeros((1, 4), np.int32), np.ones(1, np.int32), x)
+        mra.compress(tg)
+        ref, st = mra.apply_ns(op, tg, precision="fp64", screen=screen)
+        got, stt = mra.apply_ns(op, tg, precision=precision, screen=screen)
+        assert stt["n_items"] == st["n_items"] > 0
+        assert rel(got.export()[2], ref.export()[2]) <= (2e-6 if precision == "tc" else 1e-5), top
