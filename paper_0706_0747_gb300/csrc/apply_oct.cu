@@ -200,7 +200,7 @@ struct OctCfg {
     static constexpr int FIT = 100 * 1024 / (PER * (int)sizeof(T));
     static constexpr int PC = FIT >= 4 ? 4 : (FIT >= 2 ? 2 : 1);
     static constexpr int NT = (4 * K2 + 31) / 32 * 32 < 64 ? 64 : (4 * K2 + 31) / 32 * 32;
-    static size_t smem(int M) { return (size_t)PC * PER * sizeof(T) + 216 * sizeof(int) + 4 * (size_t)M * sizeof(uint32_t); }
+    static size_t smem(int M) { return (size_t)PC * PER * sizeof(T) + 216 * sizeof(int) + OCT_TERM_PIECES * (size_t)M * sizeof(uint32_t); }
 };
 
 template <typename T, int K>

@@ -63,9 +63,9 @@ struct OtcSmem {
     static constexpr int TIN = Z + OTC_P * 128 + 128;          // per slot 216 int
     static constexpr int TG = TIN + 2 * 864;           // per slot 216 float
     static constexpr int LIST = TG + 2 * 864;          // pieces of the group being set up
-    static size_t bytes(int M) { return LIST + 4 * (size_t)M * sizeof(uint32_t); }
+    static size_t bytes(int M) { return LIST + OCT_TERM_PIECES * (size_t)M * sizeof(uint32_t); }
 };
-static_assert(OtcSmem::LIST + 4 * MRA_MAX_TERMS * 4 + 2048 <= 232448, "shared memory of one CTA");
+static_assert(OtcSmem::LIST + OCT_TERM_PIECES * MRA_MAX_TERMS * 4 + 2048 <= 232448, "shared memory of one CTA");
 
 // a unit as its roles see it
 struct OtcUnit {

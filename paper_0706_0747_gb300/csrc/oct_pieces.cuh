@@ -36,12 +36,27 @@ constexpr bool pieces_cover_classes(int dims) {
 }
 static_assert(pieces_cover_classes(3), "a term's pieces are its kept classes");
 
+// most pieces of a term: its classes' products, or (J_m > j, leaf and internal siblings) those of the
+// classes but the core, and the core for the leaves.  {0, 2} beside the core takes five.
+constexpr int most_pieces() {
+    const PieceTable T = make_pieces();
+    int most = 0;
+    for (int A = 0; A < 16; ++A) {
+        const int n = (A & 8) && T.p[A & 7].n + 1 > T.p[A].n ? T.p[A & 7].n + 1 : T.p[A].n;
+        most = n > most ? n : most;
+    }
+    return most;
+}
+#define OCT_TERM_PIECES 5  // entries of a group's piece list per term
+static_assert(most_pieces() <= OCT_TERM_PIECES, "a group's pieces fit its list");
+
 static __constant__ PieceTable c_pieces = make_pieces();
 
 #define PIECE_CCC 0x15  // core in every direction
 
 // The pieces of a group at level j, by one warp: non-core pieces first, then the core
-// ones, each in increasing m.  out[i] = m | box << 16 | leaf_only << 24 (NULL: count only).
+// ones, each in increasing m.  out[i] = m | box << 16 | leaf_only << 24 (NULL: count only); at most
+// OCT_TERM_PIECES M of them.
 static __device__ int oct_pieces(const int32_t* sched, int M, int lm, int j, bool any_leaf, bool any_int, uint32_t* out) {
     const int lane = threadIdx.x & 31;
     const int32_t* m1 = sched + M + 4 * j;
