@@ -93,8 +93,8 @@ __global__ void __launch_bounds__(OTC_THREADS, 1) k_apply_oct_tc(OctTcArgs Q) {
     extern __shared__ __align__(1024) unsigned char sm[];
     __shared__ uint32_t s_tmem;
     // X full / empty, D_I full / empty; per pair: operands full, MMAs done; per slot: set up, done with;
-    // the pairs' sums written, read
-    __shared__ __align__(8) uint64_t b_xf[2], b_xe[2], b_df[2], b_de[2], b_af[4], b_ae[4], b_sf[2], b_se[2], b_y, b_yr;
+    // the pairs' sums written, read; the issuing warps' MMAs done (after a wait that gave up)
+    __shared__ __align__(8) uint64_t b_xf[2], b_xe[2], b_df[2], b_de[2], b_af[4], b_ae[4], b_sf[2], b_se[2], b_y, b_yr, b_end[5];
     __shared__ volatile int s_abort;
     __shared__ int s_unit, s_emin;
     __shared__ unsigned s_xmax;
@@ -116,6 +116,7 @@ __global__ void __launch_bounds__(OTC_THREADS, 1) k_apply_oct_tc(OctTcArgs Q) {
         }
         tc::mbar_init(&b_y, 16);
         tc::mbar_init(&b_yr, 16);
+        for (int i = 0; i < 5; ++i) tc::mbar_init(&b_end[i], 1);
         for (int i = 0; i < 4; ++i) {
             tc::mbar_init(&b_af[i], 4);
             tc::mbar_init(&b_ae[i], 1);
@@ -614,7 +615,15 @@ __global__ void __launch_bounds__(OTC_THREADS, 1) k_apply_oct_tc(OctTcArgs Q) {
 #undef OTC_ALL
     tc::fence_before();
     __syncthreads();
-    if (s_abort && tid == 0) atomicExch(Q.err, 4);
+    if (s_abort) {
+        if (tid == 0) atomicExch(Q.err, 4);
+        // a role stops where it stands: what the issuing warps have sent may still write tensor memory
+        if (warp >= 20 && warp <= 24) {
+            tc::commit_warp(&b_end[warp - 20]);
+            tc::mbar_wait(&b_end[warp - 20], 0, OTC_WAIT_MIN);
+        }
+        __syncthreads();
+    }
     if (warp == 0) tc::tmem_dealloc(tbase, 512);
 }
 
