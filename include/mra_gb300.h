@@ -311,9 +311,10 @@ typedef struct {
                             /* of Algorithm 3 (same items; for comparison)    */
     int screen_mode;        /* MRA_SCREEN_*                                   */
     int margin;             /* learned screen: terms added on each side        */
-    int wait_limit;         /* tensor-core apply: polls of one MMA completion  */
-                            /* wait before it gives up (MRA_ETIMEOUT); 0 means */
-                            /* the default 2^26                                */
+    int wait_limit;         /* tensor-core apply: polls (about 4 us each) of   */
+                            /* one completion wait before it gives up         */
+                            /* (MRA_ETIMEOUT), at least 4096; 0 means the      */
+                            /* default 2^20 (four seconds)                     */
     int test_flags;         /* 0 in normal use; MRA_TEST_WITHHOLD_MMA for the  */
                             /* test of the bounded wait                        */
     const mra_mlp* schedule;  /* learned screen: a 16 -> 12 network (mra_mlp_*) */

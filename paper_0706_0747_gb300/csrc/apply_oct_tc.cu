@@ -45,9 +45,6 @@ namespace mra {
 
 #define OTC_THREADS 896
 #define OTC_SETUP 96  // threads that set up units
-// polls of one completion wait (TC_SUSPEND_NS each at most)
-#define OTC_WAIT_LIMIT (1u << 20)
-#define OTC_WAIT_MIN 4096u
 #define OTC_P 8  // pieces per chunk
 
 struct OtcSmem {
@@ -620,7 +617,7 @@ __global__ void __launch_bounds__(OTC_THREADS, 1) k_apply_oct_tc(OctTcArgs Q) {
         // a role stops where it stands: what the issuing warps have sent may still write tensor memory
         if (warp >= 20 && warp <= 24) {
             tc::commit_warp(&b_end[warp - 20]);
-            tc::mbar_wait(&b_end[warp - 20], 0, OTC_WAIT_MIN);
+            tc::mbar_wait(&b_end[warp - 20], 0, TC_WAIT_MIN);
         }
         __syncthreads();
     }
@@ -639,7 +636,7 @@ int oct_slice_tc() { return OTC_P; }
 // oct_part_alloc(S, oct_slice_tc(), sizeof(float), ...).  oct_tc_configure() first.
 int oct_tc_launch(OctTcArgs Q, const ScreenOut& S, void* part, double* out, cudaStream_t st) {
     const int k = Q.P.k;
-    Q.wait_limit = Q.wait_limit ? std::max(Q.wait_limit, OTC_WAIT_MIN) : OTC_WAIT_LIMIT;
+    Q.wait_limit = tc::wait_polls(Q.wait_limit);
     Q.part = part;
     Q.P.ns = std::max(1, (S.max_pieces + OTC_P - 1) / OTC_P);
     const int per = oct_part_groups(S, OTC_P, sizeof(float), k);

@@ -42,10 +42,6 @@
 namespace mra {
 
 #define TC_THREADS 256
-// polls of one completion wait: the default, and the smallest accepted (far above the
-// time one group of MMAs takes)
-#define TC_WAIT_LIMIT (1u << 26)
-#define TC_WAIT_MIN 4096u
 // MMA-issuing threads (lane 0 of warps 0..TC_ISSUERS-1): warps 0-3 issue stages II and III
 // for a quarter of a chunk's terms each, warp 4 issues stage I; each commits to the mbarrier
 #define TC_ISSUERS 5
@@ -854,7 +850,7 @@ TcArgs tc_args(const ApplyArgs& A, const TcBuffers& B, int* err) {
     T.n_lowp = nullptr;
     T.Fh = B.Fh; T.Fl = B.Fl; T.sF = B.sF; T.maxF = B.maxF;
     T.err = err;  // the apply's error word: a wait that reaches its limit writes 4
-    T.wait_limit = TC_WAIT_LIMIT;
+    T.wait_limit = tc::wait_polls(0);
     T.withhold = 0;
     T.counter = B.counter;
     T.order = nullptr;
@@ -906,7 +902,7 @@ int launch_apply_tc(const ApplyArgs& A, const ScreenOut& S, GhostBlocks ghosts, 
     TcArgs T = tc_args(A, G.B, err);
     T.lpb = lpb;
     T.n_lowp = n_lowp;
-    T.wait_limit = wait_limit ? std::max(wait_limit, TC_WAIT_MIN) : TC_WAIT_LIMIT;
+    T.wait_limit = tc::wait_polls(wait_limit);
     T.withhold = withhold;
     return tc_launch(T, 8, 3, st);
 }

@@ -39,6 +39,16 @@ __device__ __forceinline__ void mbar_init(uint64_t* mbar, uint32_t count) {
     asm volatile("fence.mbarrier_init.release.cluster;");
 }
 
+// Polls of one completion wait, in every kernel: as the caller asked, at least TC_WAIT_MIN (far
+// above the time of the work that is waited for), or the default.  A poll that finds nothing takes
+// 3.8 us here (4,096 polls 15.5 ms in the group kernel, 16.0 in the pair-list one), so the default
+// is four seconds.
+#define TC_WAIT_MIN 4096u
+#define TC_WAIT_LIMIT (1u << 20)
+inline unsigned wait_polls(unsigned asked) {
+    return !asked ? TC_WAIT_LIMIT : (asked < TC_WAIT_MIN ? TC_WAIT_MIN : asked);
+}
+
 // Bounded wait for the given phase; returns false when the limit is reached.  A
 // poll that finds the phase incomplete puts the thread to sleep for TC_POLL_NS
 // nanoseconds before the next, so a waiting warp issues few instructions.
