@@ -41,6 +41,8 @@ struct mra_mlp {
     int64_t cap = 0;
     __half *h1 = nullptr, *h2 = nullptr, *h3 = nullptr;
     float *y = nullptr, *d3 = nullptr, *d2 = nullptr, *d1 = nullptr, *dy = nullptr;
+    float* part = nullptr;          // the row slices' weight gradients (room for part_n floats)
+    int64_t part_n = 0;
     double* loss = nullptr;
     mra::Alloc A;
 };
@@ -400,6 +402,26 @@ static int ensure_cap(mra_mlp* M, int64_t n) {
     return MRA_OK;
 }
 
+// Rows per slice for a batch of n, and where the slices' gradients go: a buffer that the network keeps,
+// as it keeps its activations (a block of the stream it was made on could reach another network
+// that trains on another stream); the gradient itself when there is one slice.  Fewer slices where
+// the allocator has no room for as many.
+static float* slice_room(mra_mlp* M, int64_t n, int* rows) {
+    for (int want = 64;; want /= 2) {
+        *rows = (int)std::max<int64_t>(32, ((n + want - 1) / want + 31) / 32 * 32);
+        const int64_t slices = (n + *rows - 1) / *rows;
+        if (slices == 1) return M->grad;
+        if (slices * M->np <= M->part_n) return M->part;
+        M->A.put(M->part);
+        M->part = nullptr;
+        M->part_n = 0;
+        if (dalloc(M->A, &M->part, slices * M->np) == MRA_OK) {
+            M->part_n = slices * M->np;
+            return M->part;
+        }
+    }
+}
+
 static MlpArgs mlp_args(const mra_mlp* M, const float* x, int64_t n, float* y) {
     MlpArgs A{};
     A.n = n;
@@ -441,7 +463,7 @@ static int mlp_loss_grad_impl(mra_mlp* M, const float* x, const float* t, int64_
     WgradArgs W{};
     W.n = n;
     W.np = M->np;
-    W.rows = (int)std::max<int64_t>(32, ((n + 63) / 64 + 31) / 32 * 32);
+    W.part = slice_room(M, n, &W.rows);
     const int slices = (int)((n + W.rows - 1) / W.rows);
     const float* d[4] = {M->d1, M->d2, M->d3, M->dy};
     const void* h[4] = {x, M->h1, M->h2, M->h3};
@@ -456,10 +478,9 @@ static int mlp_loss_grad_impl(mra_mlp* M, const float* x, const float* t, int64_
         W.tile0[l + 1] = W.tile0[l] + W.ti[l] * ((M->dout[l] + 127) / 128);
     }
     W.x16 = ((uintptr_t)x & 15) == 0;
-    Scratch tmp(M->A);
-    MRA_TRY(tmp.get(&W.part, (size_t)slices * M->np));
     k_mlp_wgrad<<<dim3(slices, W.tile0[4]), 256, 0, st>>>(W);
     MRA_CK_LAUNCH();
+    if (slices == 1) return MRA_OK;
     k_mlp_wsum<<<(unsigned)std::min<int64_t>(num_sms() * 4, (M->np + 255) / 256), 256, 0, st>>>(M->np, slices, W.part, M->grad);
     MRA_CK_LAUNCH();
     return MRA_OK;
@@ -624,6 +645,7 @@ int mra_mlp_free(mra_mlp* M) {
     const Alloc& A = M->A;
     A.put(M->master); A.put(M->grad); A.put(M->m); A.put(M->v); A.put(M->w16); A.put(M->loss);
     A.put(M->h1); A.put(M->h2); A.put(M->h3); A.put(M->y); A.put(M->d3); A.put(M->d2); A.put(M->d1); A.put(M->dy);
+    A.put(M->part);
     M->magic = 0;
     delete M;
     return MRA_OK;
