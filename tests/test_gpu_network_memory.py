@@ -16,6 +16,9 @@ if not torch.cuda.is_available():
 from paper_0706_0747_gb300 import mra  # noqa: E402
 
 
+HOOKS = []  # the library keeps blocks that were freed: a hook outlives its last handle
+
+
 class LimitAlloc:
     """torch caching-allocator hook that refuses blocks of more than `limit` bytes."""
 
@@ -33,6 +36,7 @@ class LimitAlloc:
 
         self._fa, self._ff = mra.ALLOC_FN(_alloc), mra.FREE_FN(_free)
         self.hook = mra.Alloc(self._fa, self._ff, None)
+        HOOKS.append(self)
 
 
 def batch(seed, rows=4096):
