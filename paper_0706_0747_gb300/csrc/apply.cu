@@ -1091,7 +1091,7 @@ int apply_impl(const mra_op* op, const mra_tree* f, const mra_apply_opts* o, cud
     if (groups) {
         OP = oct_args(aa, S, F);
         OP.skip = narrowed;
-        MRA_TRY(oct_part_alloc(S, tc ? oct_slice_tc() : oct_slice_simt(), tc ? sizeof(float) : sizeof(double), k, A, &part));
+        MRA_TRY(oct_part_alloc(&S, tc ? oct_slice_tc() : oct_slice_simt(), tc ? sizeof(float) : sizeof(double), k, A, &part));
         G.p[4] = part;
         MRA_TRY(oct_items(S, 1, narrowed, nitems, st));
     }

@@ -153,6 +153,7 @@ struct OctGroups {
     int32_t* np = nullptr;               // [n] pieces
     unsigned long long* pairs = nullptr; // [ntrees] static pairs and items (in ScreenOut's report)
     unsigned long long* items = nullptr;
+    int batch = 0;                       // groups a launch takes (oct_part_alloc)
 };
 
 // what a screen leaves: pair lists per output node, sibling groups, or both
@@ -222,8 +223,7 @@ int oct_place_ghosts(const ScreenOut& S, int n, cudaStream_t st);
 int oct_items(const ScreenOut& S, int ntrees, const int32_t* skip, unsigned long long* n_items, cudaStream_t st);
 OctArgs oct_args(const ApplyArgs& A, const ScreenOut& S, const Forest& F);
 int oct_slice_simt();
-int oct_part_alloc(const ScreenOut& S, int slice, size_t elem, int k, const Alloc& A, void** part);
-int oct_part_groups(const ScreenOut& S, int slice, size_t elem, int k);
+int oct_part_alloc(ScreenOut* S, int slice, size_t elem, int k, const Alloc& A, void** part);
 int oct_reduce(const OctArgs& P, int slice, int ng, const float* part, double* out, cudaStream_t st);
 int oct_tc_configure();
 int oct_slice_tc();

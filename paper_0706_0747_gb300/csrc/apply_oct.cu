@@ -413,19 +413,21 @@ OctArgs oct_args(const ApplyArgs& A, const ScreenOut& S, const Forest& F) {
     return P;
 }
 
-// partial sums of at most this many bytes are in flight; more groups run in batches
+// Partial sums of at most OCT_PART_BYTES are in flight; more groups run in batches.  Where the
+// allocator has no room for as many, batches shrink by halves, as long as they are of more than
+// OCT_PART_LEAST.
 #define OCT_PART_BYTES ((size_t)1 << 30)
+#define OCT_PART_LEAST ((size_t)64 << 20)
 
-int oct_part_groups(const ScreenOut& S, int slice, size_t elem, int k) {
-    const size_t per = (size_t)std::max(1, (S.max_pieces + slice - 1) / slice) * 8 * k * k * k * elem;
-    return (int)std::max<size_t>(1, std::min<size_t>((size_t)S.oct.n, OCT_PART_BYTES / per));
-}
-
-int oct_part_alloc(const ScreenOut& S, int slice, size_t elem, int k, const Alloc& A, void** part) {
+int oct_part_alloc(ScreenOut* S, int slice, size_t elem, int k, const Alloc& A, void** part) {
+    const size_t per = (size_t)std::max(1, (S->max_pieces + slice - 1) / slice) * 8 * k * k * k * elem;
+    size_t batch = std::max<size_t>(1, std::min<size_t>((size_t)S->oct.n, OCT_PART_BYTES / per));
     unsigned char* p;
-    const size_t per = (size_t)std::max(1, (S.max_pieces + slice - 1) / slice) * 8 * k * k * k * elem;
-    MRA_TRY(dalloc(A, &p, per * oct_part_groups(S, slice, elem, k)));
+    int rc;
+    while ((rc = dalloc(A, &p, per * batch)) == MRA_ENOMEM && batch > 1 && per * batch > OCT_PART_LEAST) batch = (batch + 1) / 2;
+    MRA_TRY(rc);
     *part = p;
+    S->oct.batch = (int)batch;
     return MRA_OK;
 }
 
@@ -437,7 +439,7 @@ static int oct_launch_k(OctArgs P, const ScreenOut& S, double* part, double* out
     MRA_CK(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     P.part = part;
     P.ns = std::max(1, (S.max_pieces + OCT_SLICE - 1) / OCT_SLICE);
-    const int per = oct_part_groups(S, OCT_SLICE, sizeof(double), K);
+    const int per = S.oct.batch;
     for (int g0 = 0; g0 < S.oct.n; g0 += per) {
         const int ng = std::min(per, S.oct.n - g0);
         P.g0 = g0;

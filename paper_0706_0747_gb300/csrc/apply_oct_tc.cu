@@ -635,11 +635,10 @@ int oct_slice_tc() { return OTC_P; }
 // Q.P, the operands, err, withhold and wait_limit (0: the default) set; part:
 // oct_part_alloc(S, oct_slice_tc(), sizeof(float), ...).  oct_tc_configure() first.
 int oct_tc_launch(OctTcArgs Q, const ScreenOut& S, void* part, double* out, cudaStream_t st) {
-    const int k = Q.P.k;
     Q.wait_limit = tc::wait_polls(Q.wait_limit);
     Q.part = part;
     Q.P.ns = std::max(1, (S.max_pieces + OTC_P - 1) / OTC_P);
-    const int per = oct_part_groups(S, OTC_P, sizeof(float), k);
+    const int per = S.oct.batch;
     for (int g0 = 0; g0 < S.oct.n; g0 += per) {
         const int ng = std::min(per, S.oct.n - g0);
         Q.P.g0 = g0;

@@ -291,7 +291,7 @@ static int plan_build(mra_plan* p, cudaStream_t st) {
         MRA_CK(cudaStreamSynchronize(st));  // `order` goes out of scope
     }
     if (p->groups)
-        MRA_TRY(oct_part_alloc(p->S, p->tc ? oct_slice_tc() : oct_slice_simt(), p->tc ? sizeof(float) : sizeof(double),
+        MRA_TRY(oct_part_alloc(&p->S, p->tc ? oct_slice_tc() : oct_slice_simt(), p->tc ? sizeof(float) : sizeof(double),
                                p->k, A, &p->part));
 
     if (p->tc) {

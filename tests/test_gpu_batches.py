@@ -1,0 +1,36 @@
+"""The sibling groups in batches: with room for the partial sums of a few groups at a time (an allocator that
+refuses large blocks) the results are bit for bit those of one launch, for an apply and a plan."""
+import numpy as np
+import pytest
+
+from paper_0706_0747_gb300 import workloads as W
+from tests.test_gpu_network_memory import LimitAlloc
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+if not torch.cuda.is_available():
+    pytest.skip("needs a CUDA GPU", allow_module_level=True)
+
+from paper_0706_0747_gb300 import mra  # noqa: E402
+
+DENS = dict(coef=[3.0, 1.2, 0.4], expo=[40.0, 400.0, 3000.0], centers=[[0.42, 0.55, 0.5], [0.8, 0.2, 0.9], [0.3, 0.31, 0.7]],
+            r2coef=[0.0, 0.0, 0.0])
+
+
+@pytest.mark.parametrize("precision,k", [("fp64", 6), ("fp32", 7), ("tc", 8)])
+def test_batches_of_groups(precision, k):
+    mra.release_cached()
+    out = []
+    for limit in (1 << 40, 60 << 20):
+        A = LimitAlloc(limit)
+        t, _ = mra.build_tree(W.Density(**DENS), k, 1e-5, 4, init_level=4 if precision == "tc" else 3, allocator=A.hook)
+        mra.compress(t)
+        op = mra.make_operator(0.0, 1.0, 1e-6, k, 4, allocator=A.hook)
+        g, st = mra.apply_ns(op, t, precision=precision)
+        plan = mra.plan_create(op, [t, t], precision=precision)
+        plan.execute()
+        out.append((st["n_items"], g.export()[2], plan.output(0).export()[2], plan.output(1).export()[2]))
+        assert (A.refused > 0) == (limit == 60 << 20)
+    for a, b in zip(*out):
+        assert np.array_equal(a, b)
