@@ -850,17 +850,18 @@ __global__ void k_schedule2(int M, int nlev, double eps, const double* w, const 
 #define D2_PLANES 20
 #define D2_Q 8     // entries of F^{t1} a block
 #define D2_MB 16   // terms staged at a time
+#define D2_LEAST ((size_t)1 << 20)
 
 // One block per (level, plane |t1| <= |t2|, D2_Q entries (c1, i1)); thread (i2, c2), the sums in
 // registers.  The plane with |t1| and |t2| exchanged is the same matrix with directions exchanged.
 // Layout [i][c]: the apply's threads read consecutive c.
 template <int K>
-__global__ void __launch_bounds__((K * K + 31) / 32 * 32) k_dense2(int M, int nlev, const double* F, const double* w,
+__global__ void __launch_bounds__((K * K + 31) / 32 * 32) k_dense2(int M, int nlev, int j0, const double* F, const double* w,
                                                                   const int32_t* sched, double* D) {
     constexpr int KK = K * K;
     constexpr int U1[13] = {0, 0, 0, 0, 1, 1, 1, 2, 2, 3, 0, 0, 1}, U2[13] = {0, 1, 2, 3, 1, 2, 3, 2, 3, 3, 0, 1, 1};
     __shared__ double f1[D2_MB][D2_Q], f2[D2_MB][KK];
-    const int j = blockIdx.x, q0 = blockIdx.z * D2_Q, tid = threadIdx.x, lane = tid & 31;
+    const int j = j0 + blockIdx.x, q0 = blockIdx.z * D2_Q, tid = threadIdx.x, lane = tid & 31;
     int u1 = 0, u2 = 0;
 #pragma unroll
     for (int p = 0; p < 13; ++p)
@@ -903,8 +904,8 @@ __global__ void __launch_bounds__((K * K + 31) / 32 * 32) k_dense2(int M, int nl
     }
     if (tid >= KK) return;
     const int i2 = tid / K, c2 = tid % K;
-    double* D0 = D + ((size_t)j * D2_PLANES + (inner ? 16 + 2 * u1 + u2 : 4 * u1 + u2)) * KK * KK;
-    double* D1 = D + ((size_t)j * D2_PLANES + (inner ? 16 + 2 * u2 + u1 : 4 * u2 + u1)) * KK * KK;
+    double* D0 = D + ((size_t)blockIdx.x * D2_PLANES + (inner ? 16 + 2 * u1 + u2 : 4 * u1 + u2)) * KK * KK;
+    double* D1 = D + ((size_t)blockIdx.x * D2_PLANES + (inner ? 16 + 2 * u2 + u1 : 4 * u2 + u1)) * KK * KK;
 #pragma unroll
     for (int q = 0; q < D2_Q; ++q) {
         if (q0 + q >= KK) break;
@@ -928,7 +929,7 @@ struct Apply2Smem {
 };
 
 template <int K>
-__global__ void __launch_bounds__(A2_NT) k_apply2(int M, int nlev, Offs2 off, const uint64_t* key,
+__global__ void __launch_bounds__(A2_NT) k_apply2(int M, int nlev, int j0, int g0, Offs2 off, const uint64_t* key,
                                                               const int32_t* coord, const int32_t* leaf, const double* s,
                                                               const double* D, const int32_t* sched,
                                                               const double* filt, double* gout, unsigned long long* counters) {
@@ -940,7 +941,7 @@ __global__ void __launch_bounds__(A2_NT) k_apply2(int M, int nlev, Offs2 off, co
     double* H = Z;             // H^(0), H^(1) while inputs are refined
     __shared__ int s_cnt[4], s_base[9], s_anc[9], s_lev[9], s_nout;
     __shared__ unsigned s_leaf, s_need[9];
-    const int tid = threadIdx.x, lane = tid & 31, g = blockIdx.x;
+    const int tid = threadIdx.x, lane = tid & 31, g = g0 + blockIdx.x;
     const int i0 = g == 0 ? 0 : 1 + 4 * (g - 1);
     const int j = coord[3 * i0], nout = j ? 4 : 1;
     const int p1 = coord[3 * i0 + 1] >> 1, p2 = coord[3 * i0 + 2] >> 1;
@@ -1063,7 +1064,7 @@ __global__ void __launch_bounds__(A2_NT) k_apply2(int M, int nlev, Offs2 off, co
         }
     }
     const int c = tid % KK, part = tid / KK, pc1 = (c / K) & 1, pc2 = (c % K) & 1;
-    const double* Dj = D + (size_t)j * D2_PLANES * KK * KK;
+    const double* Dj = D + (size_t)(j - j0) * D2_PLANES * KK * KK;
     const bool inner = s_cnt[3] > 0 && leafm != 0xfu;  // some internal output keeps core terms
     double y[4] = {0.0, 0.0, 0.0, 0.0};
 #pragma unroll 1
@@ -1140,16 +1141,19 @@ __global__ void __launch_bounds__(A2_NT) k_apply2(int M, int nlev, Offs2 off, co
     }
 }
 
+// levels j0 .. j1 - 1, whose matrices D holds
 template <int K>
-static int apply2_launch(int n, int M, int nlev, const Offs2& off, const mra_tree2* f, const mra_op* op, const int32_t* sched,
-                         double* D, double* gout, unsigned long long* counters, cudaStream_t st) {
+static int apply2_launch(int j0, int j1, int M, const mra_tree2* f, const mra_op* op, const int32_t* sched, double* D,
+                         double* gout, unsigned long long* counters, cudaStream_t st) {
     constexpr int KK = K * K;
     constexpr size_t bytes = Apply2Smem<K>::bytes;
-    k_dense2<K><<<dim3(nlev, 13, (KK + D2_Q - 1) / D2_Q), (KK + 31) / 32 * 32, 0, st>>>(M, nlev, op->F, op->w, sched, D);
+    Offs2 off;
+    memcpy(off.v, f->off, sizeof(off.v));
+    k_dense2<K><<<dim3(j1 - j0, 13, (KK + D2_Q - 1) / D2_Q), (KK + 31) / 32 * 32, 0, st>>>(M, f->nlev, j0, op->F, op->w, sched, D);
     MRA_CK_LAUNCH();
     MRA_CK(cudaFuncSetAttribute(k_apply2<K>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
-    k_apply2<K><<<1 + (n - 1) / 4, A2_NT, bytes, st>>>(M, nlev, off, f->key, f->coord, f->leaf, f->s, D, sched, f->filt, gout,
-                                                     counters);
+    const int g0 = (f->off[j0] + 3) / 4, ng = (f->off[j1] + 3) / 4 - g0;  // the root alone, then fours
+    k_apply2<K><<<ng, A2_NT, bytes, st>>>(M, f->nlev, j0, g0, off, f->key, f->coord, f->leaf, f->s, D, sched, f->filt, gout, counters);
     MRA_CK_LAUNCH();
     return MRA_OK;
 }
@@ -1173,8 +1177,14 @@ static int apply2_impl(const mra_op* op, const mra_tree2* f, cudaStream_t st, mr
     MRA_TRY(leaf_norm2(f, part, dv, st));
     double* ym;
     MRA_TRY(tmp.get(&ym, (size_t)M * kk));
+    // the matrices of all levels; of fewer at a time where the allocator has no room for them, as long
+    // as they take more than D2_LEAST bytes (k = 12: 3.3 MB a level)
     double* D;
-    MRA_TRY(tmp.get(&D, (size_t)nlev * D2_PLANES * kk * kk));
+    int per = nlev, rc;
+    while ((rc = tmp.get(&D, (size_t)per * D2_PLANES * kk * kk)) == MRA_ENOMEM && per > 1 &&
+           (size_t)per * D2_PLANES * kk * kk * sizeof(double) > D2_LEAST)
+        per = (per + 1) / 2;
+    MRA_TRY(rc);
     k_pilot2_terms<<<M, (kk + 31) / 32 * 32, 0, st>>>(k, op->w, op->F, f->s, ym);
     MRA_CK_LAUNCH();
     k_pilot2_sum<<<1, 640, 0, st>>>(kk, M, ym, dv);
@@ -1187,8 +1197,6 @@ static int apply2_impl(const mra_op* op, const mra_tree2* f, cudaStream_t st, mr
     MRA_TRY(tree2_clone_skeleton(f, &g));
     Tree2Guard tg{g};
     g->state = MRA_TREE_NSFORM;
-    Offs2 off;
-    memcpy(off.v, f->off, sizeof(off.v));
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     MRA_CK(cudaEventCreate(&e0));
     struct Ev {
@@ -1201,9 +1209,9 @@ static int apply2_impl(const mra_op* op, const mra_tree2* f, cudaStream_t st, mr
     } ev{e0, e1};
     MRA_CK(cudaEventCreate(&e1));
     MRA_CK(cudaEventRecord(e0, st));
-    using Fn = int (*)(int, int, int, const Offs2&, const mra_tree2*, const mra_op*, const int32_t*, double*, double*, unsigned long long*, cudaStream_t);
+    using Fn = int (*)(int, int, int, const mra_tree2*, const mra_op*, const int32_t*, double*, double*, unsigned long long*, cudaStream_t);
     static const Fn fn[] = FOR_EVERY_K(apply2_launch);
-    MRA_TRY(fn[k](n, M, nlev, off, f, op, sched, D, g->s, counters, st));
+    for (int j = 0; j < nlev; j += per) MRA_TRY(fn[k](j, std::min(nlev, j + per), M, f, op, sched, D, g->s, counters, st));
     MRA_CK(cudaEventRecord(e1, st));
     MRA_CK(cudaMemsetAsync(g->dnorm, 0, n * sizeof(double), st));
     unsigned long long hc[4];

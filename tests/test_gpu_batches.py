@@ -34,3 +34,20 @@ def test_batches_of_groups(precision, k):
         assert (A.refused > 0) == (limit == 60 << 20)
     for a, b in zip(*out):
         assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("k", [8, 12])
+def test_d2_level_by_level(k):
+    """d = 2 with room for the matrices of a few levels at a time (20 k^4 doubles a level)."""
+    dens = W.unit_mass2(np.array([300.0, 5000.0]), np.array([[0.4, 0.55], [0.71, 0.27]]))
+    out = []
+    for limit in (1 << 40, 8 << 20 if k == 12 else 3 << 20):
+        A = LimitAlloc(limit)
+        t, _ = mra.build_tree2(dens, k, 1e-5, 6, init_level=4, allocator=A.hook)
+        mra.compress2(t)
+        op = mra.make_operator2(0.0, 0.5, 1e-3, k, 6, allocator=None)
+        g, st = mra.apply_ns2(op, t)
+        out.append((st["n_items"], st["n_ghosts"], g.export()[2]))
+        assert (A.refused > 0) == (limit < 1 << 40)
+    for a, b in zip(*out):
+        assert np.array_equal(a, b)
