@@ -299,7 +299,7 @@ __device__ int dens_factors(const DensDev& D, int g0, const double* X, double rc
     constexpr int N = H * K, OCT = H == 2 ? 8 : 1;
     __shared__ int s_na;
     __shared__ float2 span[DG_CHUNK][3 * H];  // smallest and largest distance squared per direction and half
-    __shared__ float3 size[DG_CHUNK];         // |c| / cut, |b| / cut, a
+    __shared__ float3 size[DG_CHUNK];         // |c| / cut (negative: no term), |b| / cut, a
     const int tid = threadIdx.x, lane = tid & 31, ng = min(DG_CHUNK, D.n - g0);
     __syncthreads();
     for (int e = tid; e < ng * 3 * H; e += BuildSmem<K>::NT) {
@@ -310,10 +310,11 @@ __device__ int dens_factors(const DensDev& D, int g0, const double* X, double rc
         span[g][r] = make_float2(dn * dn, dx * dx);
     }
     for (int g = tid; g < ng; g += BuildSmem<K>::NT) {
-        const double c = fabs(D.coef[g0 + g]), r2 = fabs(D.r2[g0 + g]);
-        // (a term that is not a number reaches nothing)
-        size[g] = c == c && r2 == r2 ? make_float3((float)(c * rcut), (float)(r2 * rcut), (float)D.expo[g0 + g])
-                                     : make_float3(0.0f, 0.0f, 1.0f);
+        const double c = fabs(D.coef[g0 + g]), r2 = fabs(D.r2[g0 + g]), *p = D.cen + 3 * (g0 + g);
+        // a term that is not a number, or one that is zero in all of the cube, reaches nothing
+        const bool some = c == c && r2 == r2 && fabs(p[0]) < 1e150 && fabs(p[1]) < 1e150 && fabs(p[2]) < 1e150 &&
+                          isfinite(D.expo[g0 + g]);
+        size[g] = some ? make_float3((float)(c * rcut), (float)(r2 * rcut), (float)D.expo[g0 + g]) : make_float3(-1.0f, 0.0f, 0.0f);
     }
     __syncthreads();
     for (int e = tid; e < DG_CHUNK * OCT; e += BuildSmem<K>::NT) {  // (a multiple of 32: whole warps)
@@ -324,7 +325,7 @@ __device__ int dens_factors(const DensDev& D, int g0, const double* X, double rc
                          s3 = span[g][H == 2 ? 4 + (o & 1) : 2];
             const float3 z = size[g];
             // a dmin^2 <= log of the rest over the cut
-            on = !(z.z * (s1.x + s2.x + s3.x) > __logf(z.x + z.y * (s1.y + s2.y + s3.y)) + 1e-2f);
+            on = !(z.x < 0.0f) && !(z.z * (s1.x + s2.x + s3.x) > __logf(z.x + z.y * (s1.y + s2.y + s3.y)) + 1e-2f);
         }
         const unsigned b = __ballot_sync(0xffffffffu, on);
         if (o == 0) mask[e / OCT] = OCT == 1 ? (b >> lane) & 1u : (b >> lane) & 0xffu;
