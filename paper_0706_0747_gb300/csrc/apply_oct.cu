@@ -218,7 +218,7 @@ __global__ void __launch_bounds__(OctCfg<T, K>::NT) k_apply_oct(OctArgs P) {
     int* tin = (int*)(Fw + PC * 7 * K2);            // 216
     uint32_t* list = (uint32_t*)(tin + 216);
     __shared__ unsigned s_leaf;
-    __shared__ unsigned s_line[36];  // (b2, b3): the boxes b1 that are there
+    __shared__ unsigned s_lines[6];  // per plane b3 the lines b2 with an input box
     __shared__ float s_wh[PC], s_wl[PC];
     if (P.skip && *P.skip != P.run_if) return;
     const int g = P.g0 + blockIdx.x / P.ns, sl = blockIdx.x % P.ns, tid = threadIdx.x;
@@ -226,17 +226,17 @@ __global__ void __launch_bounds__(OctCfg<T, K>::NT) k_apply_oct(OctArgs P) {
     if (q0 >= np) return;
     const int i0 = P.first[g], tree = P.node_tree ? P.node_tree[i0] : 0;
     const int j = P.coord[4 * i0], nout = j ? 8 : 1;
-    for (int e = tid; e < 216; e += NT) tin[e] = P.in[(size_t)g * 216 + e];
+    if (tid < 6) s_lines[tid] = 0u;
+    __syncthreads();
+    for (int e = tid; e < 216; e += NT) {
+        const int in = P.in[(size_t)g * 216 + e];
+        tin[e] = in;
+        if (in >= 0) atomicOr(&s_lines[e % 6], 1u << ((e / 6) % 6));
+    }
     if (tid < 32) {
         const unsigned lf = __ballot_sync(0xffffffffu, tid < nout && P.leaf[i0 + (tid < nout ? tid : 0)]);
         if (tid == 0) s_leaf = lf;
         oct_pieces(P.sched + (size_t)tree * P.sl, P.M, P.lm, j, lf != 0, lf != (1u << nout) - 1u, list);
-    }
-    __syncthreads();
-    for (int e = tid; e < 36; e += NT) {
-        unsigned b = 0;
-        for (int b1 = 0; b1 < 6; ++b1) b |= (unsigned)(tin[b1 * 36 + e] >= 0) << b1;
-        s_line[e] = b;
     }
     __syncthreads();
     const unsigned leafm = s_leaf;
@@ -272,8 +272,7 @@ __global__ void __launch_bounds__(OctCfg<T, K>::NT) k_apply_oct(OctArgs P) {
         }
         for (int b3 = 0; b3 < 6; ++b3) {
             if (!((m3 >> b3) & 1u)) continue;
-            unsigned lines = 0;  // lines b2 with a box to read; a plane without one adds nothing
-            for (int b2 = 0; b2 < 6; ++b2) lines |= (unsigned)((m2 >> b2) & 1u && s_line[b2 * 6 + b3] & m1) << b2;
+            const unsigned lines = m2 & s_lines[b3];  // a plane without an input adds nothing
             if (!lines) continue;
             for (int a1p = 0; a1p < 2 / NA; ++a1p) {
                 __syncthreads();
