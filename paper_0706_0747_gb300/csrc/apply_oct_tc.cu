@@ -68,7 +68,8 @@ static_assert(OtcSmem::LIST + OCT_TERM_PIECES * MRA_MAX_TERMS * 4 + 2048 <= 2324
 struct OtcUnit {
     int unit;            // -1: no more units
     int npc, ps;         // pieces; positions (4 or 8) of a tile row
-    unsigned m1, m2, m3; // boxes the pieces read, per direction
+    int s1, s2;          // first box of the pieces' pairs of boxes per direction: 0, or 1 (core sets only)
+    unsigned m1, m2, m3; // boxes the pieces read, per direction, where the group has inputs
     int nout;
     unsigned leaf;       // leaf outputs
     uint32_t piece[OTC_P];
@@ -94,7 +95,7 @@ __global__ void __launch_bounds__(OTC_THREADS, 1) k_apply_oct_tc(OctTcArgs Q) {
     __shared__ __align__(8) uint64_t b_xf[2], b_xe[2], b_df[2], b_de[2], b_af[4], b_ae[4], b_sf[2], b_se[2], b_y, b_yr, b_end[5];
     __shared__ volatile int s_abort;
     __shared__ int s_unit, s_emin;
-    __shared__ unsigned s_xmax;
+    __shared__ unsigned s_xmax, s_there, s_reads;  // (boxes of directions 1, 2, 3 in bytes 0, 1, 2)
     __shared__ OtcUnit s_u[2];
     const OctArgs& P = Q.P;
     if (P.skip && *P.skip != P.run_if) return;
@@ -157,6 +158,7 @@ __global__ void __launch_bounds__(OTC_THREADS, 1) k_apply_oct_tc(OctTcArgs Q) {
                     s_unit = u;
                     s_emin = INT_MAX;
                     s_xmax = 0u;
+                    s_there = 0u;
                 }
                 sync();
                 unit = s_unit;
@@ -171,6 +173,7 @@ __global__ void __launch_bounds__(OTC_THREADS, 1) k_apply_oct_tc(OctTcArgs Q) {
 #pragma unroll
                 for (int r = 0; r < 3; ++r)
                     if (t + OTC_SETUP * r < 216) in[r] = P.in[(size_t)g * 216 + t + OTC_SETUP * r];
+                unsigned there = 0u;
 #pragma unroll
                 for (int r = 0; r < 3; ++r)
                     if (in[r] >= 0) {
@@ -179,7 +182,11 @@ __global__ void __launch_bounds__(OTC_THREADS, 1) k_apply_oct_tc(OctTcArgs Q) {
                         frexpf(sx[r], &e);
                         atomicMin(&s_emin, e);
                         atomicMax(&s_xmax, __float_as_uint(Q.xmax[in[r]]));  // non-negative floats order as ints
+                        const int q = t + OTC_SETUP * r;
+                        there |= 1u << (q / 36) | 256u << ((q / 6) % 6) | 65536u << (q % 6);
                     }
+                there = __reduce_or_sync(0xffffffffu, there);
+                if (lane == 0) atomicOr(&s_there, there);
                 if (warp == 25) {
                     const unsigned lf = __ballot_sync(0xffffffffu, lane < nout && P.leaf[i0 + (lane < nout ? lane : 0)]);
                     const int tree = P.node_tree ? P.node_tree[i0] : 0;
@@ -198,22 +205,30 @@ __global__ void __launch_bounds__(OTC_THREADS, 1) k_apply_oct_tc(OctTcArgs Q) {
                         U.unit = unit;
                         U.npc = npc;
                         U.ps = npc <= 4 ? 4 : 8;
-                        U.m1 = m1;
-                        U.m2 = m2;
-                        U.m3 = m3;
+                        U.s1 = m1 == 0x1e;
+                        U.s2 = m2 == 0x1e;
                         U.nout = nout;
                         U.leaf = lf;
+                        s_reads = m1 | m2 << 8 | m3 << 16;
                     }
                 }
                 sync();
                 const float xmax = __uint_as_float(s_xmax);
                 const int es = s_emin - 1;  // the common scale 2^es
                 if (!(xmax <= FLT_MAX) && t == 0) atomicExch(Q.err, 5);  // input values beyond FP32's range
-                if (!(xmax > 0.0f && xmax <= FLT_MAX)) {
+                // (boxes that only other chunks' pieces read do not count; planes and pairs of lines without
+                // an input are passed over by all roles)
+                const unsigned m = s_reads & s_there, m1 = m & 0xffu, m2 = (m >> 8) & 0xffu, m3 = m >> 16;
+                if (!(xmax > 0.0f && xmax <= FLT_MAX) || !m1 || !m2 || !m3) {
                     const int k3 = P.k * P.k * P.k;
                     for (int e = t; e < nout * k3; e += OTC_SETUP) ((float*)Q.part)[(size_t)unit * 8 * k3 + e] = 0.0f;
                     sync();
                     continue;
+                }
+                if (t == 0) {
+                    U.m1 = m1;
+                    U.m2 = m2;
+                    U.m3 = m3;
                 }
 #pragma unroll
                 for (int r = 0; r < 3; ++r)
@@ -286,8 +301,9 @@ __global__ void __launch_bounds__(OTC_THREADS, 1) k_apply_oct_tc(OctTcArgs Q) {
                 const int slot = k & 1;
                 ok = OTC_WAITW(&b_sf[slot], (k >> 1) & 1);
                 if (!ok || tc::uniform(s_u[slot].unit) < 0) break;
-                const unsigned m1 = tc::uniform(s_u[slot].m1), m2 = tc::uniform(s_u[slot].m2), m3 = tc::uniform(s_u[slot].m3);
-                const int s1 = m1 == 0x1e, s2 = m2 == 0x1e, n1 = 3 - s1, n2 = 3 - s2, ps = tc::uniform(s_u[slot].ps);
+                const unsigned m2 = tc::uniform(s_u[slot].m2), m3 = tc::uniform(s_u[slot].m3);
+                const int s1 = tc::uniform(s_u[slot].s1), s2 = tc::uniform(s_u[slot].s2), n1 = 3 - s1, n2 = 3 - s2;
+                const int ps = tc::uniform(s_u[slot].ps);
                 const uint32_t id = tc::idesc_f16(128, 16 * ps);
                 const uint64_t th = tc::sdesc(sbase + L::T + slot * 6 * L::TAB + s1 * ps * 128, ps * 128, 128);
                 int lines = 0;
@@ -326,7 +342,7 @@ __global__ void __launch_bounds__(OTC_THREADS, 1) k_apply_oct_tc(OctTcArgs Q) {
             ok = OTC_WAITW(&b_sf[slot], (k >> 1) & 1);
             if (!ok || s_u[slot].unit < 0) break;
             const unsigned m1 = s_u[slot].m1, m2 = s_u[slot].m2, m3 = s_u[slot].m3;
-            const int s1 = m1 == 0x1e, s2 = m2 == 0x1e, n1 = 3 - s1, n2 = 3 - s2;
+            const int s1 = s_u[slot].s1, s2 = s_u[slot].s2, n1 = 3 - s1, n2 = 3 - s2;
             const int* tin = (const int*)(sm + L::TIN + slot * 864);
             const float* tg = (const float*)(sm + L::TG + slot * 864);
             for (int b3 = 0; b3 < 6 && ok; ++b3) {
@@ -382,7 +398,7 @@ __global__ void __launch_bounds__(OTC_THREADS, 1) k_apply_oct_tc(OctTcArgs Q) {
             if (!ok || tc::uniform(s_u[slot].unit) < 0) break;
             const unsigned m2 = tc::uniform(s_u[slot].m2), m3 = tc::uniform(s_u[slot].m3);
             const int npc = tc::uniform(s_u[slot].npc), n = otc_pieces(g, npc);
-            const int s2 = m2 == 0x1e, n2 = 3 - s2;
+            const int s2 = tc::uniform(s_u[slot].s2), n2 = 3 - s2;
             const int ps = tc::uniform(s_u[slot].ps);
             const uint32_t tab = sbase + L::T + slot * 6 * L::TAB + (ps == 8 ? 2 * g : g) * 128;
             for (int b3 = 0; b3 < 6 && ok && n > 0; ++b3) {
@@ -454,7 +470,7 @@ __global__ void __launch_bounds__(OTC_THREADS, 1) k_apply_oct_tc(OctTcArgs Q) {
             const unsigned m2 = U.m2;
             const int npc = U.npc, nplane = __popc(U.m3), n = otc_pieces(g, npc);
             const int ps = U.ps;
-            const int s2 = m2 == 0x1e, n2 = 3 - s2;
+            const int s2 = U.s2, n2 = 3 - s2;
             int lpp = 0;  // lines per plane
             for (int q = 0; q < n2; ++q) lpp += ((m2 >> (s2 + 2 * q)) & 3u) != 0;
             float2 y[2][8];  // [a2'][(a3', c3)] of lane (a1', c1, c2), this pair's pieces
