@@ -87,11 +87,9 @@ struct mra_plan {
     unsigned long long* nitems = nullptr;  // per tree, then the single-FP16 items of all trees
     double* lpb = nullptr;                 // precision-ladder budgets per tree
     bool tc = false;
-    // Step 3 by sibling groups (apply_oct.cu), by the pair lists, or (learned screen) by the one
-    // that `narrowed` on the device asks for
+    // Step 3 by sibling groups (apply_oct.cu) or by the pair lists
     bool groups = false, pairs = true;
     void* part = nullptr;
-    int32_t* narrowed = nullptr;
     mra::TcBuffers tcb;
     int32_t* order_heavy = nullptr;
     // apply variant
@@ -122,8 +120,6 @@ static int plan_apply_args(const mra_plan* p, ApplyArgs* aa) {
     aa->Jm = p->S.sched; aa->node_tree = p->node_tree; aa->jm_stride = p->S.sl;
     aa->eta_blk = -1.0; aa->out = p->out; aa->n_items = p->nitems;
     aa->F = p->precision == MRA_PREC_FP64 ? (const void*)op->F : (const void*)op->F32;
-    aa->skip = p->narrowed;
-    aa->run_if = 1;
     return MRA_OK;
 }
 
@@ -133,11 +129,8 @@ static int plan_tc_launch(const mra_plan* p, int mc, int ctas, int ordered, cuda
     ApplyArgs aa;
     plan_apply_args(p, &aa);
     if (p->groups) {
-        OctArgs P = oct_args(aa, p->S, p->F);
-        P.skip = p->narrowed;
-        MRA_TRY(oct_tc_launch(oct_tc_args(P, p->tcb, p->S.err + 1), p->S, p->part, p->out, st));
+        return oct_tc_launch(oct_tc_args(oct_args(aa, p->S, p->F), p->tcb, p->S.err + 1), p->S, p->part, p->out, st);
     }
-    if (!p->pairs) return MRA_OK;
     TcArgs T = tc_args(aa, p->tcb, p->S.err + 1);
     T.order = ordered ? p->order_heavy : nullptr;
     T.lpb = p->lpb;
@@ -155,19 +148,15 @@ static int plan_enqueue(const mra_plan* p, cudaStream_t st) {
     const GhostBlocks ghosts = ghost_blocks_of(p->precision, p->screen_mode);
     MRA_TRY(ghost_refine_forest(p->F, p->S, p->gblk, st, ghosts));
     MRA_CK(cudaMemsetAsync(p->nitems, 0, ((size_t)p->ntrees + 1) * sizeof(unsigned long long), st));
-    if (p->groups) MRA_TRY(oct_items(p->S, p->ntrees, p->narrowed, p->nitems, st));
+    if (p->groups) MRA_TRY(oct_items(p->S, p->ntrees, nullptr, p->nitems, st));
     if (p->tc) {
         MRA_TRY(tc_prep_blocks(p->n + p->S.nghost, p->k, p->n, p->s, p->gblk, ghosts, p->tcb, st));
         MRA_TRY(plan_tc_launch(p, p->mc, p->ctas, p->use_order, st));
     } else {
         ApplyArgs aa;
         plan_apply_args(p, &aa);
-        if (p->groups) {
-            OctArgs P = oct_args(aa, p->S, p->F);
-            P.skip = p->narrowed;
-            MRA_TRY(oct_launch(P, p->S, p->precision, (double*)p->part, p->out, st));
-        }
-        if (p->pairs) MRA_TRY(launch_apply_fact(aa, p->precision, st));
+        if (p->groups) MRA_TRY(oct_launch(oct_args(aa, p->S, p->F), p->S, p->precision, (double*)p->part, p->out, st));
+        else MRA_TRY(launch_apply_fact(aa, p->precision, st));
     }
     return MRA_OK;
 }
@@ -188,7 +177,7 @@ static void plan_release(mra_plan* p) {
     if (p->op) tc_release(p->op, &p->tcb);
     A.put(p->tref); A.put(p->dbase); A.put(p->coord); A.put(p->leaf); A.put(p->off); A.put(p->node_tree);
     A.put(p->nlev); A.put(p->key); A.put(p->s); A.put(p->gblk); A.put(p->out); A.put(p->nitems);
-    A.put(p->order_heavy); A.put(p->lpb); A.put(p->part); A.put(p->narrowed);
+    A.put(p->order_heavy); A.put(p->lpb); A.put(p->part);
     p->magic = 0;
     delete p;
 }
@@ -254,20 +243,27 @@ static int plan_build(mra_plan* p, cudaStream_t st) {
         // screen, or the network's per-box ranges with every miss restored
         Scratch tmp(A);
         unsigned long long* counts;
-        MRA_TRY(tmp.get(&counts, 2));
-        MRA_CK(cudaMemsetAsync(counts, 0, 2 * sizeof(unsigned long long), st));
+        MRA_TRY(tmp.get(&counts, 3));  // misses, empty pairs, whether a pair was narrowed
+        MRA_CK(cudaMemsetAsync(counts, 0, 3 * sizeof(unsigned long long), st));
         MRA_TRY(ghost_refine_forest(F, p->S, p->gblk, st));
-        if (p->groups) {
-            MRA_TRY(dalloc(A, &p->narrowed, 1));
-            MRA_CK(cudaMemsetAsync(p->narrowed, 0, sizeof(int32_t), st));
-        }
         MRA_TRY(schedule_narrow(op, F, p->S, p->gblk, p->screen_mode == MRA_SCREEN_PAIR ? 1 : 2, p->schedule,
-                                p->margin, nullptr, nullptr, counts, p->narrowed, A, st));
-        unsigned long long hc[2] = {0, 0};
+                                p->margin, nullptr, nullptr, counts, (int32_t*)(counts + 2), A, st));
+        unsigned long long hc[3] = {0, 0, 0};
         MRA_CK(cudaMemcpyAsync(hc, counts, sizeof(hc), cudaMemcpyDeviceToHost, st));
         MRA_CK(cudaStreamSynchronize(st));
         p->n_misses = (long long)hc[0];
         p->n_pairs_empty = (long long)hc[1];
+        // a learned screen that narrowed no pair is the static schedule, by groups; what the other way
+        // would have used is given back
+        if (p->groups && hc[2]) {
+            p->groups = false;
+            oct_release(A, &p->S.oct);
+        } else if (p->groups) {
+            p->pairs = false;
+            A.put(p->S.count); A.put(p->S.pair_off); A.put(p->S.pairs);
+            p->S.count = p->S.pair_off = nullptr;
+            p->S.pairs = nullptr;
+        }
     }
     MRA_TRY(dalloc(A, &p->out, (size_t)n * k3));
     MRA_TRY(dalloc(A, &p->nitems, (size_t)nt + 1));
@@ -500,7 +496,7 @@ int mra_plan_get_info(const mra_plan* p, mra_plan_info* info, void* stream) {
     memset(info, 0, sizeof(*info));
     info->n_trees = p->ntrees;
     info->n_nodes = p->n;
-    info->n_pairs = p->S.npairs;
+    info->n_pairs = p->pairs ? p->S.npairs : 0;
     if (!p->pairs) {
         std::vector<unsigned long long> np(p->ntrees);
         MRA_CK(cudaMemcpyAsync(np.data(), p->S.oct.pairs, p->ntrees * sizeof(unsigned long long), cudaMemcpyDeviceToHost, st));

@@ -51,3 +51,34 @@ def test_d2_level_by_level(k):
         assert (A.refused > 0) == (limit < 1 << 40)
     for a, b in zip(*out):
         assert np.array_equal(a, b)
+
+
+def test_learned_plan_keeps_one_way():
+    """A plan whose network narrows pairs holds no more than a plan of the exact screen, and one whose network
+    keeps every term no more than a static one, but for the network's own."""
+    k = 6
+
+    def held(screen, logits=None):
+        mra.release_cached()
+        A = LimitAlloc(1 << 40)
+        t, _ = mra.build_tree(W.Density(**DENS), k, 1e-4, 4, init_level=2, allocator=A.hook)
+        mra.compress(t)
+        op = mra.make_operator(0.0, 1.0, 1e-5, k, 4)
+        net = None
+        if logits:
+            theta = np.zeros(mra.mlp_create().n_params, dtype=np.float32)
+            theta[-12:] = np.tile(logits, 4)
+            net = mra.mlp_create(params=theta)
+        plan = mra.plan_create(op, [t], precision="tc", use_graph=False, screen=screen, schedule=net, margin=0)
+        plan.execute()
+        out = plan.output(0).export()[2]
+        info = plan.info()
+        torch.cuda.synchronize()
+        mra.release_cached()  # what is cached, not held
+        size = A.held
+        return size, out, info["n_pairs"], info["n_items"]
+
+    pair, empty = held("pair"), held("learned", [10.0, 0.0, 0.0])
+    static, full = held("static"), held("learned", [-10.0, 0.0, 1.0])
+    for a, b in ((pair, empty), (static, full)):
+        assert b[0] <= a[0] and b[2:] == a[2:] and np.array_equal(a[1], b[1])

@@ -23,20 +23,27 @@ class LimitAlloc:
     """torch caching-allocator hook that refuses blocks of more than `limit` bytes."""
 
     def __init__(self, limit):
-        self.limit, self.refused = limit, 0
+        self.limit, self.refused, self.sizes = limit, 0, {}
 
         def _alloc(nbytes, stream, ctx):
             if nbytes > self.limit:
                 self.refused += 1
                 return None
-            return torch.cuda.caching_allocator_alloc(int(nbytes), torch.cuda.current_device(), stream or 0)
+            p = torch.cuda.caching_allocator_alloc(int(nbytes), torch.cuda.current_device(), stream or 0)
+            self.sizes[p] = int(nbytes)
+            return p
 
         def _free(ptr, stream, ctx):
+            self.sizes.pop(ptr)
             torch.cuda.caching_allocator_delete(ptr)
 
         self._fa, self._ff = mra.ALLOC_FN(_alloc), mra.FREE_FN(_free)
         self.hook = mra.Alloc(self._fa, self._ff, None)
         HOOKS.append(self)
+
+    @property
+    def held(self):
+        return sum(self.sizes.values())
 
 
 def batch(seed, rows=4096):
