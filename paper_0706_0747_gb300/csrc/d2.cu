@@ -430,10 +430,10 @@ static int build_tree2_impl(const mra_density* f, int k, double eps, int max_lev
 // their parents), a lane per fiber.  Both halves of the filter come from H^(0) by parity:
 // H^(1)_{ia} = (-1)^{i+a} H^(0)_{ia}, zero for a > i (the d = 3 transforms' identities).  The
 // wavelet norm is ||children - upsampled parent|| = ||d|| (the filter matrix is orthogonal), for all
-// levels in one launch after the scaling blocks.  k = 8: 1,250 FP64 operations a group for the
-// scaling block and as many for the norm, where the full filter matrix took 8,192 (12 us per
-// level, a block per node).
-#define W2_WARPS 1
+// levels in one launch, the last one, whose first block also computes the root's scaling block (a launch
+// of its own for the norms cost trees of two or three levels more than the rest saved: 5 boxes at
+// k = 8 21 us -> 29 a call, now 25).  k = 8: 1,250 FP64 operations a group for the scaling block and as many
+// for the norm, where the full filter matrix took 8,192 (12 us per level, a block per node).
 
 // src (2 fibers' worth of K at stride st, the second half at src + h) -> y
 template <int K>
@@ -472,21 +472,18 @@ __device__ __forceinline__ void up2_fiber(const double* H, const double* src, in
     }
 }
 
-// MODE 0: scaling block of the parent; 1: its wavelet norm; 2: children += upsampled parent
+// MODE 0: scaling block of the parent; 1: the parent's wavelet norm, the first group's scaling block
+// before it; 2: children += upsampled parent
 template <int K, int MODE>
-__global__ void __launch_bounds__(32 * W2_WARPS) k_scale2(int ng, int cbase, const int32_t* parent, double* s, double* dnorm,
-                                                          const double* filt) {
+__global__ void __launch_bounds__(32) k_scale2(int cbase, const int32_t* parent, double* s, double* dnorm, const double* filt) {
     constexpr int KK = K * K, K1 = K + 1;
     __shared__ double H[KK];
-    __shared__ double buf[W2_WARPS][2 * K * K1];
-    for (int e = threadIdx.x; e < KK; e += blockDim.x) H[e] = filt[e];
-    __syncthreads();
-    const int lane = threadIdx.x & 31, wl = threadIdx.x >> 5, g = blockIdx.x * W2_WARPS + wl;
-    if (g >= ng) return;
-    const int c0 = cbase + 4 * g, par = parent[c0];
-    double* t = buf[wl];  // (2k, k), rows padded
+    __shared__ double t[2 * K * K1];  // (2k, k), rows padded
+    const int lane = threadIdx.x, c0 = cbase + 4 * blockIdx.x, par = parent[c0];
+    for (int e = lane; e < KK; e += 32) H[e] = filt[e];
+    __syncwarp();
     double* ch = s + (size_t)c0 * KK;
-    if (MODE == 0) {
+    if (MODE == 0 || (MODE == 1 && blockIdx.x == 0)) {
         // direction 1: fiber of column c (0..2k-1) of the children's square, rows r of both halves
         if (lane < 2 * K) {
             double y[K];
@@ -501,7 +498,8 @@ __global__ void __launch_bounds__(32 * W2_WARPS) k_scale2(int ng, int cbase, con
 #pragma unroll
             for (int i = 0; i < K; ++i) s[(size_t)par * KK + lane * K + i] = y[i];
         }
-        return;
+        if (MODE == 0) return;
+        __syncwarp();
     }
     // direction 1 of the parent's block: column i2 -> rows 0..2k-1
     if (lane < K) {
@@ -538,15 +536,15 @@ __global__ void __launch_bounds__(32 * W2_WARPS) k_scale2(int ng, int cbase, con
 
 template <int K>
 static int compress2_t(mra_tree2* t, cudaStream_t st) {
-    for (int j = t->nlev - 2; j >= 0; --j) {
+    for (int j = t->nlev - 2; j >= 1; --j) {
         const int ng = (t->off[j + 2] - t->off[j + 1]) / 4;
         if (ng <= 0) continue;
-        k_scale2<K, 0><<<(ng + W2_WARPS - 1) / W2_WARPS, 32 * W2_WARPS, 0, st>>>(ng, t->off[j + 1], t->parent, t->s, t->dnorm, t->filt);
+        k_scale2<K, 0><<<ng, 32, 0, st>>>(t->off[j + 1], t->parent, t->s, t->dnorm, t->filt);
         MRA_CK_LAUNCH();
     }
     const int ng = (t->n - 1) / 4;
     if (ng > 0) {
-        k_scale2<K, 1><<<(ng + W2_WARPS - 1) / W2_WARPS, 32 * W2_WARPS, 0, st>>>(ng, 1, t->parent, t->s, t->dnorm, t->filt);
+        k_scale2<K, 1><<<ng, 32, 0, st>>>(1, t->parent, t->s, t->dnorm, t->filt);
         MRA_CK_LAUNCH();
     }
     return MRA_OK;
@@ -557,7 +555,7 @@ static int assemble2_t(mra_tree2* t, cudaStream_t st) {
     for (int j = 0; j + 1 < t->nlev; ++j) {
         const int ng = (t->off[j + 2] - t->off[j + 1]) / 4;
         if (ng <= 0) continue;
-        k_scale2<K, 2><<<(ng + W2_WARPS - 1) / W2_WARPS, 32 * W2_WARPS, 0, st>>>(ng, t->off[j + 1], t->parent, t->s, t->dnorm, t->filt);
+        k_scale2<K, 2><<<ng, 32, 0, st>>>(t->off[j + 1], t->parent, t->s, t->dnorm, t->filt);
         MRA_CK_LAUNCH();
     }
     return MRA_OK;
