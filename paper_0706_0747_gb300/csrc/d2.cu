@@ -843,9 +843,13 @@ __global__ void k_schedule2(int M, int nlev, double eps, const double* w, const 
 // terms (k = 8: 0.2 M; the terms one at a time, by separable sums shared by the four siblings, took
 // 33 K each, 1.1 M on the bench's quadtree: apply 1.69 ms, 2.7 ms an output box at a time).
 //
+// A level of 2^j boxes a direction has no translations beyond 2^j - 1: of levels 0 and 1 only the
+// planes within reach are formed and read.
+//
 // Planes of a level: 4 |t1| + |t2|, the core x core ones (|t| <= 1) with the terms that a leaf
 // keeps (J_m >= j); 16 + 2 |t1| + |t2| those ones with the terms an internal box keeps (J_m = j).
 #define D2_PLANES 20
+__device__ __forceinline__ int d2_reach(int j) { return j > 1 ? 3 : j; }  // largest |t| of a level
 #define D2_Q 8     // entries of F^{t1} a block
 #define D2_MB 16   // terms staged at a time
 #define D2_LEAST ((size_t)1 << 20)
@@ -864,6 +868,7 @@ __global__ void __launch_bounds__((K * K + 31) / 32 * 32) k_dense2(int M, int nl
 #pragma unroll
     for (int p = 0; p < 13; ++p)
         if ((int)blockIdx.y == p) u1 = U1[p], u2 = U2[p];
+    if (u2 > d2_reach(j)) return;  // (u1 <= u2)
     const bool inner = blockIdx.y >= 10;
     const int S = (u1 <= 1) + (u2 <= 1);
     const int lo = sched[M + 3 * j + S], hi = sched[M + 3 * nlev + 3 * j + S];
@@ -1066,7 +1071,7 @@ __global__ void __launch_bounds__(A2_NT) k_apply2(int M, int nlev, int j0, int g
     const bool inner = s_cnt[3] > 0 && leafm != 0xfu;  // some internal output keeps core terms
     double y[4] = {0.0, 0.0, 0.0, 0.0};
 #pragma unroll 1
-    for (int u1 = 0; u1 < 4; ++u1) {
+    for (int u1 = 0; u1 <= d2_reach(j); ++u1) {
         __syncthreads();
         for (int e = tid; e < 12 * KK; e += NT) {  // (a1, b2, i)
             const int a1 = e / (6 * KK), r = e % (6 * KK);
@@ -1076,7 +1081,7 @@ __global__ void __launch_bounds__(A2_NT) k_apply2(int M, int nlev, int j0, int g
             Y[12 * KK + e] = xp - xm;
         }
 #pragma unroll 1
-        for (int u2 = 0; u2 < 4; ++u2) {
+        for (int u2 = 0; u2 <= d2_reach(j); ++u2) {
             const int S = (u1 <= 1) + (u2 <= 1);
             if (!s_cnt[S]) continue;
             __syncthreads();
