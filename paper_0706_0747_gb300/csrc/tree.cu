@@ -1031,9 +1031,10 @@ __global__ void __launch_bounds__(SLICE_NT) k_up_slice(int cbase, const int32_t*
 // Wavelet norms of every internal node at once (after the scaling blocks of all
 // levels are in place): ||cube - (U x U x U) s_parent|| = ||d|| (the filter matrix is
 // orthogonal).  Block g takes the sibling group at 1 + 8 g -- the groups of all
-// levels in turn -- and its parent.
+// levels in turn -- and its parent; block 0 computes the root's scaling block first, which no other
+// block reads (one launch less, a third of the time on a tree of two levels).
 template <int K>
-__global__ void k_wnorm_all(const int32_t* parent, const double* s, double* dnorm, const double* filt) {
+__global__ void k_wnorm_all(const int32_t* parent, double* s, double* dnorm, const double* filt) {
     using L = TriSmem<K>;
     constexpr int K2 = 2 * K, K3 = K * K * K, P1 = L::P1, P2 = L::P2;
     extern __shared__ double sm[];
@@ -1053,9 +1054,17 @@ __global__ void k_wnorm_all(const int32_t* parent, const double* s, double* dnor
         const int x1 = ((o >> 2) & 1) * K + i1, x2 = ((o >> 1) & 1) * K + i2, x3 = (o & 1) * K + i3;
         cube[(x1 * K2 + x2) * P2 + x3] = s[(size_t)(c0 + o) * K3 + r];
     }
+    if (blockIdx.x == 0) {
+        __syncthreads();
+        fiber_stage<K2, K2, K2, K2 * P2, P2, 0, K, K2 * P2, P2, TRI_D, K>(cube, ra, D);
+        fiber_stage<K, K2, K2, K2 * P2, P2, 1, K, K * P2, P2, TRI_D, K>(ra, rb, D);
+        fiber_stage<K, K, K2, K * P2, P2, 2, K, K * P1, P1, TRI_D, K>(rb, sp, D);
+    }
     for (int e = threadIdx.x; e < K3; e += blockDim.x) {
         const int i1 = e / (K * K), i2 = (e / K) % K, i3 = e % K;
-        sp[(i1 * K + i2) * P1 + i3] = s[(size_t)i * K3 + e];
+        double& v = sp[(i1 * K + i2) * P1 + i3];
+        if (blockIdx.x == 0) s[(size_t)i * K3 + e] = v;
+        else v = s[(size_t)i * K3 + e];
     }
     __syncthreads();
     fiber_stage<K, K, K, K * P1, P1, 0, K2, K * P1, P1, TRI_U, K>(sp, ra, U);       // (2k, k, k)
@@ -1079,14 +1088,13 @@ __global__ void k_wnorm_all(const int32_t* parent, const double* s, double* dnor
     if (threadIdx.x == 0) dnorm[i] = sqrt(acc);
 }
 
+// the scaling blocks of the levels from the finest internal one up to `top`
 template <int K>
-static int compress_fast_t(mra_tree* t, bool norms, cudaStream_t st) {
-    // the scaling blocks level by level, then the wavelet norms of all internal nodes in
-    // one launch
+static int compress_levels_t(mra_tree* t, int top, cudaStream_t st) {
     using L = TriSmem<K>;
     const size_t smem = (size_t)(L::MATS + L::CUBE + L::RA + L::RB + L::SP) * sizeof(double);
     MRA_CK(cudaFuncSetAttribute(k_compress_fast_level_t<K>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    for (int j = t->nlev - 2; j >= 0; --j) {
+    for (int j = t->nlev - 2; j >= top; --j) {
         const int nparents = (t->off[j + 2] - t->off[j + 1]) / 8;
         if (nparents <= 0) continue;
         // a small level: each parent over k/2 blocks (up to the order whose cube fits their
@@ -1101,6 +1109,16 @@ static int compress_fast_t(mra_tree* t, bool norms, cudaStream_t st) {
             k_compress_fast_level_t<K><<<nparents, 256, smem, st>>>(t->off[j + 1], t->a.parent, t->s, t->filt);
         MRA_CK_LAUNCH();
     }
+    return MRA_OK;
+}
+
+// the scaling blocks level by level, then (with norms) the root's and the wavelet norms of all
+// internal nodes in one launch
+template <int K>
+static int compress_fast_t(mra_tree* t, bool norms, cudaStream_t st) {
+    using L = TriSmem<K>;
+    const size_t smem = (size_t)(L::MATS + L::CUBE + L::RA + L::RB + L::SP) * sizeof(double);
+    MRA_TRY(compress_levels_t<K>(t, norms ? 1 : 0, st));
     if (norms && t->n > 1) {
         MRA_CK(cudaFuncSetAttribute(k_wnorm_all<K>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
         k_wnorm_all<K><<<(t->n - 1) / 8, 256, smem, st>>>(t->a.parent, t->s, t->dnorm, t->filt);
@@ -1110,8 +1128,8 @@ static int compress_fast_t(mra_tree* t, bool norms, cudaStream_t st) {
 }
 
 template <int K>
-static int assemble_t(mra_tree* t, cudaStream_t st) {
-    for (int j = 0; j + 1 < t->nlev; ++j) {
+static int assemble_t(mra_tree* t, cudaStream_t st, int top) {
+    for (int j = top; j + 1 < t->nlev; ++j) {
         const int nparents = (t->off[j + 2] - t->off[j + 1]) / 8;
         if (nparents <= 0) continue;
         k_up_slice<K><<<dim3(nparents, (K + 1) / 2), 2 * nparents < num_sms() ? SLICE_NT : 128, 0, st>>>(t->off[j + 1], t->a.parent, t->s, t->filt);
@@ -1171,8 +1189,11 @@ struct CubeSmem {
 // blocks), and a level of 1, 8 or 48 parents took as long as one of 122, 44 us at k = 8 (a block
 // per parent): round trip of a 7,961-node tree 0.88 ms -> 0.75 ms.
 //
-// the children's cube -> the parent's wavelet cube and norm; BLOCK: and its block (the k^3 corner)
-template <int K, bool BLOCK>
+// The root's block needs no launch of its own: nothing else in these launches reads or writes it.
+//
+// the children's cube -> the parent's wavelet cube and norm; the first block (k = 12: every one) also
+// the parent's scaling block, the k^3 corner
+template <int K>
 __global__ void __launch_bounds__(256) k_compress_cube(int cbase, const int32_t* parent, double* s, double* dnorm,
                                                        double* dcube, const double* filt) {
     using L = CubeSmem<K>;
@@ -1196,14 +1217,15 @@ __global__ void __launch_bounds__(256) k_compress_cube(int cbase, const int32_t*
         const bool corner = x1 < K && x2 < K && x3 < K;
         const double v = cube[(x1 * K2 + x2) * P2 + x3];
         if (!corner) acc += v * v;
-        else if (BLOCK) s[(size_t)i * K3 + (x1 * K + x2) * K + x3] = v;
+        else if (K == 12 || blockIdx.x == 0) s[(size_t)i * K3 + (x1 * K + x2) * K + x3] = v;
         dcube[(size_t)i * N3 + e] = corner ? 0.0 : v;
     }
     acc = block_sum(acc, red);
     if (threadIdx.x == 0) dnorm[i] = sqrt(acc);
 }
 
-// inverse: the wavelet cube's part of its children's blocks (the parent's block adds its own later)
+// inverse: the wavelet cube's part of its children's blocks (the parent's block adds its own later; the
+// root's is part of the first cube)
 template <int K>
 __global__ void __launch_bounds__(256) k_expand_cube(const int32_t* parent, double* s, const double* dcube,
                                                      const double* filt) {
@@ -1216,7 +1238,8 @@ __global__ void __launch_bounds__(256) k_expand_cube(const int32_t* parent, doub
     for (int e = threadIdx.x; e < K * K; e += blockDim.x) Ht[(e % K) * K + e / K] = filt[e];
     for (int e = threadIdx.x; e < N3; e += blockDim.x) {
         const int x3 = e % K2, x2 = (e / K2) % K2, x1 = e / (K2 * K2);
-        cube[(x1 * K2 + x2) * P2 + x3] = dcube[(size_t)i * N3 + e];  // (its corner is zero)
+        const bool root = blockIdx.x == 0 && x1 < K && x2 < K && x3 < K;
+        cube[(x1 * K2 + x2) * P2 + x3] = root ? s[(x1 * K + x2) * K + x3] : dcube[(size_t)i * N3 + e];  // (corners are zero)
     }
     __syncthreads();
     for (int d = 0; d < 3; ++d) cube_fibers<K, true>(cube, W, Ht, d);
@@ -1231,21 +1254,19 @@ __global__ void __launch_bounds__(256) k_expand_cube(const int32_t* parent, doub
 template <int K>
 static int compress_cubes_t(mra_tree* t, cudaStream_t st) {
     constexpr size_t smem = CubeSmem<K>::BYTES;
+    if (t->n <= 1) return MRA_OK;
+    MRA_CK(cudaFuncSetAttribute(k_compress_cube<K>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     if constexpr (K < 12) {
-        MRA_TRY(compress_fast_t<K>(t, false, st));
-        if (t->n <= 1) return MRA_OK;
-        MRA_CK(cudaFuncSetAttribute(k_compress_cube<K, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        k_compress_cube<K, false><<<(t->n - 1) / 8, 256, smem, st>>>(1, t->a.parent, t->s, t->dnorm, t->dcube, t->filt);
+        MRA_TRY(compress_levels_t<K>(t, 1, st));
+        k_compress_cube<K><<<(t->n - 1) / 8, 256, smem, st>>>(1, t->a.parent, t->s, t->dnorm, t->dcube, t->filt);
         MRA_CK_LAUNCH();
-        return MRA_OK;
-    }
-    // (k = 12 has no such kernel for the blocks alone: level by level)
-    MRA_CK(cudaFuncSetAttribute(k_compress_cube<K, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    for (int j = t->nlev - 2; j >= 0; --j) {
-        const int nparents = (t->off[j + 2] - t->off[j + 1]) / 8;
-        if (nparents <= 0) continue;
-        k_compress_cube<K, true><<<nparents, 256, smem, st>>>(t->off[j + 1], t->a.parent, t->s, t->dnorm, t->dcube, t->filt);
-        MRA_CK_LAUNCH();
+    } else {  // (k = 12 has no kernel for the blocks alone: level by level)
+        for (int j = t->nlev - 2; j >= 0; --j) {
+            const int nparents = (t->off[j + 2] - t->off[j + 1]) / 8;
+            if (nparents <= 0) continue;
+            k_compress_cube<K><<<nparents, 256, smem, st>>>(t->off[j + 1], t->a.parent, t->s, t->dnorm, t->dcube, t->filt);
+            MRA_CK_LAUNCH();
+        }
     }
     return MRA_OK;
 }
@@ -1257,7 +1278,7 @@ static int expand_cubes_t(mra_tree* t, cudaStream_t st) {
     MRA_CK(cudaFuncSetAttribute(k_expand_cube<K>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     k_expand_cube<K><<<(t->n - 1) / 8, 256, smem, st>>>(t->a.parent, t->s, t->dcube, t->filt);
     MRA_CK_LAUNCH();
-    return assemble_t<K>(t, st);
+    return assemble_t<K>(t, st, 1);
 }
 
 int compress_impl(mra_tree* t, int mode, cudaStream_t st) {
@@ -1312,10 +1333,10 @@ int inverse_impl(mra_tree* t, cudaStream_t st) {
 
 int assemble_impl(mra_tree* t, cudaStream_t st) {
     const int k = t->k;
-    static int (*const up[])(mra_tree*, cudaStream_t) = {nullptr,       assemble_t<1>, assemble_t<2>,  assemble_t<3>,  assemble_t<4>,
+    static int (*const up[])(mra_tree*, cudaStream_t, int) = {nullptr,       assemble_t<1>, assemble_t<2>,  assemble_t<3>,  assemble_t<4>,
                                                          assemble_t<5>, assemble_t<6>, assemble_t<7>,  assemble_t<8>,  assemble_t<9>,
                                                          assemble_t<10>, assemble_t<11>, assemble_t<12>};
-    MRA_TRY(up[k](t, st));
+    MRA_TRY(up[k](t, st, 0));
     t->state = MRA_TREE_LEAVES;
     return MRA_OK;
 }
