@@ -311,9 +311,11 @@ __device__ int dens_factors(const DensDev& D, int g0, const double* X, double rc
     }
     for (int g = tid; g < ng; g += BuildSmem<K>::NT) {
         const double c = fabs(D.coef[g0 + g]), r2 = fabs(D.r2[g0 + g]), *p = D.cen + 3 * (g0 + g);
-        // a term that is not a number, or one that is zero in all of the cube, reaches nothing
-        const bool some = c == c && r2 == r2 && fabs(p[0]) < 1e150 && fabs(p[1]) < 1e150 && fabs(p[2]) < 1e150 &&
-                          isfinite(D.expo[g0 + g]);
+        // a term that is not a number, or one that is zero in all of the cube (centre beyond 2^498, no
+        // finite exponent), reaches nothing; by the numbers' exponents, FP64 comparisons being the bound
+        auto top = [](double v) { return __double2hiint(v) & 0x7ff00000; };
+        const bool some = c == c && r2 == r2 && max(max(top(p[0]), top(p[1])), top(p[2])) < 0x5f100000 &&
+                          top(D.expo[g0 + g]) < 0x7ff00000;
         size[g] = some ? make_float3((float)(c * rcut), (float)(r2 * rcut), (float)D.expo[g0 + g]) : make_float3(-1.0f, 0.0f, 0.0f);
     }
     __syncthreads();
