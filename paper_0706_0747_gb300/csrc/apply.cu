@@ -1041,7 +1041,7 @@ int apply_impl(const mra_op* op, const mra_tree* f, const mra_apply_opts* o, cud
     const int smode = o ? o->screen_mode : MRA_SCREEN_STATIC;
     // the static schedule's items run by sibling groups (apply_oct.cu); a learned screen that
     // narrows no pair is the static schedule, which the device decides
-    const bool groups = prec != MRA_PREC_TC_LADDER && !(o && (o->block_screen || o->itemwise)) && smode != MRA_SCREEN_PAIR;
+    bool groups = prec != MRA_PREC_TC_LADDER && !(o && (o->block_screen || o->itemwise)) && smode != MRA_SCREEN_PAIR;
     const bool pairs = !groups || smode != MRA_SCREEN_STATIC;
     MRA_TRY(screen_forest(op, F, unscreened, (pairs ? SCREEN_PAIRS : 0) | (groups ? SCREEN_GROUPS : 0), A, st, &S));
     MRA_CK(cudaEventRecord(ev[1], st));
@@ -1089,13 +1089,17 @@ int apply_impl(const mra_op* op, const mra_tree* f, const mra_apply_opts* o, cud
     OctArgs OP;
     void* part = nullptr;
     if (groups) {
+        const int have = oct_part_alloc(&S, tc ? oct_slice_tc() : oct_slice_simt(), tc ? sizeof(float) : sizeof(double), k, A, &part);
+        if (have == MRA_ENOMEM && pairs) groups = false;  // no room for both ways: the pair lists serve either
+        else MRA_TRY(have);
+    }
+    if (groups) {
         OP = oct_args(aa, S, F);
         OP.skip = narrowed;
-        MRA_TRY(oct_part_alloc(&S, tc ? oct_slice_tc() : oct_slice_simt(), tc ? sizeof(float) : sizeof(double), k, A, &part));
         G.p[4] = part;
         MRA_TRY(oct_items(S, 1, narrowed, nitems, st));
     }
-    aa.skip = narrowed;
+    aa.skip = groups ? narrowed : nullptr;
     aa.run_if = 1;
     if (tc) {
         // tcgen05 FP16 hi/lo split products (apply_oct_tc.cu, apply_tc.cu); with the ladder,

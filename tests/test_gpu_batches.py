@@ -53,6 +53,30 @@ def test_d2_level_by_level(k):
         assert np.array_equal(a, b)
 
 
+def constant_net(logits):
+    theta = np.zeros(mra.mlp_create().n_params, dtype=np.float32)
+    theta[-12:] = np.tile(logits, 4)
+    return mra.mlp_create(params=theta)
+
+
+def test_learned_apply_without_room_for_the_groups():
+    """The learned screen prepares the groups beside the pair lists; where they find no room the pair lists serve."""
+    k, out = 6, []
+    for limit in (1 << 40, 20 << 20):
+        mra.release_cached()
+        A = LimitAlloc(limit)
+        t, _ = mra.build_tree(W.Density(**DENS), k, 1e-5, 4, init_level=3, allocator=A.hook)
+        mra.compress(t)
+        op = mra.make_operator(0.0, 1.0, 1e-6, k, 4)
+        for logits in ([10.0, 0.0, 0.0], [-10.0, 0.0, 1.0]):  # every pair narrowed; none
+            g, st = mra.apply_ns(op, t, precision="fp64", screen="learned", schedule=constant_net(logits), margin=0)
+            out.append((st["n_items"], g.export()[2]))
+        assert (A.refused > 0) == (limit == 20 << 20)
+    assert [a[0] for a in out[:2]] == [a[0] for a in out[2:]]
+    assert np.array_equal(out[0][1], out[2][1])
+    assert np.abs(out[1][1] - out[3][1]).max() <= 1e-12 * np.abs(out[1][1]).max()
+
+
 def test_learned_plan_keeps_one_way():
     """A plan whose network narrows pairs holds no more than a plan of the exact screen, and one whose network
     keeps every term no more than a static one, but for the network's own."""
@@ -66,9 +90,7 @@ def test_learned_plan_keeps_one_way():
         op = mra.make_operator(0.0, 1.0, 1e-5, k, 4)
         net = None
         if logits:
-            theta = np.zeros(mra.mlp_create().n_params, dtype=np.float32)
-            theta[-12:] = np.tile(logits, 4)
-            net = mra.mlp_create(params=theta)
+            net = constant_net(logits)
         plan = mra.plan_create(op, [t], precision="tc", use_graph=False, screen=screen, schedule=net, margin=0)
         plan.execute()
         out = plan.output(0).export()[2]
