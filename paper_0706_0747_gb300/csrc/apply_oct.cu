@@ -189,9 +189,10 @@ int oct_items(const ScreenOut& S, int ntrees, const int32_t* skip, unsigned long
 //             output fibers a3 = 0, 1 stay in registers.
 // A slice's sum goes to its own place and k_oct_reduce adds a group's slices in order, so
 // the result does not depend on how the slices are scheduled.  Lines and planes without an input box
-// (outside the cube, or not needed) are passed over: they are most of a coarse level's 216, where
-// a box at a time had no work for them either (an FP64 apply of one box at k = 12: 8.97 ms with
-// them, 0.83 ms without; a box at a time 1.14 ms; 585 boxes at k = 8: 2.31 and 2.04 ms).
+// (outside the cube, or not needed) are passed over, and the outputs that a root does not have:
+// they are most of a coarse level's 216 inputs, where a box at a time had no work for them either (an
+// FP64 apply of one box at k = 12: 8.97 ms with them, 0.41 ms without; a box at a time 1.14 ms; of
+// 89 boxes at k = 8 2.00, 1.56 and 2.82 ms).
 template <typename T, int K>
 struct OctCfg {
     static constexpr int K2 = K * K, K3 = K2 * K;
@@ -203,11 +204,15 @@ struct OctCfg {
     static constexpr int FIT = 100 * 1024 / (PER * (int)sizeof(T));
     static constexpr int PC = FIT >= 4 ? 4 : (FIT >= 2 ? 2 : 1);
     static constexpr int NT = (4 * K2 + 31) / 32 * 32 < 64 ? 64 : (4 * K2 + 31) / 32 * 32;
+    // FP32 blocks come two to an SM, as their shared memory allows, also at k = 8, where the compiler takes
+    // 150 registers unless it is told (an apply to 585 boxes 419 us so, 367 with 128); the smaller
+    // orders stay below their limits by themselves (0: not stated)
+    static constexpr int MIN_BLOCKS = sizeof(T) == 4 && K == 8 ? 2 : 0;
     static size_t smem(int M) { return (size_t)PC * PER * sizeof(T) + 216 * sizeof(int) + OCT_TERM_PIECES * (size_t)M * sizeof(uint32_t); }
 };
 
 template <typename T, int K>
-__global__ void __launch_bounds__(OctCfg<T, K>::NT) k_apply_oct(OctArgs P) {
+__global__ void __launch_bounds__(OctCfg<T, K>::NT, OctCfg<T, K>::MIN_BLOCKS) k_apply_oct(OctArgs P) {
     using C = OctCfg<T, K>;
     constexpr int K2 = C::K2, K3 = C::K3, PC = C::PC, NT = C::NT, NA = C::NA;
     extern __shared__ __align__(16) unsigned char oct_sm[];
@@ -218,7 +223,7 @@ __global__ void __launch_bounds__(OctCfg<T, K>::NT) k_apply_oct(OctArgs P) {
     int* tin = (int*)(Fw + PC * 7 * K2);            // 216
     uint32_t* list = (uint32_t*)(tin + 216);
     __shared__ unsigned s_leaf;
-    __shared__ unsigned s_lines[6];  // per plane b3 the lines b2 with an input box
+    __shared__ __align__(8) unsigned s_there[12];  // input boxes: 64 bits per plane b3, bit 6 b2 + b1
     __shared__ float s_wh[PC], s_wl[PC];
     if (P.skip && *P.skip != P.run_if) return;
     const int g = P.g0 + blockIdx.x / P.ns, sl = blockIdx.x % P.ns, tid = threadIdx.x;
@@ -226,12 +231,12 @@ __global__ void __launch_bounds__(OctCfg<T, K>::NT) k_apply_oct(OctArgs P) {
     if (q0 >= np) return;
     const int i0 = P.first[g], tree = P.node_tree ? P.node_tree[i0] : 0;
     const int j = P.coord[4 * i0], nout = j ? 8 : 1;
-    if (tid < 6) s_lines[tid] = 0u;
-    __syncthreads();
-    for (int e = tid; e < 216; e += NT) {
-        const int in = P.in[(size_t)g * 216 + e];
-        tin[e] = in;
-        if (in >= 0) atomicOr(&s_lines[e % 6], 1u << ((e / 6) % 6));
+    for (int e = tid; e < 384; e += NT) {
+        const int b3 = e >> 6, b2 = (e & 63) / 6, b1 = (e & 63) % 6, q = b1 * 36 + b2 * 6 + b3;
+        const int in = b2 < 6 ? P.in[(size_t)g * 216 + q] : -1;
+        if (b2 < 6) tin[q] = in;
+        const unsigned there = __ballot_sync(0xffffffffu, in >= 0);
+        if ((e & 31) == 0) s_there[e >> 5] = there;
     }
     if (tid < 32) {
         const unsigned lf = __ballot_sync(0xffffffffu, tid < nout && P.leaf[i0 + (tid < nout ? tid : 0)]);
@@ -272,18 +277,23 @@ __global__ void __launch_bounds__(OctCfg<T, K>::NT) k_apply_oct(OctArgs P) {
         }
         for (int b3 = 0; b3 < 6; ++b3) {
             if (!((m3 >> b3) & 1u)) continue;
-            const unsigned lines = m2 & s_lines[b3];  // a plane without an input adds nothing
+            const unsigned long long there = *(const unsigned long long*)(s_there + 2 * b3);
+            unsigned lines = 0;  // lines b2 with a box to read; a plane without one adds nothing
+#pragma unroll
+            for (int b2 = 0; b2 < 6; ++b2) lines |= (unsigned)(((unsigned)(there >> (6 * b2)) & m1) != 0) << b2;
+            lines &= m2;
             if (!lines) continue;
-            for (int a1p = 0; a1p < 2 / NA; ++a1p) {
+            for (int a1p = 0; a1p < (j ? 2 / NA : 1); ++a1p) {
                 __syncthreads();
                 for (int task = tid; task < 6 * K2; task += NT) {
                     const int b2 = task / K2, r = task % K2;
                     if (!((lines >> b2) & 1u)) continue;
+                    const unsigned have = (unsigned)(there >> (6 * b2)) & m1;
                     T x[6][K];
 #pragma unroll
                     for (int b1 = 0; b1 < 6; ++b1) {
                         const int in = tin[b1 * 36 + b2 * 6 + b3];
-                        if (in >= 0 && ((m1 >> b1) & 1u)) {
+                        if ((have >> b1) & 1u) {
                             const double* src = (in < P.n ? P.s + (size_t)in * K3 : P.gblk + (size_t)(in - P.n) * K3) + r;
 #pragma unroll
                             for (int i = 0; i < K; ++i) x[b1][i] = (T)src[i * K2];
@@ -297,8 +307,9 @@ __global__ void __launch_bounds__(OctCfg<T, K>::NT) k_apply_oct(OctArgs P) {
                         const int box = (list[qb + pc] >> 16) & 0xff;
 #pragma unroll
                         for (int a = 0; a < NA; ++a) {
+                            if (a && !j) break;  // (the root alone has the one output 0, 0, 0)
                             T out[K];
-                            band_sum<T, K>(Ft + pc * 7 * K2, box >> 4, NA == 2 ? a : a1p, x, out);
+                            band_sum<T, K>(Ft + pc * 7 * K2, box >> 4, NA == 2 ? a : a1p, have, x, out);
                             T* dst = W + ((pc * NA + a) * 6 + b2) * C::WB + r;
 #pragma unroll
                             for (int c = 0; c < K; ++c) dst[c * C::W1] = out[c];
@@ -319,8 +330,9 @@ __global__ void __launch_bounds__(OctCfg<T, K>::NT) k_apply_oct(OctArgs P) {
                     }
 #pragma unroll
                     for (int a = 0; a < 2; ++a) {
+                        if (a && !j) break;
                         T out[K];
-                        band_sum<T, K>(Ft + pc * 7 * K2, set, a, x, out);
+                        band_sum<T, K>(Ft + pc * 7 * K2, set, a, boxes, x, out);
                         T* dst = V + (pa * 2 + a) * C::VB + c1 * K * C::V2 + i3;
 #pragma unroll
                         for (int c = 0; c < K; ++c) dst[c * C::V2] = out[c];
@@ -340,6 +352,7 @@ __global__ void __launch_bounds__(OctCfg<T, K>::NT) k_apply_oct(OctArgs P) {
 #pragma unroll
                         for (int a = 0; a < 2; ++a) {
                             const int t = a + 2 - b3;
+                            if (a && !j) break;
                             if (!(set & (band_core(a, b3) ? 1 : 2))) continue;
                             if (leaf_only && !((leafm >> (2 * oa + a)) & 1u)) continue;
                             const T* F = Fw + (pc * 7 + t + 3) * K2;
