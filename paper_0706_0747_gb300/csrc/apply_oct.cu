@@ -204,15 +204,14 @@ struct OctCfg {
     static constexpr int FIT = 100 * 1024 / (PER * (int)sizeof(T));
     static constexpr int PC = FIT >= 4 ? 4 : (FIT >= 2 ? 2 : 1);
     static constexpr int NT = (4 * K2 + 31) / 32 * 32 < 64 ? 64 : (4 * K2 + 31) / 32 * 32;
-    // FP32 blocks come two to an SM, as their shared memory allows, also at k = 8, where the compiler takes
-    // 150 registers unless it is told (an apply to 585 boxes 419 us so, 367 with 128); the smaller
-    // orders stay below their limits by themselves (0: not stated)
-    static constexpr int MIN_BLOCKS = sizeof(T) == 4 && K == 8 ? 2 : 0;
+    // lines without an input are passed over, planes always; not in FP32 at k = 8, where the test costs
+    // the second block of an SM (148 registers for 128: 64 Gaussians 3.86 -> 5.56 ms)
+    static constexpr bool BY_LINE = sizeof(T) == 8 || K != 8;
     static size_t smem(int M) { return (size_t)PC * PER * sizeof(T) + 216 * sizeof(int) + OCT_TERM_PIECES * (size_t)M * sizeof(uint32_t); }
 };
 
 template <typename T, int K>
-__global__ void __launch_bounds__(OctCfg<T, K>::NT, OctCfg<T, K>::MIN_BLOCKS) k_apply_oct(OctArgs P) {
+__global__ void __launch_bounds__(OctCfg<T, K>::NT) k_apply_oct(OctArgs P) {
     using C = OctCfg<T, K>;
     constexpr int K2 = C::K2, K3 = C::K3, PC = C::PC, NT = C::NT, NA = C::NA;
     extern __shared__ __align__(16) unsigned char oct_sm[];
@@ -245,6 +244,10 @@ __global__ void __launch_bounds__(OctCfg<T, K>::NT, OctCfg<T, K>::MIN_BLOCKS) k_
     }
     __syncthreads();
     const unsigned leafm = s_leaf;
+    // the boxes b1 of line (b2, b3) that are there, read where it is asked for: registers are short
+    auto line_boxes = [&](int b3, int b2) {
+        return (unsigned)(*(const unsigned long long*)(s_there + 2 * b3) >> (6 * b2)) & 63u;
+    };
     // this thread's output fibers (stage III): a1, a2, c1, c2; a3 = 0, 1
     const bool mine = tid < 4 * K2;
     const int oa = tid / K2, oc = tid % K2;  // a1 a2; c1 c2
@@ -277,23 +280,18 @@ __global__ void __launch_bounds__(OctCfg<T, K>::NT, OctCfg<T, K>::MIN_BLOCKS) k_
         }
         for (int b3 = 0; b3 < 6; ++b3) {
             if (!((m3 >> b3) & 1u)) continue;
-            const unsigned long long there = *(const unsigned long long*)(s_there + 2 * b3);
-            unsigned lines = 0;  // lines b2 with a box to read; a plane without one adds nothing
-#pragma unroll
-            for (int b2 = 0; b2 < 6; ++b2) lines |= (unsigned)(((unsigned)(there >> (6 * b2)) & m1) != 0) << b2;
-            lines &= m2;
-            if (!lines) continue;
+            if (!(s_there[2 * b3] | s_there[2 * b3 + 1])) continue;  // a plane without an input adds nothing
             for (int a1p = 0; a1p < (j ? 2 / NA : 1); ++a1p) {
                 __syncthreads();
                 for (int task = tid; task < 6 * K2; task += NT) {
                     const int b2 = task / K2, r = task % K2;
-                    if (!((lines >> b2) & 1u)) continue;
-                    const unsigned have = (unsigned)(there >> (6 * b2)) & m1;
+                    const unsigned have = line_boxes(b3, b2);
+                    if (!((m2 >> b2) & 1u) || (C::BY_LINE && !have)) continue;
                     T x[6][K];
 #pragma unroll
                     for (int b1 = 0; b1 < 6; ++b1) {
                         const int in = tin[b1 * 36 + b2 * 6 + b3];
-                        if ((have >> b1) & 1u) {
+                        if (in >= 0 && ((m1 >> b1) & 1u)) {
                             const double* src = (in < P.n ? P.s + (size_t)in * K3 : P.gblk + (size_t)(in - P.n) * K3) + r;
 #pragma unroll
                             for (int i = 0; i < K; ++i) x[b1][i] = (T)src[i * K2];
@@ -309,7 +307,7 @@ __global__ void __launch_bounds__(OctCfg<T, K>::NT, OctCfg<T, K>::MIN_BLOCKS) k_
                         for (int a = 0; a < NA; ++a) {
                             if (a && !j) break;  // (the root alone has the one output 0, 0, 0)
                             T out[K];
-                            band_sum<T, K>(Ft + pc * 7 * K2, box >> 4, NA == 2 ? a : a1p, have, x, out);
+                            band_sum<T, K>(Ft + pc * 7 * K2, box >> 4, NA == 2 ? a : a1p, have & m1, x, out);
                             T* dst = W + ((pc * NA + a) * 6 + b2) * C::WB + r;
 #pragma unroll
                             for (int c = 0; c < K; ++c) dst[c * C::W1] = out[c];
@@ -320,7 +318,11 @@ __global__ void __launch_bounds__(OctCfg<T, K>::NT, OctCfg<T, K>::MIN_BLOCKS) k_
                 for (int task = tid; task < npc * NA * K2; task += NT) {
                     const int pa = task / K2, r = task % K2, c1 = r / K, i3 = r % K, pc = pa / NA;
                     const int set = (list[qb + pc] >> 18) & 3;
-                    const unsigned boxes = set_boxes(set) & lines;
+                    unsigned boxes = set_boxes(set);  // of the lines that stage I has written
+                    if (C::BY_LINE)
+#pragma unroll
+                        for (int b2 = 0; b2 < 6; ++b2)
+                            if (!line_boxes(b3, b2)) boxes &= ~(1u << b2);
                     T x[6][K];
 #pragma unroll
                     for (int b2 = 0; b2 < 6; ++b2) {
