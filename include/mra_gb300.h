@@ -270,7 +270,9 @@ int mra_op_export(const mra_op* op, double* w_host, double* tau_host, double* F_
  * these are not checked. */
 
 #define MRA_PREC_FP64     0   /* FP64 SIMT contractions                        */
-#define MRA_PREC_FP32     1   /* FP32 SIMT contractions, FP64 accumulation     */
+#define MRA_PREC_FP32     1   /* FP32 SIMT contractions; terms added to the    */
+                              /* output block in FP64 by pairs, in two floats  */
+                              /* (48 bits) by sibling groups (static screen)   */
 #define MRA_PREC_TC_SPLIT 2   /* FP16 hi+lo split products on tcgen05 tensor   */
                               /* cores with FP32 accumulation (TMEM), each    */
                               /* chunk of terms added to the output block in  */

@@ -363,8 +363,9 @@ __global__ void __launch_bounds__(OctCfg<T, K>::NT) k_apply_oct(OctArgs P) {
                                 if (t != 0) half_mul<T, K, 1>(F, v, y[a]);
                                 continue;
                             }
-                            // FP32: y += w_m (F v) in two floats, as exact as the FP64 sum it replaces:
-                            // products split by fma, sums by Knuth's two-sum
+                            // FP32: y += w_m (F v) in two floats, products split by fma, sums by Knuth's
+                            // two-sum: about 48 bits (the low words add up in FP32), far below the
+                            // rounding of the 24-bit factors in F v
                             T acc[K];
 #pragma unroll
                             for (int c = 0; c < K; ++c) acc[c] = (T)0;
@@ -397,7 +398,7 @@ __global__ void __launch_bounds__(OctCfg<T, K>::NT) k_apply_oct(OctArgs P) {
 }
 
 // ghat of a group's outputs: its slices' sums in order.  FP32 slices are added in two floats
-// (Knuth's two-sum, as exact as FP64 for so few terms) and converted once: on this part FP64
+// (Knuth's two-sum: about 48 bits, where a slice has 24) and converted once: on this part FP64
 // additions and conversions run at 1/64 of the FP32 rate (120 us on 3-D Poisson k = 8 with an FP64
 // conversion and addition per slice).
 template <typename TP>

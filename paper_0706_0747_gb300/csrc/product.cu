@@ -36,7 +36,8 @@ __device__ double pot_eval(const PotDev& V, double x1, double x2, double x3) {
 // k-1-q are the sum and difference of its even and odd terms, and back the even coefficients read
 // the sums of the values and the odd ones their differences: half the multiplications.  FP64
 // operations are the bound (k = 8, a leaf: 6 x 64 fibers x 40 and 512 potential values): a thread
-// takes whole fibers.  164 us -> 123 us on the hydrogen iteration's tree.
+// takes whole fibers.  164 us -> 83 us on the hydrogen iteration's tree (123 us before the rule came as a
+// compile-time table).
 template <int K>
 __global__ void __launch_bounds__(128) k_tree_multiply(int n, const int32_t* coord, const int32_t* leaf, const double* s,
                                                        PotDev V, double scale, double* out) {
