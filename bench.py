@@ -53,9 +53,9 @@ FP64_TFLOPS = 1.25
 # DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) per launch of the
 # apply kernel on this workload, from one ncu capture of the current kernel
 # version; absent where no capture of the current kernel exists.
-TRAFFIC_BYTES = {"tc/static": 150.528512e6, "tc/pair": 97.199008e6}
+TRAFFIC_BYTES = {"tc/static": 151.167232e6, "tc/pair": 97.283840e6}
 # k_dense2 and k_apply2 on poisson2d (ncu, one launch each): DRAM read + write
-TRAFFIC_D2 = 8.620544e6
+TRAFFIC_D2 = 7.531008e6
 
 
 class Clocks:

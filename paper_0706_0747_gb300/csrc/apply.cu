@@ -582,7 +582,7 @@ __device__ __forceinline__ void child_pair(const T* HT, const T* src, int st, Pu
 // Arithmetic T and stored blocks O: double and double; where the blocks only become FP16 hi/lo
 // operands and no screen decision reads them, two floats (F2) and float -- they are rounded to FP32
 // there in any case, and the apply's error against 64 bits stays the same to its digits; or float
-// and float (MRA_PREC_TC_FAST).  3-D Poisson k = 8: 246 us in FP64 (87 % of its rate), 110 us in two
+// and float (MRA_PREC_TC_FAST).  3-D Poisson k = 8: 246 us in FP64 (87 % of its rate), 115 us in two
 // floats (issue slots), the operand preparation 59 us and 35 us.
 // k is fixed at compile time: padded arrays and triangular contractions.
 template <int KT, typename T, typename O>

@@ -233,9 +233,7 @@ int oct_launch(const OctArgs& P, const ScreenOut& S, int precision, double* part
 int screen_forest(const mra_op* op, const Forest& F, int unscreened, int what, const Alloc& A, cudaStream_t st,
                   ScreenOut* S);
 void screen_release(const Alloc& A, ScreenOut* S);
-// Step 2 for every missing input block of a forest; fp32: refine in FP32 (for blocks that
-// only feed FP16 hi/lo tensor-core operands), else FP64
-// Step 2's blocks: FP64, or floats from arithmetic in two floats or one, in the same memory
+// Step 2 for every missing input block of a forest.  Its blocks: FP64, or floats from arithmetic in two floats or one, in the same memory
 enum GhostBlocks { GHOST_FP64, GHOST_TWO_FLOATS, GHOST_FP32 };
 // floats where the blocks only become the tensor cores' FP16 operands and no screen reads them
 inline GhostBlocks ghost_blocks_of(int precision, int screen_mode) {

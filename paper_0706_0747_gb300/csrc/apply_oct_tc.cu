@@ -26,14 +26,16 @@
 //   24     issues stage I into one of two accumulators;
 //   25-27  set up the next unit (pieces, inputs, scales, F tiles) in the other of two slots.
 // A warp waits for itself: meeting at a named barrier behind one polling warp cost a conversion 200
-// to 300 cycles.  What bounds the kernel is shared memory, 76 % busy (half of it the tensor core's: an
-// MMA of stage II or III reads 4 KB of A for 32 or 16 columns), and issue slots, 60 %: the conversions'
-// share of them is why scaling and splitting use two-lane FP32.  3-D Poisson k = 8: 0.79 ms; 0.93 ms
+// to 300 cycles.  What bounds the kernel is shared memory, 75 % busy (half of it the tensor core's: an
+// MMA of stage II or III reads 4 KB of A for 32 or 16 columns), and issue slots, 59 %: the conversions'
+// share of them is why scaling and splitting use two-lane FP32.  3-D Poisson k = 8: 0.78 ms; 0.93 ms
 // with F_hi and F_lo as products of their own and barriers; 1.38 ms in the version whose units were set
 // up and finished by the whole CTA.  Stage I in halves of 4 pieces, or pieces instead of pairs as
 // the grain of conversions and MMAs, lose (0.86 and 1.07 ms): A is read or waited for twice.
+// Planes and pairs of lines without an input box (outside the cube, or not needed) are passed over: a
+// replayed plan of one box at k = 8 takes 45 us, 75 with them.
 // Every wait is bounded: one that reaches its limit makes all roles stop, the error word is set
-// to 4 and the kernel frees its tensor memory.
+// to 4, what was sent ends, and the kernel frees its tensor memory.
 #include <cfloat>
 #include <climits>
 
