@@ -404,10 +404,12 @@ static int ensure_cap(mra_mlp* M, int64_t n) {
 
 // Rows per slice for a batch of n, and where the slices' gradients go: a buffer that the network keeps,
 // as it keeps its activations (a block of the stream it was made on could reach another network
-// that trains on another stream); the gradient itself when there is one slice.  Fewer slices where
-// the allocator has no room for as many.
+// that trains on another stream); the gradient itself when there is one slice.  It is made for the
+// most slices at once, so that a larger batch does not give it back while an earlier step uses it.
+// Fewer slices where the allocator has no room for as many.
+#define MLP_SLICES 64
 static float* slice_room(mra_mlp* M, int64_t n, int* rows) {
-    for (int want = 64;; want /= 2) {
+    for (int want = MLP_SLICES;; want /= 2) {
         *rows = (int)std::max<int64_t>(32, ((n + want - 1) / want + 31) / 32 * 32);
         const int64_t slices = (n + *rows - 1) / *rows;
         if (slices == 1) return M->grad;
@@ -415,8 +417,9 @@ static float* slice_room(mra_mlp* M, int64_t n, int* rows) {
         M->A.put(M->part);
         M->part = nullptr;
         M->part_n = 0;
-        if (dalloc(M->A, &M->part, slices * M->np) == MRA_OK) {
-            M->part_n = slices * M->np;
+        const int64_t room = (want == MLP_SLICES ? want : slices) * M->np;
+        if (dalloc(M->A, &M->part, room) == MRA_OK) {
+            M->part_n = room;
             return M->part;
         }
     }
@@ -459,7 +462,7 @@ static int mlp_loss_grad_impl(mra_mlp* M, const float* x, const float* t, int64_
     A.loss = M->loss;
     MRA_CK(cudaMemsetAsync(M->loss, 0, sizeof(double), st));
     MRA_TRY(mlp_rows<true>(A, st));
-    // row slices: about an SM each for a 128 x 128 layer, at least 32 rows, at most 64 slices
+    // row slices: about an SM each for a 128 x 128 layer, at least 32 rows, at most MLP_SLICES
     WgradArgs W{};
     W.n = n;
     W.np = M->np;
